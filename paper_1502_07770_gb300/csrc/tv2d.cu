@@ -32,6 +32,7 @@
 
 #include "tv2d_common.cuh"
 #include "tv_launch.cuh"
+#include "tv_split_launch.h"
 
 using namespace tvk;
 using namespace tvh;
@@ -666,10 +667,46 @@ Tv2dWs carve_tv2d(void *base, long long H, long long W, int max_iters)
     return o;
 }
 
+// The phases on the threshold-splitting kernel (tv_split.cuh): rows or columns of the image.
+SplitSrc split_src(SplitMode mode, const float *img, const float *w, float lam, long long H,
+                   long long W, float *x0, const Tv2dWs &ws)
+{
+    SplitSrc src{};
+    SplitView &v = src.v;
+    const bool cols = mode == SPLIT_COL;
+    v.mode = mode;
+    v.cols = cols;
+    v.p0 = img;
+    v.p1 = ws.y;
+    if (cols) v.p2 = ws.y;
+    v.pw = w;
+    v.lam = lam;
+    v.ws = 1.f;
+    v.o0 = cols ? ws.y : x0;
+    v.o1 = ws.buf1;
+    v.stride = cols ? W : 1;
+    v.wrow = W - 1;
+    v.rec = ws.rec;
+    v.spill = ws.spill;
+    v.maxlen = (int)(cols ? H : W);
+    src.nchains = cols ? W : H;
+    src.len = (int)(cols ? H : W);
+    src.buf0 = x0;
+    src.buf1 = ws.buf1;
+    src.y = ws.y;
+    src.k = &ws.st->k;
+    src.done = &ws.st->done;
+    src.prm = ws.prm;
+    src.ticket = &ws.st->ticket_row;
+    return src;
+}
+
 template <bool HAS_WH>
 tv_status launch_init(const float *img, const float *wh, float lam, long long H, long long W,
                       float *x0, const Tv2dWs &ws, cudaStream_t s)
 {
+    if (split_takes(W, H, split_max_chains(W, false, false, wh != nullptr)))
+        return launch_split(split_src(SPLIT_INIT, img, wh, lam, H, W, x0, ws), ws.hdr, s, PK_INIT);
     if (H <= coop_max_chains()) {
         CoopInitRowsP<HAS_WH> p{img, ws.y, wh, lam, H, W, x0, ws.buf1};
         return launch_coop(p, H, (int)W, ws.rec, nullptr, ws.spill, ws.hdr, s, PK_INIT);
@@ -680,8 +717,13 @@ tv_status launch_init(const float *img, const float *wh, float lam, long long H,
 
 template <bool HAS_WH>
 tv_status launch_row(const float *img, const float *wh, float lam, long long H, long long W,
-                     float *x0, const Tv2dWs &ws, cudaStream_t s)
+                     int max_iters, float *x0, const Tv2dWs &ws, cudaStream_t s)
 {
+    if (split_takes(W, H, split_max_chains(W, false, false, wh != nullptr))) {
+        SplitSrc src = split_src(SPLIT_ROW, img, wh, lam, H, W, x0, ws);
+        src.max_iters = max_iters;
+        return launch_split(src, ws.hdr, s, PK_ROW);
+    }
     if (H <= coop_max_chains()) {
         CoopRowPhaseP<HAS_WH> p{img, ws.y, wh, lam, H, W, x0, ws.buf1, ws.st, ws.prm,
                                 nullptr, nullptr, 0.f, 0.f};
@@ -696,6 +738,8 @@ template <bool HAS_WV>
 tv_status launch_col(const float *wv, float lam, long long H, long long W, float *x0,
                      const Tv2dWs &ws, cudaStream_t s)
 {
+    if (split_takes(H, W, split_max_chains(H, true, false, wv != nullptr)))
+        return launch_split(split_src(SPLIT_COL, nullptr, wv, lam, H, W, x0, ws), ws.hdr, s, PK_COL);
     if (W <= coop_max_chains()) {
         CoopColPhaseP<HAS_WV> p{wv, lam, H, W, x0, ws.buf1, ws.y, ws.st, ws.prm,
                                 nullptr, nullptr, 0.f, 0.f, 0.f};
@@ -873,8 +917,8 @@ tv_status tv2d_denoise(const float *d_img, int64_t H, int64_t W, const float *d_
         const int u = (max_iters - launched) < batch ? (max_iters - launched) : batch;
         for (int t = 0; t < u; ++t) {
             if ((st = launch_col_any(d_wv, lambda, H, W, d_x, ws, s)) != TV_OK) return st;
-            st = d_wh ? launch_row<true>(d_img, d_wh, lambda, H, W, d_x, ws, s)
-                      : launch_row<false>(d_img, d_wh, lambda, H, W, d_x, ws, s);
+            st = d_wh ? launch_row<true>(d_img, d_wh, lambda, H, W, max_iters, d_x, ws, s)
+                      : launch_row<false>(d_img, d_wh, lambda, H, W, max_iters, d_x, ws, s);
             if (st != TV_OK) return st;
             if ((st = launch_gap(d_img, d_wh, d_wv, lambda, H, W, d_x, ws, s)) != TV_OK) return st;
         }

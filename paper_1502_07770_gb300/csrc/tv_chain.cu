@@ -12,6 +12,7 @@
 #include "tv_flat.cuh"
 #include "tv_halves.cuh"
 #include "tv_launch.cuh"
+#include "tv_split_launch.h"
 
 namespace tvh {
 
@@ -185,23 +186,6 @@ using namespace tvh;
 namespace {
 
 constexpr int kRing = 32;
-
-// CSR batches: the node range [offsets[0], offsets[num_chains]) of x must not overlap
-// that of y or of w (the host checks only x == y, since the offsets live on the device).
-// Read by every thread at kernel entry; an overlap flags ERR_BAD_CHAIN and skips the
-// whole launch.
-__device__ __forceinline__ bool csr_disjoint(const float *x, const float *y, const float *w,
-                                             long long off0, long long offn)
-{
-    if (offn <= off0) return true;
-    const size_t len = (size_t)(offn - off0) * sizeof(float);
-    auto apart = [&](const float *a) {
-        if (a == nullptr) return true;
-        const uintptr_t p = (uintptr_t)(x + off0), q = (uintptr_t)(a + off0);
-        return p + len <= q || q + len <= p;
-    };
-    return apart(y) && apart(w);
-}
 
 // Contiguous chains: chain k at [off_k, off_{k+1}) (or [k*len, (k+1)*len)).
 template <bool HAS_W>
@@ -824,6 +808,25 @@ tv_status tv_chain_solve(const float *d_y, const float *d_w, float lambda,
     tv_status st = check_cuda(cudaMemsetAsync(ws.hdr, 0, sizeof(WsHeader), s), "memset header");
     if (st != TV_OK) return st;
     const bool vec_w = vec_ok(d_offsets, max_len, d_y, d_w, d_x);
+    if (split_takes(max_len, num_chains,
+                    split_max_chains(max_len, false, vec_w, d_w != nullptr))) {
+        SplitSrc src{};
+        src.v.mode = SPLIT_PLAIN;
+        src.v.p0 = d_y;
+        src.v.pw = d_w;
+        src.v.lam = d_w ? 0.f : lambda;
+        src.v.ws = 1.f;
+        src.v.o0 = d_x;
+        src.v.stride = 1;
+        src.v.wrow = max_len;
+        src.v.rec = ws.rec;
+        src.v.spill = ws.spill;
+        src.v.maxlen = (int)max_len;
+        src.nchains = num_chains;
+        src.len = (int)max_len;
+        src.offsets = d_offsets;
+        return launch_split(src, ws.hdr, s, PK_CHAIN);
+    }
     // by default, batches the fixed-shape thread kernel stages 16 bytes at a time leave
     // the warp-per-chain kernel at a smaller batch size
     const bool vec_flat = vec_w && max_len >= kHalvesMinLen && thread_split() == 2;
@@ -900,6 +903,23 @@ tv_status tv_chain_solve_columns(const float *d_y, const float *d_w, float lambd
     cudaStream_t s = (cudaStream_t)stream;
     tv_status st = check_cuda(cudaMemsetAsync(ws.hdr, 0, sizeof(WsHeader), s), "memset header");
     if (st != TV_OK) return st;
+    if (split_takes(H, W, split_max_chains(H, true, false, d_w != nullptr))) {
+        SplitSrc src{};
+        src.v.mode = SPLIT_PLAIN;
+        src.v.cols = true;
+        src.v.p0 = d_y;
+        src.v.pw = d_w;
+        src.v.lam = d_w ? 0.f : lambda;
+        src.v.ws = 1.f;
+        src.v.o0 = d_x;
+        src.v.stride = ld;
+        src.v.rec = ws.rec;
+        src.v.spill = ws.spill;
+        src.v.maxlen = (int)H;
+        src.nchains = W;
+        src.len = (int)H;
+        return launch_split(src, ws.hdr, s, PK_CHAIN);
+    }
     if (W <= coop_max_chains()) {
         if (d_w) {
             CoopColsP<true> p{d_y, d_w, 0.f, H, W, ld, d_x};

@@ -21,6 +21,7 @@
 #include <atomic>
 
 #include "tv_launch.cuh"
+#include "tv_split_launch.h"
 
 using namespace tvk;
 using namespace tvh;
@@ -1041,7 +1042,25 @@ tv_status tv2d_denoise_l1(const float *d_img, int64_t H, int64_t W, const float 
     PdlScope pdl(true);  // each kernel may become resident while its predecessor finishes
     while (k < max_iters) {
         // dual step: column chains
-        if (d_wv) {
+        if (split_takes(H, W, split_max_chains(H, true, false, d_wv != nullptr))) {
+            SplitSrc src{};
+            SplitView &v = src.v;
+            v.mode = SPLIT_COL;
+            v.cols = true;
+            v.p0 = v.p1 = ws.xbar;
+            v.p2 = v.o0 = ws.y;
+            v.pw = d_wv;
+            v.lam = lambda;
+            v.ca = v.ws = 1.f / sigma;
+            v.cb = 0.f;
+            v.sg = sigma;
+            v.stride = W;
+            v.rec = ws.rec;
+            v.spill = ws.spill;
+            v.maxlen = src.len = (int)H;
+            src.nchains = W;
+            st = launch_split(src, ws.hdr, s, PK_COL);
+        } else if (d_wv) {
             L1ColsP<true> p{ws.xbar, d_wv, ws.y, lambda, H, W, sigma, 1.f / sigma};
             st = launch_coop(p, W, (int)H, ws.rec, ws.crec, ws.spill, ws.hdr, s, PK_COL);
         } else {

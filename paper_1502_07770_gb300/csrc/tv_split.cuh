@@ -1,0 +1,918 @@
+// Chain TV-l2 by splitting at thresholds: the chain kernel of the 2D phases and of the
+// batches of tv_chain_solve whose chains have at most kSplitMaxLen nodes.
+//
+// The dynamic program of Sec. 4.1 walks a chain node by node, and each node waits for the
+// one before. Here a chain is cut top down instead. Take a run of neighbouring nodes whose
+// boundary flows u (the edge terms w_i sign(x_{i+1} - x_i), prefix sums of x - y) are known,
+// and let z be the mean it would have if it were one constant piece. For ONE threshold z the
+// forward message of Algorithm 2 is a number per node,
+//     t_i = m_{i-1} + (z - y_i),   m_i = clip(t_i, -w_i, w_i),
+// and it tells on which side of z the minimiser lies: t_i > w_i puts x_i below z whatever
+// follows, t_i < -w_i above it, and an undecided node goes with its right neighbour (the
+// backward clip of Algorithm 2). Where neighbours end on different sides, the edge between
+// them carries the flow +-w_i, so the run is cut there and the two parts are independent. A
+// run on one side only is constant at z: its mean is z, so no part can lie above. Every round
+// treats all runs of a chain at once; signals of the 1D experiment (Sec. 6.1) take 7 rounds
+// at 1024 nodes, a ramp log2(n), and every round but the last adds a cut.
+//
+// Composed maps m -> clip(m + a, lo, hi) are closed under composition, so a round is not
+// sequential: each lane holds L consecutive nodes in registers, composes its nodes' maps, a
+// warp scan (across W warps: a shared-memory exchange) gives each lane its incoming m, a
+// second walk gives the sides as two bit masks, and the undecided bits are filled from the
+// right by one carry-propagating addition. The mean of every run comes from a walk from the
+// right and a segmented scan over the lanes. Cut flows are folded into the values at the cut
+// (y_i += u, y_{i+1} -= u, w_i = 0), after which a cut needs no special case.
+//
+// Solutions are sums of the values of a run over its length: all nodes of a run are bitwise
+// equal, and the rounding is that of one mean. The folded flows cost eps * |u| per run, so a
+// chain that is to be cut at a flow above 16 max |y| goes to the warp's dynamic program
+// (coop_solve_chain, records and reserve in the workspace) instead.
+#pragma once
+#include "tv2d_common.cuh"
+#include "tv_coop.cuh"
+
+namespace tvk {
+
+constexpr int kSplitMaxLen = 4096;     // nodes of the longest chain (8 warps x 32 lanes x 16)
+constexpr float kSplitHeavy = 16.f;
+
+// What a chain's nodes are made of. PLAIN: c = y. INIT, ROW, COL: the set-up of the phases
+// of eq. pd (x^0 rows, primal rows, dual columns).
+enum SplitMode { SPLIT_PLAIN = 0, SPLIT_INIT = 1, SPLIT_ROW = 2, SPLIT_COL = 3 };
+
+struct SplitView {
+    int mode;
+    bool cols;                 // chains are columns (node stride `stride`), else rows
+    const float *p0, *p1, *p2; // PLAIN y; INIT f, y; ROW f, y, x^k; COL x^k, x^{k-1}, y
+    const float *pw;           // edge weights, or NULL: lam
+    float lam, ws;             // weight = ws * (pw or lam)
+    float ca, cb, sg;          // ROW: c = ca (f - y) + cb x; COL: 1/sigma, theta, sigma
+    float *o0, *o1;
+    long long stride, wrow;    // columns: node stride (values and weights); rows: weight row
+    float2 *rec, *spill;       // records and reserve of the fallback
+    int maxlen;                // records of one chain
+
+    __device__ __forceinline__ float unary(float a, float b, float c) const
+    {
+        if (mode == SPLIT_PLAIN) return a;
+        if (mode == SPLIT_INIT) return a - b;
+        if (mode == SPLIT_ROW) return ca * (a - b) + cb * c;
+        return c * ca + (a + cb * (a - b));
+    }
+    __device__ __forceinline__ void emit(long long o, float xv, float c) const
+    {
+        if (mode == SPLIT_COL) {
+            o0[o] = sg * (c - xv);
+        } else {
+            o0[o] = xv;
+            if (mode == SPLIT_INIT) o1[o] = xv;
+        }
+    }
+};
+
+// The fallback's policy (coop_solve_chain): one chain of the view.
+struct SplitCoopP {
+    static constexpr bool CREC = false;
+    struct Raw {
+        float a, b, c, w;
+    };
+    struct Acc {};
+    SplitView v;
+    long long wstart;
+    int n;
+
+    __device__ int max_len() const { return v.maxlen; }
+    __device__ long long at(long long start, int i) const { return start + (long long)i * v.stride; }
+    __device__ void fetch(long long, long long start, int nn, int i, Raw &r) const
+    {
+        const bool in = i < nn;
+        const long long o = at(start, i);
+        r.a = in ? v.p0[o] : 0.f;
+        r.b = in && v.p1 ? v.p1[o] : 0.f;
+        r.c = in && v.p2 ? v.p2[o] : 0.f;
+        r.w = v.lam;
+        if (v.pw) r.w = i < nn - 1 ? v.pw[wstart + (long long)i * v.stride] : 0.f;
+    }
+    __device__ void unary(long long, long long, int, int, const Raw &r, float &c, float &w,
+                          Acc &) const
+    {
+        c = v.unary(r.a, r.b, r.c);
+        w = v.ws * r.w;
+    }
+    __device__ void emit(long long k, long long start, int i, float xv, float) const
+    {
+        float c = 0.f, w;
+        if (v.mode == SPLIT_COL) unary_direct(i, n, k, start, c, w);
+        v.emit(at(start, i), xv, c);
+    }
+    __device__ void unary_direct(int i, int nn, long long k, long long start, float &c,
+                                 float &w) const
+    {
+        Raw r;
+        Acc a;
+        fetch(k, start, nn, i, r);
+        unary(k, start, nn, i, r, c, w, a);
+        if (i == nn - 1) w = 0.f;
+    }
+    __device__ void emit_direct(int i, long long k, long long start, float xv, float c) const
+    {
+        emit(k, start, i, xv, c);
+    }
+};
+
+static __device__ __noinline__ void split_fallback(const SplitView &v, long long k,
+                                                   long long start, long long wstart, int n,
+                                                   int lane, float2 *spill, WsHeader *hdr)
+{
+    SplitCoopP p{v, wstart, n};
+    SplitCoopP::Acc acc;
+    coop_solve_chain(p, acc, k, start, n, lane, (float2 *)nullptr, (float *)nullptr, 0, v.rec,
+                     (float *)nullptr, spill, hdr);
+}
+
+// Exchange between the warps of one chain (W > 1).
+template <int W>
+struct SplitX {
+    float a[W], lo[W], hi[W];     // composed map of each warp
+    float R[W], St[W], Kt[W];     // head sum, tail sum and count of each warp
+    float K[W];                   // head count
+    float u[W], u2[W];            // flow of a (new) cut after the warp's last node
+    float re[W];                  // r of that node
+    float amax[W];
+    unsigned char cut[W], side[W], more[W], heavy[W];
+    int bad;                      // the chain goes to the fallback
+};
+
+__device__ __forceinline__ float rcp_approx(float v)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float clampw(float v, float lo, float hi)
+{
+    return fminf(fmaxf(v, lo), hi);
+}
+
+// s / k: the approximate reciprocal's quotient with one residual correction
+__device__ __forceinline__ float mean_of(float s, float k)
+{
+    const float rc = rcp_approx(k), q = s * rc;
+    return fmaf(fmaf(-q, k, s), rc, q);
+}
+
+template <int W>
+__device__ __forceinline__ void split_sync(int bar)
+{
+    if constexpr (W == 1) {
+        __syncwarp();
+    } else {
+        // literal barrier names: with a name in a register the block would hold all 16, and
+        // an SM only four such blocks
+        if (bar == 0) asm volatile("bar.sync 1, %0;" ::"n"(W * WARP) : "memory");
+        else if (bar == 1) asm volatile("bar.sync 2, %0;" ::"n"(W * WARP) : "memory");
+        else if (bar == 2) asm volatile("bar.sync 3, %0;" ::"n"(W * WARP) : "memory");
+        else asm volatile("bar.sync 4, %0;" ::"n"(W * WARP) : "memory");
+    }
+}
+
+// Lane slots of L nodes in shared memory, padded so that the lanes' 16-byte accesses do not
+// share banks.
+template <int L>
+__host__ __device__ constexpr int split_lp()
+{
+    return (L / 4) % 2 == 1 ? L : L + 4;
+}
+
+// fma, clipped to [0, 1] by the instruction itself
+__device__ __forceinline__ float fma_sat(float a, float b, float c)
+{
+    float r;
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+// y0 += u, y1 -= u and r = w = 0 where bit is set: predicated, the lanes differ
+__device__ __forceinline__ void cut_at(unsigned bit, float u, float &y0, float &y1, float &r,
+                                       float &w)
+{
+    asm("{\n .reg .pred p;\n setp.ne.u32 p, %5, 0;\n @p add.f32 %0, %0, %4;\n"
+        " @p sub.f32 %1, %1, %4;\n @p mov.f32 %2, 0f00000000;\n @p mov.f32 %3, 0f00000000;\n}"
+        : "+f"(y0), "+f"(y1), "+f"(r), "+f"(w)
+        : "f"(u), "r"(bit));
+}
+__device__ __forceinline__ void cut_at_unit(unsigned bit, unsigned up, float &y0, float &y1,
+                                            float &r)
+{
+    asm("{\n .reg .pred p, q;\n setp.ne.u32 p, %3, 0;\n setp.ne.u32 q, %4, 0;\n"
+        " @q add.f32 %0, %0, 0f3F800000;\n @q add.f32 %1, %1, 0fBF800000;\n"
+        " @p mov.f32 %2, 0f00000000;\n}"
+        : "+f"(y0), "+f"(y1), "+f"(r)
+        : "r"(bit), "r"(up));
+}
+
+// Solves one chain held as L nodes per lane in sc (values) and sx (weights if !UNI); writes
+// the solution to sx. Returns false (in every lane) if the chain needs the fallback.
+//
+// The walks are bound by issue and by the half-rate ALU pipe (minima, selects, logic), so
+// what can be arithmetic on the FMA pipe is: r[j] is 1, or 0 where the chain is cut after node
+// j, and a sum that restarts at cuts is s = fma(s, r, y). Node j of a lane is bit L-1-j of
+// its masks.
+//
+// UNI: one weight lamw for every edge. Values are divided by 2 lamw and messages shifted to
+// v = m / (2 lamw) + 1/2 in [0, 1], so that a step m -> clip(m + z - y, -w, w) is one
+// saturating fma, v -> sat(v r' + (z - y)), r' of the edge before the node. After a cut v
+// restarts at 1/2: the half is folded into the values at the cut (with the flow +-1/2: both 0
+// or both 1), and a node before a cut compares with 0 alone. The last sums take the values as
+// they came, so that scaling costs no digits.
+template <int L, int W, bool UNI>
+__device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W> *xc, int n,
+                                            float lamw, int lane, int wi, int bar)
+{
+    constexpr int LP = split_lp<L>();
+    constexpr unsigned ML = L == 32 ? 0xffffffffu : (1u << L) - 1u;
+    const int base = (wi * WARP + lane) * L;
+    const float4 *yp = reinterpret_cast<const float4 *>(sc + (wi * WARP + lane) * LP);
+    float y[L], w[UNI ? 1 : L], r[L], z[L];
+    unsigned C = 0;  // cuts (the edge after the node): chain end, padding, decoupled edges
+    float amax = 0.f;
+    const int last = n - 1 - base;  // the chain's last node, in the lane's numbering
+#pragma unroll
+    for (int q = 0; q < L / 4; ++q) {
+        const float4 t = yp[q];
+        y[4 * q] = t.x;
+        y[4 * q + 1] = t.y;
+        y[4 * q + 2] = t.z;
+        y[4 * q + 3] = t.w;
+    }
+#pragma unroll
+    for (int j = 0; j < L; ++j) amax = fmaxf(amax, fabsf(y[j]));
+    if constexpr (UNI) {
+        const int k = max(0, min(L, last));  // nodes with an edge to the next one
+        C = k >= L ? 0u : ((1u << (L - k)) - 1u) & ML;
+#pragma unroll
+        for (int j = 0; j < L; ++j) r[j] = j < last ? 1.f : 0.f;
+    } else {
+        const float4 *wp = reinterpret_cast<const float4 *>(sx + (wi * WARP + lane) * LP);
+#pragma unroll
+        for (int q = 0; q < L / 4; ++q) {
+            const float4 e = wp[q];  // 0 from the chain's last node on
+            w[4 * q] = e.x;
+            w[4 * q + 1] = e.y;
+            w[4 * q + 2] = e.z;
+            w[4 * q + 3] = e.w;
+        }
+#pragma unroll
+        for (int j = 0; j < L; ++j) {
+            const bool cut = !(w[j] > 0.f);
+            w[j] = cut ? 0.f : w[j];
+            r[j] = cut ? 0.f : 1.f;
+            C = C << 1 | (cut ? 1u : 0u);
+        }
+    }
+    amax = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(amax)));
+    if constexpr (W > 1) {
+        if (lane == 0) xc->amax[wi] = amax;
+        if (lane == WARP - 1) xc->re[wi] = r[L - 1];
+        split_sync<W>(bar);
+#pragma unroll
+        for (int q = 0; q < W; ++q) amax = fmaxf(amax, xc->amax[q]);
+    }
+    unsigned H = 0;   // edges whose flow would swamp the values
+    unsigned UP = 0;  // UNI: cuts with flow +w
+    if constexpr (UNI) {
+        if (!(lamw > 1e-30f * amax && lamw > 1e-37f)) {  // no weight to speak of: x = y
+            float4 *xp = reinterpret_cast<float4 *>(sx + (wi * WARP + lane) * LP);
+#pragma unroll
+            for (int q = 0; q < L / 4; ++q) xp[q] = yp[q];
+            return true;
+        }
+        if (lamw > kSplitHeavy * amax) H = ML;
+        const float s = 0.5f / lamw;
+        const bool head = wi == 0 && lane == 0;
+#pragma unroll
+        for (int j = 0; j < L; ++j) {
+            y[j] *= s;
+            if (j == 0 && head) y[j] -= 0.5f;
+            if (j == last) y[j] += 0.5f;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < L; ++j)
+            if (w[j] > kSplitHeavy * amax) H |= 1u << (L - 1 - j);
+    }
+
+    const bool any_heavy = __any_sync(FULL, H != 0);
+    unsigned bc = __ballot_sync(FULL, C != 0);  // lanes with a cut
+    float re = 0.f;  // UNI: r of the edge into the lane's first node
+    if constexpr (UNI) {
+        const float rq = __shfl_up_sync(FULL, r[L - 1], 1);
+        if (lane > 0) re = rq;
+        else if (W > 1 && wi > 0) re = xc->re[wi - 1];
+    }
+    bool more = true;
+    for (;;) {
+        // ---- sums of the runs across lanes ----
+        float Sh = 0.f, St = 0.f, b = 1.f;  // to the lane's first cut; after its last one
+#pragma unroll
+        for (int j = L - 1; j >= 0; --j) {
+            Sh = fmaf(Sh, r[j], y[j]);
+            b *= r[j];
+            St = fmaf(b, y[j], St);
+        }
+        const float kh = C ? (float)(__clz(C) - (31 - L)) : (float)L;  // nodes of the head
+        const float kt = (float)(__ffs(C) - 1);                       // nodes after the last cut
+        // R, K: sum and count from the lane's first node to the end of its run
+        float R = Sh, K = kh;
+        int pe = lane;
+        if (bc != FULL) {
+            const unsigned ahead = bc >> lane;
+            pe = ahead ? lane + __ffs(ahead) - 1 : WARP;  // lane where that run ends
+#pragma unroll
+            for (int o = 1; o < WARP; o <<= 1) {
+                const float r2 = __shfl_down_sync(FULL, R, o);
+                if (lane + o < WARP && lane + o <= pe) R += r2;
+            }
+            const float kp = __shfl_sync(FULL, kh, pe & (WARP - 1));
+            K = pe < WARP ? (float)((pe - lane) * L) + kp : (float)((WARP - lane) * L);
+        }
+        float Rn, Kn;       // the same for the next lane's first node
+        float zprev = 0.f;  // value of the run that enters this warp
+        float zt;           // value of the run after the lane's last cut
+        if constexpr (W == 1) {
+            Rn = __shfl_down_sync(FULL, R, 1);
+            Kn = __shfl_down_sync(FULL, K, 1);
+            zt = mean_of(St + Rn, kt + Kn);  // (unused in the last lane)
+        } else {
+            // Every warp forms the sum of a run that crosses warps in the same order (tail of
+            // the warp it begins in, plus the head sums folded from the right), so that all its
+            // nodes get the same bits.
+            const int lq = bc ? 31 - __clz(bc) : 0;
+            const float Rq = __shfl_down_sync(FULL, R, 1), Kq = __shfl_down_sync(FULL, K, 1);
+            const float tS = lane < WARP - 1 ? St + Rq : St, tK = lane < WARP - 1 ? kt + Kq : kt;
+            if (lane == lq) {
+                xc->St[wi] = tS;
+                xc->Kt[wi] = tK;
+            }
+            if (lane == 0) {
+                xc->R[wi] = R;
+                xc->K[wi] = K;
+                xc->cut[wi] = bc != 0;
+            }
+            split_sync<W>(bar);
+            float Rin = 0.f, Kin = 0.f;  // the same for the next warp's first node
+            float rr = 0.f, kk = 0.f;    // from warp q's first node to the end of its run
+            bool enters = true;          // the run that enters warp wi is not found yet
+#pragma unroll
+            for (int q = W - 1; q >= 0; --q) {
+                const bool e = xc->cut[q] != 0;
+                if (q < wi && enters && e) {
+                    zprev = mean_of(xc->St[q] + rr, xc->Kt[q] + kk);
+                    enters = false;
+                }
+                rr = xc->R[q] + (e ? 0.f : rr);
+                kk = xc->K[q] + (e ? 0.f : kk);
+                if (q == wi + 1) {
+                    Rin = rr;
+                    Kin = kk;
+                }
+            }
+            if (enters) zprev = mean_of(rr, kk);  // the chain's first run
+            if (pe == WARP) {
+                R += Rin;
+                K += Kin;
+            }
+            Rn = __shfl_down_sync(FULL, R, 1);
+            Kn = __shfl_down_sync(FULL, K, 1);
+            if (lane == WARP - 1) {
+                Rn = Rin;
+                Kn = Kin;
+            }
+            const bool out = lane == lq;  // its last run leaves the warp
+            zt = mean_of((out ? tS : St) + (out ? Rin : Rn), (out ? tK : kt) + (out ? Kin : Kn));
+        }
+        // zr: value of the run at the lane's first node
+        const unsigned before = bc & ((1u << lane) - 1u);
+        float zr;
+        if constexpr (W == 1) {
+            const float zh = mean_of(R, K);  // of the lane's first node, if a run begins there
+            zr = __shfl_sync(FULL, C ? zt : zh, before ? 31 - __clz(before) : 0);
+            if (lane == 0) zr = zh;
+        } else {
+            zr = __shfl_sync(FULL, zt, before ? 31 - __clz(before) : 0);
+            if (!before) zr = zprev;
+        }
+
+        // ---- mean of every run that begins in the lane, at its first node ----
+        float s = Rn, k = Kn;
+        if (W == 1 && lane == WARP - 1) s = k = 0.f;
+        if (!more) {  // no cut in the last round: the runs are the solution
+#pragma unroll
+            for (int j = L - 1; j >= 0; --j) {
+                s = fmaf(s, r[j], y[j]);
+                k = fmaf(k, r[j], 1.f);
+                z[j] = mean_of(s, k);
+            }
+            const unsigned LC = C & (0u - C);
+            float4 *xp = reinterpret_cast<float4 *>(sx + (wi * WARP + lane) * LP);
+#pragma unroll
+            for (int q = 0; q < L / 4; ++q) {
+                float v[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int j = 4 * q + e;
+                    if (j > 0 && (C & (1u << (L - j)))) zr = z[j];
+                    if (j > 0 && (LC & (1u << (L - j)))) zr = zt;  // the bits other lanes have
+                    v[e] = zr;
+                }
+                xp[q] = make_float4(v[0], v[1], v[2], v[3]);
+            }
+            return true;
+        }
+#pragma unroll
+        for (int j = L - 1; j >= 0; --j) {
+            s = fmaf(s, r[j], y[j]);
+            k = fmaf(k, r[j], 1.f);
+            z[j] = s * rcp_approx(k);
+        }
+
+        // ---- forward: z - y per node, and the lane's composed map ----
+        float a = 0.f, lo = 0.f, hi = 0.f;
+#pragma unroll
+        for (int j = 0; j < L; ++j) {
+            if (j > 0 && r[j > 0 ? j - 1 : 0] == 0.f) zr = z[j];
+            const float d = zr - y[j];
+            z[j] = d;
+            a += d;
+            if constexpr (UNI) {
+                const float rp = j == 0 ? re : r[j > 0 ? j - 1 : 0];
+                if (j == 0) {
+                    lo = __saturatef(d);
+                    hi = __saturatef(rp + d);
+                } else {
+                    lo = fma_sat(lo, rp, d);
+                    hi = fma_sat(hi, rp, d);
+                }
+            } else {
+                if (j == 0) {
+                    lo = -w[0];
+                    hi = w[0];
+                } else {
+                    lo = clampw(lo + d, -w[j], w[j]);
+                    hi = clampw(hi + d, -w[j], w[j]);
+                }
+            }
+        }
+        // m (UNI: v) into the lane's first node. A map with lo == hi forgets its input; from
+        // such lanes the message walks through the few others, one lane a step, and only a
+        // long row of those takes a scan of the composed maps.
+        float m;
+        const unsigned kn = __ballot_sync(FULL, lo == hi) | (W == 1 ? 1u : 0u);
+        unsigned far = ~kn;
+        far &= far << 1;
+        far &= far << 2;  // rows of four and more
+        if (far == 0 && (W == 1 || (kn & 1u))) {
+            float out = W == 1 && lane == 0 ? clampw(a, lo, hi) : hi;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const float in = __shfl_up_sync(FULL, out, 1);
+                if (!((kn >> lane) & 1u)) out = clampw(in + a, lo, hi);
+            }
+            if constexpr (W > 1) {
+                if (lane == WARP - 1) xc->a[wi] = 0.f, xc->lo[wi] = xc->hi[wi] = out;
+                split_sync<W>(bar);
+            }
+            m = __shfl_up_sync(FULL, out, 1);
+        } else {
+#pragma unroll
+            for (int o = 1; o < WARP; o <<= 1) {
+                const float a2 = __shfl_up_sync(FULL, a, o);
+                const float l2 = __shfl_up_sync(FULL, lo, o);
+                const float h2 = __shfl_up_sync(FULL, hi, o);
+                if (lane >= o) {
+                    const float nl = clampw(l2 + a, lo, hi);
+                    hi = clampw(h2 + a, lo, hi);
+                    lo = nl;
+                    a += a2;
+                }
+            }
+            if constexpr (W > 1) {
+                if (lane == WARP - 1) {
+                    xc->a[wi] = a;
+                    xc->lo[wi] = lo;
+                    xc->hi[wi] = hi;
+                }
+                split_sync<W>(bar);
+            }
+            float mc = 0.f;
+            if constexpr (W > 1) {
+#pragma unroll
+                for (int q = 0; q < W; ++q)
+                    if (q < wi) mc = clampw(mc + xc->a[q], xc->lo[q], xc->hi[q]);
+            }
+            m = __shfl_up_sync(FULL, clampw(mc + a, lo, hi), 1);
+        }
+        if (lane == 0) {
+            m = 0.f;
+            if constexpr (W > 1) {
+#pragma unroll
+                for (int q = 0; q < W; ++q)
+                    if (q < wi) m = clampw(m + xc->a[q], xc->lo[q], xc->hi[q]);
+            }
+        }
+
+        // ---- sides: below z (t > w) and above (t < -w), one bit per node ----
+        unsigned below = 0, above = 0;
+#pragma unroll
+        for (int j = 0; j < L; ++j) {
+            if constexpr (UNI) {
+                const float rp = j == 0 ? re : r[j > 0 ? j - 1 : 0];
+                const float t = fmaf(m, rp, z[j]);
+                m = fma_sat(m, rp, z[j]);
+                below = __funnelshift_l(__float_as_uint(1.f - t), below, 1);
+                above = __funnelshift_l(__float_as_uint(t), above, 1);
+            } else {
+                const float t = m + z[j];
+                below = __funnelshift_l(__float_as_uint(w[j] - t), below, 1);
+                above = __funnelshift_l(__float_as_uint(t + w[j]), above, 1);
+                z[j] = m = clampw(t, -w[j], w[j]);  // the flow of a cut made here
+            }
+        }
+        if constexpr (UNI) below |= C & ~above;
+        const unsigned dec = below | above;
+        const unsigned U = ~dec & ML;
+        const bool first = dec != 0 && ((below >> (31 - __clz(dec | 1u))) & 1u);
+        const unsigned bd = __ballot_sync(FULL, dec != 0), bl = __ballot_sync(FULL, first);
+        unsigned carry;  // side of the next lane's first node
+        {
+            const unsigned nx = (bd >> lane) >> 1;
+            const int q = lane + __ffs(nx);
+            carry = nx ? (bl >> (q & 31)) & 1u : 0u;
+            if constexpr (W > 1) {
+                if (lane == 0) {
+                    const int q0 = bd ? __ffs(bd) - 1 : 0;
+                    xc->side[wi] = bd ? 2 + ((bl >> q0) & 1) : 0;
+                }
+                split_sync<W>(bar);
+                if (!nx) {
+                    unsigned sd = 0;
+#pragma unroll
+                    for (int q2 = W - 1; q2 >= 0; --q2)
+                        if (q2 > wi && xc->side[q2]) sd = xc->side[q2] & 1u;
+                    carry = sd;
+                }
+            }
+        }
+        const unsigned S = ((below << 1) | carry) & U;
+        const unsigned low = below | (U & ~(U + S));
+        const unsigned fresh = (low ^ ((low << 1) | carry)) & ~C & ML;
+
+        // ---- new cuts: fold their flows into the values ----
+        const unsigned upf = fresh & low;
+        const unsigned bf = __ballot_sync(FULL, fresh != 0);
+        more = bf != 0;
+        bc |= bf;
+        // the flow of a cut after the lane's last node (UNI: 2 with its half, 1 without)
+        float ue;
+        if constexpr (UNI) ue = (upf & 1u) ? 2.f : (float)(fresh & 1u);
+        else ue = (fresh & 1u) ? z[L - 1] : 0.f;
+        float up = __shfl_up_sync(FULL, ue, 1);
+        if (more) {
+            float dummy = 0.f;
+#pragma unroll
+            for (int j = 0; j < L; ++j) {
+                const unsigned bit = 1u << (L - 1 - j);
+                float &yn = j + 1 < L ? y[j + 1 < L ? j + 1 : 0] : dummy;
+                if constexpr (UNI) cut_at_unit(fresh & bit, upf & bit, y[j], yn, r[j]);
+                else cut_at(fresh & bit, z[j], y[j], yn, r[j], w[j]);
+            }
+        }
+        C |= fresh;
+        UP |= upf;
+        bool hv = any_heavy && __any_sync(FULL, (fresh & H) != 0);
+        if constexpr (W > 1) {
+            if (lane == WARP - 1) {
+                xc->u[wi] = ue;
+                xc->more[wi] = more;
+                xc->heavy[wi] = hv;
+            }
+            split_sync<W>(bar);
+            more = hv = false;
+#pragma unroll
+            for (int q = 0; q < W; ++q) {
+                more |= xc->more[q] != 0;
+                hv |= xc->heavy[q] != 0;
+            }
+            if (lane == 0) up = wi > 0 ? xc->u[wi - 1] : 0.f;
+        } else {
+            if (lane == 0) up = 0.f;
+        }
+        if constexpr (UNI) {
+            y[0] -= up > 1.f ? 1.f : 0.f;
+            if (up > 0.f) re = 0.f;
+        } else {
+            y[0] -= up;
+        }
+        if (hv) return false;
+        if constexpr (UNI) {
+            if (!more) {  // the values as they came, with the flows of all cuts
+                const unsigned ends = last >= L ? 0u : ML >> max(0, min(31, last));
+                const unsigned F = C & ~ends;  // cuts that carry a flow
+                float u = (F & 1u) ? ((UP & 1u) ? lamw : -lamw) : 0.f;
+                float ul = __shfl_up_sync(FULL, u, 1);
+                if (lane == 0) ul = 0.f;
+                if constexpr (W > 1) {
+                    if (lane == WARP - 1) xc->u2[wi] = u;
+                    split_sync<W>(bar);
+                    if (lane == 0 && wi > 0) ul = xc->u2[wi - 1];
+                }
+#pragma unroll
+                for (int q = 0; q < L / 4; ++q) {
+                    const float4 t = yp[q];
+                    const float v[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const unsigned bit = 1u << (L - 1 - (4 * q + e));
+                        u = (F & bit) ? ((UP & bit) ? lamw : -lamw) : 0.f;
+                        y[4 * q + e] = v[e] + (u - ul);  // equal flows cancel exactly
+                        ul = u;
+                    }
+                }
+            }
+        }
+    }
+}
+
+struct UnitStride {  // of rows: known at compile time
+    __device__ __forceinline__ operator long long() const { return 1; }
+};
+
+// Load, solve and store for the chains of one block: `nch` chains of W warps each. Rows are
+// loaded by their own warps; columns by the whole block, nch neighbouring columns of a row at
+// a time.
+template <int L, int W, bool UNI>
+__device__ __forceinline__ void split_chain(const SplitView &v, float *smem, SplitX<W> *xall,
+                                            int nch, int cs, long long k0, int cnt, long long start,
+                                            long long wstart, int n, WsHeader *hdr,
+                                            float2 *spill)
+{
+    constexpr int LP = split_lp<L>();
+    constexpr int T = W * WARP;
+    const int tid = threadIdx.x;
+    const int lane = tid & (WARP - 1), warp = tid / WARP;
+    const int g = warp / W, wi = warp % W;
+    SplitX<W> *xc = xall + g;
+    // the chain and the node lane that this thread loads and stores
+    const int cc = v.cols ? tid & (nch - 1) : g;
+    const int ll = v.cols ? tid / nch : wi * WARP + lane;
+    const bool in = cc < cnt;
+    const long long st = v.cols ? k0 + cc : start;
+    const long long wst = v.cols ? st : wstart;
+    float *lc = smem + (size_t)cc * cs, *lx = smem + (size_t)(nch + cc) * cs;
+    constexpr int UL = L % 8 == 0 ? 8 : 4;
+    auto load = [&](auto stride) {
+        const long long step = T * (long long)stride, o0 = ll * (long long)stride;
+        const float *q0 = v.p0 + st + o0, *q1 = v.p1 + st + o0, *q2 = v.p2 + st + o0,
+                    *qw = v.pw + wst + o0;
+        const bool h1 = v.p1 != nullptr, h2 = v.p2 != nullptr;
+        const int nn = in ? n : 0;
+#pragma unroll 1
+        for (int b0 = 0; b0 < L; b0 += UL) {
+            float a[UL], b[UL], c[UL], e[UL];
+#pragma unroll
+            for (int u = 0; u < UL; ++u) {
+                const int i = (b0 + u) * T + ll;
+                const bool ok = i < nn;
+                a[u] = ok ? q0[u * step] : 0.f;
+                b[u] = ok && h1 ? q1[u * step] : 0.f;
+                c[u] = ok && h2 ? q2[u * step] : 0.f;
+                if constexpr (!UNI) e[u] = i < nn - 1 ? qw[u * step] : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < UL; ++u) {
+                const int i = (b0 + u) * T + ll;
+                const int p = i + (LP - L) * (i / L);
+                lc[p] = v.unary(a[u], b[u], c[u]);
+                if constexpr (!UNI) lx[p] = v.ws * e[u];
+            }
+            q0 += UL * step;
+            q1 += UL * step;
+            q2 += UL * step;
+            qw += UL * step;
+        }
+    };
+    if (v.cols) load(v.stride);
+    else load(UnitStride());
+    if (tid % T == 0) xc->bad = 0;
+    if (v.cols) __syncthreads();
+    else split_sync<W>(g);
+    bool good = true;
+    if (g < cnt) {
+        good = split_solve<L, W, UNI>(smem + (size_t)g * cs, smem + (size_t)(nch + g) * cs, xc, n,
+                                      v.ws * v.lam, lane, wi, g);
+        if (!good && tid % T == 0) xc->bad = 1;
+    }
+    if (v.cols) __syncthreads();
+    else split_sync<W>(g);
+    if (in && !xall[cc].bad) {
+        auto store = [&](auto stride) {
+            long long o = st + ll * (long long)stride;
+#pragma unroll 4
+            for (int q = 0; q < L; ++q) {
+                const int i = q * T + ll;
+                const int p = i + (LP - L) * (i / L);
+                if (i < n) v.emit(o, lx[p], lc[p]);
+                o += T * (long long)stride;
+            }
+        };
+        if (v.cols) store(v.stride);
+        else store(UnitStride());
+    }
+    if (!good && wi == 0) {
+        SplitView vv = v;
+        split_fallback(vv, k0 + g, v.cols ? k0 + g : start, v.cols ? k0 + g : wstart, n, lane, spill,
+                       hdr);
+    }
+}
+
+// Nodes per lane for a chain of n nodes (0: longer than W warps hold). With one weight three
+// arrays of 32 registers fit a lane, with a weight per edge four of 24.
+template <int W, bool UNI>
+__host__ __device__ constexpr int split_pick(int n)
+{
+    constexpr int T = 32 * W;
+    if (W == 1 && n <= 4 * T) return 4;
+    if (W == 1 && n <= 8 * T) return 8;
+    if (!UNI && W < 8 && n <= 12 * T) return 12;
+    if (n <= 16 * T) return 16;
+    if (!UNI && W < 8 && n <= 20 * T) return 20;
+    if (W < 8 && n <= 24 * T) return 24;
+    return UNI && n <= 32 * T ? 32 : 0;
+}
+
+// Floats of one chain's slot array (values; the weights or solutions take another).
+template <int W>
+__host__ __device__ constexpr int split_slots(int l, int nch)
+{
+    return 32 * W * ((l / 4) % 2 == 1 ? l : l + 4) + 32 / nch;
+}
+
+template <int W>
+__host__ __device__ constexpr int split_threads()
+{
+    return W <= 2 ? 256 : 512;
+}
+
+// CSR batches: the node range [offsets[0], offsets[num_chains]) of x must not overlap
+// that of y or of w (the host checks only x == y, since the offsets live on the device).
+// Read by every thread at kernel entry; an overlap flags ERR_BAD_CHAIN and skips the
+// whole launch.
+__device__ __forceinline__ bool csr_disjoint(const float *x, const float *y, const float *w,
+                                             long long off0, long long offn)
+{
+    if (offn <= off0) return true;
+    const size_t len = (size_t)(offn - off0) * sizeof(float);
+    auto apart = [&](const float *a) {
+        if (a == nullptr) return true;
+        const uintptr_t p = (uintptr_t)(x + off0), q = (uintptr_t)(a + off0);
+        return p + len <= q || q + len <= p;
+    };
+    return apart(y) && apart(w);
+}
+
+// Chains of one array (tv_chain_solve, tv_chain_solve_columns) or of one image (the phases of
+// the 2D solvers).
+struct SplitSrc {
+    SplitView v;  // filled by the host; the phases resolve iterates and step sizes here
+    long long nchains;
+    int len;                 // chain length, or with offsets the longest
+    const int64_t *offsets;  // CSR rows, or NULL
+    int n_lo;                // with offsets: chains of n_lo < n <= what the kernel holds
+    long long off0;
+    // phases of eq. pd
+    float *buf0, *buf1, *y;
+    int *k;                  // iteration (NULL: step sizes given in v)
+    const int *done;
+    int max_iters;
+    const Tv2dParams *prm;
+    unsigned *ticket;        // ROW: blocks finished; the last one advances *k
+
+    __device__ bool bind(unsigned blk, int nch, SplitView &o, long long &k0, int &cnt,
+                         WsHeader *hdr)
+    {
+        k0 = (long long)blk * nch;
+        cnt = (int)min((long long)nch, nchains - k0);
+        o = v;
+        off0 = 0;
+        if (offsets) {
+            off0 = (long long)offsets[0];
+            if (!csr_disjoint(v.o0, v.p0, v.pw, off0, (long long)offsets[nchains])) {
+                if (threadIdx.x == 0) atomicOr(&hdr->status, ERR_BAD_CHAIN);
+                return false;
+            }
+        }
+        if (v.mode >= SPLIT_ROW && k) {
+            const int it = *k;
+            if (*done || (v.mode == SPLIT_ROW && it >= max_iters)) return false;
+            const Tv2dParams &p = prm[it];
+            float *xc = (it & 1) ? buf1 : buf0, *xo = (it & 1) ? buf0 : buf1;
+            if (v.mode == SPLIT_ROW) {
+                o.p2 = xc;
+                o.o0 = xo;
+                o.ca = o.ws = (float)(p.tau / (p.tau + 1.0));
+                o.cb = (float)(1.0 / (p.tau + 1.0));
+            } else {
+                o.p0 = xc;
+                o.p1 = xo;
+                o.ca = o.ws = (float)(1.0 / p.sigma);
+                o.cb = (float)p.theta_prev;
+                o.sg = (float)p.sigma;
+            }
+        }
+        return true;
+    }
+    __device__ void chain(const SplitView &o, long long c, long long &start, long long &wstart,
+                          int &n, WsHeader *hdr) const
+    {
+        n = len;
+        if (o.cols) {
+            start = wstart = c;
+        } else if (offsets) {
+            const long long a = offsets[c], b = offsets[c + 1];
+            // monotone offsets keep every chain inside the first (c+1)*len nodes after
+            // offsets[0]; that also bounds its slice of the reserve
+            if (a < off0 || b < a || b - a > len || b - off0 > (c + 1) * (long long)len) {
+                atomicOr(&hdr->status, ERR_BAD_CHAIN);
+                n = 0;
+                return;
+            }
+            start = wstart = a;
+            n = (int)(b - a);
+        } else {
+            start = c * (long long)len;
+            wstart = c * o.wrow;
+        }
+    }
+    __device__ float2 *spill(const SplitView &o, long long c, long long start, int n) const
+    {
+        return o.spill + (offsets ? 2 * (start - off0) + 2 * c : c * (2LL * n + 2));
+    }
+    __device__ void done_block() const
+    {
+        if (v.mode != SPLIT_ROW || !ticket) return;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            if (atomicAdd(ticket, 1u) == gridDim.x - 1) {
+                __threadfence();
+                *ticket = 0;
+                *k = *k + 1;
+            }
+        }
+    }
+};
+
+// SRC: bind(block, nch, view, k0, cnt) the chains k0 .. k0 + cnt - 1 of this block;
+// chain(view, k, start, wstart, n) one of them (n = 0: skip); spill(view, k, start, n);
+// done_block() at the block's end.
+template <int W, bool UNI, class SRC>
+__global__ void __launch_bounds__(split_threads<W>(), W <= 2 ? 2 : 1)
+    split_kernel(SRC src, WsHeader *hdr, int nch, int cs)
+{
+    pdl_enter();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ SplitX<W> xall[split_threads<W>() / (WARP * W)];
+    float *smem = reinterpret_cast<float *>(smem_raw);
+    SplitView v;
+    long long k0;
+    int cnt;
+    if (!src.bind(blockIdx.x, nch, v, k0, cnt, hdr)) return;
+    const int g = threadIdx.x / (WARP * W);
+    long long start = 0, wstart = 0;
+    int n = 0;
+    if (v.cols) src.chain(v, k0, start, wstart, n, hdr);
+    else if (g < cnt) src.chain(v, k0 + g, start, wstart, n, hdr);
+    // chains that a launch for other lengths takes, and empty ones
+    if (split_pick<W, UNI>(n) == 0 || n <= src.n_lo) n = 0;
+    float2 *spill = src.spill(v, k0 + g, start, n);
+    if (n > 0) {
+        const int l = split_pick<W, UNI>(n);
+        if constexpr (W == 1) {
+            if (l == 4) split_chain<4, W, UNI>(v, smem, xall, nch, cs, k0, cnt, start, wstart, n, hdr, spill);
+            if (l == 8) split_chain<8, W, UNI>(v, smem, xall, nch, cs, k0, cnt, start, wstart, n, hdr, spill);
+        }
+        if constexpr (!UNI && W < 8) {
+            if (l == 12) split_chain<12, W, UNI>(v, smem, xall, nch, cs, k0, cnt, start, wstart, n, hdr, spill);
+            if (l == 20) split_chain<20, W, UNI>(v, smem, xall, nch, cs, k0, cnt, start, wstart, n, hdr, spill);
+        }
+        if (l == 16) split_chain<16, W, UNI>(v, smem, xall, nch, cs, k0, cnt, start, wstart, n, hdr, spill);
+        if constexpr (W < 8) {
+            if (l == 24) split_chain<24, W, UNI>(v, smem, xall, nch, cs, k0, cnt, start, wstart, n, hdr, spill);
+        }
+        if constexpr (UNI) {
+            if (l == 32) split_chain<32, W, UNI>(v, smem, xall, nch, cs, k0, cnt, start, wstart, n, hdr, spill);
+        }
+    }
+    src.done_block();
+}
+
+}  // namespace tvk
