@@ -25,7 +25,7 @@
 //
 // Solutions are sums of the values of a run over its length: all nodes of a run are bitwise
 // equal, and the rounding is that of one mean. The folded flows cost eps * |u| per run, so a
-// chain that is to be cut at a flow above 16 max |y| goes to the warp's dynamic program
+// chain that is to be cut at a flow above 16 max |y|, or whose values are not finite, goes to the warp's dynamic program
 // (coop_solve_chain, records and reserve in the workspace) instead.
 #pragma once
 #include "tv2d_common.cuh"
@@ -138,7 +138,7 @@ struct SplitX {
     float K[W];                   // head count
     float u[W], u2[W];            // flow of a (new) cut after the warp's last node
     float re[W];                  // r of that node
-    float amax[W];
+    unsigned amax[W];
     unsigned char cut[W], side[W], more[W], heavy[W];
     int bad;                      // the chain goes to the fallback
 };
@@ -234,7 +234,7 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
     const float4 *yp = reinterpret_cast<const float4 *>(sc + (wi * WARP + lane) * LP);
     float y[L], w[UNI ? 1 : L], r[L], z[L];
     unsigned C = 0;  // cuts (the edge after the node): chain end, padding, decoupled edges
-    float amax = 0.f;
+    unsigned ab = 0;  // bits of the largest |y|
     const int last = n - 1 - base;  // the chain's last node, in the lane's numbering
 #pragma unroll
     for (int q = 0; q < L / 4; ++q) {
@@ -245,7 +245,7 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
         y[4 * q + 3] = t.w;
     }
 #pragma unroll
-    for (int j = 0; j < L; ++j) amax = fmaxf(amax, fabsf(y[j]));
+    for (int j = 0; j < L; ++j) ab = max(ab, __float_as_uint(y[j]) & 0x7fffffffu);
     if constexpr (UNI) {
         const int k = max(0, min(L, last));  // nodes with an edge to the next one
         C = k >= L ? 0u : ((1u << (L - k)) - 1u) & ML;
@@ -269,14 +269,16 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
             C = C << 1 | (cut ? 1u : 0u);
         }
     }
-    amax = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(amax)));
+    ab = __reduce_max_sync(FULL, ab);
     if constexpr (W > 1) {
-        if (lane == 0) xc->amax[wi] = amax;
+        if (lane == 0) xc->amax[wi] = ab;
         if (lane == WARP - 1) xc->re[wi] = r[L - 1];
         split_sync<W>(bar);
 #pragma unroll
-        for (int q = 0; q < W; ++q) amax = fmaxf(amax, xc->amax[q]);
+        for (int q = 0; q < W; ++q) ab = max(ab, xc->amax[q]);
     }
+    if (ab >= 0x7f800000u) return false;  // not finite: as the dynamic program has it
+    const float amax = __uint_as_float(ab);
     unsigned H = 0;   // edges whose flow would swamp the values
     unsigned UP = 0;  // UNI: cuts with flow +w
     if constexpr (UNI) {
