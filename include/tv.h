@@ -240,6 +240,14 @@ tv_status tv_chain_solve_backward(const float *d_x, const float *d_grad_x,
                                   float *d_grad_y, float *d_grad_w, void *d_workspace,
                                   size_t workspace_bytes, tv_stream_t stream);
 
+/* tv_chain_solve_backward that also writes grad_w at a chain's last node, as 0 (no edge), so
+ * that a caller need not clear the array first. */
+tv_status tv_chain_solve_backward_full(const float *d_x, const float *d_grad_x,
+                                       const int64_t *d_offsets, int64_t num_chains,
+                                       int64_t max_len, float *d_grad_y, float *d_grad_w,
+                                       void *d_workspace, size_t workspace_bytes,
+                                       tv_stream_t stream);
+
 /* Bytes of workspace tv_chain_solve_columns needs for an H x W array. */
 size_t tv_columns_workspace_size(int64_t H, int64_t W);
 

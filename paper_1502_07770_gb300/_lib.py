@@ -47,6 +47,7 @@ SIGNATURES = {
     "tv_chain_solve": (ctypes.c_int, [_p, _p, ctypes.c_float, _p, _i64, _i64, _p, _p, _sz, _p]),
     "tv_chain_solve_noalloc": (ctypes.c_int, [_p, _p, ctypes.c_float, _p, _i64, _i64, _p, _p]),
     "tv_chain_solve_backward": (ctypes.c_int, [_p, _p, _p, _i64, _i64, _p, _p, _p, _sz, _p]),
+    "tv_chain_solve_backward_full": (ctypes.c_int, [_p, _p, _p, _i64, _i64, _p, _p, _p, _sz, _p]),
     "tv_columns_workspace_size": (_sz, [_i64, _i64]),
     "tv_chain_solve_columns": (ctypes.c_int,
                                [_p, _p, ctypes.c_float, _i64, _i64, _i64, _p, _p, _sz, _p]),
@@ -339,11 +340,14 @@ def chain_prox_backward(x, grad_x, offsets=None, max_len=None, with_w=False, ws=
             raise ValueError("max_len is required with offsets")
         offp = _ptr(offsets)
     gy = torch.empty_like(x)
-    gw = torch.zeros_like(x) if with_w else None
+    # rows: the kernel writes every entry; CSR chains need not cover the array
+    gw = None
+    if with_w:
+        gw = torch.empty_like(x) if offsets is None else torch.zeros_like(x)
     wsb = ws if ws is not None else workspace(256, x.device, "grad")
-    _check(lib.tv_chain_solve_backward(_ptr(x), _ptr(grad_x), offp, num_chains, max_len,
-                                       _ptr(gy), _ptr(gw), _ptr(wsb), wsb.numel(),
-                                       _stream(x.device)))
+    _check(lib.tv_chain_solve_backward_full(_ptr(x), _ptr(grad_x), offp, num_chains, max_len,
+                                            _ptr(gy), _ptr(gw), _ptr(wsb), wsb.numel(),
+                                            _stream(x.device)))
     return gy, gw
 
 
