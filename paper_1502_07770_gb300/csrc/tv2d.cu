@@ -69,6 +69,12 @@ __global__ void tv2d_init_state(Tv2dState *st, Tv2dParams *prm, int max_iters, d
     st->gap = nan("");
 }
 
+__global__ void tv2d_start(Tv2dState *st, Tv2dState first, WsHeader *hdr)
+{
+    if (threadIdx.x == 0) *st = first;
+    if (threadIdx.x < sizeof(WsHeader) / sizeof(int)) reinterpret_cast<int *>(hdr)[threadIdx.x] = 0;
+}
+
 // Warp-level completion counter: returns true in lane 0 of the last warp of the grid.
 __device__ __forceinline__ bool last_warp_done(unsigned *ticket, int lane)
 {
@@ -542,61 +548,81 @@ struct CoopColPhaseP {
 // neighbour of every pixel. One pass over the image; FP32 within a thread, FP64
 // across threads; the last block reduces the block partials in a fixed order and
 // raises the stop flag.
+//
+// A warp takes 32 columns of kGapRows consecutive rows and issues all their loads before it
+// uses one (the kernel is one image pass between two phases, bound by latency: 1024 x 1024
+// walked pixel by pixel with state, step size and FP64 division read first took 16 us); the
+// lower neighbour is the next row's value, the right one the next lane's.
 constexpr int kGapThreads = 256;
+constexpr int kGapRows = 8;
+constexpr int kGapTileRows = kGapThreads / WARP * kGapRows;
+constexpr int kGapMaxBlocks = 4096;
+
+__device__ __forceinline__ double warp_sum(double v)
+{
+#pragma unroll
+    for (int o = WARP / 2; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+    return v;
+}
+
+// Sum over the block in a fixed order; valid in thread 0.
+__device__ __forceinline__ double block_sum(double v, double *red)
+{
+    v = warp_sum(v);
+    __syncthreads();
+    if ((threadIdx.x & (WARP - 1)) == 0) red[threadIdx.x / WARP] = v;
+    __syncthreads();
+    double b = 0.0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < kGapThreads / WARP; ++w) b += red[w];
+    return b;
+}
 
 __global__ void __launch_bounds__(kGapThreads)
-    tv2d_gap_kernel(const float *f, const float *wh, const float *wv, float lam, long long H,
-                    long long W, const float *buf0, const float *buf1, Tv2dState *st,
-                    const Tv2dParams *prm, double *partials, double *gaps, unsigned *ticket)
+    tv2d_gap_kernel(const float *f, const float *wh, const float *wv, float lam, int H, int W,
+                    const float *x1, const float *x0, int k, float inv_tau, long long ctiles,
+                    long long tiles,
+                    Tv2dState *st, double *partials, double *gaps, unsigned *ticket)
 {
-    __shared__ double red[kGapThreads];
+    __shared__ double red[kGapThreads / WARP];
     __shared__ bool last;
     pdl_enter();
     if (st->done) return;
-    const int kp1 = st->k;  // x^{k+1} is the newest iterate
-    if (kp1 < 1) return;
-    const int k = kp1 - 1;
-    const float *x1 = (kp1 & 1) ? buf1 : buf0;  // x^{k+1}
-    const float *x0 = (kp1 & 1) ? buf0 : buf1;  // x^k
-    const float inv_tau = (float)(1.0 / prm[k].tau);
-    const long long N = H * W;
-    // grid-stride walk over the pixels; row and column advance incrementally
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    const long long dr = stride / W, dc = stride - dr * W;
-    long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    long long r = q / W, c = q - r * W;
+    const int lane = threadIdx.x & (WARP - 1), warp = threadIdx.x / WARP;
     double acc = 0.0;
-    float part = 0.f;
-    int cnt = 0;
-    for (; q < N; q += stride) {
-        const float xv = x1[q], fv = f[q];
-        const float z = xv + (xv - x0[q]) * inv_tau;
-        float t = 0.5f * (xv - fv) * (xv - fv) + 0.5f * (z - fv) * (z + fv);
-        if (c + 1 < W) t += (wh ? wh[r * (W - 1) + c] : lam) * fabsf(x1[q + 1] - xv);
-        if (r + 1 < H) t += (wv ? wv[q] : lam) * fabsf(x1[q + W] - xv);
-        part += t;
-        if (++cnt == 32) {  // FP32 over at most 32 pixels, FP64 beyond
-            acc += (double)part;
-            part = 0.f;
-            cnt = 0;
+    for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int c = (int)(tile % ctiles) * WARP + lane;
+        const int r0 = (int)(tile / ctiles) * kGapTileRows + warp * kGapRows;
+        float xv[kGapRows + 1], fv[kGapRows], xo[kGapRows], wd[kGapRows], wr[kGapRows], xe[kGapRows];
+#pragma unroll
+        for (int u = 0; u <= kGapRows; ++u) {
+            const int r = r0 + u;
+            const bool in = c < W && r < H;
+            const long long q = (long long)r * W + c;
+            xv[u] = in ? x1[q] : 0.f;
+            if (u == kGapRows) break;
+            fv[u] = in ? f[q] : 0.f;
+            xo[u] = in ? x0[q] : 0.f;
+            xe[u] = in && lane == WARP - 1 && c + 1 < W ? x1[q + 1] : 0.f;
+            wr[u] = in && c + 1 < W ? (wh ? wh[q - r] : lam) : 0.f;
+            wd[u] = in && r + 1 < H ? (wv ? wv[q] : lam) : 0.f;
         }
-        c += dc;
-        r += dr;
-        if (c >= W) {
-            c -= W;
-            ++r;
+        float part = 0.f;
+#pragma unroll
+        for (int u = 0; u < kGapRows; ++u) {
+            const float xn = __shfl_down_sync(FULL, xv[u], 1);
+            const float xr = lane == WARP - 1 ? xe[u] : xn;
+            const float z = xv[u] + (xv[u] - xo[u]) * inv_tau;
+            float t = 0.5f * (xv[u] - fv[u]) * (xv[u] - fv[u]) + 0.5f * (z - fv[u]) * (z + fv[u]);
+            if (wr[u] != 0.f) t += wr[u] * fabsf(xr - xv[u]);
+            if (wd[u] != 0.f) t += wd[u] * fabsf(xv[u + 1] - xv[u]);
+            part += t;
         }
+        acc += (double)part;  // FP32 over a thread's 8 pixels, FP64 beyond
     }
-    acc += (double)part;
-    // block sum in a fixed order
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int h = kGapThreads / 2; h > 0; h >>= 1) {
-        if ((int)threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
-        __syncthreads();
-    }
+    acc = block_sum(acc, red);
     if (threadIdx.x == 0) {
-        partials[blockIdx.x] = red[0];
+        partials[blockIdx.x] = acc;
         __threadfence();
         last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     }
@@ -605,18 +631,13 @@ __global__ void __launch_bounds__(kGapThreads)
     // the last block sums the block partials in a fixed order
     __threadfence();
     double b = 0.0;
-    for (unsigned bq = threadIdx.x; bq < gridDim.x; bq += blockDim.x)
-        b += __ldcg(partials + bq);
-    red[threadIdx.x] = b;
-    __syncthreads();
-    for (int h = kGapThreads / 2; h > 0; h >>= 1) {
-        if ((int)threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
-        __syncthreads();
-    }
+    for (unsigned bq = threadIdx.x; bq < gridDim.x; bq += blockDim.x) b += __ldcg(partials + bq);
+    b = block_sum(b, red);
     if (threadIdx.x == 0) {
-        const double g = red[0] * st->inv_N;
+        const double g = b * st->inv_N;
         st->gap = g;
         st->gap_k = k;
+        st->k = k + 1;
         gaps[k] = g;
         if (st->tol > 0.0 && g <= st->tol) st->done = 1;
         *ticket = 0;
@@ -636,6 +657,7 @@ struct Tv2dWs {
     double *gaps, *partials;
     WsHeader *hdr;
     float *y, *buf1;
+    const float *y0;  // where the first phases read the dual (NULL: 0)
     float2 *rec;
     float *crec;
     float2 *spill;
@@ -653,9 +675,10 @@ Tv2dWs carve_tv2d(void *base, long long H, long long W, int max_iters)
     o.st = cv.take<Tv2dState>(1);
     o.prm = cv.take<Tv2dParams>((size_t)max_iters + 2);
     o.gaps = cv.take<double>((size_t)max_iters + 2);
-    o.partials = cv.take<double>((size_t)4096);  // one per block of the gap kernel
+    o.partials = cv.take<double>((size_t)kGapMaxBlocks);  // one per block of the gap kernel
     o.hdr = cv.take<WsHeader>(1);
     o.y = cv.take<float>((size_t)(H * W));
+    o.y0 = o.y;
     o.buf1 = cv.take<float>((size_t)(H * W));
     const long long rec_rows = wr * W, rec_cols = wc * H;
     o.rec = cv.take<float2>((size_t)((rec_rows > rec_cols ? rec_rows : rec_cols) * WARP));
@@ -667,46 +690,81 @@ Tv2dWs carve_tv2d(void *base, long long H, long long W, int max_iters)
     return o;
 }
 
+// One iteration's step sizes and place in the schedule (the host's copy of Tv2dParams).
+struct Step {
+    int k = 0;
+    double tau = 1.0, sigma = 1.0, theta_prev = 0.0;
+    void next()
+    {
+        const double theta = 1.0 / sqrt(1.0 + 2.0 * tau);
+        tau *= theta;
+        sigma /= theta;
+        theta_prev = theta;
+        ++k;
+    }
+};
+
 // The phases on the threshold-splitting kernel (tv_split.cuh): rows or columns of the image.
 SplitSrc split_src(SplitMode mode, const float *img, const float *w, float lam, long long H,
-                   long long W, float *x0, const Tv2dWs &ws)
+                   long long W, const Step &it, float *x0, const Tv2dWs &ws)
 {
     SplitSrc src{};
     SplitView &v = src.v;
     const bool cols = mode == SPLIT_COL;
+    float *xc = (it.k & 1) ? ws.buf1 : x0, *xo = (it.k & 1) ? x0 : ws.buf1;
     v.mode = mode;
     v.cols = cols;
-    v.p0 = img;
-    v.p1 = ws.y;
-    if (cols) v.p2 = ws.y;
     v.pw = w;
     v.lam = lam;
     v.ws = 1.f;
-    v.o0 = cols ? ws.y : x0;
-    v.o1 = ws.buf1;
+    if (mode == SPLIT_INIT) {
+        v.p0 = img;
+        v.p1 = ws.y0;
+        v.o0 = x0;
+        v.o1 = ws.buf1;
+    } else if (mode == SPLIT_ROW) {
+        v.p0 = img;
+        v.p1 = ws.y;
+        v.p2 = xc;
+        v.o0 = xo;
+        v.ca = v.ws = (float)(it.tau / (it.tau + 1.0));
+        v.cb = (float)(1.0 / (it.tau + 1.0));
+    } else {
+        v.p0 = xc;
+        v.p1 = xo;
+        v.p2 = it.k == 0 ? ws.y0 : ws.y;
+        v.o0 = ws.y;
+        v.ca = v.ws = (float)(1.0 / it.sigma);
+        v.cb = (float)it.theta_prev;
+        v.sg = (float)it.sigma;
+    }
     v.stride = cols ? W : 1;
     v.wrow = W - 1;
     v.rec = ws.rec;
     v.spill = ws.spill;
     v.maxlen = (int)(cols ? H : W);
     src.nchains = cols ? W : H;
-    src.len = (int)(cols ? H : W);
-    src.buf0 = x0;
-    src.buf1 = ws.buf1;
-    src.y = ws.y;
-    src.k = &ws.st->k;
-    src.done = &ws.st->done;
-    src.prm = ws.prm;
-    src.ticket = &ws.st->ticket_row;
+    src.len = v.maxlen;
+    src.done = mode == SPLIT_INIT ? nullptr : &ws.st->done;
     return src;
+}
+
+bool split_rows(long long H, long long W, const float *wh)
+{
+    return split_takes(W, H, split_max_chains(W, false, false, wh != nullptr));
+}
+bool split_cols(long long H, long long W, const float *wv)
+{
+    return split_takes(H, W, split_max_chains(H, true, false, wv != nullptr));
 }
 
 template <bool HAS_WH>
 tv_status launch_init(const float *img, const float *wh, float lam, long long H, long long W,
                       float *x0, const Tv2dWs &ws, cudaStream_t s)
 {
-    if (split_takes(W, H, split_max_chains(W, false, false, wh != nullptr)))
-        return launch_split(split_src(SPLIT_INIT, img, wh, lam, H, W, x0, ws), ws.hdr, s, PK_INIT);
+    if (split_rows(H, W, wh))
+        return launch_split(split_src(SPLIT_INIT, img, wh, lam, H, W, Step(), x0, ws), ws.hdr, s,
+                            PK_INIT);
     if (H <= coop_max_chains()) {
         CoopInitRowsP<HAS_WH> p{img, ws.y, wh, lam, H, W, x0, ws.buf1};
         return launch_coop(p, H, (int)W, ws.rec, nullptr, ws.spill, ws.hdr, s, PK_INIT);
@@ -717,13 +775,10 @@ tv_status launch_init(const float *img, const float *wh, float lam, long long H,
 
 template <bool HAS_WH>
 tv_status launch_row(const float *img, const float *wh, float lam, long long H, long long W,
-                     int max_iters, float *x0, const Tv2dWs &ws, cudaStream_t s)
+                     const Step &it, float *x0, const Tv2dWs &ws, cudaStream_t s)
 {
-    if (split_takes(W, H, split_max_chains(W, false, false, wh != nullptr))) {
-        SplitSrc src = split_src(SPLIT_ROW, img, wh, lam, H, W, x0, ws);
-        src.max_iters = max_iters;
-        return launch_split(src, ws.hdr, s, PK_ROW);
-    }
+    if (split_rows(H, W, wh))
+        return launch_split(split_src(SPLIT_ROW, img, wh, lam, H, W, it, x0, ws), ws.hdr, s, PK_ROW);
     if (H <= coop_max_chains()) {
         CoopRowPhaseP<HAS_WH> p{img, ws.y, wh, lam, H, W, x0, ws.buf1, ws.st, ws.prm,
                                 nullptr, nullptr, 0.f, 0.f};
@@ -735,11 +790,12 @@ tv_status launch_row(const float *img, const float *wh, float lam, long long H, 
 }
 
 template <bool HAS_WV>
-tv_status launch_col(const float *wv, float lam, long long H, long long W, float *x0,
-                     const Tv2dWs &ws, cudaStream_t s)
+tv_status launch_col(const float *wv, float lam, long long H, long long W, const Step &it,
+                     float *x0, const Tv2dWs &ws, cudaStream_t s)
 {
-    if (split_takes(H, W, split_max_chains(H, true, false, wv != nullptr)))
-        return launch_split(split_src(SPLIT_COL, nullptr, wv, lam, H, W, x0, ws), ws.hdr, s, PK_COL);
+    if (split_cols(H, W, wv))
+        return launch_split(split_src(SPLIT_COL, nullptr, wv, lam, H, W, it, x0, ws), ws.hdr, s,
+                            PK_COL);
     if (W <= coop_max_chains()) {
         CoopColPhaseP<HAS_WV> p{wv, lam, H, W, x0, ws.buf1, ws.y, ws.st, ws.prm,
                                 nullptr, nullptr, 0.f, 0.f, 0.f};
@@ -750,28 +806,24 @@ tv_status launch_col(const float *wv, float lam, long long H, long long W, float
     return launch(p, W, ws.rec, ws.crec, ws.spill, ws.hdr, s, PK_COL);
 }
 
-tv_status launch_col_any(const float *wv, float lam, long long H, long long W, float *x0,
-                         const Tv2dWs &ws, cudaStream_t s)
+tv_status launch_col_any(const float *wv, float lam, long long H, long long W, const Step &it,
+                         float *x0, const Tv2dWs &ws, cudaStream_t s)
 {
-    return wv ? launch_col<true>(wv, lam, H, W, x0, ws, s)
-              : launch_col<false>(wv, lam, H, W, x0, ws, s);
-}
-
-int gap_blocks(long long H, long long W)
-{
-    long long b = (H * W + kGapThreads * 8 - 1) / (kGapThreads * 8);
-    const long long cap = 4LL * sm_count_current();
-    return (int)(b < 1 ? 1 : (b > cap ? cap : b));
+    return wv ? launch_col<true>(wv, lam, H, W, it, x0, ws, s)
+              : launch_col<false>(wv, lam, H, W, it, x0, ws, s);
 }
 
 tv_status launch_gap(const float *img, const float *wh, const float *wv, float lam, long long H,
-                     long long W, float *x0, const Tv2dWs &ws, cudaStream_t s)
+                     long long W, const Step &it, float *x0, const Tv2dWs &ws, cudaStream_t s)
 {
-    const int blocks = gap_blocks(H, W);
+    const float *xn = (it.k & 1) ? x0 : ws.buf1, *xp = (it.k & 1) ? ws.buf1 : x0;
+    const long long ctiles = (W + WARP - 1) / WARP;
+    const long long tiles = ctiles * ((H + kGapTileRows - 1) / kGapTileRows);
+    const int blocks = (int)std::min<long long>(tiles, kGapMaxBlocks);
     tv_status st = check_cuda(launch_k(tv2d_gap_kernel, dim3(blocks), dim3(kGapThreads), 0, s, img,
-                                       wh, wv, lam, H, W, (const float *)x0,
-                                       (const float *)ws.buf1, ws.st, (const Tv2dParams *)ws.prm,
-                                       ws.partials, ws.gaps, &ws.st->ticket_col),
+                                       wh, wv, lam, (int)H, (int)W, xn, xp, it.k,
+                                       (float)(1.0 / it.tau), ctiles, tiles, ws.st, ws.partials,
+                                       ws.gaps, &ws.st->ticket_col),
                               "gap kernel launch");
     if (st == TV_OK) note_launch();
     return st;
@@ -854,32 +906,35 @@ tv_status tv2d_denoise(const float *d_img, int64_t H, int64_t W, const float *d_
     ws.vec_rows = ws.vec_cols = (W % 4 == 0) && aligned16(d_img) && aligned16(d_x);
     cudaStream_t s = (cudaStream_t)stream;
     tv_status st;
-    {
+    const bool split = split_rows(H, W, d_wh) && split_cols(H, W, d_wv);
+    if (split) {
+        // the phases take step sizes from the host, and the first ones read d_y0 itself, or 0
+        ws.y0 = d_y0;
+        Tv2dState first{};
+        first.max_iters = max_iters;
+        first.gap_k = -1;
+        first.tol = gap_tol;
+        first.inv_N = 1.0 / ((double)H * W);
+        first.gap = NAN;
+        tv2d_start<<<1, WARP, 0, s>>>(ws.st, first, ws.hdr);
+        if ((st = check_cuda(cudaGetLastError(), "start")) != TV_OK) return st;
+        note_launch();
+    } else {
         // step sizes of eq. pd, FP64 on the host
         static thread_local ParamChunk chunk;
-        double tau = 1.0, sigma = 1.0, theta_prev = 0.0, tau_prev = 1.0;
         for (int first = 0; first <= max_iters; first += kParamChunk) {
-            chunk.first = first;
-            chunk.count = (max_iters + 1 - first) < kParamChunk ? (max_iters + 1 - first) : kParamChunk;
-            for (int q = 0; q < chunk.count; ++q) {
-                chunk.p[q] = Tv2dParams{tau, sigma, theta_prev, tau_prev};
-                const double theta = 1.0 / sqrt(1.0 + 2.0 * tau);
-                tau_prev = tau;
-                tau *= theta;
-                sigma /= theta;
-                theta_prev = theta;
-            }
+            fill_params(chunk, first, std::min(kParamChunk, max_iters + 1 - first));
             tv2d_init_state<<<1, 128, 0, s>>>(ws.st, ws.prm, max_iters, gap_tol,
                                               1.0 / ((double)H * W), chunk);
             if ((st = check_cuda(cudaGetLastError(), "init state")) != TV_OK) return st;
             note_launch();
         }
+        if ((st = check_cuda(cudaMemsetAsync(ws.hdr, 0, sizeof(WsHeader), s), "memset")) != TV_OK)
+            return st;
+        st = d_y0 ? check_cuda(cudaMemcpyAsync(ws.y, d_y0, npx, cudaMemcpyDeviceToDevice, s), "copy y0")
+                  : check_cuda(cudaMemsetAsync(ws.y, 0, npx, s), "zero y");
+        if (st != TV_OK) return st;
     }
-    if ((st = check_cuda(cudaMemsetAsync(ws.hdr, 0, sizeof(WsHeader), s), "memset")) != TV_OK)
-        return st;
-    st = d_y0 ? check_cuda(cudaMemcpyAsync(ws.y, d_y0, npx, cudaMemcpyDeviceToDevice, s), "copy y0")
-              : check_cuda(cudaMemsetAsync(ws.y, 0, npx, s), "zero y");
-    if (st != TV_OK) return st;
     // launches of the two phases timed before this call (benchmark profiling only)
     const bool prof = prof_on();
     const size_t prof_col0 = prof ? prof_pending(PK_COL) : 0;
@@ -910,17 +965,19 @@ tv_status tv2d_denoise(const float *d_img, int64_t H, int64_t W, const float *d_
         return r;
     };
     Tv2dState hs;
+    Step it;
     int launched = 0;
     bool done = false;
     while (launched < max_iters && !done) {
         const int batch = launched == 0 ? 6 : 3;
         const int u = (max_iters - launched) < batch ? (max_iters - launched) : batch;
         for (int t = 0; t < u; ++t) {
-            if ((st = launch_col_any(d_wv, lambda, H, W, d_x, ws, s)) != TV_OK) return st;
-            st = d_wh ? launch_row<true>(d_img, d_wh, lambda, H, W, max_iters, d_x, ws, s)
-                      : launch_row<false>(d_img, d_wh, lambda, H, W, max_iters, d_x, ws, s);
+            if ((st = launch_col_any(d_wv, lambda, H, W, it, d_x, ws, s)) != TV_OK) return st;
+            st = d_wh ? launch_row<true>(d_img, d_wh, lambda, H, W, it, d_x, ws, s)
+                      : launch_row<false>(d_img, d_wh, lambda, H, W, it, d_x, ws, s);
             if (st != TV_OK) return st;
-            if ((st = launch_gap(d_img, d_wh, d_wv, lambda, H, W, d_x, ws, s)) != TV_OK) return st;
+            if ((st = launch_gap(d_img, d_wh, d_wv, lambda, H, W, it, d_x, ws, s)) != TV_OK) return st;
+            it.next();
         }
         launched += u;
         if ((st = launch_copy()) != TV_OK) return st;

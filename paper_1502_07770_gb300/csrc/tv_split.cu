@@ -34,38 +34,42 @@ tv_status launch_u(SplitSrc src, WsHeader *hdr, cudaStream_t s)
     tv_status st = TV_OK;
     const int n = src.len;
     src.n_lo = 0;
-    // warps per chain: what one, two and four hold (eight: 16 nodes a lane)
-    constexpr int N1 = (UNI ? 32 : 24) * WARP, N2 = 2 * N1, N4 = 4 * N1;
-    static_assert(N4 >= kSplitMaxLen || !UNI, "lengths");
+    src.lanes = 0;
+    constexpr int N1 = 32 * WARP, N2 = 2 * N1;  // what one warp and two hold
+    static_assert(kSplitMaxLen <= 4 * N1, "lengths");
     if (src.v.cols) {
         // neighbouring columns share a block: 16- to 32-byte pieces of each row, unless there
         // are too few columns to occupy every SM that way
-        int nch = n <= N1 ? 8 : (n <= N4 ? 4 : 2);
+        int nch = n <= N1 ? 8 : 4;
         while (nch > 2 && src.nchains < 3LL * sms * nch / 2) nch /= 2;
-        if (n <= N1) return launch_w<1, UNI>(src, split_pick<1, UNI>(n), nch, hdr, s);
-        if (n <= N2) return launch_w<2, UNI>(src, split_pick<2, UNI>(n), nch, hdr, s);
-        if (n <= N4) return launch_w<4, UNI>(src, split_pick<4, UNI>(n), nch, hdr, s);
-        if constexpr (!UNI) return launch_w<8, UNI>(src, split_pick<8, UNI>(n), nch, hdr, s);
-        return TV_OK;
+        if (n <= N1) return launch_w<1, UNI>(src, split_pick<1>(n), nch, hdr, s);
+        if (n <= N2) return launch_w<2, UNI>(src, split_pick<2>(n), nch, hdr, s);
+        return launch_w<4, UNI>(src, split_pick<4>(n), nch, hdr, s);
     }
     const int nch = src.nchains <= 16LL * sms ? 1 : 2;
-    const bool all = src.offsets != nullptr;  // lengths vary: one launch per length class
-    if (all || n <= N1)
-        st = launch_w<1, UNI>(src, split_pick<1, UNI>(n <= N1 ? n : N1), nch, hdr, s);
-    if (st == TV_OK && n > N1 && (all || n <= N2)) {
-        src.n_lo = all ? N1 : 0;
-        st = launch_w<2, UNI>(src, split_pick<2, UNI>(n <= N2 ? n : N2), 1, hdr, s);
+    if (!src.offsets) {
+        if (n <= N1) return launch_w<1, UNI>(src, split_pick<1>(n), nch, hdr, s);
+        if (n <= N2) return launch_w<2, UNI>(src, split_pick<2>(n), 1, hdr, s);
+        return launch_w<4, UNI>(src, split_pick<4>(n), 1, hdr, s);
     }
-    if (st == TV_OK && n > N2 && (all || n <= N4)) {
-        src.n_lo = all ? N2 : 0;
-        st = launch_w<4, UNI>(src, split_pick<4, UNI>(n <= N4 ? n : N4), 1, hdr, s);
+    // Lengths vary: one launch per number of warps, each with the one variant that holds its
+    // longest chain (and 4 or 8 nodes a lane up to 256). The unrolled loop of a variant (up to
+    // 20 KB) fits the instruction cache and several do not: 6000 chains of 1 to 2500 nodes, each
+    // with the variant of its own length, took 239-415 us, most of it waiting for instructions.
+    auto place = [&](int n_lo, int lanes) {
+        src.n_lo = n_lo;
+        src.lanes = lanes;
+    };
+    if (n > N2) {
+        place(N2, split_pick<4>(n));
+        st = launch_w<4, UNI>(src, src.lanes, 1, hdr, s);
     }
-    if constexpr (!UNI) {
-        if (st == TV_OK && n > N4) {
-            src.n_lo = all ? N4 : 0;
-            st = launch_w<8, UNI>(src, split_pick<8, UNI>(n), 1, hdr, s);
-        }
+    if (st == TV_OK && n > N1) {
+        place(N1, split_pick<2>(n <= N2 ? n : N2));
+        st = launch_w<2, UNI>(src, src.lanes, 1, hdr, s);
     }
+    place(0, split_pick<1>(n <= N1 ? n : N1));
+    if (st == TV_OK) st = launch_w<1, UNI>(src, src.lanes, nch, hdr, s);
     return st;
 }
 

@@ -33,8 +33,9 @@
 
 namespace tvk {
 
-constexpr int kSplitMaxLen = 4096;     // nodes of the longest chain (8 warps x 32 lanes x 16)
+constexpr int kSplitMaxLen = 4096;     // nodes of the longest chain (4 warps x 32 lanes x 32)
 constexpr float kSplitHeavy = 16.f;
+constexpr float kSplitTiny = 1e-37f;  // weights up to here decouple
 
 // What a chain's nodes are made of. PLAIN: c = y. INIT, ROW, COL: the set-up of the phases
 // of eq. pd (x^0 rows, primal rows, dual columns).
@@ -191,13 +192,12 @@ __device__ __forceinline__ float fma_sat(float a, float b, float c)
     asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
-// y0 += u, y1 -= u and r = w = 0 where bit is set: predicated, the lanes differ
-__device__ __forceinline__ void cut_at(unsigned bit, float u, float &y0, float &y1, float &r,
-                                       float &w)
+// y0 += u, y1 -= u and w = 0 where bit is set: predicated, the lanes differ
+__device__ __forceinline__ void cut_at(unsigned bit, float u, float &y0, float &y1, float &w)
 {
-    asm("{\n .reg .pred p;\n setp.ne.u32 p, %5, 0;\n @p add.f32 %0, %0, %4;\n"
-        " @p sub.f32 %1, %1, %4;\n @p mov.f32 %2, 0f00000000;\n @p mov.f32 %3, 0f00000000;\n}"
-        : "+f"(y0), "+f"(y1), "+f"(r), "+f"(w)
+    asm("{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n @p add.f32 %0, %0, %3;\n"
+        " @p sub.f32 %1, %1, %3;\n @p mov.f32 %2, 0f00000000;\n}"
+        : "+f"(y0), "+f"(y1), "+f"(w)
         : "f"(u), "r"(bit));
 }
 __device__ __forceinline__ void cut_at_unit(unsigned bit, unsigned up, float &y0, float &y1,
@@ -214,8 +214,8 @@ __device__ __forceinline__ void cut_at_unit(unsigned bit, unsigned up, float &y0
 // the solution to sx. Returns false (in every lane) if the chain needs the fallback.
 //
 // The walks are bound by issue and by the half-rate ALU pipe (minima, selects, logic), so
-// what can be arithmetic on the FMA pipe is: r[j] is 1, or 0 where the chain is cut after node
-// j, and a sum that restarts at cuts is s = fma(s, r, y). Node j of a lane is bit L-1-j of
+// what can be arithmetic on the FMA pipe is: with r = 1, or 0 where the chain is cut after a
+// node, a sum that restarts at cuts is s = fma(s, r, y). Node j of a lane is bit L-1-j of
 // its masks.
 //
 // UNI: one weight lamw for every edge. Values are divided by 2 lamw and messages shifted to
@@ -232,7 +232,7 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
     constexpr unsigned ML = L == 32 ? 0xffffffffu : (1u << L) - 1u;
     const int base = (wi * WARP + lane) * L;
     const float4 *yp = reinterpret_cast<const float4 *>(sc + (wi * WARP + lane) * LP);
-    float y[L], w[UNI ? 1 : L], r[L], z[L];
+    float y[L], w[UNI ? 1 : L], r[UNI ? L : 1], z[L];
     unsigned C = 0;  // cuts (the edge after the node): chain end, padding, decoupled edges
     unsigned ab = 0;  // bits of the largest |y|
     const int last = n - 1 - base;  // the chain's last node, in the lane's numbering
@@ -263,16 +263,15 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
         }
 #pragma unroll
         for (int j = 0; j < L; ++j) {
-            const bool cut = !(w[j] > 0.f);
+            const bool cut = !(w[j] > kSplitTiny);
             w[j] = cut ? 0.f : w[j];
-            r[j] = cut ? 0.f : 1.f;
             C = C << 1 | (cut ? 1u : 0u);
         }
     }
     ab = __reduce_max_sync(FULL, ab);
     if constexpr (W > 1) {
         if (lane == 0) xc->amax[wi] = ab;
-        if (lane == WARP - 1) xc->re[wi] = r[L - 1];
+        if (UNI && lane == WARP - 1) xc->re[wi] = r[UNI ? L - 1 : 0];
         split_sync<W>(bar);
 #pragma unroll
         for (int q = 0; q < W; ++q) ab = max(ab, xc->amax[q]);
@@ -282,7 +281,7 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
     unsigned H = 0;   // edges whose flow would swamp the values
     unsigned UP = 0;  // UNI: cuts with flow +w
     if constexpr (UNI) {
-        if (!(lamw > 1e-30f * amax && lamw > 1e-37f)) {  // no weight to speak of: x = y
+        if (!(lamw > 1e-30f * amax && lamw > kSplitTiny)) {  // no weight to speak of: x = y
             float4 *xp = reinterpret_cast<float4 *>(sx + (wi * WARP + lane) * LP);
 #pragma unroll
             for (int q = 0; q < L / 4; ++q) xp[q] = yp[q];
@@ -303,6 +302,12 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
             if (w[j] > kSplitHeavy * amax) H |= 1u << (L - 1 - j);
     }
 
+    // 1, or 0 where the chain is cut after node j: kept for one weight, for a weight per edge
+    // made from it (a register per node less, so 32 nodes a lane fit)
+    auto keep = [&](int j) {
+        if constexpr (UNI) return r[j];
+        else return __saturatef(w[j] * 3e38f);
+    };
     const bool any_heavy = __any_sync(FULL, H != 0);
     unsigned bc = __ballot_sync(FULL, C != 0);  // lanes with a cut
     float re = 0.f;  // UNI: r of the edge into the lane's first node
@@ -317,8 +322,9 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
         float Sh = 0.f, St = 0.f, b = 1.f;  // to the lane's first cut; after its last one
 #pragma unroll
         for (int j = L - 1; j >= 0; --j) {
-            Sh = fmaf(Sh, r[j], y[j]);
-            b *= r[j];
+            const float rj = keep(j);
+            Sh = fmaf(Sh, rj, y[j]);
+            b *= rj;
             St = fmaf(b, y[j], St);
         }
         const float kh = C ? (float)(__clz(C) - (31 - L)) : (float)L;  // nodes of the head
@@ -410,8 +416,9 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
         if (!more) {  // no cut in the last round: the runs are the solution
 #pragma unroll
             for (int j = L - 1; j >= 0; --j) {
-                s = fmaf(s, r[j], y[j]);
-                k = fmaf(k, r[j], 1.f);
+                const float rj = keep(j);
+                s = fmaf(s, rj, y[j]);
+                k = fmaf(k, rj, 1.f);
                 z[j] = mean_of(s, k);
             }
             const unsigned LC = C & (0u - C);
@@ -432,8 +439,9 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
         }
 #pragma unroll
         for (int j = L - 1; j >= 0; --j) {
-            s = fmaf(s, r[j], y[j]);
-            k = fmaf(k, r[j], 1.f);
+            const float rj = keep(j);
+            s = fmaf(s, rj, y[j]);
+            k = fmaf(k, rj, 1.f);
             z[j] = s * rcp_approx(k);
         }
 
@@ -441,7 +449,7 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
         float a = 0.f, lo = 0.f, hi = 0.f;
 #pragma unroll
         for (int j = 0; j < L; ++j) {
-            if (j > 0 && r[j > 0 ? j - 1 : 0] == 0.f) zr = z[j];
+            if (j > 0 && (UNI ? r : w)[j > 0 ? j - 1 : 0] == 0.f) zr = z[j];
             const float d = zr - y[j];
             z[j] = d;
             a += d;
@@ -585,7 +593,7 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
                 const unsigned bit = 1u << (L - 1 - j);
                 float &yn = j + 1 < L ? y[j + 1 < L ? j + 1 : 0] : dummy;
                 if constexpr (UNI) cut_at_unit(fresh & bit, upf & bit, y[j], yn, r[j]);
-                else cut_at(fresh & bit, z[j], y[j], yn, r[j], w[j]);
+                else cut_at(fresh & bit, z[j], y[j], yn, w[j]);
             }
         }
         C |= fresh;
@@ -653,9 +661,9 @@ struct UnitStride {  // of rows: known at compile time
 // a time.
 template <int L, int W, bool UNI>
 __device__ __forceinline__ void split_chain(const SplitView &v, float *smem, SplitX<W> *xall,
-                                            int nch, int cs, long long k0, int cnt, long long start,
-                                            long long wstart, int n, WsHeader *hdr,
-                                            float2 *spill)
+                                            int nch, int cs, long long k0, int cnt, long long kc,
+                                            long long start, long long wstart, int n,
+                                            WsHeader *hdr, float2 *spill)
 {
     constexpr int LP = split_lp<L>();
     constexpr int T = W * WARP;
@@ -675,7 +683,7 @@ __device__ __forceinline__ void split_chain(const SplitView &v, float *smem, Spl
         const long long step = T * (long long)stride, o0 = ll * (long long)stride;
         const float *q0 = v.p0 + st + o0, *q1 = v.p1 + st + o0, *q2 = v.p2 + st + o0,
                     *qw = v.pw + wst + o0;
-        const bool h1 = v.p1 != nullptr, h2 = v.p2 != nullptr;
+        const bool h1 = v.p1 != nullptr, h2 = v.p2 != nullptr, hw = v.pw != nullptr;
         const int nn = in ? n : 0;
 #pragma unroll 1
         for (int b0 = 0; b0 < L; b0 += UL) {
@@ -687,7 +695,7 @@ __device__ __forceinline__ void split_chain(const SplitView &v, float *smem, Spl
                 a[u] = ok ? q0[u * step] : 0.f;
                 b[u] = ok && h1 ? q1[u * step] : 0.f;
                 c[u] = ok && h2 ? q2[u * step] : 0.f;
-                if constexpr (!UNI) e[u] = i < nn - 1 ? qw[u * step] : 0.f;
+                if constexpr (!UNI) e[u] = i < nn - 1 ? (hw ? qw[u * step] : v.lam) : 0.f;
             }
 #pragma unroll
             for (int u = 0; u < UL; ++u) {
@@ -731,24 +739,24 @@ __device__ __forceinline__ void split_chain(const SplitView &v, float *smem, Spl
     }
     if (!good && wi == 0) {
         SplitView vv = v;
-        split_fallback(vv, k0 + g, v.cols ? k0 + g : start, v.cols ? k0 + g : wstart, n, lane, spill,
-                       hdr);
+        split_fallback(vv, kc, v.cols ? kc : start, v.cols ? kc : wstart, n, lane, spill, hdr);
     }
 }
 
-// Nodes per lane for a chain of n nodes (0: longer than W warps hold). With one weight three
-// arrays of 32 registers fit a lane, with a weight per edge four of 24.
-template <int W, bool UNI>
+// Nodes per lane for a chain of n nodes (0: longer than W warps hold). Three arrays of 32
+// registers fit a lane.
+template <int W>
 __host__ __device__ constexpr int split_pick(int n)
 {
     constexpr int T = 32 * W;
     if (W == 1 && n <= 4 * T) return 4;
     if (W == 1 && n <= 8 * T) return 8;
-    if (!UNI && W < 8 && n <= 12 * T) return 12;
+    if (W == 1 && n <= 12 * T) return 12;
     if (n <= 16 * T) return 16;
-    if (!UNI && W < 8 && n <= 20 * T) return 20;
-    if (W < 8 && n <= 24 * T) return 24;
-    return UNI && n <= 32 * T ? 32 : 0;
+    if (n <= 20 * T) return 20;
+    if (n <= 24 * T) return 24;
+    if (n <= 28 * T) return 28;
+    return n <= 32 * T ? 32 : 0;
 }
 
 // Floats of one chain's slot array (values; the weights or solutions take another).
@@ -756,6 +764,14 @@ template <int W>
 __host__ __device__ constexpr int split_slots(int l, int nch)
 {
     return 32 * W * ((l / 4) % 2 == 1 ? l : l + 4) + 32 / nch;
+}
+
+// Shared memory of the largest block of split_kernel<W>.
+template <int W>
+constexpr size_t split_smem_most()
+{
+    const int nch = W == 1 ? 8 : 4;
+    return 2 * (size_t)nch * split_slots<W>(32, nch) * sizeof(float);
 }
 
 template <int W>
@@ -782,21 +798,17 @@ __device__ __forceinline__ bool csr_disjoint(const float *x, const float *y, con
 }
 
 // Chains of one array (tv_chain_solve, tv_chain_solve_columns) or of one image (the phases of
-// the 2D solvers).
+// the 2D solvers). The host fills the view, iterates and step sizes included: read from device
+// state they cost each phase a chain of dependent loads and FP64 divisions.
 struct SplitSrc {
-    SplitView v;  // filled by the host; the phases resolve iterates and step sizes here
+    SplitView v;
     long long nchains;
     int len;                 // chain length, or with offsets the longest
     const int64_t *offsets;  // CSR rows, or NULL
-    int n_lo;                // with offsets: chains of n_lo < n <= what the kernel holds
+    int n_lo;                // chains of more than n_lo nodes only
+    int lanes;               // nodes a lane takes (0: by the chain's length)
     long long off0;
-    // phases of eq. pd
-    float *buf0, *buf1, *y;
-    int *k;                  // iteration (NULL: step sizes given in v)
-    const int *done;
-    int max_iters;
-    const Tv2dParams *prm;
-    unsigned *ticket;        // ROW: blocks finished; the last one advances *k
+    const int *done;         // phases of eq. pd: the solve's stop flag, or NULL
 
     __device__ bool bind(unsigned blk, int nch, SplitView &o, long long &k0, int &cnt,
                          WsHeader *hdr)
@@ -812,24 +824,7 @@ struct SplitSrc {
                 return false;
             }
         }
-        if (v.mode >= SPLIT_ROW && k) {
-            const int it = *k;
-            if (*done || (v.mode == SPLIT_ROW && it >= max_iters)) return false;
-            const Tv2dParams &p = prm[it];
-            float *xc = (it & 1) ? buf1 : buf0, *xo = (it & 1) ? buf0 : buf1;
-            if (v.mode == SPLIT_ROW) {
-                o.p2 = xc;
-                o.o0 = xo;
-                o.ca = o.ws = (float)(p.tau / (p.tau + 1.0));
-                o.cb = (float)(1.0 / (p.tau + 1.0));
-            } else {
-                o.p0 = xc;
-                o.p1 = xo;
-                o.ca = o.ws = (float)(1.0 / p.sigma);
-                o.cb = (float)p.theta_prev;
-                o.sg = (float)p.sigma;
-            }
-        }
+        if (done && *done) return false;
         return true;
     }
     __device__ void chain(const SplitView &o, long long c, long long &start, long long &wstart,
@@ -858,24 +853,10 @@ struct SplitSrc {
     {
         return o.spill + (offsets ? 2 * (start - off0) + 2 * c : c * (2LL * n + 2));
     }
-    __device__ void done_block() const
-    {
-        if (v.mode != SPLIT_ROW || !ticket) return;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            if (atomicAdd(ticket, 1u) == gridDim.x - 1) {
-                __threadfence();
-                *ticket = 0;
-                *k = *k + 1;
-            }
-        }
-    }
 };
 
 // SRC: bind(block, nch, view, k0, cnt) the chains k0 .. k0 + cnt - 1 of this block;
-// chain(view, k, start, wstart, n) one of them (n = 0: skip); spill(view, k, start, n);
-// done_block() at the block's end.
+// chain(view, k, start, wstart, n) one of them (n = 0: skip); spill(view, k, start, n).
 template <int W, bool UNI, class SRC>
 __global__ void __launch_bounds__(split_threads<W>(), W <= 2 ? 2 : 1)
     split_kernel(SRC src, WsHeader *hdr, int nch, int cs)
@@ -889,32 +870,27 @@ __global__ void __launch_bounds__(split_threads<W>(), W <= 2 ? 2 : 1)
     int cnt;
     if (!src.bind(blockIdx.x, nch, v, k0, cnt, hdr)) return;
     const int g = threadIdx.x / (WARP * W);
+    const long long kc = k0 + g;
     long long start = 0, wstart = 0;
     int n = 0;
     if (v.cols) src.chain(v, k0, start, wstart, n, hdr);
-    else if (g < cnt) src.chain(v, k0 + g, start, wstart, n, hdr);
+    else if (g < cnt) src.chain(v, kc, start, wstart, n, hdr);
     // chains that a launch for other lengths takes, and empty ones
-    if (split_pick<W, UNI>(n) == 0 || n <= src.n_lo) n = 0;
-    float2 *spill = src.spill(v, k0 + g, start, n);
+    if (split_pick<W>(n) == 0 || n <= src.n_lo) n = 0;
+    float2 *spill = src.spill(v, kc, start, n);
     if (n > 0) {
-        const int l = split_pick<W, UNI>(n);
+        const int l = src.lanes && n > 256 ? src.lanes : split_pick<W>(n);
         if constexpr (W == 1) {
-            if (l == 4) split_chain<4, W, UNI>(v, smem, xall, nch, cs, k0, cnt, start, wstart, n, hdr, spill);
-            if (l == 8) split_chain<8, W, UNI>(v, smem, xall, nch, cs, k0, cnt, start, wstart, n, hdr, spill);
+            if (l == 4) split_chain<4, W, UNI>(v, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
+            if (l == 8) split_chain<8, W, UNI>(v, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
+            if (l == 12) split_chain<12, W, UNI>(v, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
         }
-        if constexpr (!UNI && W < 8) {
-            if (l == 12) split_chain<12, W, UNI>(v, smem, xall, nch, cs, k0, cnt, start, wstart, n, hdr, spill);
-            if (l == 20) split_chain<20, W, UNI>(v, smem, xall, nch, cs, k0, cnt, start, wstart, n, hdr, spill);
-        }
-        if (l == 16) split_chain<16, W, UNI>(v, smem, xall, nch, cs, k0, cnt, start, wstart, n, hdr, spill);
-        if constexpr (W < 8) {
-            if (l == 24) split_chain<24, W, UNI>(v, smem, xall, nch, cs, k0, cnt, start, wstart, n, hdr, spill);
-        }
-        if constexpr (UNI) {
-            if (l == 32) split_chain<32, W, UNI>(v, smem, xall, nch, cs, k0, cnt, start, wstart, n, hdr, spill);
-        }
+        if (l == 16) split_chain<16, W, UNI>(v, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
+        if (l == 20) split_chain<20, W, UNI>(v, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
+        if (l == 24) split_chain<24, W, UNI>(v, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
+        if (l == 28) split_chain<28, W, UNI>(v, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
+        if (l == 32) split_chain<32, W, UNI>(v, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
     }
-    src.done_block();
 }
 
 }  // namespace tvk
