@@ -22,6 +22,7 @@
 #include "tv2d_common.cuh"
 #include "tv_halves.cuh"
 #include "tv_launch.cuh"
+#include "tv_split_launch.h"
 
 using namespace tvk;
 using namespace tvh;
@@ -37,6 +38,7 @@ struct BImg {
     float *crec;
     float2 *spill;
     double inv_N;
+    const float *y0;  // the dual to start from (NULL: 0)
 };
 
 struct BState {
@@ -467,6 +469,74 @@ struct BColsTP {
     __device__ void finish_empty() const {}
 };
 
+// ------------------------------------------------ threshold splitting -------
+// The phases on the kernel of tv_split.cuh (every image's chains fit it): a block takes the
+// neighbouring rows or columns of one image that a group names. Chains of one length class
+// (warps per chain) share a launch.
+struct SGroup {
+    int img, first, count;
+};
+
+struct BSplitSrc {
+    const BImg *imgs;
+    const BState *st;
+    const SGroup *groups;
+    const Tv2dParams *prm;
+    SplitMode mode;
+    int n_lo, lanes;  // 0, 0: every length, by its own number of nodes a lane
+    const BImg *im;
+
+    __device__ bool bind(unsigned blk, int, SplitView &v, long long &k0, int &cnt, WsHeader *)
+    {
+        const SGroup g = groups[blk];
+        const BState &s = st[g.img];
+        if (mode != SPLIT_INIT && s.done) return false;
+        im = imgs + g.img;
+        k0 = g.first;
+        cnt = g.count;
+        const int k = s.k;
+        float *xc = (k & 1) ? im->x1 : im->x0, *xo = (k & 1) ? im->x0 : im->x1;
+        v.mode = mode;
+        v.cols = mode == SPLIT_COL;
+        v.p0 = v.cols ? xc : im->f;
+        // the first phases read the caller's dual, or none: y itself is written first
+        v.p1 = v.cols ? xo : (mode == SPLIT_ROW ? im->y : im->y0);
+        v.p2 = v.cols ? (k == 0 ? im->y0 : im->y) : (mode == SPLIT_ROW ? xc : nullptr);
+        v.pw = v.cols ? im->wv : im->wh;
+        v.lam = im->lam;
+        v.ws = 1.f;
+        v.ca = v.cb = v.sg = 0.f;
+        v.o0 = v.cols ? im->y : (mode == SPLIT_ROW ? xo : im->x0);
+        v.o1 = im->x1;
+        if (mode == SPLIT_ROW) {
+            const double tau = prm[k].tau;
+            v.ca = v.ws = (float)(tau / (tau + 1.0));
+            v.cb = (float)(1.0 / (tau + 1.0));
+        } else if (v.cols) {
+            v.ca = v.ws = (float)(1.0 / prm[k].sigma);
+            v.cb = (float)prm[k].theta_prev;
+            v.sg = (float)prm[k].sigma;
+        }
+        v.stride = v.cols ? im->W : 1;
+        v.wrow = im->W - 1;
+        v.rec = im->rec;
+        v.spill = im->spill;
+        v.maxlen = v.cols ? im->H : im->W;
+        return true;
+    }
+    __device__ void chain(const SplitView &v, long long c, long long &start, long long &wstart,
+                          int &n, WsHeader *) const
+    {
+        n = v.maxlen;
+        start = v.cols ? c : c * im->W;
+        wstart = v.cols ? c : c * v.wrow;
+    }
+    __device__ float2 *spill(const SplitView &v, long long c, long long, int n) const
+    {
+        return v.spill + c * (2LL * n + 2);
+    }
+};
+
 constexpr int kBGapThreads = 256;
 constexpr int kGapBatch = 4;  // pixels of a thread whose loads are in flight together
 
@@ -591,6 +661,11 @@ struct Plan {
     std::vector<BGroup> rgroups, cgroups;  // one-thread-per-chain groups
     bool thread_rows = false, thread_cols = false;
     bool halves = false;  // thread-per-chain batches run a thread per chain half
+    // threshold splitting: groups of rows and of columns by warps per chain (1, 2, 4), the
+    // longest chain of each class, and whether any image has weights in that direction
+    bool split = false, split_w[2] = {false, false};
+    std::vector<SGroup> sgroups[2][3];
+    int smax[2][3] = {{0, 0, 0}, {0, 0, 0}};
     std::vector<GapTile> tiles;
     std::vector<int> ntiles, tile0;
     int max_h = 0, max_w = 0;
@@ -603,6 +678,7 @@ struct BatchedWs {
     BState *st;
     ChainRef *cols, *rows;
     BGroup *rgroups, *cgroups;
+    SGroup *sgroups[2][3];
     float2 *trec;  // records of the one-thread-per-chain launches
     float *tcrec;
     GapTile *tiles;
@@ -644,6 +720,11 @@ BatchedWs carve_batched(void *base, const tv_image_desc *d, int n, int max_iters
     o.cgroups = cv.take<BGroup>((size_t)ncg);
     o.trec = cv.take<float2>((size_t)std::max(rrec, crec));
     o.tcrec = cv.take<float>((size_t)crec);
+    SGroup *sg = cv.take<SGroup>((size_t)(nrows + ncols));
+    for (int q = 0; q < 6; ++q) {
+        o.sgroups[q / 3][q % 3] = sg;
+        sg += plan.sgroups[q / 3][q % 3].size();
+    }
     o.ntiles = cv.take<int>((size_t)n);
     o.tile0 = cv.take<int>((size_t)n);
     o.partials = cv.take<double>((size_t)ntiles);
@@ -668,6 +749,7 @@ BatchedWs carve_batched(void *base, const tv_image_desc *d, int n, int max_iters
         const long long sp = std::max(H * (2 * W + 2), W * (2 * H + 2));
         b.spill = cv.take<float2>((size_t)sp);
         b.inv_N = 1.0 / (double)N;
+        b.y0 = d[m].y0;
     }
     o.bytes = align_up(cv.used, 256);
     return o;
@@ -721,6 +803,43 @@ void build_plan(const tv_image_desc *d, int n, Plan &plan)
         }
         plan.max_h = std::max(plan.max_h, (int)d[m].H);
         plan.max_w = std::max(plan.max_w, (int)d[m].W);
+    }
+}
+
+// Warps per chain (as a power of two) of the splitting kernel, and chains per block.
+int split_class(int n) { return n <= 32 * WARP ? 0 : (n <= 64 * WARP ? 1 : 2); }
+int split_group(int cls, bool cols)
+{
+    if (cols) return cls == 0 ? 8 : 4;  // 16- and 32-byte pieces of each row
+    return cls == 0 ? 2 : 1;
+}
+
+// Before the workspace is laid out: whether the batch runs on the splitting kernel, and its
+// groups, longest chains first.
+void plan_split(const tv_image_desc *d, int n, Plan &plan)
+{
+    plan.split = true;
+    plan.split_w[0] = plan.split_w[1] = false;
+    for (int m = 0; m < n; ++m) {
+        plan.split = plan.split && split_takes(d[m].W, d[m].H, INT64_MAX) &&
+                     split_takes(d[m].H, d[m].W, INT64_MAX);
+        plan.split_w[0] = plan.split_w[0] || d[m].wh != nullptr;
+        plan.split_w[1] = plan.split_w[1] || d[m].wv != nullptr;
+    }
+    if (!plan.split) return;
+    std::vector<int> order(n);
+    for (int dir = 0; dir < 2; ++dir) {
+        auto len = [&](int m) { return dir ? d[m].H : d[m].W; };
+        for (int m = 0; m < n; ++m) order[m] = m;
+        std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return len(a) > len(b); });
+        for (int m : order) {
+            const int c = split_class((int)len(m));
+            const long long g = split_group(c, dir == 1), chains = dir ? d[m].W : d[m].H;
+            plan.smax[dir][c] = std::max(plan.smax[dir][c], (int)len(m));
+            for (long long k = 0; k < chains; k += g)
+                plan.sgroups[dir][c].push_back(
+                    SGroup{m, (int)k, (int)std::min<long long>(g, chains - k)});
+        }
     }
 }
 
@@ -825,10 +944,57 @@ tv_status launch_thread(const BatchedWs &ws, const Plan &plan, bool cols, cudaSt
     return check_cuda(cudaGetLastError(), "batched thread-per-chain launch");
 }
 
+// One phase on the splitting kernel; with `prepare` only its shared-memory opt-in.
+template <int W, bool UNI>
+tv_status split_one(const BatchedWs &ws, const Plan &plan, SplitMode mode, int cls, bool prepare,
+                    cudaStream_t s)
+{
+    const int dir = mode == SPLIT_COL ? 1 : 0;
+    const size_t blocks = plan.sgroups[dir][cls].size();
+    if (blocks == 0) return TV_OK;
+    const int nch = split_group(cls, dir == 1);
+    const int cs = split_slots<W>(split_pick<W>(plan.smax[dir][cls]), nch);
+    const size_t smem = 2 * (size_t)nch * cs * sizeof(float);
+    auto kern = split_kernel<W, UNI, BSplitSrc>;
+    if (prepare)
+        return check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)split_smem_most<W>()),
+                          "cudaFuncSetAttribute");
+    const BSplitSrc src{ws.imgs, ws.st, ws.sgroups[dir][cls], ws.prm, mode, 0, 0, nullptr};
+    kern<<<(unsigned)blocks, nch * W * WARP, smem, s>>>(src, ws.hdr, nch, cs);
+    return check_cuda(cudaGetLastError(), "batched phase launch");
+}
+
+template <bool UNI>
+tv_status split_phase_u(const BatchedWs &ws, const Plan &plan, SplitMode mode, bool prepare,
+                        cudaStream_t s)
+{
+    tv_status st = split_one<4, UNI>(ws, plan, mode, 2, prepare, s);
+    if (st == TV_OK) st = split_one<2, UNI>(ws, plan, mode, 1, prepare, s);
+    if (st == TV_OK) st = split_one<1, UNI>(ws, plan, mode, 0, prepare, s);
+    return st;
+}
+
+tv_status split_phase(const BatchedWs &ws, const Plan &plan, SplitMode mode, bool prepare,
+                      cudaStream_t s)
+{
+    return plan.split_w[mode == SPLIT_COL ? 1 : 0] ? split_phase_u<false>(ws, plan, mode, prepare, s)
+                                                   : split_phase_u<true>(ws, plan, mode, prepare, s);
+}
+
 tv_status launch_iteration(const BatchedWs &ws, const Plan &plan, cudaStream_t s,
                            cudaGraphConditionalHandle cond, int use_cond)
 {
-    tv_status st = plan.thread_cols ? launch_thread<BColsTP>(ws, plan, true, s)
+    tv_status st;
+    if (plan.split) {
+        st = split_phase(ws, plan, SPLIT_COL, false, s);
+        if (st == TV_OK) st = split_phase(ws, plan, SPLIT_ROW, false, s);
+        if (st != TV_OK) return st;
+        batched_gap_kernel<<<(unsigned)plan.tiles.size(), kBGapThreads, 0, s>>>(
+            ws.imgs, ws.st, ws.tiles, ws.prm, ws.partials, ws.ctl, cond, use_cond);
+        return check_cuda(cudaGetLastError(), "batched gap launch");
+    }
+    st = plan.thread_cols ? launch_thread<BColsTP>(ws, plan, true, s)
                                     : launch_phase<2>(ws, plan, ws.cols, (int)plan.cols.size(), s);
     if (st != TV_OK) return st;
     st = plan.thread_rows ? launch_thread<BRowsTP<1>>(ws, plan, false, s)
@@ -934,6 +1100,7 @@ tv_status tv2d_denoise_batched(const tv_image_desc *imgs, int n_imgs, int max_it
         }
     }
     Plan plan;
+    plan_split(imgs, n_imgs, plan);
     BatchedWs ws = carve_batched(d_workspace, imgs, n_imgs, max_iters, plan);
     if (workspace_bytes < ws.bytes) {
         set_error("tv2d_denoise_batched: workspace of %zu bytes, %zu needed", workspace_bytes,
@@ -944,19 +1111,29 @@ tv_status tv2d_denoise_batched(const tv_image_desc *imgs, int n_imgs, int max_it
     cudaStream_t s = (cudaStream_t)stream;
     tv_status st;
     if ((st = upload(ws.imgs, plan.imgs, s)) != TV_OK) return st;
-    if ((st = upload(ws.cols, plan.cols, s)) != TV_OK) return st;
-    if ((st = upload(ws.rows, plan.rows, s)) != TV_OK) return st;
+    if (!plan.split) {
+        if ((st = upload(ws.cols, plan.cols, s)) != TV_OK) return st;
+        if ((st = upload(ws.rows, plan.rows, s)) != TV_OK) return st;
+    }
     if ((st = upload(ws.tiles, plan.tiles, s)) != TV_OK) return st;
     if ((st = upload(ws.ntiles, plan.ntiles, s)) != TV_OK) return st;
     if ((st = upload(ws.tile0, plan.tile0, s)) != TV_OK) return st;
-    if ((st = prepare_phase<0>(plan, (int)plan.rows.size(), plan.max_w)) != TV_OK) return st;
-    if ((st = prepare_phase<1>(plan, (int)plan.rows.size(), plan.max_w)) != TV_OK) return st;
-    if ((st = prepare_phase<2>(plan, (int)plan.cols.size(), plan.max_h)) != TV_OK) return st;
-    if ((st = upload(ws.rgroups, plan.rgroups, s)) != TV_OK) return st;
-    if ((st = upload(ws.cgroups, plan.cgroups, s)) != TV_OK) return st;
-    if ((st = prepare_thread<BRowsTP<0>>()) != TV_OK) return st;
-    if ((st = prepare_thread<BRowsTP<1>>()) != TV_OK) return st;
-    if ((st = prepare_thread<BColsTP>()) != TV_OK) return st;
+    if (plan.split) {
+        for (int q = 0; q < 6; ++q)
+            if ((st = upload(ws.sgroups[q / 3][q % 3], plan.sgroups[q / 3][q % 3], s)) != TV_OK)
+                return st;
+        if ((st = split_phase(ws, plan, SPLIT_ROW, true, s)) != TV_OK) return st;
+        if ((st = split_phase(ws, plan, SPLIT_COL, true, s)) != TV_OK) return st;
+    } else {
+        if ((st = prepare_phase<0>(plan, (int)plan.rows.size(), plan.max_w)) != TV_OK) return st;
+        if ((st = prepare_phase<1>(plan, (int)plan.rows.size(), plan.max_w)) != TV_OK) return st;
+        if ((st = prepare_phase<2>(plan, (int)plan.cols.size(), plan.max_h)) != TV_OK) return st;
+        if ((st = upload(ws.rgroups, plan.rgroups, s)) != TV_OK) return st;
+        if ((st = upload(ws.cgroups, plan.cgroups, s)) != TV_OK) return st;
+        if ((st = prepare_thread<BRowsTP<0>>()) != TV_OK) return st;
+        if ((st = prepare_thread<BRowsTP<1>>()) != TV_OK) return st;
+        if ((st = prepare_thread<BColsTP>()) != TV_OK) return st;
+    }
     {
         static thread_local ParamChunk chunk;
         for (int first = 0; first <= max_iters; first += kParamChunk) {
@@ -969,14 +1146,15 @@ tv_status tv2d_denoise_batched(const tv_image_desc *imgs, int n_imgs, int max_it
     }
     if ((st = check_cuda(cudaMemsetAsync(ws.hdr, 0, sizeof(WsHeader), s), "memset")) != TV_OK)
         return st;
-    for (int m = 0; m < n_imgs; ++m) {
+    for (int m = 0; m < n_imgs && !(plan.split && max_iters > 0); ++m) {
         const size_t bytes = sizeof(float) * (size_t)(imgs[m].H * imgs[m].W);
         st = imgs[m].y0 ? check_cuda(cudaMemcpyAsync(plan.imgs[m].y, imgs[m].y0, bytes,
                                                      cudaMemcpyDeviceToDevice, s), "copy y0")
                         : check_cuda(cudaMemsetAsync(plan.imgs[m].y, 0, bytes, s), "zero y");
         if (st != TV_OK) return st;
     }
-    st = plan.thread_rows ? launch_thread<BRowsTP<0>>(ws, plan, false, s)
+    st = plan.split ? split_phase(ws, plan, SPLIT_INIT, false, s)
+         : plan.thread_rows ? launch_thread<BRowsTP<0>>(ws, plan, false, s)
                           : launch_phase<0>(ws, plan, ws.rows, (int)plan.rows.size(), s);
     if (st != TV_OK) return st;
     note_launch();
