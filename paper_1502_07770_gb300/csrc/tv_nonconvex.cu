@@ -9,16 +9,21 @@
 //
 // Two warps per chain, one per half of a chain rooted at its middle node (see
 // nc_chain_kernel). A message is a list of breakpoints (lambda_p, h(lambda_p)) in shared
-// memory plus the slopes of its two ends; each lane owns a contiguous chunk of the list.
-//  - sum: the two sorted lists are merged by merge-path partitioning (one binary search
-//    per lane, then a sequential merge of the lane's output chunk), every point taking
-//    the other function's value by interpolation;
+// memory plus the slopes of its two ends; a warp goes over a list 32 points at a time, one
+// point a lane, so that every lane works, shared accesses do not conflict and the record of
+// M^_i is stored in whole lines.
+//  - sum: the place of a point in the merged list is its own index plus its rank in the other
+//    list (a binary search; for a grid of labels the rounded-up coordinate), every point
+//    taking the other function's value by interpolation;
 //  - Algorithm 1 as a scan: with g(z) = h(z) - w z, (h (x) f^1)(z) = w z + min_{y<=z} g(y),
-//    so a warp prefix-minimum of g over the breakpoints decides which points stay (those
-//    on the running minimum) and where a falling segment re-crosses the running minimum
-//    (the new breakpoint of Algorithm 1); survivors are compacted by a warp scan of
-//    counts. f^2 is the same pass run from the right end with g(z) = h(z) + w z;
-//  - f^3: a warp minimum gives min h; points are clipped to min h + C, crossings added.
+//    so a prefix minimum of g decides which points stay (those on the running minimum) and
+//    where a falling segment re-crosses it (the new breakpoint of Algorithm 1); votes give
+//    each survivor its place. f^2 is the same pass run from the right end with g(z) = h(z) +
+//    w z, its survivors written from the end of the buffer;
+//  - f^3: values are relative to the minimum; points are clipped to C, crossings added.
+// A node costs about 1700 warp instructions at 126 labels and 250 points. With a contiguous
+// chunk of the list per lane (a counting and a writing walk each, 18.9 of 32 lanes active) it
+// cost 3870, and 1000 x 1482 x 126 took 13.7 ms.
 // Values are kept relative to the minimum of M^_i (the minimum is the same after every
 // min-convolution, since each f^k >= 0 with f^k(0) = 0); the minima are summed in FP64 into
 // the chain's optimum energy. Every M^_i goes to the workspace; the backward pass takes
@@ -62,8 +67,6 @@ struct NcArgs {
     float2 *tails;        // per node: end slopes of M^_i
 };
 
-__device__ __forceinline__ int chunk_of(int t) { return ((t + WARP - 1) / WARP) | 1; }
-
 // value of the list (P, t; end slopes sl, sr; constant c0 when t == 0) at z, on the
 // segment left of index j (P[j-1] <= z <= P[j])
 __device__ __forceinline__ float interp_at(const float2 *P, int t, float sl, float sr, float c0,
@@ -84,136 +87,122 @@ __device__ __forceinline__ float warp_min(float v)
     return v;
 }
 
-__device__ __forceinline__ int warp_excl_sum(int v, int lane, int &total)
+__device__ __forceinline__ unsigned lanes_below(int lane) { return (1u << lane) - 1u; }
+
+// Points of P (t of them, sorted) left of x: P[q].x < x, or <= x with EQ.
+template <bool EQ>
+__device__ __forceinline__ int rank_of(const float2 *P, int t, float x)
 {
-    int inc = v;
-#pragma unroll
-    for (int o = 1; o < WARP; o <<= 1) {
-        const int u = __shfl_up_sync(FULL, inc, o);
-        if (lane >= o) inc += u;
+    int lo = 0;
+    for (int s = t > 0 ? 1 << (31 - __clz(t)) : 0; s > 0; s >>= 1) {
+        const int q = lo + s;
+        if (q <= t) {
+            const float v = P[q - 1].x;
+            if (EQ ? v <= x : v < x) lo = q;
+        }
     }
-    total = __shfl_sync(FULL, inc, WARP - 1);
-    return inc - v;
+    return lo;
 }
 
 // merge A (ta) and B (tb) into O: O = A + B as functions; returns min of O's values (or
-// the constant when ta + tb == 0). Ties: A's point first.
+// the constant when ta + tb == 0). Ties: A's point first. GRID: B's points lie at 0, 1, ...
+template <bool GRID>
 __device__ float nc_merge(const float2 *A, int ta, float slA, float srA, float cA, const float2 *B,
                           int tb, float slB, float srB, float2 *O, int lane)
 {
-    const int t = ta + tb;
-    const int per = chunk_of(t);
-    const int k0 = min(t, lane * per), k1 = min(t, k0 + per);
-    // merge path: i elements of A and k0 - i of B come before output k0
-    int lo = max(0, k0 - tb), hi = min(k0, ta);
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (A[mid].x <= B[k0 - 1 - mid].x) lo = mid + 1;
-        else hi = mid;
-    }
-    int i = lo, j = k0 - lo;
     float mn = INFINITY;
-    for (int k = k0; k < k1; ++k) {
-        float2 o;
-        if (j >= tb || (i < ta && A[i].x <= B[j].x)) {
-            o.x = A[i].x;
-            o.y = A[i].y + interp_at(B, tb, slB, srB, 0.f, j, o.x);
-            ++i;
-        } else {
-            o.x = B[j].x;
-            o.y = B[j].y + interp_at(A, ta, slA, srA, cA, i, o.x);
-            ++j;
-        }
-        O[k] = o;
-        mn = fminf(mn, o.y);
+    for (int q = lane; q < ta; q += WARP) {
+        const float2 e = A[q];
+        const int j = GRID ? (int)fminf(fmaxf(ceilf(e.x), 0.f), (float)tb) : rank_of<false>(B, tb, e.x);
+        const float v = e.y + interp_at(B, tb, slB, srB, 0.f, j, e.x);
+        O[q + j] = make_float2(e.x, v);
+        mn = fminf(mn, v);
+    }
+    for (int q = lane; q < tb; q += WARP) {
+        const float2 e = B[q];
+        const int i = rank_of<true>(A, ta, e.x);
+        const float v = e.y + interp_at(A, ta, slA, srA, cA, i, e.x);
+        O[q + i] = make_float2(e.x, v);
+        mn = fminf(mn, v);
     }
     mn = warp_min(mn);
-    return t ? mn : cA;
+    return ta + tb ? mn : cA;
 }
 
-// Algorithm 1 as a scan: O = (H - m) (x) f^1 (REV = false) or (x) f^2 (REV = true), H of
-// t points with end slopes sl, sr; values are shifted by -m on the way. With REV the list
-// is read from its right end in mirrored coordinates (z -> -z). Optionally copies the
-// shifted input to `store` (the record of M^_i). Returns the output count (never above
-// t); sets the output's end slopes.
+// Algorithm 1 as a scan: (H - m) (x) f^1 (REV = false) or (x) f^2 (REV = true), H of t points
+// with end slopes sl, sr; values are shifted by -m on the way. With REV the list is read from
+// its right end in mirrored coordinates (z -> -z). The result goes to O[0..] or, with REV, to
+// the end of O (O[T - count..T)). Optionally copies the shifted input to `store` (the record of
+// M^_i). Returns the output count (never above t); sets the output's end slopes.
 template <bool REV>
 __device__ int nc_mc12(const float2 *H, int t, float sl, float sr, float m, float w, float2 *O,
-                       float2 *store, int lane, float &osl, float &osr)
+                       int T, float2 *store, int lane, float &osl, float &osr)
 {
-    // mirrored view: element q of the view is H[REV ? t-1-q : q] at z' = REV ? -x : x
-    auto at = [&](int q) -> float2 {
-        const float2 e = H[REV ? t - 1 - q : q];
-        return make_float2(REV ? -e.x : e.x, e.y - m);
-    };
     const float vsl = REV ? -sr : sl, vsr = REV ? -sl : sr;  // end slopes of the view
-    const int per = chunk_of(t);
-    const int p0 = min(t, lane * per), p1 = min(t, p0 + per);
-    if (store) {
-        for (int p = p0; p < p1; ++p) {
-            const float2 e = H[p];
-            store[p] = make_float2(e.x, e.y - m);
+    float Rc = INFINITY;            // minimum of g over the points before this block
+    float px = 0.f, pg = INFINITY;  // last point before this block (first of its duplicates)
+    float lastx = 0.f;              // x of the point before this block
+    int cnt = 0;
+    auto put = [&](int pos, float z, float v) {
+        O[REV ? T - 1 - pos : pos] = make_float2(REV ? -z : z, v);
+    };
+    for (int b = 0; b < t; b += WARP) {
+        const int q = b + lane;
+        const bool in = q < t;
+        float2 e = make_float2(0.f, 0.f);
+        if (in) {
+            const float2 h = H[REV ? t - 1 - q : q];
+            e = make_float2(REV ? -h.x : h.x, h.y - m);
+            if (store) store[q] = e;
         }
-    }
-    // prefix minimum of g = h - w z over the non-duplicate points (a point equal in z to
-    // its predecessor adds nothing)
-    float cm = INFINITY;
-    for (int q = p0; q < p1; ++q) {
-        const float2 e = at(q);
-        const bool dup = q > 0 && at(q - 1).x == e.x;
-        if (!dup) cm = fminf(cm, fmaf(-w, e.x, e.y));
-    }
-    float inc = cm;
+        // a point equal in z to its predecessor adds nothing
+        float xb = __shfl_up_sync(FULL, e.x, 1);
+        if (lane == 0) xb = lastx;
+        const bool nd = in && !(q > 0 && xb == e.x);
+        const float g = nd ? fmaf(-w, e.x, e.y) : INFINITY;
+        float inc = g;
 #pragma unroll
-    for (int o = 1; o < WARP; o <<= 1) {
-        const float u = __shfl_up_sync(FULL, inc, o);
-        if (lane >= o) inc = fminf(inc, u);
+        for (int o = 1; o < WARP; o <<= 1) {
+            const float u = __shfl_up_sync(FULL, inc, o);
+            if (lane >= o) inc = fminf(inc, u);
+        }
+        const float ex = __shfl_up_sync(FULL, inc, 1);
+        const float R = lane == 0 ? Rc : fminf(Rc, ex);  // minimum over the points before q
+        const unsigned ndm = __ballot_sync(FULL, nd);
+        const unsigned below = ndm & lanes_below(lane);
+        const int src = below ? 31 - __clz(below) : 0;
+        float qx = __shfl_sync(FULL, e.x, src), qg = __shfl_sync(FULL, g, src);
+        if (!below) {
+            qx = px;
+            qg = pg;
+        }
+        // a falling segment re-crosses the running minimum between its ends
+        bool cross = nd && q > 0 && qg > R && g < R;
+        float z = 0.f;
+        if (cross) {
+            z = qx + (e.x - qx) * ((R - qg) / (g - qg));
+            cross = z > qx && z < e.x;
+        }
+        const bool keep = nd && g <= R;
+        const unsigned cm = __ballot_sync(FULL, cross), km = __ballot_sync(FULL, keep);
+        const int pos = cnt + __popc(cm & lanes_below(lane)) + __popc(km & lanes_below(lane));
+        if (cross) put(pos, z, fmaf(w, z, R));
+        if (keep) put(pos + (cross ? 1 : 0), e.x, e.y);
+        cnt += __popc(cm) + __popc(km);
+        Rc = fminf(Rc, __shfl_sync(FULL, inc, WARP - 1));
+        if (ndm) {
+            const int l = 31 - __clz(ndm);
+            px = __shfl_sync(FULL, e.x, l);
+            pg = __shfl_sync(FULL, g, l);
+        }
+        lastx = __shfl_sync(FULL, e.x, WARP - 1);
     }
-    float excl = __shfl_up_sync(FULL, inc, 1);
-    if (lane == 0) excl = INFINITY;
-    const float R_all = __shfl_sync(FULL, inc, WARP - 1);
-    // count, then write. Point q (not a duplicate): its predecessor pq (the last non-duplicate
-    // before it); crossing on (pq, q) iff g_pq > R_pq and g_q < R_pq; point kept iff
-    // g_q <= R_{q-1}.
-    int pos = 0, total = 0;
-    for (int pass = 0; pass < 2; ++pass) {
-        float R = excl;  // running minimum over the view's points before q
-        float2 prev = make_float2(0.f, 0.f);
-        float gprev = INFINITY;
-        if (p0 > 0 && p0 < p1) {
-            int pq = p0 - 1;
-            while (pq > 0 && at(pq - 1).x == at(pq).x) --pq;
-            prev = at(pq);
-            gprev = fmaf(-w, prev.x, prev.y);
-        }
-        int c = 0;
-        auto emit = [&](float z, float v) {
-            if (pass == 1) {
-                const int o = REV ? total - 1 - pos - c : pos + c;
-                O[o] = make_float2(REV ? -z : z, v);
-            }
-            ++c;
-        };
-        for (int q = p0; q < p1; ++q) {
-            const float2 e = at(q);
-            if (q > 0 && at(q - 1).x == e.x) continue;  // duplicate
-            const float g = fmaf(-w, e.x, e.y);
-            if (q > 0 && gprev > R && g < R) {
-                // the falling segment re-crosses the running minimum
-                const float z = prev.x + (e.x - prev.x) * ((R - gprev) / (g - gprev));
-                if (z > prev.x && z < e.x) emit(z, fmaf(w, z, R));
-            }
-            if (g <= R) emit(e.x, e.y);
-            R = fminf(R, g);
-            prev = e;
-            gprev = g;
-        }
-        // the right end of the view: its last point off the running minimum and g
-        // falling there: the end re-crosses the minimum
-        if (t > 0 && p1 == t && p0 < p1 && gprev > R_all && vsr < w) {
-            const float z = prev.x + (R_all - gprev) / (vsr - w);
-            emit(z, fmaf(w, z, R_all));
-        }
-        if (pass == 0) pos = warp_excl_sum(c, lane, total);
+    // the right end of the view: its last point off the running minimum and g falling there:
+    // the end re-crosses the minimum
+    if (t > 0 && pg > Rc && vsr < w) {
+        const float z = px + (Rc - pg) / (vsr - w);
+        if (lane == 0) put(cnt, z, fmaf(w, z, Rc));
+        ++cnt;
     }
     // end slopes: the left end keeps its slope (<= 0 <= w); the right end follows h where
     // g falls (slope < w), else rises with slope w
@@ -221,54 +210,68 @@ __device__ int nc_mc12(const float2 *H, int t, float sl, float sr, float m, floa
     osl = REV ? -nsr : vsl;
     osr = REV ? -vsl : nsr;
     __syncwarp();
-    return total;
+    return cnt;
 }
 
 // O = min(H, min H + C) for 0 < C < inf; H has minimum 0 (values relative). End slopes
 // become 0. Points whose two neighbouring segments are both flat at the cap are dropped.
-// Returns the output count, or -1 (nothing written) if it would exceed `cap_out`.
+// Returns the output count, or -1 if it exceeds `cap_out` (then O is not complete).
 __device__ int nc_mc3(const float2 *H, int t, float sl, float sr, float C, float2 *O, int cap_out,
                       int lane)
 {
     const float cap = C;
-    const int per = chunk_of(t);
-    const int p0 = min(t, lane * per), p1 = min(t, p0 + per);
-    int pos = 0, total = 0;
-    for (int pass = 0; pass < 2; ++pass) {
-        int c = 0;
-        auto emit = [&](float z, float v) {
-            if (pass == 1) O[pos + c] = make_float2(z, v);
-            ++c;
-        };
-        for (int p = p0; p < p1; ++p) {
-            const float2 e = H[p];
-            if (p == 0 && e.y < cap && sl < 0.f) {
-                const float z = e.x + (cap - e.y) / sl;
-                if (z < e.x) emit(z, cap);
-            }
-            const bool lflat = p == 0 ? true : H[p - 1].y >= cap;
-            const bool rflat = p == t - 1 ? true : H[p + 1].y >= cap;
-            if (!(e.y >= cap && lflat && rflat)) emit(e.x, fminf(e.y, cap));
-            if (p + 1 < t) {
-                const float2 f = H[p + 1];
-                const float a = e.y - cap, b = f.y - cap;
-                if ((a < 0.f && b > 0.f) || (a > 0.f && b < 0.f)) {
-                    const float z = e.x + (f.x - e.x) * (a / (a - b));
-                    if (z > e.x && z < f.x) emit(z, cap);
-                }
-            }
-            if (p == t - 1 && e.y < cap && sr > 0.f) {
-                const float z = e.x + (cap - e.y) / sr;
-                if (z > e.x) emit(z, cap);
+    int cnt = 0;
+    auto put = [&](int pos, float z, float v) {
+        if (pos < cap_out) O[pos] = make_float2(z, v);
+    };
+    if (t > 0) {
+        const float2 e = H[0];
+        if (e.y < cap && sl < 0.f) {
+            const float z = e.x + (cap - e.y) / sl;
+            if (z < e.x) {
+                if (lane == 0) put(0, z, cap);
+                cnt = 1;
             }
         }
-        if (pass == 0) {
-            pos = warp_excl_sum(c, lane, total);
-            if (total > cap_out) return -1;
+    }
+    for (int b = 0; b < t; b += WARP) {
+        const int p = b + lane;
+        bool keep = false, cross = false;
+        float2 e = make_float2(0.f, 0.f);
+        float z = 0.f;
+        if (p < t) {
+            e = H[p];
+            const bool lflat = p == 0 || H[p - 1].y >= cap;
+            bool rflat = true;
+            if (p + 1 < t) {
+                const float2 f = H[p + 1];
+                rflat = f.y >= cap;
+                const float u = e.y - cap, v = f.y - cap;
+                if ((u < 0.f && v > 0.f) || (u > 0.f && v < 0.f)) {
+                    z = e.x + (f.x - e.x) * (u / (u - v));
+                    cross = z > e.x && z < f.x;
+                }
+            }
+            keep = !(e.y >= cap && lflat && rflat);
+        }
+        const unsigned km = __ballot_sync(FULL, keep), cm = __ballot_sync(FULL, cross);
+        const int pos = cnt + __popc(km & lanes_below(lane)) + __popc(cm & lanes_below(lane));
+        if (keep) put(pos, e.x, fminf(e.y, cap));
+        if (cross) put(pos + (keep ? 1 : 0), z, cap);
+        cnt += __popc(km) + __popc(cm);
+    }
+    if (t > 0) {
+        const float2 e = H[t - 1];
+        if (e.y < cap && sr > 0.f) {
+            const float z = e.x + (cap - e.y) / sr;
+            if (z > e.x) {
+                if (lane == 0) put(cnt, z, cap);
+                ++cnt;
+            }
         }
     }
     __syncwarp();
-    return total;
+    return cnt > cap_out ? -1 : cnt;
 }
 
 struct BestZ {
@@ -295,56 +298,38 @@ __device__ __forceinline__ BestZ warp_best(BestZ b)
 }
 
 // argmin over z of H(z) + min(w |xn - z|, C) (pair = true) or of H(z) (pair = false),
-// candidates and order as in the file comment; H in global memory.
+// candidates and order as in the file comment; H in shared memory. The points are shared out
+// over the lanes; xn and xn -+ C/w, which may lie between them, take a lane each.
 __device__ float nc_argmin(const float2 *H, int t, float sl, float sr, bool pair, float xn, float w,
                            float C, int lane)
 {
     if (t == 0) return pair ? xn : 0.f;
-    const int per = chunk_of(t);
-    const int p0 = min(t, lane * per), p1 = min(t, p0 + per);
     BestZ b{INFINITY, 0x7fffffff, 0.f};
     const bool trunc = pair && isfinite(C) && w > 0.f;
-    const float r = trunc ? C / w : 0.f;
-    const float zs[3] = {xn, xn - r, xn + r};
-    const int prs[3] = {0, t + 1, t + 2};
     auto pen = [&](float z) {
         if (!pair) return 0.f;
         return fminf(w * fabsf(xn - z), C);
     };
-    float2 prevp = make_float2(0.f, 0.f);
-    if (p0 > 0 && p0 < p1) prevp = H[p0 - 1];
-    for (int p = p0; p < p1; ++p) {
+    if (pair && lane < (trunc ? 3 : 1)) {
+        const float r = trunc ? C / w : 0.f;
+        const float z = lane == 0 ? xn : (lane == 1 ? xn - r : xn + r);
+        const int q = rank_of<true>(H, t, z);  // the segment left of point q, or an end
+        float hz;
+        if (q == 0) {
+            hz = H[0].y + sl * (z - H[0].x);
+        } else if (q == t) {
+            const float2 e = H[t - 1];
+            hz = e.y + sr * (z - e.x);
+        } else {
+            const float2 l = H[q - 1], e = H[q];
+            const float d = e.x - l.x;
+            hz = d > 0.f ? l.y + (e.y - l.y) * ((z - l.x) / d) : l.y;
+        }
+        best_of(b, hz + pen(z), lane == 0 ? 0 : t + lane, z);
+    }
+    for (int p = lane; p < t; p += WARP) {
         const float2 e = H[p];
         best_of(b, e.y + pen(e.x), 1 + p, e.x);
-        // special candidates on the segment left of p (or the left end)
-        if (pair) {
-#pragma unroll
-            for (int s = 0; s < 3; ++s) {
-                if (s > 0 && !trunc) break;
-                const float z = zs[s];
-                bool in;
-                float hz;
-                if (p == 0) {
-                    in = z < e.x;
-                    hz = e.y + sl * (z - e.x);
-                } else {
-                    in = z >= prevp.x && z < e.x;
-                    const float d = e.x - prevp.x;
-                    hz = d > 0.f ? prevp.y + (e.y - prevp.y) * ((z - prevp.x) / d) : prevp.y;
-                }
-                if (in) best_of(b, hz + pen(z), prs[s], z);
-            }
-        }
-        prevp = e;
-    }
-    if (pair && p1 == t && p0 < p1) {  // right end
-        const float2 e = H[t - 1];
-#pragma unroll
-        for (int s = 0; s < 3; ++s) {
-            if (s > 0 && !trunc) break;
-            const float z = zs[s];
-            if (z >= e.x) best_of(b, e.y + sr * (z - e.x) + pen(z), prs[s], z);
-        }
     }
     b = warp_best(b);
     return b.z;
@@ -353,12 +338,17 @@ __device__ float nc_argmin(const float2 *H, int t, float sl, float sr, bool pair
 // What the two warps of a chain tell each other at the root (shared memory).
 struct NcPairXchg {
     double esum[2];   // each half's sum of message minima
-    int ta[2], mi[2];  // each half's final message: count, buffer
+    int ta[2], mi[2], at[2];  // each half's final message: count, buffer, first point
     float sl[2], sr[2], cA[2];
     int bad[2];
 };
 
-__device__ __forceinline__ void pair_bar(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+// (at most kNcMaxWarps / 2 = 2 pairs; literal names, or a block would hold all 16 barriers)
+__device__ __forceinline__ void pair_bar(int pair)
+{
+    if (pair == 0) asm volatile("bar.sync 1, 64;" ::: "memory");
+    else asm volatile("bar.sync 2, 64;" ::: "memory");
+}
 
 // Two warps per chain, rooted at node mid = n/2 (Algorithm 2 may take any root): warp 0
 // of the pair runs the forward pass over nodes 0..mid-1, warp 1 over nodes n-1..mid+1
@@ -406,6 +396,16 @@ __global__ void nc_chain_kernel(NcArgs p, WsHeader *hdr)
     auto node_of = [&](int j) { return role == 0 ? j : n - 1 - j; };
     auto edge_of = [&](int i) { return role == 0 ? i : i - 1; };  // index of w / C of the edge
 
+    // Grid unaries of up to kPre * 32 labels are fetched a node ahead (ahead[]).
+    constexpr int kPre = 8;
+    float ahead[kPre];
+    const bool pre = !p.uoff && p.grid_len <= kPre * WARP;
+    auto fetch = [&](long long node) {
+        const float *v = p.uval + node * (long long)p.grid_len;
+#pragma unroll
+        for (int q = 0; q < kPre; ++q)
+            if (q * WARP + lane < p.grid_len) ahead[q] = v[q * WARP + lane];
+    };
     auto load_unary = [&](long long node, float2 *F, int &tf, float &slF, float &srF) -> bool {
         if (p.uoff) {
             const long long u0 = p.uoff[node], u1 = p.uoff[node + 1];
@@ -415,17 +415,30 @@ __global__ void nc_chain_kernel(NcArgs p, WsHeader *hdr)
         } else {
             tf = p.grid_len;
             if (tf > T) return false;
-            for (int q = lane; q < tf; q += WARP)
-                F[q] = make_float2((float)q, p.uval[node * (long long)p.grid_len + q]);
+            if (pre) {
+#pragma unroll
+                for (int q = 0; q < kPre; ++q)
+                    if (q * WARP + lane < tf)
+                        F[q * WARP + lane] = make_float2((float)(q * WARP + lane), ahead[q]);
+            } else {
+                for (int q = lane; q < tf; q += WARP)
+                    F[q] = make_float2((float)q, p.uval[node * (long long)p.grid_len + q]);
+            }
         }
         slF = p.sl ? p.sl[node] : p.sl_s;
         srF = p.sr ? p.sr[node] : p.sr_s;
         if (tf == 0) slF = srF = 0.f;
         return true;
     };
+    auto merge = [&](const float2 *A, int tA, float slA, float srA, float cA, const float2 *B, int tB,
+                     float slB, float srB, float2 *O) {
+        return p.uoff ? nc_merge<false>(A, tA, slA, srA, cA, B, tB, slB, srB, O, lane)
+                      : nc_merge<true>(A, tA, slA, srA, cA, B, tB, slB, srB, O, lane);
+    };
 
     // ---------------- forward pass over this warp's half ----------------
-    int mi = 0, ta = 0;
+    int mi = 0, ta = 0, at = 0;  // the message: ta points of buffer mi from point `at`
+    if (pre && cnt > 0) fetch(start + node_of(0));
     float slA = 0.f, srA = 0.f, cA = 0.f;
     double energy = 0.0;
     unsigned aoff = 0;
@@ -443,9 +456,10 @@ __global__ void nc_chain_kernel(NcArgs p, WsHeader *hdr)
             break;
         }
         __syncwarp();
+        if (pre) fetch(start + (j + 1 < cnt ? node_of(j + 1) : mid));
         float2 *Mh = P(2);
         const int th = ta + tf;
-        const float m = nc_merge(P(mi), ta, slA, srA, cA, F, tf, slF, srF, Mh, lane);
+        const float m = merge(P(mi) + at, ta, slA, srA, cA, F, tf, slF, srF, Mh);
         const float slH = slA + slF, srH = srA + srF;
         energy += (double)m;
         __syncwarp();
@@ -458,21 +472,23 @@ __global__ void nc_chain_kernel(NcArgs p, WsHeader *hdr)
         const float Ci = p.C ? p.C[start + e] : p.C_s;
         // (x) f^1 into F's buffer (free now), recording M^_i; (x) f^2 into mi's buffer
         float s1l, s1r, s2l, s2r;
-        const int t1 = nc_mc12<false>(Mh, th, slH, srH, m, wi, F, arena + aoff, lane, s1l, s1r);
+        const int t1 = nc_mc12<false>(Mh, th, slH, srH, m, wi, F, T, arena + aoff, lane, s1l, s1r);
         aoff += (unsigned)th;
-        const int t2 = nc_mc12<true>(F, t1, s1l, s1r, 0.f, wi, P(mi), nullptr, lane, s2l, s2r);
+        const int t2 = nc_mc12<true>(F, t1, s1l, s1r, 0.f, wi, P(mi), T, nullptr, lane, s2l, s2r);
+        at = T - t2;
         if (isfinite(Ci)) {
             if (Ci <= 0.f) {
                 ta = 0;
                 cA = 0.f;
                 slA = srA = 0.f;
             } else {
-                const int t3 = nc_mc3(P(mi), t2, s2l, s2r, Ci, F, T, lane);
+                const int t3 = nc_mc3(P(mi) + at, t2, s2l, s2r, Ci, F, T, lane);
                 if (t3 < 0) {
                     bad = true;
                     break;
                 }
                 mi = fi;
+                at = 0;
                 ta = t3;
                 slA = srA = 0.f;
                 cA = 0.f;
@@ -490,12 +506,13 @@ __global__ void nc_chain_kernel(NcArgs p, WsHeader *hdr)
         xs->esum[role] = energy;
         xs->ta[role] = ta;
         xs->mi[role] = mi;
+        xs->at[role] = at;
         xs->sl[role] = slA;
         xs->sr[role] = srA;
         xs->cA[role] = cA;
         xs->bad[role] = bad ? 1 : 0;
     }
-    pair_bar(1 + pair);
+    pair_bar(pair);
 
     // ---------------- root: M^_mid = M_L + M_R + f_mid, both warps alike ----------------
     const bool any_bad = xs->bad[0] || xs->bad[1];
@@ -505,26 +522,28 @@ __global__ void nc_chain_kernel(NcArgs p, WsHeader *hdr)
     float slr = 0.f, srr = 0.f, mr = 0.f;
     if (!any_bad) {
         const int tL = xs->ta[0], tR = xs->ta[1];
-        const float2 *ML = Pw(2 * pair, xs->mi[0]), *MR = Pw(2 * pair + 1, xs->mi[1]);
+        const float2 *ML = Pw(2 * pair, xs->mi[0]) + xs->at[0],
+                     *MR = Pw(2 * pair + 1, xs->mi[1]) + xs->at[1];
         const int other = 1 - xs->mi[role];  // my free message buffer
         if (tL + tR > T) {
             root_bad = true;
         } else {
-            nc_merge(ML, tL, xs->sl[0], xs->sr[0], xs->cA[0], MR, tR, xs->sl[1], xs->sr[1], P(2),
-                     lane);
+            nc_merge<false>(ML, tL, xs->sl[0], xs->sr[0], xs->cA[0], MR, tR, xs->sl[1], xs->sr[1],
+                            P(2), lane);
         }
         int tf = 0;
         float slF = 0.f, srF = 0.f;
+        if (pre && cnt == 0) fetch(start + mid);
         if (!root_bad && !load_unary(start + mid, P(other), tf, slF, srF)) root_bad = true;
         if (!root_bad && tL + tR + tf > T) root_bad = true;
         __syncwarp();
         // both warps have read both messages before either overwrites its own
-        pair_bar(1 + pair);
+        pair_bar(pair);
         if (!root_bad) {
             const float cLR = (tL + tR == 0) ? xs->cA[0] + xs->cA[1] : 0.f;
             const float slLR = xs->sl[0] + xs->sl[1], srLR = xs->sr[0] + xs->sr[1];
             float2 *R = P(xs->mi[role]);
-            mr = nc_merge(P(2), tL + tR, slLR, srLR, cLR, P(other), tf, slF, srF, R, lane);
+            mr = merge(P(2), tL + tR, slLR, srLR, cLR, P(other), tf, slF, srF, R);
             tr = tL + tR + tf;
             slr = slLR + slF;
             srr = srLR + srF;
@@ -532,7 +551,7 @@ __global__ void nc_chain_kernel(NcArgs p, WsHeader *hdr)
             xmid = nc_argmin(R, tr, slr, srr, false, 0.f, 0.f, 0.f, lane);
         }
     } else {
-        pair_bar(1 + pair);
+        pair_bar(pair);
     }
     if (root_bad) {
         if (role == 0) {
@@ -553,19 +572,46 @@ __global__ void nc_chain_kernel(NcArgs p, WsHeader *hdr)
     __syncwarp();
     __threadfence_block();
     // ---------------- backward: clip this half outwards from the root ----------------
+    // The records do not depend on x: they are copied a node ahead into two of the buffers, and
+    // the places of the records two ahead.
+    auto place = [&](int j, int2 &mt, float2 &tl) {
+        if (j < 0) return;
+        const long long node = start + node_of(j);
+        mt = p.meta[node];
+        tl = p.tails[node];
+    };
+    auto copy = [&](int j, const int2 &mt) {
+        if (j >= 0)
+            for (int q = lane; q < mt.y; q += WARP) cp_async8(P(j & 1) + q, arena + mt.x + q);
+        cp_async_commit();
+    };
     float xn = xmid;
+    int2 m0 = make_int2(0, 0), m1 = m0;
+    float2 t0 = make_float2(0.f, 0.f), t1 = t0;
+    place(cnt - 1, m0, t0);
+    place(cnt - 2, m1, t1);
+    copy(cnt - 1, m0);
     for (int j = cnt - 1; j >= 0; --j) {
+        copy(j - 1, m1);
+        int2 m2 = make_int2(0, 0);
+        float2 t2 = make_float2(0.f, 0.f);
+        place(j - 2, m2, t2);
+        cp_async_wait<1>();
+        __syncwarp();
         const int i = node_of(j);
-        const long long node = start + i;
-        const int2 mt = p.meta[node];
-        const float2 tl = p.tails[node];
         const int e = edge_of(i);
         const float wi = p.w ? p.w[start + e] : p.w_s;
         const float Ci = p.C ? p.C[start + e] : p.C_s;
-        const float xi = nc_argmin(arena + mt.x, mt.y, tl.x, tl.y, true, xn, wi, Ci, lane);
-        if (lane == 0) p.x[node] = xi;
+        const float xi = nc_argmin(P(j & 1), m0.y, t0.x, t0.y, true, xn, wi, Ci, lane);
+        if (lane == 0) p.x[start + i] = xi;
         xn = xi;
+        m0 = m1;
+        t0 = t1;
+        m1 = m2;
+        t1 = t2;
+        __syncwarp();
     }
+    cp_async_wait<0>();
 }
 
 struct NcWs {
