@@ -439,7 +439,7 @@ tv_status tv_set_programmatic_launch(int on);
  * tile's epilogue, one issuing thread per block). Both accumulate the same BF16 products
  * in FP32, in a different order. With 16 or 32 output channels each tcgen05 MMA is only
  * 128 x 32 x 16 and the forward pass of the network is faster on mma.sync (0.38 against
- * 0.53 ms at 1024 x 1024). The backward kernels always use mma.sync. */
+ * 0.53 ms at 1024 x 1024). The NHWC backward kernels always use mma.sync. */
 tv_status tv_net_set_tensor_path(int mode);
 /* Mode 2: the same tcgen05 GEMM per 128-pixel row tile, fed by TMA and run by warp roles
  * over vertical strips: a block walks runs of consecutive rows of one 128-pixel column, so
@@ -518,6 +518,31 @@ tv_status tv_net_conv3x3_dual_head(const void *d_x, int B, int H, int W, int cin
 tv_status tv_net_dual_head(const float *d_o, int B, int H, int W, const float *d_lam,
                            const float *d_target, float *d_y, float *d_loss, void *d_grad_o,
                            void *d_ws, size_t ws_bytes, tv_stream_t stream);
+/* The layers of one training step in the grouped layout (32 channels between layers; the
+ * tcgen05 kernel of tv_net_conv3x3_grouped forward and for the gradient of the input). A
+ * 32-output ReLU layer writes its activation and, per pixel, the word of its ReLU mask (bit
+ * c: channel c of conv + bias > 0; B x H x W uint32). d_x NULL: the first layer, whose input
+ * is the image f with its lambda (as tv_net_first_layer, weights [32][3][3][16]); otherwise
+ * x is grouped, weights [32][3][3][32]. */
+tv_status tv_net_train_layer(const void *d_x, const float *d_f, const float *d_lam, int B, int H,
+                             int W, const void *d_w, const float *d_bias, void *d_act_out,
+                             uint32_t *d_mask_out, tv_stream_t stream);
+/* The last layer (weights [16][3][3][32], channel 0 of its output kept in d_o, B x H x W
+ * FP32) and the head: *d_loss and the gradient d_grad_o (B x H x W FP32) of
+ * tv_net_dual_head. d_ws: tv_net_workspace_size bytes. */
+tv_status tv_net_train_head(const void *d_x, int B, int H, int W, const void *d_w, const float *d_bias,
+                            const float *d_lam, const float *d_target, float *d_o, float *d_loss,
+                            float *d_grad_o, void *d_ws, size_t ws_bytes, tv_stream_t stream);
+/* Backward of one layer: its weight and bias gradients are ADDED to d_dw and d_db (may be
+ * NULL), and d_dx (grouped) = (conv^T dy) * mask, the mask of the layer below. The input is
+ * x (grouped, 32 channels), or, with d_x NULL, the image f and its lambda (first layer: no
+ * mask, no dx, w not read). The output gradient is d_dy (grouped, 32 channels), or, with
+ * d_dy NULL, d_grad_o, channel 0 of the 16-channel last layer (FP32, rounded to BF16).
+ * Pointers of BF16 tensors and d_ws 16-byte aligned. */
+tv_status tv_net_train_backward(const void *d_x, const float *d_f, const float *d_lam,
+                                const void *d_dy, const float *d_grad_o, int B, int H, int W,
+                                const void *d_w, const uint32_t *d_mask, void *d_dx, float *d_dw,
+                                float *d_db, void *d_ws, size_t ws_bytes, tv_stream_t stream);
 /* out[i] = bfloat16(a[i]) (round to nearest even), i < n. */
 tv_status tv_net_cast_bf16(const float *d_a, int64_t n, void *d_out, tv_stream_t stream);
 /* One Adam step on n FP32 parameters (step counts from 1); the gradient is read and

@@ -8,7 +8,11 @@
 //   forward:        M = pixels, N = Cout, K = 9 * Cin
 //   backward data:  the same with the kernel flipped and Cin/Cout swapped
 //   backward weight: M = Cout, N = 9 * Cin, K = pixels (persistent blocks, FP32
-//                    partial tiles, atomics into the FP32 gradient)
+//                    partial gradients, summed in a fixed order)
+// That is the general NHWC set. Inference and training run the forward and backward-data
+// GEMMs on tcgen05 in the grouped layout instead (conv3x3_tw below): for a training step on
+// 8 x 512 x 512 its seven convolutions take 390 us against 1100 us for conv3x3_persist, which
+// moved 32 FP32 pre-activations per pixel and layer where one word of signs is enough.
 // Each block of the two pixel-major kernels computes an 8 x 16 pixel tile for all
 // output channels from a zero-padded 10 x 18 input patch in shared memory; A and B
 // fragments are read with ldmatrix from rows padded by 16 bytes (conflict-free).
@@ -72,25 +76,7 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], unsigned a0, unsigned a1
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// Load the zero-padded (TH+2) x (TW+2) x C input patch of tile (ty, tx) of image b.
-template <int C>
-__device__ __forceinline__ void load_patch(__nv_bfloat16 *patch, const __nv_bfloat16 *X, int b,
-                                           int H, int W, int y0, int x0)
-{
-    constexpr int PS = C + 8;   // padded pixel stride (bf16)
-    constexpr int V = C / 8;    // 16-byte vectors per pixel
-    for (int t = threadIdx.x; t < PH * PW * V; t += blockDim.x) {
-        const int v = t % V, pix = t / V;
-        const int py = pix / PW, px = pix % PW;
-        const int gy = y0 + py - 1, gx = x0 + px - 1;
-        uint4 val = make_uint4(0, 0, 0, 0);
-        if (gy >= 0 && gy < H && gx >= 0 && gx < W)
-            val = *reinterpret_cast<const uint4 *>(X + (((long long)b * H + gy) * W + gx) * C + v * 8);
-        *reinterpret_cast<uint4 *>(patch + pix * PS + v * 8) = val;
-    }
-}
-
-// The same patch with 16-byte asynchronous copies (zero-filled outside the image).
+// 16-byte asynchronous copy into shared memory, zero-filled where !valid.
 __device__ __forceinline__ void cp_async16_zfill(void *smem, const void *gmem, bool valid)
 {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
@@ -105,6 +91,7 @@ __device__ __forceinline__ void cp_async_wait_net()
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
+// Load the zero-padded (TH+2) x (TW+2) x C input patch of tile (y0, x0) of image b.
 template <int C>
 __device__ __forceinline__ void load_patch_async(__nv_bfloat16 *patch, const __nv_bfloat16 *X,
                                                  int b, int H, int W, int y0, int x0)
@@ -255,48 +242,137 @@ __global__ void __launch_bounds__(NTHR)
 // Partial sums of dW[co][tap][ci] = sum over pixels p of dY[p][co] * X[p + tap][ci]
 // and db[co] = sum_p dY[p][co]. Each block walks tiles blockIdx.x, +gridDim.x, ...,
 // keeps its partial dW in registers (warp w owns the n8 column tiles w, w+4, ... of
-// N = 9 * CIN; both m16 tiles (co 0..31) or one (co 0..15)) and stores it, with its
-// partial db, to row blockIdx.x of P (row length 9 * CIN * COUT + COUT); the rows
-// are summed in a fixed order by wgrad_reduce, so the result is deterministic.
-template <int CIN, int COUT>
-__global__ void __launch_bounds__(NTHR)
-    conv3x3_wgrad(const __nv_bfloat16 *X, const __nv_bfloat16 *dY, int B, int H, int W,
-                  float *P)
+// N = 9 * XC; both m16 tiles (co 0..31) or one (co 0..15)) and stores it, with its
+// partial db, to row blockIdx.x of P; the rows are summed in a fixed order by
+// wgrad_reduce, so the result is deterministic. db comes from the same tensor-core pass
+// (a column tile of ones, warp w taking tile rows w and w + 4).
+// The kernel is bound by the tensor pipe once the loads are out of its way: the next tile
+// is copied asynchronously into a second buffer while the current one is multiplied (one
+// barrier per tile). 32 -> 32 channels, 8 x 512 x 512: 128 us, against 268 us with
+// one buffer, synchronous loads and db summed serially by 32 threads.
+// XL and DL say how X and dY lie in memory:
+//   WG_NHWC     [image][row][pixel][C] BF16
+//   WG_GROUPED  [image][row][C/8][pixel][8] BF16
+//   WG_PLANE    FP32 planes, rounded to BF16 on the way in. X: the image and its lambda
+//               (the 16-channel input's channels 0 and 1; channels 2..15 are zero, their
+//               gradients too, so 8 columns per tap are computed: XC = 8); dY: channel 0
+//               of 16 (the others are zero: only row co = 0 is stored).
+constexpr int WG_NHWC = 0, WG_GROUPED = 1, WG_PLANE = 2;
+
+template <int CIN, int COUT, int XL, int DL>
+struct Wgrad {
+    static constexpr int XC = XL == WG_PLANE ? 8 : CIN;     // columns per tap
+    static constexpr int CO = DL == WG_PLANE ? 1 : COUT;    // rows stored
+    // padded pixel strides (bf16); 16-byte rows need no padding
+    static constexpr int PS = XC == 8 ? 8 : XC + 8, DS = COUT + 8;
+    static constexpr int PATCH = PH * PW * PS, TILE = TH * TW * DS;
+    static constexpr int N = 9 * XC, NT = N / 8, NTW = (NT + 3) / 4, MT = COUT / 16;
+    static constexpr size_t smem = sizeof(__nv_bfloat16) * 2 * (size_t)(PATCH + TILE);
+    static constexpr int row = (CO * N + CO + 3) / 4 * 4;   // floats per block in P (16-byte rows)
+};
+
+template <int CIN, int COUT, int XL, int DL>
+__global__ void __launch_bounds__(NTHR, 4)
+    conv3x3_wgrad(const void *X, const float *lam, const void *dY, int B, int H, int W, float *P)
 {
-    constexpr int PS = CIN + 8;
-    constexpr int DS = COUT + 8;
-    constexpr int N = 9 * CIN;
-    constexpr int NT = N / 8;
-    constexpr int NTW = (NT + 3) / 4;   // column tiles per warp
-    constexpr int MT = COUT / 16;
-    __shared__ __align__(16) __nv_bfloat16 patch[PH * PW * PS];
-    __shared__ __align__(16) __nv_bfloat16 dys[TH * TW * DS];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    using G = Wgrad<CIN, COUT, XL, DL>;
+    constexpr int PS = G::PS, DS = G::DS, N = G::N, NT = G::NT, NTW = G::NTW, MT = G::MT, XC = G::XC;
+    extern __shared__ __align__(16) unsigned char smem_wg[];
+    __nv_bfloat16 *xbuf = reinterpret_cast<__nv_bfloat16 *>(smem_wg);
+    __nv_bfloat16 *dbuf = xbuf + 2 * G::PATCH;
+    __shared__ float bpart[4][COUT];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tiles_x = (W + TW - 1) / TW, tiles_y = (H + TH - 1) / TH;
-    const long long ntiles = (long long)B * tiles_x * tiles_y;
-    float acc[MT][NTW][4];
+    const int per_img = tiles_x * tiles_y;
+    const long long ntiles = (long long)B * per_img;
+
+    constexpr int XR = (PH * PW + NTHR - 1) / NTHR;  // plane pixels of a patch per thread
+    [[maybe_unused]] float xv[XR], dv = 0.f, lv = 0.f;
+    [[maybe_unused]] unsigned xin = 0u;
+    // start the loads of a tile: asynchronous copies into buffer nb, planes into registers
+    auto stage = [&](long long tile, int nb) {
+        const int b = (int)(tile / per_img), rem = (int)(tile - (long long)b * per_img);
+        const int y0 = (rem / tiles_x) * TH, x0 = (rem % tiles_x) * TW;
+        if constexpr (XL == WG_PLANE) {
+            lv = lam[b];
+            xin = 0u;
 #pragma unroll
-    for (int m = 0; m < MT; ++m)
+            for (int k = 0; k < XR; ++k) {
+                const int pix = tid + k * NTHR, gy = y0 + pix / PW - 1, gx = x0 + pix % PW - 1;
+                const bool in = pix < PH * PW && gy >= 0 && gy < H && gx >= 0 && gx < W;
+                xv[k] = in ? static_cast<const float *>(X)[((long long)b * H + gy) * W + gx] : 0.f;
+                xin |= in ? 1u << k : 0u;
+            }
+        } else {
+            const __nv_bfloat16 *xb = static_cast<const __nv_bfloat16 *>(X) + (long long)b * H * W * CIN;
+            constexpr int V = CIN / 8;
+            for (int t = tid; t < PH * PW * V; t += NTHR) {
+                const int v = XL == WG_NHWC ? t % V : t / (PH * PW);
+                const int pix = XL == WG_NHWC ? t / V : t % (PH * PW);
+                const int gy = y0 + pix / PW - 1, gx = x0 + pix % PW - 1;
+                const bool in = gy >= 0 && gy < H && gx >= 0 && gx < W;
+                const long long at = XL == WG_NHWC ? ((long long)gy * W + gx) * CIN + v * 8
+                                                   : (((long long)gy * V + v) * W + gx) * 8;
+                cp_async16_zfill(xbuf + nb * G::PATCH + pix * PS + v * 8, xb + (in ? at : 0), in);
+            }
+        }
+        if constexpr (DL == WG_PLANE) {
+            const int yy = y0 + tid / TW, xx = x0 + tid % TW;
+            dv = yy < H && xx < W ? static_cast<const float *>(dY)[((long long)b * H + yy) * W + xx] : 0.f;
+        } else {
+            const __nv_bfloat16 *db = static_cast<const __nv_bfloat16 *>(dY) + (long long)b * H * W * COUT;
+            constexpr int V = COUT / 8;
+            for (int t = tid; t < TH * TW * V; t += NTHR) {
+                const int v = DL == WG_NHWC ? t % V : t / (TH * TW);
+                const int pix = DL == WG_NHWC ? t / V : t % (TH * TW);
+                const int yy = y0 + pix / TW, xx = x0 + pix % TW;
+                const bool in = yy < H && xx < W;
+                const long long at = DL == WG_NHWC ? ((long long)yy * W + xx) * COUT + v * 8
+                                                   : (((long long)yy * V + v) * W + xx) * 8;
+                cp_async16_zfill(dbuf + nb * G::TILE + pix * DS + v * 8, db + (in ? at : 0), in);
+            }
+        }
+        cp_async_commit_net();
+    };
+    // the planes of the staged tile, rounded to BF16, into buffer nb
+    auto put = [&](int nb) {
+        if constexpr (XL == WG_PLANE) {
+#pragma unroll
+            for (int k = 0; k < XR; ++k) {
+                const int pix = tid + k * NTHR;
+                if (pix < PH * PW)
+                    *reinterpret_cast<__nv_bfloat162 *>(xbuf + nb * G::PATCH + pix * PS) =
+                        __floats2bfloat162_rn(xv[k], xin >> k & 1u ? lv : 0.f);
+            }
+        }
+        if constexpr (DL == WG_PLANE) dbuf[nb * G::TILE + tid * DS] = __float2bfloat16(dv);
+    };
+    static_assert(TH * TW == NTHR, "one pixel of a dY plane per thread");
+    if constexpr (XL == WG_PLANE || DL == WG_PLANE) {  // the channels no plane fills stay zero
+        for (int t = tid; t < (int)(G::smem / 16); t += NTHR)
+            reinterpret_cast<uint4 *>(smem_wg)[t] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+    }
+
+    float acc[MT][NTW][4], bacc[MT][4];
+#pragma unroll
+    for (int m = 0; m < MT; ++m) {
+        bacc[m][0] = bacc[m][1] = bacc[m][2] = bacc[m][3] = 0.f;
 #pragma unroll
         for (int j = 0; j < NTW; ++j) acc[m][j][0] = acc[m][j][1] = acc[m][j][2] = acc[m][j][3] = 0.f;
-    float bsum = 0.f;  // thread t < COUT sums channel t
-    for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int b = (int)(tile / (tiles_x * tiles_y));
-        const int rem = (int)(tile % (tiles_x * tiles_y));
-        const int y0 = (rem / tiles_x) * TH, x0 = (rem % tiles_x) * TW;
-        __syncthreads();
-        load_patch<CIN>(patch, X, b, H, W, y0, x0);
-        for (int t = threadIdx.x; t < TH * TW * (COUT / 8); t += blockDim.x) {
-            const int v = t % (COUT / 8), pix = t / (COUT / 8);
-            const int yy = y0 + pix / TW, xx = x0 + pix % TW;
-            uint4 val = make_uint4(0, 0, 0, 0);
-            if (yy < H && xx < W)
-                val = *reinterpret_cast<const uint4 *>(dY + (((long long)b * H + yy) * W + xx) * COUT + v * 8);
-            *reinterpret_cast<uint4 *>(dys + pix * DS + v * 8) = val;
-        }
-        __syncthreads();
-        if (threadIdx.x < COUT)
-            for (int pix = 0; pix < TH * TW; ++pix) bsum += __bfloat162float(dys[pix * DS + threadIdx.x]);
+    }
+    long long tile = blockIdx.x;
+    if (tile < ntiles) {
+        stage(tile, 0);
+        put(0);
+    }
+    cp_async_wait_net<0>();
+    __syncthreads();
+    int buf = 0;
+    for (; tile < ntiles; tile += gridDim.x) {
+        const bool more = tile + gridDim.x < ntiles;
+        if (more) stage(tile + gridDim.x, buf ^ 1);
+        const __nv_bfloat16 *patch = xbuf + buf * G::PATCH, *dys = dbuf + buf * G::TILE;
         // K loop over the 128 pixels of the tile, 16 at a time (one tile row)
 #pragma unroll 1
         for (int r = 0; r < TH; ++r) {
@@ -315,7 +391,7 @@ __global__ void __launch_bounds__(NTHR)
                 const int nt = warp + 4 * j;
                 if (nt < NT) {
                     // B (k = pixel, n = (tap, ci)) from the patch: rows = pixels, ci contiguous
-                    const int n0 = nt * 8, tap = n0 / CIN, ci = n0 % CIN;
+                    const int n0 = nt * 8, tap = n0 / XC, ci = n0 % XC;
                     const int ky = tap / 3, kx = tap % 3;
                     const int mat = (lane >> 3) & 1, rr = lane & 7;
                     const int px = mat * 8 + rr;  // pixel within the 16-pixel row
@@ -326,50 +402,63 @@ __global__ void __launch_bounds__(NTHR)
                         mma_bf16(acc[m][j], af[m][0], af[m][1], af[m][2], af[m][3], b0, b1);
                 }
             }
+            if ((r & 3) == warp) {  // db: the same rows times ones (BF16 1.0 in every element)
+#pragma unroll
+                for (int m = 0; m < MT; ++m)
+                    mma_bf16(bacc[m], af[m][0], af[m][1], af[m][2], af[m][3], 0x3F803F80u, 0x3F803F80u);
+            }
         }
+        if (more) put(buf ^ 1);
+        cp_async_wait_net<0>();
+        __syncthreads();  // the next tile is there, and every warp is done with this one
+        buf ^= 1;
     }
     // store the block's partial gradient
-    float *row = P + (long long)blockIdx.x * (COUT * N + COUT);
+    float *row = P + (long long)blockIdx.x * G::row;
     const int g = lane >> 2, tq = lane & 3;
 #pragma unroll
     for (int m = 0; m < MT; ++m)
 #pragma unroll
-        for (int j = 0; j < NTW; ++j) {
-            const int nt = warp + 4 * j;
-            if (nt >= NT) continue;
-            const int n = nt * 8 + tq * 2;
+        for (int half = 0; half < 2; ++half) {
+            const int co = m * 16 + g + half * 8;
+            if (tq == 0) bpart[warp][co] = bacc[m][half * 2];  // every column holds the sum
+            if (co >= G::CO) continue;
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                const int co = m * 16 + g + half * 8;
-                *reinterpret_cast<float2 *>(row + co * N + n) =
+            for (int j = 0; j < NTW; ++j) {
+                const int nt = warp + 4 * j;
+                if (nt >= NT) continue;
+                *reinterpret_cast<float2 *>(row + co * N + nt * 8 + tq * 2) =
                     make_float2(acc[m][j][half * 2], acc[m][j][half * 2 + 1]);
             }
         }
-    if (threadIdx.x < COUT) row[COUT * N + threadIdx.x] = bsum;
+    __syncthreads();
+    if (tid < G::CO) row[G::CO * N + tid] = (bpart[0][tid] + bpart[1][tid]) + (bpart[2][tid] + bpart[3][tid]);
 }
 
-// dW[e] += sum_b P[b][e] (e < nw) and db[e - nw] += sum_b P[b][e] (nw <= e < stride),
-// summed in a fixed order: 32 consecutive e per block row of threads, 8 interleaved
-// groups of b per column, the 8 group sums combined in order.
+// dW[e'] += sum_b P[b][e] (e < nw; e = (co, tap, c < xc) goes to e' = (co, tap, c) of cin
+// channels) and db[e - nw] += sum_b P[b][e] (nw <= e < n), summed in a fixed order: 32
+// consecutive e per block row of threads, 8 interleaved groups of b per column, the 8 group
+// sums combined in order.
 constexpr int RED_E = 32, RED_G = 8;
 __global__ void __launch_bounds__(RED_E * RED_G)
-    wgrad_reduce(const float *P, int nblocks, int stride, int nw, float *dW, float *db)
+    wgrad_reduce(const float *P, int nblocks, int stride, int nw, int n, int xc, int cin, float *dW,
+                 float *db)
 {
     __shared__ float part[RED_G][RED_E];
     const int te = threadIdx.x % RED_E, tg = threadIdx.x / RED_E;
     const int e = blockIdx.x * RED_E + te;
     float sum = 0.f;
-    if (e < stride) {
+    if (e < n) {
 #pragma unroll 4
         for (int b = tg; b < nblocks; b += RED_G) sum += P[(long long)b * stride + e];
     }
     part[tg][te] = sum;
     __syncthreads();
-    if (tg == 0 && e < stride) {
+    if (tg == 0 && e < n) {
         float tot = 0.f;
 #pragma unroll
         for (int q = 0; q < RED_G; ++q) tot += part[q][te];
-        if (e < nw) dW[e] += tot;
+        if (e < nw) dW[e / xc * cin + e % xc] += tot;
         else if (db) db[e - nw] += tot;
     }
 }
@@ -414,18 +503,32 @@ tv_status launch_conv(const __nv_bfloat16 *X, int B, int H, int W, const __nv_bf
     return st;
 }
 
-template <int CIN, int COUT>
-tv_status launch_wgrad(const __nv_bfloat16 *X, const __nv_bfloat16 *dY, int B, int H, int W,
-                       float *dW, float *db, float *P, cudaStream_t s)
+template <int CIN, int COUT, int XL = WG_NHWC, int DL = WG_NHWC>
+tv_status launch_wgrad(const void *X, const void *dY, int B, int H, int W, float *dW, float *db,
+                       float *P, cudaStream_t s, const float *lam = nullptr)
 {
+    using G = Wgrad<CIN, COUT, XL, DL>;
+    auto kern = conv3x3_wgrad<CIN, COUT, XL, DL>;
+    static bool attr = false;
+    if (!attr) {
+        tv_status st0 = check_cuda(
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem),
+            "cudaFuncSetAttribute");
+        if (st0 != TV_OK) return st0;
+        st0 = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                              (int)cudaSharedmemCarveoutMaxShared),
+                         "cudaFuncSetAttribute");
+        if (st0 != TV_OK) return st0;
+        attr = true;
+    }
     const long long blocks = wgrad_blocks(B, H, W);
-    conv3x3_wgrad<CIN, COUT><<<(unsigned)blocks, NTHR, 0, s>>>(X, dY, B, H, W, P);
+    kern<<<(unsigned)blocks, NTHR, G::smem, s>>>(X, lam, dY, B, H, W, P);
     tv_status st = check_cuda(cudaGetLastError(), "weight-gradient launch");
     if (st != TV_OK) return st;
     note_launch();
-    constexpr int nw = COUT * 9 * CIN, stride = nw + COUT;
-    wgrad_reduce<<<(stride + RED_E - 1) / RED_E, RED_E * RED_G, 0, s>>>(P, (int)blocks, stride, nw,
-                                                                        dW, db);
+    constexpr int nw = G::CO * G::N, n = nw + G::CO;
+    wgrad_reduce<<<(n + RED_E - 1) / RED_E, RED_E * RED_G, 0, s>>>(P, (int)blocks, G::row, nw, n, G::XC,
+                                                                   CIN, dW, db);
     st = check_cuda(cudaGetLastError(), "weight-gradient reduction");
     if (st == TV_OK) note_launch();
     return st;
@@ -553,6 +656,60 @@ __global__ void dual_head_grad(const float *o, int B, int H, int W, const float 
         dst[0] = __float2bfloat16(g);
 #pragma unroll
         for (int c = 1; c < 16; ++c) dst[c] = __float2bfloat16(0.f);
+    }
+}
+
+// The head in training, on the one-channel output o of the last layer (FP32 plane): the loss
+// partials of dual_head and the gradient of dual_head_grad as a plane, with y only in
+// registers. One thread walks TR rows of a column and carries p and dL/dy from row to row,
+// so that o and the target are read once (12 bytes per pixel: 13 us for
+// 8 x 512 x 512, against 251 us for the two kernels over 16-channel tensors).
+constexpr int TR = 16;
+__global__ void __launch_bounds__(256)
+    head_train(const float *o, int B, int H, int W, const float *lam, const float *target, float *grad,
+               float *loss_part, float inv_count)
+{
+    const int strips = (H + TR - 1) / TR;
+    const long long items = (long long)B * strips * W, stride = (long long)gridDim.x * blockDim.x;
+    float lsum = 0.f;
+    for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < items; it += stride) {
+        const long long sx = it / W;
+        const int x = (int)(it - sx * W), b = (int)(sx / strips), r0 = (int)(sx - (long long)b * strips) * TR;
+        const long long at = (long long)b * H * W + x;
+        const float L = lam[b];
+        auto load = [&](const float *a, int r) { return r >= 0 && r < H ? a[at + (long long)r * W] : 0.f; };
+        auto vert = [&](int r, float th) { return r >= 0 && r < H - 1 ? L * th : 0.f; };
+        // row r needs p at r - 1, r, r + 1 and the target at r, r + 1
+        float th = tanhf(load(o, r0)), p = vert(r0, th);
+        float y = vert(r0 - 1, tanhf(load(o, r0 - 1))) - p;
+        float e = y - load(target, r0);
+#pragma unroll 4
+        for (int k = 0; k < TR; ++k) {
+            const int r = r0 + k;
+            if (r >= H) break;
+            lsum += e * e;
+            const float th1 = tanhf(load(o, r + 1)), p1 = vert(r + 1, th1);
+            const float e1 = (p - p1) - load(target, r + 1);
+            float g = 0.f;
+            if (r < H - 1) {
+                const float dy_next = 2.f * e1 * inv_count, dy_here = 2.f * e * inv_count;
+                g = (dy_next - dy_here) * L * (1.f - th * th);
+            }
+            grad[at + (long long)r * W] = g;
+            th = th1;
+            p = p1;
+            e = e1;
+        }
+    }
+    __shared__ float wsum[8];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, off);
+    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = lsum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float t = 0.f;
+        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) t += wsum[q];
+        loss_part[blockIdx.x] = t * inv_count;
     }
 }
 
@@ -911,7 +1068,12 @@ __global__ void __launch_bounds__(NTHR)
 //    group 0 of the slot (channels 2..15 stay zero); act_out grouped.
 //  * TW_HEAD (the last layer, COUT = 16): x grouped; the epilogue keeps only channel 0, o,
 //    and writes p = lambda tanh(o) on the vertical edges (rows 0 .. H - 2, 0 on the last
-//    row) for the dual head.
+//    row) for the dual head; in training (lam null) it writes o itself.
+// Training runs the forward layers in the grouped layout and the backward-data ones with
+// the taps reversed as the weights are staged (TwTrain); TW_IMAGE with lam null reads the
+// one-channel gradient of o that way. Each accumulator adds its taps and K steps in the
+// order of the mma.sync kernel and gets the same bits (measured over whole gradients, three
+// batch shapes).
 // Every wait gives up after kTcSpin polls (counted in g_tc_timeouts; the tile is then not
 // written) and the other roles stop at their next wait.
 constexpr int TW_NHWC = 0, TW_GROUPED = 1, TW_IMAGE = 2, TW_HEAD = 3;
@@ -988,6 +1150,15 @@ __device__ __forceinline__ TwChunk tw_chunk(long long c, int cpc, int L, int til
     return r;
 }
 
+// What training adds to the convolution (all null / false at inference). Only the sign of
+// a pre-activation is needed again on the way back, so a layer leaves one word per pixel
+// (bit c: channel c > 0, exact) instead of its 32 FP32 pre-activations.
+struct TwTrain {
+    unsigned *mask_out;       // forward: the ReLU masks of this layer's 32 outputs
+    const unsigned *mask_in;  // backward data: the masks its 32 outputs are multiplied by
+    bool flip;                // backward data: Wt is the forward layer's [CIN][3][3][COUT]
+};
+
 // Walks the input rows of a block's chunks in load order (n + 2 rows per chunk).
 struct TwRows {
     long long c, nchunks;
@@ -1026,7 +1197,8 @@ template <int CIN, int COUT, int IO>
 __global__ void __launch_bounds__(TW_THREADS, 4)
     conv3x3_tw(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap_tail,
                int B, int H, int W, int L, const __nv_bfloat16 *Wt, const float *bias, int relu,
-               float *pre_out, __nv_bfloat16 *act_out, const float *img, const float *lam, float *p_out)
+               float *pre_out, __nv_bfloat16 *act_out, const float *img, const float *lam, float *p_out,
+               TwTrain tr)
 {
     static_assert(IO != TW_IMAGE || CIN == 16, "the image input has 16 (2 non-zero) channels");
     static_assert(IO != TW_HEAD || COUT == 16, "the head reads a 16-channel output");
@@ -1086,8 +1258,19 @@ __global__ void __launch_bounds__(TW_THREADS, 4)
     // weights: [dx][group][dy][co][8 channels]
     for (int t = tid; t < 9 * KG * COUT; t += TW_THREADS) {
         const int co = t % COUT, dy = (t / COUT) % 3, g = (t / (3 * COUT)) % KG, dx = t / (3 * COUT * KG);
-        *reinterpret_cast<uint4 *>(bbuf + (size_t)t * 16) =
-            *reinterpret_cast<const uint4 *>(Wt + ((long long)co * 9 + dy * 3 + dx) * CIN + g * 8);
+        uint4 *dst = reinterpret_cast<uint4 *>(bbuf + (size_t)t * 16);
+        if (tr.flip) {  // the taps in reverse, the channel roles swapped
+            unsigned u[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const __nv_bfloat16 *src = Wt + ((long long)(g * 8 + 2 * e) * 9 + 8 - dy * 3 - dx) * COUT + co;
+                const __nv_bfloat162 h = __halves2bfloat162(src[0], src[9 * COUT]);
+                u[e] = *reinterpret_cast<const unsigned *>(&h);
+            }
+            *dst = make_uint4(u[0], u[1], u[2], u[3]);
+        } else {
+            *dst = *reinterpret_cast<const uint4 *>(Wt + ((long long)co * 9 + dy * 3 + dx) * CIN + g * 8);
+        }
     }
     if (tid < COUT) bias_s[tid] = bias ? bias[tid] : 0.f;
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // weights for the MMAs
@@ -1118,7 +1301,7 @@ __global__ void __launch_bounds__(TW_THREADS, 4)
         auto load_row = [&](const TwRows &rw, float (&v)[5], unsigned &mask, float &lv) {
             const int y = rw.ch.y0 - 1 + rw.r;
             const float *src = img + ((long long)rw.ch.b * H + (y < 0 ? 0 : y)) * W;
-            lv = lam[rw.ch.b];
+            lv = lam ? lam[rw.ch.b] : 0.f;
             mask = 0u;
 #pragma unroll
             for (int kk = 0; kk < 5; ++kk) {
@@ -1325,6 +1508,10 @@ __global__ void __launch_bounds__(TW_THREADS, 4)
             const TwChunk ch = tw_chunk(ck, cpc, L, tiles_x, H);
             for (int j = 0; j < ch.n; ++j, ++o) {
                 const int k = tw_block<TW_R>(o);
+                const long long row = (long long)ch.b * H + ch.y0 + j;
+                const int x = ch.x0 + lg * 32 + lane;
+                unsigned keep = 0xffffffffu;  // read ahead of the wait
+                if (tr.mask_in && x < W) keep = tr.mask_in[row * W + x];
                 int got = 1;
                 if (lane == 0) got = tw_wait(c_full(k), (o / TW_R) & 1u, bad) ? 1 : 0;
                 got = __shfl_sync(0xffffffffu, got, 0);
@@ -1341,17 +1528,21 @@ __global__ void __launch_bounds__(TW_THREADS, 4)
                 asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                 __syncwarp();
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(c_empty(k)) : "memory");
-                const long long row = (long long)ch.b * H + ch.y0 + j;
-                const int x = ch.x0 + lg * 32 + lane;
                 if (IO == TW_HEAD && x < W) {
-                    p_out[row * W + x] = ch.y0 + j < H - 1 ? lam[ch.b] * tanhf(v[0] + bias_s[0]) : 0.f;
+                    const float o0 = v[0] + bias_s[0];
+                    p_out[row * W + x] = !lam ? o0 : ch.y0 + j < H - 1 ? lam[ch.b] * tanhf(o0) : 0.f;
                 } else if (x < W) {
                     const long long pbase = (row * W + x) * COUT;
+                    unsigned signs = 0u;
 #pragma unroll
                     for (int c = 0; c < COUT; c += 8) {
                         float q[8];
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) q[e] = v[c + e] + bias_s[c + e];
+                        for (int e = 0; e < 8; ++e) {
+                            q[e] = v[c + e] + bias_s[c + e];
+                            signs |= q[e] > 0.f ? 1u << (c + e) : 0u;
+                            if (!(keep >> (c + e) & 1u)) q[e] = 0.f;
+                        }
                         if (pre_out) {
                             *reinterpret_cast<float4 *>(pre_out + pbase + c) = make_float4(q[0], q[1], q[2], q[3]);
                             *reinterpret_cast<float4 *>(pre_out + pbase + c + 4) = make_float4(q[4], q[5], q[6], q[7]);
@@ -1373,6 +1564,7 @@ __global__ void __launch_bounds__(TW_THREADS, 4)
                             *reinterpret_cast<uint4 *>(act_out + o8) = make_uint4(u[0], u[1], u[2], u[3]);
                         }
                     }
+                    if (tr.mask_out) tr.mask_out[row * W + x] = signs;
                 }
             }
         }
@@ -1410,7 +1602,7 @@ template <int CIN, int COUT, int IO>
 tv_status launch_conv_tw(const __nv_bfloat16 *X, int B, int H, int W, const __nv_bfloat16 *Wt,
                          const float *bias, int relu, float *pre_out, __nv_bfloat16 *act_out,
                          cudaStream_t s, const float *img = nullptr, const float *lam = nullptr,
-                         float *p_out = nullptr)
+                         float *p_out = nullptr, TwTrain tr = {nullptr, nullptr, false})
 {
     TmapEncodeFn enc = tmap_encoder();
     if (!enc) {
@@ -1496,7 +1688,7 @@ tv_status launch_conv_tw(const __nv_bfloat16 *X, int B, int H, int W, const __nv
     PdlScope pdl(true);
     tv_status st = check_cuda(launch_k(kern, dim3((unsigned)blocks), dim3(TW_THREADS), smem, s, tmap,
                                        tmap_tail, B, H, W, (int)L, Wt, bias, relu, pre_out, act_out,
-                                       img, lam, p_out),
+                                       img, lam, p_out, tr),
                               "conv launch");
     if (st == TV_OK) note_launch();
     return st;
@@ -1918,6 +2110,93 @@ tv_status tv_net_dual_head(const float *d_o, int B, int H, int W, const float *d
         if (st == TV_OK) note_launch();
     }
     return st;
+}
+
+tv_status tv_net_train_layer(const void *d_x, const float *d_f, const float *d_lam, int B, int H,
+                             int W, const void *d_w, const float *d_bias, void *d_act_out,
+                             uint32_t *d_mask_out, tv_stream_t stream)
+{
+    clear_error();
+    if ((!d_x && (!d_f || !d_lam)) || !d_w || !d_act_out || !d_mask_out || !valid_shape(B, H, W) ||
+        !aligned16(d_x) || !aligned16(d_w) || !aligned16(d_act_out)) {
+        set_error("tv_net_train_layer: need x (or f and lam), w, act_out and mask_out, 16-byte aligned "
+                  "x, w and act_out, 1 <= B <= 65535, H, W >= 1");
+        return TV_ERR_INVALID;
+    }
+    cudaStream_t s = (cudaStream_t)stream;
+    auto X = static_cast<const __nv_bfloat16 *>(d_x);
+    auto Wt = static_cast<const __nv_bfloat16 *>(d_w);
+    auto A = static_cast<__nv_bfloat16 *>(d_act_out);
+    const TwTrain tr{d_mask_out, nullptr, false};
+    if (X) return launch_conv_tw<32, 32, TW_GROUPED>(X, B, H, W, Wt, d_bias, 1, nullptr, A, s, nullptr, nullptr, nullptr, tr);
+    return launch_conv_tw<16, 32, TW_IMAGE>(nullptr, B, H, W, Wt, d_bias, 1, nullptr, A, s, d_f, d_lam, nullptr, tr);
+}
+
+tv_status tv_net_train_head(const void *d_x, int B, int H, int W, const void *d_w, const float *d_bias,
+                            const float *d_lam, const float *d_target, float *d_o, float *d_loss,
+                            float *d_grad_o, void *d_ws, size_t ws_bytes, tv_stream_t stream)
+{
+    clear_error();
+    if (!d_x || !d_w || !d_lam || !d_target || !d_o || !d_loss || !d_grad_o || !d_ws ||
+        !valid_shape(B, H, W) || !aligned16(d_x) || !aligned16(d_w)) {
+        set_error("tv_net_train_head: bad arguments (null, shape or alignment)");
+        return TV_ERR_INVALID;
+    }
+    const long long N = (long long)B * H * W;
+    const long long items = (long long)B * ((H + TR - 1) / TR) * W;
+    const int blocks = (int)std::min<long long>((items + 255) / 256, ew_blocks(N));
+    if (ws_bytes < (size_t)blocks * sizeof(float)) {
+        set_error("tv_net_train_head: workspace smaller than tv_net_workspace_size");
+        return TV_ERR_INVALID;
+    }
+    cudaStream_t s = (cudaStream_t)stream;
+    tv_status st = launch_conv_tw<32, 16, TW_HEAD>(static_cast<const __nv_bfloat16 *>(d_x), B, H, W,
+                                                   static_cast<const __nv_bfloat16 *>(d_w), d_bias, 0,
+                                                   nullptr, nullptr, s, nullptr, nullptr, d_o);
+    if (st != TV_OK) return st;
+    float *part = static_cast<float *>(d_ws);
+    head_train<<<blocks, 256, 0, s>>>(d_o, B, H, W, d_lam, d_target, d_grad_o, part, 1.f / (float)N);
+    st = check_cuda(cudaGetLastError(), "dual head gradient");
+    if (st != TV_OK) return st;
+    note_launch();
+    sum_partials<<<1, 256, 0, s>>>(part, blocks, d_loss);
+    st = check_cuda(cudaGetLastError(), "loss sum");
+    if (st == TV_OK) note_launch();
+    return st;
+}
+
+tv_status tv_net_train_backward(const void *d_x, const float *d_f, const float *d_lam,
+                                const void *d_dy, const float *d_grad_o, int B, int H, int W,
+                                const void *d_w, const uint32_t *d_mask, void *d_dx, float *d_dw,
+                                float *d_db, void *d_ws, size_t ws_bytes, tv_stream_t stream)
+{
+    clear_error();
+    if ((!d_x && (!d_f || !d_lam)) || !d_dy == !d_grad_o || (!d_x && !d_dy) || !d_dw || !d_ws ||
+        (d_x && (!d_w || !d_mask || !d_dx)) || !valid_shape(B, H, W) || !aligned16(d_x) ||
+        !aligned16(d_dy) || !aligned16(d_w) || !aligned16(d_dx) || !aligned16(d_ws)) {
+        set_error("tv_net_train_backward: bad arguments (null, shape or alignment)");
+        return TV_ERR_INVALID;
+    }
+    if (ws_bytes < tv_net_workspace_size(B, H, W)) {
+        set_error("tv_net_train_backward: workspace smaller than tv_net_workspace_size");
+        return TV_ERR_INVALID;
+    }
+    cudaStream_t s = (cudaStream_t)stream;
+    float *P = static_cast<float *>(d_ws);
+    if (!d_x)  // the first layer: no gradient of its input
+        return launch_wgrad<16, 32, WG_PLANE, WG_GROUPED>(d_f, d_dy, B, H, W, d_dw, d_db, P, s, d_lam);
+    const TwTrain tr{nullptr, d_mask, true};
+    auto Wt = static_cast<const __nv_bfloat16 *>(d_w);
+    auto dX = static_cast<__nv_bfloat16 *>(d_dx);
+    tv_status st;
+    if (d_grad_o) {  // the last layer: one channel of dY
+        st = launch_wgrad<32, 16, WG_GROUPED, WG_PLANE>(d_x, d_grad_o, B, H, W, d_dw, d_db, P, s);
+        if (st != TV_OK) return st;
+        return launch_conv_tw<16, 32, TW_IMAGE>(nullptr, B, H, W, Wt, nullptr, 0, nullptr, dX, s, d_grad_o, nullptr, nullptr, tr);
+    }
+    st = launch_wgrad<32, 32, WG_GROUPED, WG_GROUPED>(d_x, d_dy, B, H, W, d_dw, d_db, P, s);
+    if (st != TV_OK) return st;
+    return launch_conv_tw<32, 32, TW_GROUPED>(static_cast<const __nv_bfloat16 *>(d_dy), B, H, W, Wt, nullptr, 0, nullptr, dX, s, nullptr, nullptr, nullptr, tr);
 }
 
 tv_status tv_net_adam(float *d_w, float *d_m, float *d_v, float *d_g, int64_t n, float lr,

@@ -80,7 +80,6 @@ class WarmStartNet:
         self.meta = {}
         # inference activations in the channel-group layout on the TMA-fed tcgen05 kernel
         self.grouped_inference = True
-        self._flip = torch.empty(32 * 9 * 32, dtype=torch.bfloat16, device=self.device)
         self._bufs = {}
         self._refresh_bf16()
 
@@ -130,23 +129,25 @@ class WarmStartNet:
             nws = self.lib.tv_net_workspace_size(B, H, W)
             if nws == 0:
                 raise ValueError(f"unsupported batch shape {(B, H, W)}")
-            bufs = {"x0": torch.empty(n * 16, dtype=bf, device=dev),
-                    "ws": torch.empty(nws, dtype=torch.uint8, device=dev),
-                    "o": torch.empty(n * 16, dtype=torch.float32, device=dev),
-                    "y": torch.empty(B, H, W, dtype=torch.float32, device=dev),
-                    "loss": torch.zeros(1, dtype=torch.float32, device=dev)}
-            bufs["acts"] = [torch.empty(n * cout, dtype=bf, device=dev) for _, cout, _ in LAYERS[:-1]]
+            bufs = {"ws": torch.empty(nws, dtype=torch.uint8, device=dev),
+                    "acts": [torch.empty(n * cout, dtype=bf, device=dev) for _, cout, _ in LAYERS[:-1]]}
             if train:
-                bufs["pres"] = [torch.empty(n * cout, dtype=torch.float32, device=dev)
-                                for _, cout, _ in LAYERS[:-1]]
-                bufs["g_o"] = torch.empty(n * 16, dtype=bf, device=dev)
+                # per pixel one word of ReLU signs per hidden layer, o and its gradient
+                bufs["masks"] = [torch.empty(n, dtype=torch.int32, device=dev) for _ in LAYERS[:-1]]
+                bufs["o"] = torch.empty(n, dtype=torch.float32, device=dev)
+                bufs["g_o"] = torch.empty(n, dtype=torch.float32, device=dev)
                 bufs["g_a"] = torch.empty(n * 32, dtype=bf, device=dev)
                 bufs["g_b"] = torch.empty(n * 32, dtype=bf, device=dev)
+                bufs["loss"] = torch.zeros(1, dtype=torch.float32, device=dev)
+            else:
+                bufs["x0"] = torch.empty(n * 16, dtype=bf, device=dev)
+                bufs["o"] = torch.empty(n * 16, dtype=torch.float32, device=dev)
+                bufs["y"] = torch.empty(B, H, W, dtype=torch.float32, device=dev)
             self._bufs = {key: bufs}  # keep one shape at a time
         return bufs
 
     # ---------------------------------------------------------------- forward --
-    def _forward(self, f, lam, bufs, train):
+    def _forward(self, f, lam, bufs):
         B, H, W = f.shape
         s = _lib._stream(self.device)
         lib = self.lib
@@ -154,7 +155,7 @@ class WarmStartNet:
         x = bufs["x0"]
         for li, ((cin, cout, relu), (w_off, b_off)) in enumerate(zip(LAYERS, self.offsets)):
             last = li == len(LAYERS) - 1
-            pre = bufs["o"] if last else (bufs["pres"][li] if train else None)
+            pre = bufs["o"] if last else None
             act = None if last else bufs["acts"][li]
             _lib._check(lib.tv_net_conv3x3(_vp(x), B, H, W, cin, _vp(self.params_bf16, w_off),
                                            _vp(self.params, b_off), cout, int(relu), _lib._ptr(pre),
@@ -171,7 +172,7 @@ class WarmStartNet:
         ``grouped`` (default ``self.grouped_inference``) the activations are kept in the
         channel-group layout, every layer runs on tcgen05 (the first from the image rows,
         the others fed by TMA) and the last layer's epilogue applies the head.
-        ``predict_dual_layers`` computes the same through the kernels of training."""
+        ``predict_dual_layers`` computes the same through the general NHWC kernels."""
         f, lam = self._inputs(f, lam)
         B, H, W = f.shape
         bufs = self._buffers(B, H, W, train=False)
@@ -207,7 +208,7 @@ class WarmStartNet:
         f, lam = self._inputs(f, lam)
         B, H, W = f.shape
         bufs = self._buffers(B, H, W, train=False)
-        self._forward(f, lam, bufs, train=False)
+        self._forward(f, lam, bufs)
         _lib._check(self.lib.tv_net_dual_head(_vp(bufs["o"]), B, H, W, _vp(lam), None,
                                               _vp(bufs["y"]), None, None, None, 0,
                                               _lib._stream(self.device)))
@@ -238,28 +239,30 @@ class WarmStartNet:
         bufs = self._buffers(B, H, W, train=True)
         s = _lib._stream(self.device)
         lib = self.lib
-        self._forward(f, lam, bufs, train=True)
         ws, nws = bufs["ws"], bufs["ws"].numel()
-        _lib._check(lib.tv_net_dual_head(_vp(bufs["o"]), B, H, W, _vp(lam), _vp(target),
-                                         _vp(bufs["y"]), _vp(bufs["loss"]), _vp(bufs["g_o"]),
-                                         _vp(ws), nws, s))
-        dy = bufs["g_o"]
+        acts, masks, offs = bufs["acts"], bufs["masks"], self.offsets
+        last = len(LAYERS) - 1
+        for li in range(last):
+            _lib._check(lib.tv_net_train_layer(_vp(acts[li - 1]) if li else None, _vp(f), _vp(lam),
+                                               B, H, W, _vp(self.params_bf16, offs[li][0]),
+                                               _vp(self.params, offs[li][1]), _vp(acts[li]),
+                                               _vp(masks[li]), s))
+        _lib._check(lib.tv_net_train_head(_vp(acts[-1]), B, H, W,
+                                          _vp(self.params_bf16, offs[last][0]),
+                                          _vp(self.params, offs[last][1]), _vp(lam), _vp(target),
+                                          _vp(bufs["o"]), _vp(bufs["loss"]), _vp(bufs["g_o"]),
+                                          _vp(ws), nws, s))
+        dy = None
         spare = [bufs["g_a"], bufs["g_b"]]
-        for li in range(len(LAYERS) - 1, -1, -1):
-            cin, cout, _ = LAYERS[li]
-            w_off, b_off = self.offsets[li]
-            x_in = bufs["x0"] if li == 0 else bufs["acts"][li - 1]
-            _lib._check(lib.tv_net_conv3x3_backward_weight(_vp(x_in), _vp(dy), B, H, W, cin, cout,
-                                                           _vp(self.grad, w_off),
-                                                           _vp(self.grad, b_off), _vp(ws), nws,
-                                                           s))
-            if li > 0:
-                dx = spare[li % 2]
-                _lib._check(lib.tv_net_conv3x3_backward_data(_vp(dy), B, H, W, cout,
-                                                             _vp(self.params_bf16, w_off), cin,
-                                                             _vp(bufs["pres"][li - 1]), _vp(dx),
-                                                             _vp(self._flip), s))
-                dy = dx
+        for li in range(last, -1, -1):
+            dx = spare[li % 2] if li else None
+            _lib._check(lib.tv_net_train_backward(
+                _vp(acts[li - 1]) if li else None, _vp(f), _vp(lam), _lib._ptr(dy),
+                _vp(bufs["g_o"]) if li == last else None, B, H, W,
+                _vp(self.params_bf16, offs[li][0]), _vp(masks[li - 1]) if li else None,
+                _lib._ptr(dx), _vp(self.grad, offs[li][0]), _vp(self.grad, offs[li][1]), _vp(ws),
+                nws, s))
+            dy = dx
         return bufs["loss"]
 
     def optimizer_step(self):
