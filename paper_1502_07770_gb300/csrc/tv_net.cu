@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(NTHR)
 // Partial sums of dW[co][tap][ci] = sum over pixels p of dY[p][co] * X[p + tap][ci]
 // and db[co] = sum_p dY[p][co]. Each block walks tiles blockIdx.x, +gridDim.x, ...,
 // keeps its partial dW in registers (warp w owns the n8 column tiles w, w+4, ... of
-// N = 9 * XC; both m16 tiles (co 0..31) or one (co 0..15)) and stores it, with its
+// N = 9 * CIN; both m16 tiles (co 0..31) or one (co 0..15)) and stores it, with its
 // partial db, to row blockIdx.x of P; the rows are summed in a fixed order by
 // wgrad_reduce, so the result is deterministic. db comes from the same tensor-core pass
 // (a column tile of ones, warp w taking tile rows w and w + 4).
@@ -250,33 +250,22 @@ __global__ void __launch_bounds__(NTHR)
 // is copied asynchronously into a second buffer while the current one is multiplied (one
 // barrier per tile). 32 -> 32 channels, 8 x 512 x 512: 128 us, against 268 us with
 // one buffer, synchronous loads and db summed serially by 32 threads.
-// XL and DL say how X and dY lie in memory:
-//   WG_NHWC     [image][row][pixel][C] BF16
-//   WG_GROUPED  [image][row][C/8][pixel][8] BF16
-//   WG_PLANE    FP32 planes, rounded to BF16 on the way in. X: the image and its lambda
-//               (the 16-channel input's channels 0 and 1; channels 2..15 are zero, their
-//               gradients too, so 8 columns per tap are computed: XC = 8); dY: channel 0
-//               of 16 (the others are zero: only row co = 0 is stored).
-constexpr int WG_NHWC = 0, WG_GROUPED = 1, WG_PLANE = 2;
-
-template <int CIN, int COUT, int XL, int DL>
+// X and dY lie in memory as [image][row][pixel][C], or GROUPED, [image][row][C/8][pixel][8].
+template <int CIN, int COUT>
 struct Wgrad {
-    static constexpr int XC = XL == WG_PLANE ? 8 : CIN;     // columns per tap
-    static constexpr int CO = DL == WG_PLANE ? 1 : COUT;    // rows stored
-    // padded pixel strides (bf16); 16-byte rows need no padding
-    static constexpr int PS = XC == 8 ? 8 : XC + 8, DS = COUT + 8;
+    static constexpr int PS = CIN + 8, DS = COUT + 8;       // padded pixel strides (bf16)
     static constexpr int PATCH = PH * PW * PS, TILE = TH * TW * DS;
-    static constexpr int N = 9 * XC, NT = N / 8, NTW = (NT + 3) / 4, MT = COUT / 16;
+    static constexpr int N = 9 * CIN, NT = N / 8, NTW = (NT + 3) / 4, MT = COUT / 16;
     static constexpr size_t smem = sizeof(__nv_bfloat16) * 2 * (size_t)(PATCH + TILE);
-    static constexpr int row = (CO * N + CO + 3) / 4 * 4;   // floats per block in P (16-byte rows)
+    static constexpr int row = COUT * N + COUT;             // floats per block in P
 };
 
-template <int CIN, int COUT, int XL, int DL>
+template <int CIN, int COUT, bool GROUPED>
 __global__ void __launch_bounds__(NTHR, 4)
-    conv3x3_wgrad(const void *X, const float *lam, const void *dY, int B, int H, int W, float *P)
+    conv3x3_wgrad(const __nv_bfloat16 *X, const __nv_bfloat16 *dY, int B, int H, int W, float *P)
 {
-    using G = Wgrad<CIN, COUT, XL, DL>;
-    constexpr int PS = G::PS, DS = G::DS, N = G::N, NT = G::NT, NTW = G::NTW, MT = G::MT, XC = G::XC;
+    using G = Wgrad<CIN, COUT>;
+    constexpr int PS = G::PS, DS = G::DS, N = G::N, NT = G::NT, NTW = G::NTW, MT = G::MT;
     extern __shared__ __align__(16) unsigned char smem_wg[];
     __nv_bfloat16 *xbuf = reinterpret_cast<__nv_bfloat16 *>(smem_wg);
     __nv_bfloat16 *dbuf = xbuf + 2 * G::PATCH;
@@ -286,73 +275,28 @@ __global__ void __launch_bounds__(NTHR, 4)
     const int per_img = tiles_x * tiles_y;
     const long long ntiles = (long long)B * per_img;
 
-    constexpr int XR = (PH * PW + NTHR - 1) / NTHR;  // plane pixels of a patch per thread
-    [[maybe_unused]] float xv[XR], dv = 0.f, lv = 0.f;
-    [[maybe_unused]] unsigned xin = 0u;
-    // start the loads of a tile: asynchronous copies into buffer nb, planes into registers
+    // start the copies of a tile into buffer nb
     auto stage = [&](long long tile, int nb) {
         const int b = (int)(tile / per_img), rem = (int)(tile - (long long)b * per_img);
         const int y0 = (rem / tiles_x) * TH, x0 = (rem % tiles_x) * TW;
-        if constexpr (XL == WG_PLANE) {
-            lv = lam[b];
-            xin = 0u;
-#pragma unroll
-            for (int k = 0; k < XR; ++k) {
-                const int pix = tid + k * NTHR, gy = y0 + pix / PW - 1, gx = x0 + pix % PW - 1;
-                const bool in = pix < PH * PW && gy >= 0 && gy < H && gx >= 0 && gx < W;
-                xv[k] = in ? static_cast<const float *>(X)[((long long)b * H + gy) * W + gx] : 0.f;
-                xin |= in ? 1u << k : 0u;
-            }
-        } else {
-            const __nv_bfloat16 *xb = static_cast<const __nv_bfloat16 *>(X) + (long long)b * H * W * CIN;
-            constexpr int V = CIN / 8;
-            for (int t = tid; t < PH * PW * V; t += NTHR) {
-                const int v = XL == WG_NHWC ? t % V : t / (PH * PW);
-                const int pix = XL == WG_NHWC ? t / V : t % (PH * PW);
-                const int gy = y0 + pix / PW - 1, gx = x0 + pix % PW - 1;
-                const bool in = gy >= 0 && gy < H && gx >= 0 && gx < W;
-                const long long at = XL == WG_NHWC ? ((long long)gy * W + gx) * CIN + v * 8
-                                                   : (((long long)gy * V + v) * W + gx) * 8;
-                cp_async16_zfill(xbuf + nb * G::PATCH + pix * PS + v * 8, xb + (in ? at : 0), in);
-            }
+        const __nv_bfloat16 *xb = X + (long long)b * H * W * CIN, *db = dY + (long long)b * H * W * COUT;
+        auto at = [&](int y, int x, int v, int V) {
+            return GROUPED ? (((long long)y * V + v) * W + x) * 8 : (((long long)y * W + x) * V + v) * 8;
+        };
+        for (int t = tid; t < PH * PW * (CIN / 8); t += NTHR) {
+            const int v = GROUPED ? t / (PH * PW) : t % (CIN / 8), pix = GROUPED ? t % (PH * PW) : t / (CIN / 8);
+            const int gy = y0 + pix / PW - 1, gx = x0 + pix % PW - 1;
+            const bool in = gy >= 0 && gy < H && gx >= 0 && gx < W;
+            cp_async16_zfill(xbuf + nb * G::PATCH + pix * PS + v * 8, xb + (in ? at(gy, gx, v, CIN / 8) : 0), in);
         }
-        if constexpr (DL == WG_PLANE) {
-            const int yy = y0 + tid / TW, xx = x0 + tid % TW;
-            dv = yy < H && xx < W ? static_cast<const float *>(dY)[((long long)b * H + yy) * W + xx] : 0.f;
-        } else {
-            const __nv_bfloat16 *db = static_cast<const __nv_bfloat16 *>(dY) + (long long)b * H * W * COUT;
-            constexpr int V = COUT / 8;
-            for (int t = tid; t < TH * TW * V; t += NTHR) {
-                const int v = DL == WG_NHWC ? t % V : t / (TH * TW);
-                const int pix = DL == WG_NHWC ? t / V : t % (TH * TW);
-                const int yy = y0 + pix / TW, xx = x0 + pix % TW;
-                const bool in = yy < H && xx < W;
-                const long long at = DL == WG_NHWC ? ((long long)yy * W + xx) * COUT + v * 8
-                                                   : (((long long)yy * V + v) * W + xx) * 8;
-                cp_async16_zfill(dbuf + nb * G::TILE + pix * DS + v * 8, db + (in ? at : 0), in);
-            }
+        for (int t = tid; t < TH * TW * (COUT / 8); t += NTHR) {
+            const int v = GROUPED ? t / (TH * TW) : t % (COUT / 8), pix = GROUPED ? t % (TH * TW) : t / (COUT / 8);
+            const int yy = y0 + pix / TW, xx = x0 + pix % TW;
+            const bool in = yy < H && xx < W;
+            cp_async16_zfill(dbuf + nb * G::TILE + pix * DS + v * 8, db + (in ? at(yy, xx, v, COUT / 8) : 0), in);
         }
         cp_async_commit_net();
     };
-    // the planes of the staged tile, rounded to BF16, into buffer nb
-    auto put = [&](int nb) {
-        if constexpr (XL == WG_PLANE) {
-#pragma unroll
-            for (int k = 0; k < XR; ++k) {
-                const int pix = tid + k * NTHR;
-                if (pix < PH * PW)
-                    *reinterpret_cast<__nv_bfloat162 *>(xbuf + nb * G::PATCH + pix * PS) =
-                        __floats2bfloat162_rn(xv[k], xin >> k & 1u ? lv : 0.f);
-            }
-        }
-        if constexpr (DL == WG_PLANE) dbuf[nb * G::TILE + tid * DS] = __float2bfloat16(dv);
-    };
-    static_assert(TH * TW == NTHR, "one pixel of a dY plane per thread");
-    if constexpr (XL == WG_PLANE || DL == WG_PLANE) {  // the channels no plane fills stay zero
-        for (int t = tid; t < (int)(G::smem / 16); t += NTHR)
-            reinterpret_cast<uint4 *>(smem_wg)[t] = make_uint4(0u, 0u, 0u, 0u);
-        __syncthreads();
-    }
 
     float acc[MT][NTW][4], bacc[MT][4];
 #pragma unroll
@@ -362,16 +306,12 @@ __global__ void __launch_bounds__(NTHR, 4)
         for (int j = 0; j < NTW; ++j) acc[m][j][0] = acc[m][j][1] = acc[m][j][2] = acc[m][j][3] = 0.f;
     }
     long long tile = blockIdx.x;
-    if (tile < ntiles) {
-        stage(tile, 0);
-        put(0);
-    }
+    if (tile < ntiles) stage(tile, 0);
     cp_async_wait_net<0>();
     __syncthreads();
     int buf = 0;
     for (; tile < ntiles; tile += gridDim.x) {
-        const bool more = tile + gridDim.x < ntiles;
-        if (more) stage(tile + gridDim.x, buf ^ 1);
+        if (tile + gridDim.x < ntiles) stage(tile + gridDim.x, buf ^ 1);
         const __nv_bfloat16 *patch = xbuf + buf * G::PATCH, *dys = dbuf + buf * G::TILE;
         // K loop over the 128 pixels of the tile, 16 at a time (one tile row)
 #pragma unroll 1
@@ -391,7 +331,7 @@ __global__ void __launch_bounds__(NTHR, 4)
                 const int nt = warp + 4 * j;
                 if (nt < NT) {
                     // B (k = pixel, n = (tap, ci)) from the patch: rows = pixels, ci contiguous
-                    const int n0 = nt * 8, tap = n0 / XC, ci = n0 % XC;
+                    const int n0 = nt * 8, tap = n0 / CIN, ci = n0 % CIN;
                     const int ky = tap / 3, kx = tap % 3;
                     const int mat = (lane >> 3) & 1, rr = lane & 7;
                     const int px = mat * 8 + rr;  // pixel within the 16-pixel row
@@ -408,7 +348,6 @@ __global__ void __launch_bounds__(NTHR, 4)
                     mma_bf16(bacc[m], af[m][0], af[m][1], af[m][2], af[m][3], 0x3F803F80u, 0x3F803F80u);
             }
         }
-        if (more) put(buf ^ 1);
         cp_async_wait_net<0>();
         __syncthreads();  // the next tile is there, and every warp is done with this one
         buf ^= 1;
@@ -422,7 +361,6 @@ __global__ void __launch_bounds__(NTHR, 4)
         for (int half = 0; half < 2; ++half) {
             const int co = m * 16 + g + half * 8;
             if (tq == 0) bpart[warp][co] = bacc[m][half * 2];  // every column holds the sum
-            if (co >= G::CO) continue;
 #pragma unroll
             for (int j = 0; j < NTW; ++j) {
                 const int nt = warp + 4 * j;
@@ -432,14 +370,158 @@ __global__ void __launch_bounds__(NTHR, 4)
             }
         }
     __syncthreads();
-    if (tid < G::CO) row[G::CO * N + tid] = (bpart[0][tid] + bpart[1][tid]) + (bpart[2][tid] + bpart[3][tid]);
+    if (tid < COUT) row[COUT * N + tid] = (bpart[0][tid] + bpart[1][tid]) + (bpart[2][tid] + bpart[3][tid]);
+}
+
+// The weight gradients of the training step's first and last layer, where one side of the
+// product is a plane: (FIRST) X is the image and its lambda, dY the 32-channel tensor T; else
+// dY is channel 0 of 16, an FP32 plane, and X is T. The plane is unfolded into the columns of
+// each pixel (rounded to BF16), which makes the nine taps one GEMM over pixels,
+//     S[c][n] = sum over pixels q of T[q][c] * col[q][n],
+//   FIRST: col[q][2 tap + i] = channel i of x at q + tap, col[q][18] = 1 (the bias gradient);
+//   last:  col[q][tap] = dY at q - tap; the bias gradient is the column sum of the centre tap.
+// A 16-pixel row of T (grouped, M = 32) is then read from shared memory once for all taps,
+// with 2 n8 tiles (3 if FIRST) instead of the general kernel's 36 (18): what is left is the
+// read of T. Warp w takes the tile's rows w and w + 4; the four sums are added at the end.
+// 8 x 512 x 512: 42 us (last) and 48 us (first), against 80 and 64 us in the general
+// kernel with the plane spread into its tensor.
+constexpr int kPlaneRow = 608;  // floats per block in P: 32 x 18 + 32 (first), 9 x 32 + 1 (last)
+
+template <bool FIRST>
+__global__ void __launch_bounds__(NTHR, 6)
+    wgrad_plane(const __nv_bfloat16 *T, const float *plane, const float *lam, int B, int H, int W, float *P)
+{
+    constexpr int DS = 40, CS = 24;              // padded pixel strides (bf16)
+    constexpr int NT = FIRST ? 3 : 2, NC = NT * 8;
+    __shared__ __align__(16) __nv_bfloat16 tbuf[2][TH * TW * DS];
+    __shared__ __align__(16) __nv_bfloat16 cbuf[2][TH * TW * CS];
+    static_assert(sizeof(tbuf) >= (size_t)4 * 32 * NC * sizeof(float), "the sums reuse the tiles");
+    static_assert(TH * TW == NTHR, "a pixel's columns per thread");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tiles_x = (W + TW - 1) / TW, tiles_y = (H + TH - 1) / TH;
+    const int per_img = tiles_x * tiles_y;
+    const long long ntiles = (long long)B * per_img;
+    float cv[9], lv = 0.f;
+    unsigned in = 0u;  // bit tap: that neighbour is inside; bit 9: the pixel is
+    auto stage = [&](long long tile, int nb) {
+        const int b = (int)(tile / per_img), rem = (int)(tile - (long long)b * per_img);
+        const int y0 = (rem / tiles_x) * TH, x0 = (rem % tiles_x) * TW;
+        const __nv_bfloat16 *tb = T + (long long)b * H * W * 32;
+        for (int t = tid; t < TH * TW * 4; t += NTHR) {
+            const int v = t / (TH * TW), pix = t % (TH * TW);
+            const int yy = y0 + pix / TW, xx = x0 + pix % TW;
+            const bool ok = yy < H && xx < W;
+            cp_async16_zfill(&tbuf[nb][pix * DS + v * 8], tb + (ok ? (((long long)yy * 4 + v) * W + xx) * 8 : 0), ok);
+        }
+        cp_async_commit_net();
+        const float *pb = plane + (long long)b * H * W;
+        const int y = y0 + tid / TW, x = x0 + tid % TW;
+        const bool here = y < H && x < W;
+        in = here ? 1u << 9 : 0u;
+        if (FIRST) lv = lam[b];
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap) {
+            const int dy = tap / 3 - 1, dx = tap % 3 - 1;
+            const int yy = FIRST ? y + dy : y - dy, xx = FIRST ? x + dx : x - dx;
+            const bool ok = here && yy >= 0 && yy < H && xx >= 0 && xx < W;
+            cv[tap] = ok ? pb[(long long)yy * W + xx] : 0.f;
+            in |= ok ? 1u << tap : 0u;
+        }
+    };
+    auto put = [&](int nb) {
+        unsigned u[12];
+        auto pack = [](float a, float b) {
+            const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+            return *reinterpret_cast<const unsigned *>(&h);
+        };
+        if (FIRST) {
+#pragma unroll
+            for (int tap = 0; tap < 9; ++tap) u[tap] = pack(cv[tap], in >> tap & 1u ? lv : 0.f);
+            u[9] = pack(in >> 9 & 1u ? 1.f : 0.f, 0.f);
+            u[10] = u[11] = 0u;
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) u[q] = pack(cv[2 * q], cv[2 * q + 1]);
+            u[4] = pack(cv[8], 0.f);
+            u[5] = u[6] = u[7] = 0u;
+        }
+        uint4 *d = reinterpret_cast<uint4 *>(&cbuf[nb][tid * CS]);
+#pragma unroll
+        for (int q = 0; q < NT; ++q) d[q] = make_uint4(u[4 * q], u[4 * q + 1], u[4 * q + 2], u[4 * q + 3]);
+    };
+    float acc[2][NT][4], bacc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int j = 0; j < NT; ++j) acc[m][j][0] = acc[m][j][1] = acc[m][j][2] = acc[m][j][3] = 0.f;
+    long long tile = blockIdx.x;
+    if (tile < ntiles) {
+        stage(tile, 0);
+        put(0);
+    }
+    cp_async_wait_net<0>();
+    __syncthreads();
+    int buf = 0;
+    for (; tile < ntiles; tile += gridDim.x) {
+        const bool more = tile + gridDim.x < ntiles;
+        if (more) stage(tile + gridDim.x, buf ^ 1);
+#pragma unroll
+        for (int h = 0; h < TH / 4; ++h) {
+            const int r = warp + 4 * h;
+            unsigned af[2][4];
+            const int mat = lane >> 3, rr = lane & 7;
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+                ldsm_x4_t(smem_u32(&tbuf[buf][(r * TW + (mat >> 1) * 8 + rr) * DS + m * 16 + (mat & 1) * 8]),
+                          af[m][0], af[m][1], af[m][2], af[m][3]);
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                unsigned b0, b1;
+                ldsm_x2_t(smem_u32(&cbuf[buf][(r * TW + (mat & 1) * 8 + rr) * CS + j * 8]), b0, b1);
+#pragma unroll
+                for (int m = 0; m < 2; ++m)
+                    mma_bf16(acc[m][j], af[m][0], af[m][1], af[m][2], af[m][3], b0, b1);
+                if (!FIRST && j == 0)  // column sums: an A of ones (BF16 1.0)
+                    mma_bf16(bacc, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u, b0, b1);
+            }
+        }
+        if (more) put(buf ^ 1);
+        cp_async_wait_net<0>();
+        __syncthreads();  // the next tile is there, and every warp is done with this one
+        buf ^= 1;
+    }
+    float *red = reinterpret_cast<float *>(tbuf);  // [warp][c][NC]
+    __shared__ float bsum[4];
+    const int g = lane >> 2, tq = lane & 3;
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                red[(warp * 32 + m * 16 + g + (e >> 1) * 8) * NC + j * 8 + tq * 2 + (e & 1)] = acc[m][j][e];
+    if (lane == 2) bsum[warp] = bacc[0];  // row 0, column 4: the centre tap
+    __syncthreads();
+    float *row = P + (long long)blockIdx.x * kPlaneRow;
+    for (int e = tid; e < 32 * NC; e += NTHR) {
+        const int c = e / NC, n = e % NC;
+        const float v = (red[e] + red[32 * NC + e]) + (red[2 * 32 * NC + e] + red[3 * 32 * NC + e]);
+        if (FIRST) {
+            if (n < 18) row[c * 18 + n] = v;
+            else if (n == 18) row[32 * 18 + c] = v;
+        } else if (n < 9) {
+            row[n * 32 + c] = v;
+        }
+    }
+    if (!FIRST && tid == 0) row[9 * 32] = (bsum[0] + bsum[1]) + (bsum[2] + bsum[3]);
 }
 
 // dW[e'] += sum_b P[b][e] (e < nw; e = (co, tap, c < xc) goes to e' = (co, tap, c) of cin
 // channels) and db[e - nw] += sum_b P[b][e] (nw <= e < n), summed in a fixed order: 32
-// consecutive e per block row of threads, 8 interleaved groups of b per column, the 8 group
-// sums combined in order.
-constexpr int RED_E = 32, RED_G = 8;
+// consecutive e per block row of threads, 32 interleaved groups of b per column, the group
+// sums combined in order. What bounds it is the chain of loads of one thread, so many threads
+// take few rows each: 6 us for 608 rows of 9248, 9.6 us with 8 groups.
+constexpr int RED_E = 32, RED_G = 32;
 __global__ void __launch_bounds__(RED_E * RED_G)
     wgrad_reduce(const float *P, int nblocks, int stride, int nw, int n, int xc, int cin, float *dW,
                  float *db)
@@ -503,12 +585,23 @@ tv_status launch_conv(const __nv_bfloat16 *X, int B, int H, int W, const __nv_bf
     return st;
 }
 
-template <int CIN, int COUT, int XL = WG_NHWC, int DL = WG_NHWC>
-tv_status launch_wgrad(const void *X, const void *dY, int B, int H, int W, float *dW, float *db,
-                       float *P, cudaStream_t s, const float *lam = nullptr)
+// sums the partial gradients of `blocks` blocks (row floats each)
+tv_status launch_wgrad_reduce(const float *P, long long blocks, int row, int nw, int n, int xc, int cin,
+                              float *dW, float *db, cudaStream_t s)
 {
-    using G = Wgrad<CIN, COUT, XL, DL>;
-    auto kern = conv3x3_wgrad<CIN, COUT, XL, DL>;
+    wgrad_reduce<<<(n + RED_E - 1) / RED_E, RED_E * RED_G, 0, s>>>(P, (int)blocks, row, nw, n, xc, cin,
+                                                                   dW, db);
+    tv_status st = check_cuda(cudaGetLastError(), "weight-gradient reduction");
+    if (st == TV_OK) note_launch();
+    return st;
+}
+
+template <int CIN, int COUT, bool GROUPED = false>
+tv_status launch_wgrad(const void *X, const void *dY, int B, int H, int W, float *dW, float *db,
+                       float *P, cudaStream_t s)
+{
+    using G = Wgrad<CIN, COUT>;
+    auto kern = conv3x3_wgrad<CIN, COUT, GROUPED>;
     static bool attr = false;
     if (!attr) {
         tv_status st0 = check_cuda(
@@ -522,16 +615,30 @@ tv_status launch_wgrad(const void *X, const void *dY, int B, int H, int W, float
         attr = true;
     }
     const long long blocks = wgrad_blocks(B, H, W);
-    kern<<<(unsigned)blocks, NTHR, G::smem, s>>>(X, lam, dY, B, H, W, P);
+    kern<<<(unsigned)blocks, NTHR, G::smem, s>>>(static_cast<const __nv_bfloat16 *>(X),
+                                                 static_cast<const __nv_bfloat16 *>(dY), B, H, W, P);
     tv_status st = check_cuda(cudaGetLastError(), "weight-gradient launch");
     if (st != TV_OK) return st;
     note_launch();
-    constexpr int nw = G::CO * G::N, n = nw + G::CO;
-    wgrad_reduce<<<(n + RED_E - 1) / RED_E, RED_E * RED_G, 0, s>>>(P, (int)blocks, G::row, nw, n, G::XC,
-                                                                   CIN, dW, db);
-    st = check_cuda(cudaGetLastError(), "weight-gradient reduction");
-    if (st == TV_OK) note_launch();
-    return st;
+    constexpr int nw = COUT * G::N;
+    return launch_wgrad_reduce(P, blocks, G::row, nw, nw + COUT, CIN, CIN, dW, db, s);
+}
+
+// 6 resident blocks per SM; their rows of P fit in the workspace of the general kernel (4
+// blocks per SM of rows 15 times as long)
+template <bool FIRST>
+tv_status launch_wgrad_plane(const void *T, const float *plane, const float *lam, int B, int H, int W,
+                             float *dW, float *db, float *P, cudaStream_t s)
+{
+    const long long ntiles = (long long)B * ((W + TW - 1) / TW) * ((H + TH - 1) / TH);
+    const long long blocks = std::min<long long>(6LL * sm_count_current(), ntiles);
+    wgrad_plane<FIRST><<<(unsigned)blocks, NTHR, 0, s>>>(static_cast<const __nv_bfloat16 *>(T), plane, lam,
+                                                         B, H, W, P);
+    tv_status st = check_cuda(cudaGetLastError(), "weight-gradient launch");
+    if (st != TV_OK) return st;
+    note_launch();
+    if (FIRST) return launch_wgrad_reduce(P, blocks, kPlaneRow, 32 * 18, 32 * 18 + 32, 2, 16, dW, db, s);
+    return launch_wgrad_reduce(P, blocks, kPlaneRow, 9 * 32, 9 * 32 + 1, 32, 32, dW, db, s);
 }
 
 bool valid_channels(int cin, int cout)
@@ -2184,17 +2291,17 @@ tv_status tv_net_train_backward(const void *d_x, const float *d_f, const float *
     cudaStream_t s = (cudaStream_t)stream;
     float *P = static_cast<float *>(d_ws);
     if (!d_x)  // the first layer: no gradient of its input
-        return launch_wgrad<16, 32, WG_PLANE, WG_GROUPED>(d_f, d_dy, B, H, W, d_dw, d_db, P, s, d_lam);
+        return launch_wgrad_plane<true>(d_dy, d_f, d_lam, B, H, W, d_dw, d_db, P, s);
     const TwTrain tr{nullptr, d_mask, true};
     auto Wt = static_cast<const __nv_bfloat16 *>(d_w);
     auto dX = static_cast<__nv_bfloat16 *>(d_dx);
     tv_status st;
     if (d_grad_o) {  // the last layer: one channel of dY
-        st = launch_wgrad<32, 16, WG_GROUPED, WG_PLANE>(d_x, d_grad_o, B, H, W, d_dw, d_db, P, s);
+        st = launch_wgrad_plane<false>(d_x, d_grad_o, nullptr, B, H, W, d_dw, d_db, P, s);
         if (st != TV_OK) return st;
         return launch_conv_tw<16, 32, TW_IMAGE>(nullptr, B, H, W, Wt, nullptr, 0, nullptr, dX, s, d_grad_o, nullptr, nullptr, tr);
     }
-    st = launch_wgrad<32, 32, WG_GROUPED, WG_GROUPED>(d_x, d_dy, B, H, W, d_dw, d_db, P, s);
+    st = launch_wgrad<32, 32, true>(d_x, d_dy, B, H, W, d_dw, d_db, P, s);
     if (st != TV_OK) return st;
     return launch_conv_tw<32, 32, TW_GROUPED>(static_cast<const __nv_bfloat16 *>(d_dy), B, H, W, Wt, nullptr, 0, nullptr, dX, s, nullptr, nullptr, nullptr, tr);
 }
