@@ -11,7 +11,7 @@
 //                    partial gradients, summed in a fixed order)
 // That is the general NHWC set. Inference and training run the forward and backward-data
 // GEMMs on tcgen05 in the grouped layout instead (conv3x3_tw below): for a training step on
-// 8 x 512 x 512 its seven convolutions take 390 us against 1100 us for conv3x3_persist, which
+// 8 x 512 x 512 its seven convolutions take 391 us against 1100 us for conv3x3_persist, which
 // moved 32 FP32 pre-activations per pixel and layer where one word of signs is enough.
 // Each block of the two pixel-major kernels computes an 8 x 16 pixel tile for all
 // output channels from a zero-padded 10 x 18 input patch in shared memory; A and B
@@ -250,7 +250,6 @@ __global__ void __launch_bounds__(NTHR)
 // is copied asynchronously into a second buffer while the current one is multiplied (one
 // barrier per tile). 32 -> 32 channels, 8 x 512 x 512: 128 us, against 268 us with
 // one buffer, synchronous loads and db summed serially by 32 threads.
-// X and dY lie in memory as [image][row][pixel][C], or GROUPED, [image][row][C/8][pixel][8].
 template <int CIN, int COUT>
 struct Wgrad {
     static constexpr int PS = CIN + 8, DS = COUT + 8;       // padded pixel strides (bf16)
@@ -260,7 +259,7 @@ struct Wgrad {
     static constexpr int row = COUT * N + COUT;             // floats per block in P
 };
 
-template <int CIN, int COUT, bool GROUPED>
+template <int CIN, int COUT>
 __global__ void __launch_bounds__(NTHR, 4)
     conv3x3_wgrad(const __nv_bfloat16 *X, const __nv_bfloat16 *dY, int B, int H, int W, float *P)
 {
@@ -280,17 +279,15 @@ __global__ void __launch_bounds__(NTHR, 4)
         const int b = (int)(tile / per_img), rem = (int)(tile - (long long)b * per_img);
         const int y0 = (rem / tiles_x) * TH, x0 = (rem % tiles_x) * TW;
         const __nv_bfloat16 *xb = X + (long long)b * H * W * CIN, *db = dY + (long long)b * H * W * COUT;
-        auto at = [&](int y, int x, int v, int V) {
-            return GROUPED ? (((long long)y * V + v) * W + x) * 8 : (((long long)y * W + x) * V + v) * 8;
-        };
+        auto at = [&](int y, int x, int v, int V) { return (((long long)y * W + x) * V + v) * 8; };
         for (int t = tid; t < PH * PW * (CIN / 8); t += NTHR) {
-            const int v = GROUPED ? t / (PH * PW) : t % (CIN / 8), pix = GROUPED ? t % (PH * PW) : t / (CIN / 8);
+            const int v = t % (CIN / 8), pix = t / (CIN / 8);
             const int gy = y0 + pix / PW - 1, gx = x0 + pix % PW - 1;
             const bool in = gy >= 0 && gy < H && gx >= 0 && gx < W;
             cp_async16_zfill(xbuf + nb * G::PATCH + pix * PS + v * 8, xb + (in ? at(gy, gx, v, CIN / 8) : 0), in);
         }
         for (int t = tid; t < TH * TW * (COUT / 8); t += NTHR) {
-            const int v = GROUPED ? t / (TH * TW) : t % (COUT / 8), pix = GROUPED ? t % (TH * TW) : t / (COUT / 8);
+            const int v = t % (COUT / 8), pix = t / (COUT / 8);
             const int yy = y0 + pix / TW, xx = x0 + pix % TW;
             const bool in = yy < H && xx < W;
             cp_async16_zfill(dbuf + nb * G::TILE + pix * DS + v * 8, db + (in ? at(yy, xx, v, COUT / 8) : 0), in);
@@ -596,12 +593,12 @@ tv_status launch_wgrad_reduce(const float *P, long long blocks, int row, int nw,
     return st;
 }
 
-template <int CIN, int COUT, bool GROUPED = false>
+template <int CIN, int COUT>
 tv_status launch_wgrad(const void *X, const void *dY, int B, int H, int W, float *dW, float *db,
                        float *P, cudaStream_t s)
 {
     using G = Wgrad<CIN, COUT>;
-    auto kern = conv3x3_wgrad<CIN, COUT, GROUPED>;
+    auto kern = conv3x3_wgrad<CIN, COUT>;
     static bool attr = false;
     if (!attr) {
         tv_status st0 = check_cuda(
@@ -1683,6 +1680,216 @@ __global__ void __launch_bounds__(TW_THREADS, 4)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "n"(NCOL) : "memory");
 }
 
+// ------------------------------------- weight gradient on tcgen05 (grouped layout) --
+// dW of a 32 -> 32 layer as a GEMM whose K runs over pixels, on tcgen05: mma.sync cannot go
+// faster here (its kernel above runs at 512 multiply-adds per clock and SM, which is all that
+// m16n8k16 gives). Step u is a pair of rows y, y + 1 of a 128-pixel column. Its operands are
+// the four input rows y - 1 .. y + 2 (32 channels each, so M = 128 with row i, channel ci at
+// 32 i + ci) and the two rows of dY (N = 64: row j, channel co at 32 j + co); K = 16 pixels
+// per MMA, and shift dx starts the input rows dx pixels in. Both operands are stored as they
+// lie in memory, 8 channels of a pixel together, which is the M- (N-) major layout without
+// swizzle: core matrices of 8 pixels x 8 channels, the next 8 pixels 128 bytes on (leading
+// byte offset), the next 8 channels one group on (stride byte offset). Accumulator dx
+// (TMEM columns 64 dx ..) then holds at (i, j) the tap dy = i - j of those pixels: 6 of its 8
+// blocks are taps (3/4 of the work is useful), the two others are dropped. 24 MMAs of
+// 128 x 64 x 16 per 256 pixels; the 3 shifts re-read shared memory, not the L2.
+// A block takes a contiguous run of steps, along the rows first (the input rows overlap those
+// of the next pair, which the L2 serves; a ragged last column is spread over the blocks), one
+// accumulator for all of them, so that as many products are added in a row as in the general
+// kernel; warp 0 loads (two stages of 50 KB, two
+// blocks per SM), warp 1 issues the MMAs, warps 2-5 add up dY for the bias gradient and at
+// the end read the accumulators, add the two blocks of each tap in shared memory and store
+// the block's row of P. 8 x 512 x 512: 63 us, 130 us on mma.sync; the tensors are 268 MB.
+// Waits are bounded as in conv3x3_tw; a block whose wait gave up stores NaN.
+constexpr int WT_THREADS = 192, WT_NS = 2;
+constexpr int WT_X = 16 * TW_GS, WT_D = 8 * 2048, WT_STAGE = WT_X + WT_D;
+constexpr unsigned WT_BYTES = 16 * TW_ROWB + WT_D;    // what the loads of a stage deliver
+constexpr int WT_ROW = 32 * 288 + 32;                 // floats per block in P
+constexpr size_t WT_SMEM = 1024 + (size_t)WT_NS * WT_STAGE + 8 * (2 * WT_NS + 1) + 16;
+static_assert((size_t)WT_NS * WT_STAGE >= WT_ROW * sizeof(float), "the sums reuse the stages");
+
+__global__ void __launch_bounds__(WT_THREADS, 2)
+    wgrad_tc(const __grid_constant__ CUtensorMap tx, const __grid_constant__ CUtensorMap tx_tail,
+             const __grid_constant__ CUtensorMap td, int B, int H, int W, float *P)
+{
+    extern __shared__ __align__(1024) unsigned char smem_wt[];
+    unsigned char *base = smem_wt + ((1024u - (smem_u32(smem_wt) & 1023u)) & 1023u);
+    unsigned char *barp = base + WT_NS * WT_STAGE;
+    unsigned *tslot = reinterpret_cast<unsigned *>(barp + 8 * (2 * WT_NS + 1));
+    volatile int *bad = reinterpret_cast<volatile int *>(tslot + 1);
+    const unsigned s0 = smem_u32(base), bar0 = smem_u32(barp);
+    auto full = [&](int s) { return bar0 + 8u * s; };
+    auto empty = [&](int s) { return bar0 + 8u * (WT_NS + s); };
+    const unsigned done = bar0 + 8u * (2 * WT_NS);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tiles_x = (W + TC_M - 1) / TC_M, pairs = (H + 1) / 2;
+    const long long steps = (long long)B * tiles_x * pairs;
+    const long long lo = steps * blockIdx.x / gridDim.x, hi = steps * (blockIdx.x + 1) / gridDim.x;
+
+    if (tid == 0) {
+        for (int s = 0; s < WT_NS; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(full(s)) : "memory");
+            // the MMAs' commit and the four warps that read dY
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 5;\n" ::"r"(empty(s)) : "memory");
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(done) : "memory");
+        *bad = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;\n" ::"r"(smem_u32(tslot))
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const unsigned tmem = *tslot;
+
+    float bsum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (warp == 0) {
+        if (lane == 0) {
+            int n = 0;  // steps whose loads were issued
+            for (long long u = lo; u < hi; ++u, ++n) {
+                const int s = n % WT_NS;
+                if (!tw_wait(empty(s), ((unsigned)(n / WT_NS) & 1u) ^ 1u, bad)) break;
+                const long long yp = u / tiles_x;  // image and pair of rows
+                const int x0 = (int)(u - yp * tiles_x) * TC_M, b = (int)(yp / pairs);
+                const int y = (int)(yp - (long long)b * pairs) * 2;
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(full(s)), "r"(WT_BYTES)
+                             : "memory");
+                const unsigned d0 = s0 + s * WT_STAGE;
+                auto load = [&](const CUtensorMap &m, unsigned dst, int x, int g, int yy) {
+                    asm volatile(
+                        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
+                        " [%0], [%1, {%2, %3, %4, %5}], [%6];\n" ::"r"(dst),
+                        "l"(reinterpret_cast<uint64_t>(&m)), "r"(2 * x), "r"(g), "r"(yy), "r"(b), "r"(full(s))
+                        : "memory");
+                };
+                load(td, d0 + WT_X, x0, 0, y);
+#pragma unroll 4
+                for (int q = 0; q < 16; ++q) {  // row y - 1 + q / 4, group q % 4: 128 pixels and 2 more
+                    load(tx, d0 + q * TW_GS, x0 - 1, q & 3, y - 1 + (q >> 2));
+                    load(tx_tail, d0 + q * TW_GS + 2048, x0 + 127, q & 3, y - 1 + (q >> 2));
+                }
+            }
+            if (*bad)  // let the loads in flight land before the block exits
+                for (int k = max(0, n - WT_NS); k < n; ++k)
+                    for (unsigned it = 0; it < kTcSpin; ++it) {
+                        unsigned ok;
+                        asm volatile(
+                            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+                            " selp.u32 %0, 1, 0, p;\n}\n"
+                            : "=r"(ok)
+                            : "r"(full(k % WT_NS)), "r"((unsigned)(k / WT_NS) & 1u)
+                            : "memory");
+                        if (ok) break;
+                    }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            // M- and N-major operands (bits 15 and 16)
+            constexpr uint32_t idesc = tc_idesc(128, 64) | (1u << 15) | (1u << 16);
+            for (long long u = lo; u < hi; ++u) {
+                const int n = (int)(u - lo), s = n % WT_NS;
+                if (!tw_wait(full(s), (unsigned)(n / WT_NS) & 1u, bad)) break;
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                const uint64_t a0 = tc_desc(s0 + s * WT_STAGE, 128, TW_GS);
+                const uint64_t b0 = tc_desc(s0 + s * WT_STAGE + WT_X, 128, 2048);
+                const unsigned acc = n > 0 ? 1u : 0u;
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+                    for (int ks = 0; ks < TC_M / 16; ++ks)
+                        asm volatile(
+                            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + 64u * dx),
+                            "l"(a0 + (uint64_t)(dx + 16 * ks)), "l"(b0 + (uint64_t)(16 * ks)), "r"(idesc),
+                            "r"(ks ? 1u : acc)
+                            : "memory");
+                asm volatile(
+                    "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(empty(s))
+                    : "memory");
+            }
+            // every MMA issued completes before the accumulators are read or released
+            asm volatile(
+                "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(done)
+                : "memory");
+            bool ok = false;
+            for (unsigned it = 0; it < kTcSpin && !ok; ++it) {
+                unsigned d;
+                asm volatile(
+                    "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+                    " selp.u32 %0, 1, 0, p;\n}\n"
+                    : "=r"(d)
+                    : "r"(done), "r"(0u)
+                    : "memory");
+                ok = d != 0;
+            }
+            if (!ok && atomicExch((int *)bad, 1) == 0) atomicAdd(&g_tc_timeouts, 1u);
+        }
+    } else {
+        const int g = warp - 2;  // the 8-channel group that this warp adds up
+        for (long long u = lo; u < hi; ++u) {
+            const int n = (int)(u - lo), s = n % WT_NS;
+            const bool ok = tw_wait(full(s), (unsigned)(n / WT_NS) & 1u, bad);
+            if (!__all_sync(0xffffffffu, ok)) break;
+            const unsigned char *d = base + s * WT_STAGE + WT_X + g * 2048 + lane * 16;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {  // 2 rows x 4 x 32 pixels
+                const uint4 v = *reinterpret_cast<const uint4 *>(d + (q >> 2) * 8192 + (q & 3) * 512);
+                const unsigned w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    bsum[2 * e] += __uint_as_float(w[e] << 16);
+                    bsum[2 * e + 1] += __uint_as_float(w[e] & 0xffff0000u);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(empty(s)) : "memory");
+        }
+    }
+    __syncwarp();
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    // [co][tap][ci] and the bias gradient, in the stages' memory
+    float *sum = reinterpret_cast<float *>(base);
+    const int i = warp & 3;  // TMEM lanes 32 i ..: input row i, ci = lane
+    for (int j = 0; j < 2; ++j) {  // tap dy = i - j
+        const int dy = i - j;
+        if (warp >= 2 && dy >= 0 && dy < 3) {
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) {
+                float v[32];
+                tc_ld<32>(tmem + ((unsigned)(i * 32) << 16) + (unsigned)(64 * dx + 32 * j), v);
+                float *dst = sum + (dy * 3 + dx) * 32 + lane;
+#pragma unroll
+                for (int co = 0; co < 32; ++co) dst[co * 288] = j ? dst[co * 288] + v[co] : v[co];
+            }
+        }
+        __syncthreads();
+    }
+    if (warp >= 2) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) bsum[e] += __shfl_xor_sync(0xffffffffu, bsum[e], off);
+            if (lane == 0) sum[32 * 288 + (warp - 2) * 8 + e] = bsum[e];
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const bool lost = *bad != 0;
+    float4 *row = reinterpret_cast<float4 *>(P + (long long)blockIdx.x * WT_ROW);
+    const float nan = __int_as_float(0x7fffffff);
+    for (int e = tid; e < WT_ROW / 4; e += WT_THREADS)
+        row[e] = lost ? make_float4(nan, nan, nan, nan) : reinterpret_cast<const float4 *>(sum)[e];
+    if (warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;\n" ::"r"(tmem) : "memory");
+}
+
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link to the driver library)
 typedef CUresult (*TmapEncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                                  const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
@@ -1703,6 +1910,21 @@ TmapEncodeFn tmap_encoder()
         return (TmapEncodeFn)f;
     }();
     return fn;
+}
+
+// A grouped activation of KG 8-channel groups as a 4-D tensor of 8-byte elements (2 W x KG x
+// H x B), with boxes of `px` pixels x `groups` x `rows`.
+CUresult grouped_map(TmapEncodeFn enc, CUtensorMap *map, const __nv_bfloat16 *X, int B, int H, int W, int KG,
+                     int px, int groups, int rows)
+{
+    const cuuint64_t dims[4] = {2 * (cuuint64_t)W, (cuuint64_t)KG, (cuuint64_t)H, (cuuint64_t)B};
+    const cuuint64_t strides[3] = {(cuuint64_t)W * 16, (cuuint64_t)W * KG * 16, (cuuint64_t)H * W * KG * 16};
+    const cuuint32_t box[4] = {2 * (cuuint32_t)px, (cuuint32_t)groups, (cuuint32_t)rows, 1};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, const_cast<__nv_bfloat16 *>(X), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+               px >= 16 ? CU_TENSOR_MAP_L2_PROMOTION_L2_256B : CU_TENSOR_MAP_L2_PROMOTION_NONE,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
 template <int CIN, int COUT, int IO>
@@ -1727,16 +1949,8 @@ tv_status launch_conv_tw(const __nv_bfloat16 *X, int B, int H, int W, const __nv
         memset(&tmap, 0, sizeof(tmap));  // not read: the rows come from the image
         tmap_tail = tmap;
     } else if (IO != TW_NHWC) {
-        const cuuint64_t dims[4] = {2 * (cuuint64_t)W, KG, (cuuint64_t)H, (cuuint64_t)B};
-        const cuuint64_t strides[3] = {(cuuint64_t)W * 16, (cuuint64_t)W * CIN * 2,
-                                       (cuuint64_t)H * W * CIN * 2};
-        const cuuint32_t box[4] = {256, 1, 1, 1}, box_tail[4] = {4, 1, 1, 1};
-        r0 = enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, const_cast<__nv_bfloat16 *>(X), dims, strides, box,
-                 estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        r1 = enc(&tmap_tail, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, const_cast<__nv_bfloat16 *>(X), dims, strides,
-                 box_tail, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                 CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        r0 = grouped_map(enc, &tmap, X, B, H, W, (int)KG, TC_M, 1, 1);
+        r1 = grouped_map(enc, &tmap_tail, X, B, H, W, (int)KG, 2, 1, 1);
     } else {
         const cuuint64_t dims[5] = {8, KG, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
         const cuuint64_t strides[4] = {16, 16 * KG, (cuuint64_t)W * CIN * 2, (cuuint64_t)H * W * CIN * 2};
@@ -1799,6 +2013,43 @@ tv_status launch_conv_tw(const __nv_bfloat16 *X, int B, int H, int W, const __nv
                               "conv launch");
     if (st == TV_OK) note_launch();
     return st;
+}
+
+tv_status launch_wgrad_tc(const __nv_bfloat16 *X, const __nv_bfloat16 *dY, int B, int H, int W, float *dW,
+                          float *db, float *P, cudaStream_t s)
+{
+    TmapEncodeFn enc = tmap_encoder();
+    if (!enc) {
+        set_error("weight gradient: cuTensorMapEncodeTiled is not available from the driver");
+        return TV_ERR_CUDA;
+    }
+    CUtensorMap tx, tx_tail, td;
+    if (grouped_map(enc, &tx, X, B, H, W, 4, TC_M, 1, 1) != CUDA_SUCCESS ||
+        grouped_map(enc, &tx_tail, X, B, H, W, 4, 2, 1, 1) != CUDA_SUCCESS ||
+        grouped_map(enc, &td, dY, B, H, W, 4, TC_M, 4, 2) != CUDA_SUCCESS) {
+        set_error("weight gradient: cuTensorMapEncodeTiled rejected the activation layout");
+        return TV_ERR_INVALID;
+    }
+    static bool attr = false;
+    if (!attr) {
+        tv_status st0 = check_cuda(
+            cudaFuncSetAttribute(wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WT_SMEM),
+            "cudaFuncSetAttribute");
+        if (st0 != TV_OK) return st0;
+        st0 = check_cuda(cudaFuncSetAttribute(wgrad_tc, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                              (int)cudaSharedmemCarveoutMaxShared),
+                         "cudaFuncSetAttribute");
+        if (st0 != TV_OK) return st0;
+        attr = true;
+    }
+    // two blocks per SM (shared memory and TMEM), no more than steps or rows of P
+    const long long steps = (long long)B * ((W + TC_M - 1) / TC_M) * ((H + 1) / 2);
+    const long long blocks = std::min(std::min(2LL * sm_count_current(), steps), wgrad_blocks(B, H, W));
+    wgrad_tc<<<(unsigned)blocks, WT_THREADS, WT_SMEM, s>>>(tx, tx_tail, td, B, H, W, P);
+    tv_status st = check_cuda(cudaGetLastError(), "weight-gradient launch");
+    if (st != TV_OK) return st;
+    note_launch();
+    return launch_wgrad_reduce(P, blocks, WT_ROW, 32 * 288, WT_ROW, 32, 32, dW, db, s);
 }
 
 static std::atomic<int> g_net_tc{0};  // mma.sync by default: faster for N = 16/32 (see tv.h)
@@ -2301,7 +2552,7 @@ tv_status tv_net_train_backward(const void *d_x, const float *d_f, const float *
         if (st != TV_OK) return st;
         return launch_conv_tw<16, 32, TW_IMAGE>(nullptr, B, H, W, Wt, nullptr, 0, nullptr, dX, s, d_grad_o, nullptr, nullptr, tr);
     }
-    st = launch_wgrad<32, 32, true>(d_x, d_dy, B, H, W, d_dw, d_db, P, s);
+    st = launch_wgrad_tc(static_cast<const __nv_bfloat16 *>(d_x), static_cast<const __nv_bfloat16 *>(d_dy), B, H, W, d_dw, d_db, P, s);
     if (st != TV_OK) return st;
     return launch_conv_tw<32, 32, TW_GROUPED>(static_cast<const __nv_bfloat16 *>(d_dy), B, H, W, Wt, nullptr, 0, nullptr, dX, s, nullptr, nullptr, nullptr, tr);
 }
