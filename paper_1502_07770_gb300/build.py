@@ -14,8 +14,8 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libtv.so")
-SOURCES = ["tv_split.cu", "tv_chain.cu", "tv2d.cu", "tv2d_batched.cu", "tv2d_lagrangian.cu", "tv_grad.cu",
-           "tv_net.cu", "tv_pq.cu", "tv_nonconvex.cu"]
+SOURCES = ["tv_split.cu", "tv_split_gap.cu", "tv_chain.cu", "tv2d.cu", "tv2d_batched.cu",
+           "tv2d_lagrangian.cu", "tv_grad.cu", "tv_net.cu", "tv_pq.cu", "tv_nonconvex.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-diag-suppress", "177",
          "-I", INCLUDE]

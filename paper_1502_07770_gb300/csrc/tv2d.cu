@@ -2,9 +2,10 @@
 // accelerated primal-dual iteration eq. pd on the saddle-point problem
 // eq. rof-saddle, where both proximal maps are batches of chain problems.
 //
-// Per iteration k, two fused kernels run the chain dynamic program of
-// Algorithm 2 / Sec. 4.1 with the proximal arithmetic folded into their loads
-// and stores (one warp per chain for up to 2048 chains, else one thread):
+// Per iteration k, two fused kernels solve the chains with the proximal arithmetic folded
+// into their loads and stores: by threshold splitting (tv_split.cuh; sides of at most 4096
+// pixels), else by the dynamic program of Algorithm 2 / Sec. 4.1 (one warp per chain for up
+// to 2048 chains, else one thread):
 //   column (dual) phase, one chain per image column:
 //       eta = y + sigma_k (x^k + theta_{k-1} (x^k - x^{k-1}))
 //       xhat = argmin TV_v(x) + sigma_k/2 ||x - eta/sigma_k||^2  (chains: c = eta/sigma_k,
@@ -21,16 +22,15 @@
 // f - D_h^T p_h - D_v^T p_v = x^{k+1} + (x^{k+1} - x^k)/tau_k),
 //   G_k = P(x^{k+1}) - D(p) = 1/2||x^{k+1} - f||^2 + TV(x^{k+1}) - 1/2||f||^2
 //         + 1/2||x^{k+1} + (x^{k+1} - x^k)/tau_k||^2 >= 0.
-// A gap kernel after each row phase reads x^{k+1}, x^k and f, accumulates G_k per
-// pixel (FP32 over at most 32 pixels per thread, FP64 beyond); its last block sums
-// the block partials in a fixed order and raises the stop flag. Later kernels see
-// the flag and return at once, so a batch of launched iterations costs little after it.
+// The gap pass after each row phase (tv2d_gap.cuh) raises the stop flag on the device. Later
+// kernels see it and return at once, so a batch of launched iterations costs little after it.
 #include <cuda_runtime.h>
 #include <math.h>
 
 #include <algorithm>
 
 #include "tv2d_common.cuh"
+#include "tv2d_gap.cuh"
 #include "tv_launch.cuh"
 #include "tv_split_launch.h"
 
@@ -40,18 +40,6 @@ using namespace tvh;
 namespace {
 
 constexpr int kRing = 32;
-
-struct Tv2dState {
-    int k;                // completed primal (row) steps
-    int done;             // per-pixel gap reached the tolerance
-    unsigned ticket_col;  // warps finished in the running column phase
-    unsigned ticket_row;  // warps finished in the running row phase
-    int max_iters;
-    int gap_k;            // index of the last gap written (-1: none yet)
-    double tol;           // per-pixel tolerance; 0 never stops early
-    double inv_N;         // 1 / (H W)
-    double gap;           // last per-pixel gap G_{gap_k} / (H W)
-};
 
 __global__ void tv2d_init_state(Tv2dState *st, Tv2dParams *prm, int max_iters, double tol,
                                 double inv_N, ParamChunk chunk)
@@ -541,107 +529,12 @@ struct CoopColPhaseP {
     __device__ void finish_empty() const {}
 };
 
-// ------------------------------------------------------------------ gap ------
-// G_k after the primal step of iteration k (k = st->k - 1 once the row kernel has
-// counted itself): the per-pixel terms 1/2 (x - f)^2 + 1/2 (z - f)(z + f) with
-// z = x^{k+1} + (x^{k+1} - x^k)/tau_k, plus w |difference| over the right and lower
-// neighbour of every pixel. One pass over the image; FP32 within a thread, FP64
-// across threads; the last block reduces the block partials in a fixed order and
-// raises the stop flag.
-//
-// A warp takes 32 columns of kGapRows consecutive rows and issues all their loads before it
-// uses one (the kernel is one image pass between two phases, bound by latency: 1024 x 1024
-// walked pixel by pixel with state, step size and FP64 division read first took 16 us); the
-// lower neighbour is the next row's value, the right one the next lane's.
-constexpr int kGapThreads = 256;
-constexpr int kGapRows = 8;
-constexpr int kGapTileRows = kGapThreads / WARP * kGapRows;
-constexpr int kGapMaxBlocks = 4096;
-
-__device__ __forceinline__ double warp_sum(double v)
+// The gap as a pass of its own (tv2d_gap.cuh): the last iteration of a batch, and the phases
+// that are not on the splitting kernel.
+__global__ void __launch_bounds__(kGapThreads) tv2d_gap_kernel(GapView v)
 {
-#pragma unroll
-    for (int o = WARP / 2; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-    return v;
-}
-
-// Sum over the block in a fixed order; valid in thread 0.
-__device__ __forceinline__ double block_sum(double v, double *red)
-{
-    v = warp_sum(v);
-    __syncthreads();
-    if ((threadIdx.x & (WARP - 1)) == 0) red[threadIdx.x / WARP] = v;
-    __syncthreads();
-    double b = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < kGapThreads / WARP; ++w) b += red[w];
-    return b;
-}
-
-__global__ void __launch_bounds__(kGapThreads)
-    tv2d_gap_kernel(const float *f, const float *wh, const float *wv, float lam, int H, int W,
-                    const float *x1, const float *x0, int k, float inv_tau, long long ctiles,
-                    long long tiles,
-                    Tv2dState *st, double *partials, double *gaps, unsigned *ticket)
-{
-    __shared__ double red[kGapThreads / WARP];
-    __shared__ bool last;
     pdl_enter();
-    if (st->done) return;
-    const int lane = threadIdx.x & (WARP - 1), warp = threadIdx.x / WARP;
-    double acc = 0.0;
-    for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        const int c = (int)(tile % ctiles) * WARP + lane;
-        const int r0 = (int)(tile / ctiles) * kGapTileRows + warp * kGapRows;
-        float xv[kGapRows + 1], fv[kGapRows], xo[kGapRows], wd[kGapRows], wr[kGapRows], xe[kGapRows];
-#pragma unroll
-        for (int u = 0; u <= kGapRows; ++u) {
-            const int r = r0 + u;
-            const bool in = c < W && r < H;
-            const long long q = (long long)r * W + c;
-            xv[u] = in ? x1[q] : 0.f;
-            if (u == kGapRows) break;
-            fv[u] = in ? f[q] : 0.f;
-            xo[u] = in ? x0[q] : 0.f;
-            xe[u] = in && lane == WARP - 1 && c + 1 < W ? x1[q + 1] : 0.f;
-            wr[u] = in && c + 1 < W ? (wh ? wh[q - r] : lam) : 0.f;
-            wd[u] = in && r + 1 < H ? (wv ? wv[q] : lam) : 0.f;
-        }
-        float part = 0.f;
-#pragma unroll
-        for (int u = 0; u < kGapRows; ++u) {
-            const float xn = __shfl_down_sync(FULL, xv[u], 1);
-            const float xr = lane == WARP - 1 ? xe[u] : xn;
-            const float z = xv[u] + (xv[u] - xo[u]) * inv_tau;
-            float t = 0.5f * (xv[u] - fv[u]) * (xv[u] - fv[u]) + 0.5f * (z - fv[u]) * (z + fv[u]);
-            if (wr[u] != 0.f) t += wr[u] * fabsf(xr - xv[u]);
-            if (wd[u] != 0.f) t += wd[u] * fabsf(xv[u + 1] - xv[u]);
-            part += t;
-        }
-        acc += (double)part;  // FP32 over a thread's 8 pixels, FP64 beyond
-    }
-    acc = block_sum(acc, red);
-    if (threadIdx.x == 0) {
-        partials[blockIdx.x] = acc;
-        __threadfence();
-        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    // the last block sums the block partials in a fixed order
-    __threadfence();
-    double b = 0.0;
-    for (unsigned bq = threadIdx.x; bq < gridDim.x; bq += blockDim.x) b += __ldcg(partials + bq);
-    b = block_sum(b, red);
-    if (threadIdx.x == 0) {
-        const double g = b * st->inv_N;
-        st->gap = g;
-        st->gap_k = k;
-        st->k = k + 1;
-        gaps[k] = g;
-        if (st->tol > 0.0 && g <= st->tol) st->done = 1;
-        *ticket = 0;
-    }
+    gap_pass(v, blockIdx.x, gridDim.x);
 }
 
 template <class P>
@@ -745,7 +638,7 @@ SplitSrc split_src(SplitMode mode, const float *img, const float *w, float lam, 
     v.maxlen = (int)(cols ? H : W);
     src.nchains = cols ? W : H;
     src.len = v.maxlen;
-    src.done = mode == SPLIT_INIT ? nullptr : &ws.st->done;
+    src.done = &ws.st->done;  // (clear before the first phase)
     return src;
 }
 
@@ -791,11 +684,12 @@ tv_status launch_row(const float *img, const float *wh, float lam, long long H, 
 
 template <bool HAS_WV>
 tv_status launch_col(const float *wv, float lam, long long H, long long W, const Step &it,
-                     float *x0, const Tv2dWs &ws, cudaStream_t s)
+                     float *x0, const Tv2dWs &ws, const GapView *gap, cudaStream_t s)
 {
-    if (split_cols(H, W, wv))
-        return launch_split(split_src(SPLIT_COL, nullptr, wv, lam, H, W, it, x0, ws), ws.hdr, s,
-                            PK_COL);
+    if (split_cols(H, W, wv)) {
+        const SplitSrc src = split_src(SPLIT_COL, nullptr, wv, lam, H, W, it, x0, ws);
+        return gap ? launch_split_gap(src, *gap, ws.hdr, s, PK_COL) : launch_split(src, ws.hdr, s, PK_COL);
+    }
     if (W <= coop_max_chains()) {
         CoopColPhaseP<HAS_WV> p{wv, lam, H, W, x0, ws.buf1, ws.y, ws.st, ws.prm,
                                 nullptr, nullptr, 0.f, 0.f, 0.f};
@@ -807,23 +701,25 @@ tv_status launch_col(const float *wv, float lam, long long H, long long W, const
 }
 
 tv_status launch_col_any(const float *wv, float lam, long long H, long long W, const Step &it,
-                         float *x0, const Tv2dWs &ws, cudaStream_t s)
+                         float *x0, const Tv2dWs &ws, const GapView *gap, cudaStream_t s)
 {
-    return wv ? launch_col<true>(wv, lam, H, W, it, x0, ws, s)
-              : launch_col<false>(wv, lam, H, W, it, x0, ws, s);
+    return wv ? launch_col<true>(wv, lam, H, W, it, x0, ws, gap, s)
+              : launch_col<false>(wv, lam, H, W, it, x0, ws, gap, s);
 }
 
-tv_status launch_gap(const float *img, const float *wh, const float *wv, float lam, long long H,
-                     long long W, const Step &it, float *x0, const Tv2dWs &ws, cudaStream_t s)
+// the gap of iteration it.k
+GapView gap_view(const float *img, const float *wh, const float *wv, float lam, long long H, long long W,
+                 const Step &it, const float *x0, const Tv2dWs &ws)
 {
     const float *xn = (it.k & 1) ? x0 : ws.buf1, *xp = (it.k & 1) ? ws.buf1 : x0;
-    const long long ctiles = (W + WARP - 1) / WARP;
-    const long long tiles = ctiles * ((H + kGapTileRows - 1) / kGapTileRows);
-    const int blocks = (int)std::min<long long>(tiles, kGapMaxBlocks);
-    tv_status st = check_cuda(launch_k(tv2d_gap_kernel, dim3(blocks), dim3(kGapThreads), 0, s, img,
-                                       wh, wv, lam, (int)H, (int)W, xn, xp, it.k,
-                                       (float)(1.0 / it.tau), ctiles, tiles, ws.st, ws.partials,
-                                       ws.gaps, &ws.st->ticket_col),
+    return GapView{img, wh, wv, lam, (int)H, (int)W, xn, xp, it.k, (float)(1.0 / it.tau), 0, 0,
+                   ws.st, ws.partials, ws.gaps, &ws.st->ticket_col};
+}
+
+tv_status launch_gap(GapView v, cudaStream_t s)
+{
+    const int blocks = gap_tiles(v, kGapThreads / WARP);
+    tv_status st = check_cuda(launch_k(tv2d_gap_kernel, dim3(blocks), dim3(kGapThreads), 0, s, v),
                               "gap kernel launch");
     if (st == TV_OK) note_launch();
     return st;
@@ -964,6 +860,11 @@ tv_status tv2d_denoise(const float *d_img, int64_t H, int64_t W, const float *d_
         if (r == TV_OK) note_launch();
         return r;
     };
+    // On the splitting kernel the gap of an iteration rides in the next one's column phase;
+    // the last of a batch is a kernel of its own. 1024 x 1024 at 5 iterations: 353 us
+    // against 374 with a gap kernel after every iteration; 297 x 401 at 6: 229 against 247.
+    const bool fused = split_cols(H, W, d_wv);
+    GapView gap;
     Tv2dState hs;
     Step it;
     int launched = 0;
@@ -972,11 +873,14 @@ tv_status tv2d_denoise(const float *d_img, int64_t H, int64_t W, const float *d_
         const int batch = launched == 0 ? 6 : 3;
         const int u = (max_iters - launched) < batch ? (max_iters - launched) : batch;
         for (int t = 0; t < u; ++t) {
-            if ((st = launch_col_any(d_wv, lambda, H, W, it, d_x, ws, s)) != TV_OK) return st;
+            st = launch_col_any(d_wv, lambda, H, W, it, d_x, ws, fused && t > 0 ? &gap : nullptr, s);
+            if (st != TV_OK) return st;
             st = d_wh ? launch_row<true>(d_img, d_wh, lambda, H, W, it, d_x, ws, s)
                       : launch_row<false>(d_img, d_wh, lambda, H, W, it, d_x, ws, s);
             if (st != TV_OK) return st;
-            if ((st = launch_gap(d_img, d_wh, d_wv, lambda, H, W, it, d_x, ws, s)) != TV_OK) return st;
+            gap = gap_view(d_img, d_wh, d_wv, lambda, H, W, it, d_x, ws);
+            if (!fused || t + 1 == u)
+                if ((st = launch_gap(gap, s)) != TV_OK) return st;
             it.next();
         }
         launched += u;

@@ -479,6 +479,7 @@ struct SGroup {
 
 struct BSplitSrc {
     const BImg *imgs;
+    static constexpr bool GAP = false;
     const BState *st;
     const SGroup *groups;
     const Tv2dParams *prm;

@@ -29,6 +29,7 @@
 // (coop_solve_chain, records and reserve in the workspace) instead.
 #pragma once
 #include "tv2d_common.cuh"
+#include "tv2d_gap.cuh"
 #include "tv_coop.cuh"
 
 namespace tvk {
@@ -140,8 +141,8 @@ struct SplitX {
     float u[W], u2[W];            // flow of a (new) cut after the warp's last node
     float re[W];                  // r of that node
     unsigned amax[W];
-    unsigned char cut[W], side[W], more[W], heavy[W];
-    int bad;                      // the chain goes to the fallback
+    unsigned char cut[W], side[W], more[W], heavy[W];  // heavy: 1; the stop flag: 2
+    int bad;                      // the chain goes to the fallback, or was stopped
 };
 
 __device__ __forceinline__ float rcp_approx(float v)
@@ -211,7 +212,8 @@ __device__ __forceinline__ void cut_at_unit(unsigned bit, unsigned up, float &y0
 }
 
 // Solves one chain held as L nodes per lane in sc (values) and sx (weights if !UNI); writes
-// the solution to sx. Returns false (in every lane) if the chain needs the fallback.
+// the solution to sx. Returns (the same in every lane) whether it did, or the chain needs the
+// fallback, or (STOP) *stop was raised meanwhile, which is looked at once a round.
 //
 // The walks are bound by issue and by the half-rate ALU pipe (minima, selects, logic), so
 // what can be arithmetic on the FMA pipe is: with r = 1, or 0 where the chain is cut after a
@@ -224,9 +226,12 @@ __device__ __forceinline__ void cut_at_unit(unsigned bit, unsigned up, float &y0
 // restarts at 1/2: the half is folded into the values at the cut (with the flow +-1/2: both 0
 // or both 1), and a node before a cut compares with 0 alone. The last sums take the values as
 // they came, so that scaling costs no digits.
-template <int L, int W, bool UNI>
-__device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W> *xc, int n,
-                                            float lamw, int lane, int wi, int bar)
+enum SplitEnd { SPLIT_DONE = 0, SPLIT_FALLBACK = 1, SPLIT_STOPPED = 2 };
+
+template <int L, int W, bool UNI, bool STOP>
+__device__ __forceinline__ int split_solve(const float *sc, float *sx, SplitX<W> *xc, int n,
+                                           float lamw, int lane, int wi, int bar,
+                                           [[maybe_unused]] const int *stop)
 {
     constexpr int LP = split_lp<L>();
     constexpr unsigned ML = L == 32 ? 0xffffffffu : (1u << L) - 1u;
@@ -276,7 +281,7 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
 #pragma unroll
         for (int q = 0; q < W; ++q) ab = max(ab, xc->amax[q]);
     }
-    if (ab >= 0x7f800000u) return false;  // not finite: as the dynamic program has it
+    if (ab >= 0x7f800000u) return SPLIT_FALLBACK;  // not finite: as the dynamic program has it
     const float amax = __uint_as_float(ab);
     unsigned H = 0;   // edges whose flow would swamp the values
     unsigned UP = 0;  // UNI: cuts with flow +w
@@ -285,7 +290,7 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
             float4 *xp = reinterpret_cast<float4 *>(sx + (wi * WARP + lane) * LP);
 #pragma unroll
             for (int q = 0; q < L / 4; ++q) xp[q] = yp[q];
-            return true;
+            return SPLIT_DONE;
         }
         if (lamw > kSplitHeavy * amax) H = ML;
         const float s = 0.5f / lamw;
@@ -435,7 +440,7 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
                 }
                 xp[q] = make_float4(v[0], v[1], v[2], v[3]);
             }
-            return true;
+            return SPLIT_DONE;
         }
 #pragma unroll
         for (int j = L - 1; j >= 0; --j) {
@@ -530,6 +535,9 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
             }
         }
 
+        int halt = 0;  // on its way while the sides are walked
+        if constexpr (STOP) halt = *(const volatile int *)stop;
+
         // ---- sides: below z (t > w) and above (t < -w), one bit per node ----
         unsigned below = 0, above = 0;
 #pragma unroll
@@ -603,18 +611,21 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
             if (lane == WARP - 1) {
                 xc->u[wi] = ue;
                 xc->more[wi] = more;
-                xc->heavy[wi] = hv;
+                xc->heavy[wi] = (hv ? 1 : 0) | (halt ? 2 : 0);
             }
             split_sync<W>(bar);
             more = hv = false;
+            halt = 0;
 #pragma unroll
             for (int q = 0; q < W; ++q) {
                 more |= xc->more[q] != 0;
-                hv |= xc->heavy[q] != 0;
+                hv |= (xc->heavy[q] & 1) != 0;
+                halt |= xc->heavy[q] & 2;
             }
             if (lane == 0) up = wi > 0 ? xc->u[wi - 1] : 0.f;
         } else {
             if (lane == 0) up = 0.f;
+            if constexpr (STOP) halt = __any_sync(FULL, halt);
         }
         if constexpr (UNI) {
             y[0] -= up > 1.f ? 1.f : 0.f;
@@ -622,7 +633,8 @@ __device__ __forceinline__ bool split_solve(const float *sc, float *sx, SplitX<W
         } else {
             y[0] -= up;
         }
-        if (hv) return false;
+        if (STOP && halt) return SPLIT_STOPPED;
+        if (hv) return SPLIT_FALLBACK;
         if constexpr (UNI) {
             if (!more) {  // the values as they came, with the flows of all cuts
                 const unsigned ends = last >= L ? 0u : ML >> max(0, min(31, last));
@@ -659,8 +671,8 @@ struct UnitStride {  // of rows: known at compile time
 // Load, solve and store for the chains of one block: `nch` chains of W warps each. Rows are
 // loaded by their own warps; columns by the whole block, nch neighbouring columns of a row at
 // a time.
-template <int L, int W, bool UNI>
-__device__ __forceinline__ void split_chain(const SplitView &v, float *smem, SplitX<W> *xall,
+template <int L, int W, bool UNI, bool STOP>
+__device__ __forceinline__ void split_chain(const SplitView &v, const int *stop, float *smem, SplitX<W> *xall,
                                             int nch, int cs, long long k0, int cnt, long long kc,
                                             long long start, long long wstart, int n,
                                             WsHeader *hdr, float2 *spill)
@@ -715,11 +727,11 @@ __device__ __forceinline__ void split_chain(const SplitView &v, float *smem, Spl
     if (tid % T == 0) xc->bad = 0;
     if (v.cols) __syncthreads();
     else split_sync<W>(g);
-    bool good = true;
+    int end = SPLIT_DONE;
     if (g < cnt) {
-        good = split_solve<L, W, UNI>(smem + (size_t)g * cs, smem + (size_t)(nch + g) * cs, xc, n,
-                                      v.ws * v.lam, lane, wi, g);
-        if (!good && tid % T == 0) xc->bad = 1;
+        end = split_solve<L, W, UNI, STOP>(smem + (size_t)g * cs, smem + (size_t)(nch + g) * cs, xc, n,
+                                           v.ws * v.lam, lane, wi, g, stop);
+        if (end != SPLIT_DONE && tid % T == 0) xc->bad = 1;
     }
     if (v.cols) __syncthreads();
     else split_sync<W>(g);
@@ -737,7 +749,7 @@ __device__ __forceinline__ void split_chain(const SplitView &v, float *smem, Spl
         if (v.cols) store(v.stride);
         else store(UnitStride());
     }
-    if (!good && wi == 0) {
+    if (end == SPLIT_FALLBACK && wi == 0) {
         SplitView vv = v;
         split_fallback(vv, kc, v.cols ? kc : start, v.cols ? kc : wstart, n, lane, spill, hdr);
     }
@@ -809,6 +821,7 @@ struct SplitSrc {
     int lanes;               // nodes a lane takes (0: by the chain's length)
     long long off0;
     const int *done;         // phases of eq. pd: the solve's stop flag, or NULL
+    static constexpr bool GAP = false;
 
     __device__ bool bind(unsigned blk, int nch, SplitView &o, long long &k0, int &cnt,
                          WsHeader *hdr)
@@ -855,6 +868,15 @@ struct SplitSrc {
     }
 };
 
+// The column phase of a 2D solve with the gap pass of the iteration before in the first blocks
+// of the grid. (A source of its own: with the look at the flag in every chain kernel the others
+// were up to 4 % slower.)
+struct SplitGapSrc : SplitSrc {  // (done is given)
+    static constexpr bool GAP = true;
+    GapView gap;
+    int gap_blocks;
+};
+
 // SRC: bind(block, nch, view, k0, cnt) the chains k0 .. k0 + cnt - 1 of this block;
 // chain(view, k, start, wstart, n) one of them (n = 0: skip); spill(view, k, start, n).
 template <int W, bool UNI, class SRC>
@@ -868,7 +890,18 @@ __global__ void __launch_bounds__(split_threads<W>(), W <= 2 ? 2 : 1)
     SplitView v;
     long long k0;
     int cnt;
-    if (!src.bind(blockIdx.x, nch, v, k0, cnt, hdr)) return;
+    unsigned blk = blockIdx.x;
+    if constexpr (SRC::GAP) {
+        if (blk < (unsigned)src.gap_blocks) {
+            gap_pass(src.gap, blk, src.gap_blocks);
+            return;
+        }
+        blk -= src.gap_blocks;
+    }
+    bool bound = src.bind(blk, nch, v, k0, cnt, hdr);
+    // the gap pass may raise the flag meanwhile: the whole block sees it or none of it
+    if constexpr (SRC::GAP) bound = !__syncthreads_or(!bound);
+    if (!bound) return;
     const int g = threadIdx.x / (WARP * W);
     const long long kc = k0 + g;
     long long start = 0, wstart = 0;
@@ -878,18 +911,20 @@ __global__ void __launch_bounds__(split_threads<W>(), W <= 2 ? 2 : 1)
     // chains that a launch for other lengths takes, and empty ones
     if (split_pick<W>(n) == 0 || n <= src.n_lo) n = 0;
     float2 *spill = src.spill(v, kc, start, n);
+    const int *stop = nullptr;
+    if constexpr (SRC::GAP) stop = src.done;
     if (n > 0) {
         const int l = src.lanes && n > 256 ? src.lanes : split_pick<W>(n);
         if constexpr (W == 1) {
-            if (l == 4) split_chain<4, W, UNI>(v, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
-            if (l == 8) split_chain<8, W, UNI>(v, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
-            if (l == 12) split_chain<12, W, UNI>(v, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
+            if (l == 4) split_chain<4, W, UNI, SRC::GAP>(v, stop, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
+            if (l == 8) split_chain<8, W, UNI, SRC::GAP>(v, stop, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
+            if (l == 12) split_chain<12, W, UNI, SRC::GAP>(v, stop, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
         }
-        if (l == 16) split_chain<16, W, UNI>(v, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
-        if (l == 20) split_chain<20, W, UNI>(v, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
-        if (l == 24) split_chain<24, W, UNI>(v, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
-        if (l == 28) split_chain<28, W, UNI>(v, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
-        if (l == 32) split_chain<32, W, UNI>(v, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
+        if (l == 16) split_chain<16, W, UNI, SRC::GAP>(v, stop, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
+        if (l == 20) split_chain<20, W, UNI, SRC::GAP>(v, stop, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
+        if (l == 24) split_chain<24, W, UNI, SRC::GAP>(v, stop, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
+        if (l == 28) split_chain<28, W, UNI, SRC::GAP>(v, stop, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
+        if (l == 32) split_chain<32, W, UNI, SRC::GAP>(v, stop, smem, xall, nch, cs, k0, cnt, kc, start, wstart, n, hdr, spill);
     }
 }
 

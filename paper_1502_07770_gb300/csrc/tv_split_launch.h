@@ -7,6 +7,10 @@ namespace tvh {
 
 // Chains of at most kSplitMaxLen nodes, on `s`; the source's fields as tv_split.cuh says.
 tv_status launch_split(tvk::SplitSrc src, tvk::WsHeader *hdr, cudaStream_t s, int kind);
+// The columns of `src`, a phase of a 2D solve, with the gap pass `gap` of the iteration before
+// in the same launch.
+tv_status launch_split_gap(const tvk::SplitSrc &src, const tvk::GapView &gap, tvk::WsHeader *hdr,
+                           cudaStream_t s, int kind);
 
 // Whether a batch of chains runs on it. It is the warp-per-chain kernel of TV-l2 chains that
 // fit its registers, unless another was asked for (tv_set_coop_split); a batch above the
