@@ -690,7 +690,46 @@ __device__ __forceinline__ void split_chain(const SplitView &v, const int *stop,
     const long long st = v.cols ? k0 + cc : start;
     const long long wst = v.cols ? st : wstart;
     float *lc = smem + (size_t)cc * cs, *lx = smem + (size_t)(nch + cc) * cs;
-    constexpr int UL = L % 8 == 0 ? 8 : 4;
+    // What counts here is the number of round trips to memory. With one weight a lane has the
+    // registers for two: rows whose arrays all start on 16-byte boundaries go four nodes at a
+    // time, and other chains L / 2 (1024 x 1024 rows 24.2 -> 22.2 us). With weights per edge the
+    // same made the solve spill (4096 x 1024: 61 -> 69 us), so those take 8 at a time.
+    const uintptr_t bits = (uintptr_t)(v.p0 + st) | (uintptr_t)(v.o0 + st) |
+                           (v.p1 ? (uintptr_t)(v.p1 + st) : 0) | (v.p2 ? (uintptr_t)(v.p2 + st) : 0) |
+                           (v.o1 ? (uintptr_t)(v.o1 + st) : 0);
+    const bool vec = UNI && !v.cols && (bits & 15) == 0;
+    auto load4 = [&] {
+        constexpr int QL = L >= 16 ? 4 : L / 4;  // 16-byte pieces in flight
+        const bool h1 = v.p1 != nullptr, h2 = v.p2 != nullptr;
+        const int nn = in ? n : 0;
+        auto ld = [nn](const float *q, int i) {
+            if (i + 3 < nn) return *reinterpret_cast<const float4 *>(q + i);
+            return make_float4(i < nn ? q[i] : 0.f, i + 1 < nn ? q[i + 1] : 0.f,
+                               i + 2 < nn ? q[i + 2] : 0.f, 0.f);
+        };
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+        for (int b0 = 0; b0 < L / 4; b0 += QL) {
+            float4 a[QL], b[QL], c[QL];
+#pragma unroll
+            for (int u = 0; u < QL; ++u) {
+                if (b0 + u >= L / 4) break;
+                const int i = 4 * ((b0 + u) * T + ll);
+                a[u] = ld(v.p0 + st, i);
+                b[u] = h1 ? ld(v.p1 + st, i) : zero;
+                c[u] = h2 ? ld(v.p2 + st, i) : zero;
+            }
+#pragma unroll
+            for (int u = 0; u < QL; ++u) {
+                if (b0 + u >= L / 4) break;
+                const int i = 4 * ((b0 + u) * T + ll), p = i + (LP - L) * (i / L);
+                *reinterpret_cast<float4 *>(lc + p) =
+                    make_float4(v.unary(a[u].x, b[u].x, c[u].x), v.unary(a[u].y, b[u].y, c[u].y),
+                                v.unary(a[u].z, b[u].z, c[u].z), v.unary(a[u].w, b[u].w, c[u].w));
+            }
+        }
+    };
+    constexpr int UL = UNI ? (L <= 16 ? L : L / 2) : L % 8 == 0 ? 8 : 4;
     auto load = [&](auto stride) {
         const long long step = T * (long long)stride, o0 = ll * (long long)stride;
         const float *q0 = v.p0 + st + o0, *q1 = v.p1 + st + o0, *q2 = v.p2 + st + o0,
@@ -723,6 +762,7 @@ __device__ __forceinline__ void split_chain(const SplitView &v, const int *stop,
         }
     };
     if (v.cols) load(v.stride);
+    else if (UNI && vec) load4();
     else load(UnitStride());
     if (tid % T == 0) xc->bad = 0;
     if (v.cols) __syncthreads();
@@ -746,8 +786,26 @@ __device__ __forceinline__ void split_chain(const SplitView &v, const int *stop,
                 o += T * (long long)stride;
             }
         };
-        if (v.cols) store(v.stride);
-        else store(UnitStride());
+        if (UNI && vec) {
+#pragma unroll 4
+            for (int q = 0; q < L / 4; ++q) {
+                const int i = 4 * (q * T + ll), p = i + (LP - L) * (i / L);
+                const float4 t = *reinterpret_cast<const float4 *>(lx + p);
+                if (i + 3 < n) {
+                    *reinterpret_cast<float4 *>(v.o0 + st + i) = t;
+                    if (v.mode == SPLIT_INIT) *reinterpret_cast<float4 *>(v.o1 + st + i) = t;
+                } else {
+                    const float x[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (i + e < n) v.emit(st + i + e, x[e], 0.f);
+                }
+            }
+        } else if (v.cols) {
+            store(v.stride);
+        } else {
+            store(UnitStride());
+        }
     }
     if (end == SPLIT_FALLBACK && wi == 0) {
         SplitView vv = v;
