@@ -15,9 +15,10 @@ tv_status launch_w(SRC src, int lmax, int nch, WsHeader *hdr, cudaStream_t s)
     const int cs = split_slots<W>(lmax, nch);
     const size_t smem = 2 * (size_t)nch * cs * sizeof(float);
     auto kern = split_kernel<W, UNI, SRC>;
-    tv_status st = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)smem),
-                              "cudaFuncSetAttribute");
+    tv_status st = TV_OK;
+    if (smem > 47 * 1024)  // beyond what needs no opt-in (with the exchange): a call less, 1 us
+        st = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                        "cudaFuncSetAttribute");
     if (st != TV_OK) return st;
     long long blocks = (src.nchains + nch - 1) / nch;
     if constexpr (SRC::GAP) {

@@ -1,5 +1,7 @@
 // Host entry of the threshold-splitting chain kernel.
 #pragma once
+#include <algorithm>
+
 #include "tv_launch.cuh"
 #include "tv_split.cuh"
 
@@ -22,21 +24,34 @@ inline bool split_takes(long long max_len, long long chains, long long max_chain
            chains <= (coop_max_auto() ? max_chains : coop_max_chains());
 }
 
-// Crossovers, measured (us, splitting / thread kernel):
-//  - rows that the fixed-shape thread kernel stages 16 bytes at a time: at 1024 nodes 49 / 113
-//    for 4096 chains and 166 / 176 for 16384, at 256 nodes 24 / 35 and 69 / 49, at 4096 nodes
-//    220 / 453 and 819 / 675; with a weight per edge, at 1024 nodes 75 / 119 and 263 / 193, at
-//    4096 nodes 353 / 471 and 1362 / 737;
-//  - other rows: at 1023 nodes 166 / 234 for 16384 chains and 623 / 890 for 65536, with weights
-//    262 / 543 and 1004 / 1281; chains of under 64 nodes leave most of a warp idle;
+// Largest batch for the splitting kernel. Crossovers, measured (us, splitting / thread kernel;
+// chain_prox called from Python, about 15 us of which are the call):
+//  - rows that the fixed-shape thread kernel stages 16 bytes at a time (vec). Splitting costs
+//    about the same for any short chain, the thread kernel in proportion to its length, so the
+//    line goes with the length: 64 nodes 17 / 18 for 2048 chains and 21 / 16 for 4096, 128 nodes
+//    22 / 22 for 4096 and 28 / 23 for 6144, 192 nodes 25 / 29 and 32 / 30 for 6000, 256 nodes
+//    32 / 37 for 6000 and 40 / 37 for 8192. Long ones: at 512 nodes 54 / 64 for 8192 and 95 / 91
+//    for 16384, at 1024 nodes 91 / 122 and 180 / 177, at 4096 nodes 441 / 475 and 853 / 675. With
+//    a weight per edge as above up to 256 nodes, then at 1024 nodes 86 / 126 for 6000 and
+//    129 / 129 for 8192.
+//  - other rows, one weight: 130 nodes 24 / 23 for 3072 chains, 201 nodes 27 / 31 for 4096 and
+//    36 / 35 for 6144, 257 nodes 41 / 41 for 6144, 385 nodes 48 / 59 and 62 / 60 for 8192, 514
+//    nodes 239 / 266 for 32768 and 469 / 449 for 65536, 770 nodes 636 / 708 for 65536;
+//  - other rows with a weight per edge (the thread kernel stages those worst): 65 nodes 31 / 39
+//    for 8192 and 51 / 41 for 16384, 130 nodes 66 / 78 for 16384 and 120 / 91 for 32768, 201
+//    nodes 248 / 266 for 65536, 1023 nodes 61 / 167 for 4096;
 //  - columns (the thread kernel runs one thread per chain): at 1024 nodes 57 / 889 for 4096 and
 //    650 / 1119 for 65536, at 100 nodes 56 / 93 for 16384 and 195 / 114 for 65536.
-constexpr long long kSplitMaxChainsVec = 8192, kSplitMaxChainsVecW = 6144;
+// Chains of under 64 nodes leave most of a warp idle. Up to 2048 chains the alternative is
+// another warp-per-chain kernel, which is never faster.
 inline long long split_max_chains(long long len, bool cols, bool vec, bool has_w)
 {
     if (len < 64) return kCoopMaxChainsDefault;
-    if (vec && !cols) return has_w ? kSplitMaxChainsVecW : kSplitMaxChainsVec;
-    return cols && len < 256 ? 16384 : INT64_MAX;
+    if (cols) return len < 256 ? 16384 : INT64_MAX;
+    if (vec) return std::max(2048LL, std::min(28 * len, has_w ? 6144LL : 8192LL));
+    if (has_w) return len < 192 ? 150 * len : INT64_MAX;
+    if (len < 400) return std::max(2048LL, 23 * len);
+    return len < 640 ? 32768 : INT64_MAX;
 }
 
 }  // namespace tvh
