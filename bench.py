@@ -85,8 +85,10 @@ def peaks():
 
 # the sources each recorded kernel is built from (its translation unit and the
 # shared headers): a change to any of them voids that kernel's recorded traffic
+SPLIT_SOURCES = ["tv_split.cuh", "tv_split.cu", "tv_split_gap.cu", "tv_split_grid.cuh", "tv_split_launch.h"]
 KERNEL_SOURCES = {
-    "tv2d": ["tv2d.cu", "tv2d_common.cuh", "tv_coop.cuh", "tv_dp.cuh", "tv_launch.cuh", "tv_host.h"],
+    "tv2d": ["tv2d.cu", "tv2d_common.cuh", "tv2d_gap.cuh", "tv_coop.cuh", "tv_dp.cuh", "tv_launch.cuh",
+             "tv_host.h"] + SPLIT_SOURCES,
     "chain": ["tv_chain.cu", "tv_flat.cuh", "tv_halves.cuh", "tv_coop.cuh", "tv_dp.cuh", "tv_launch.cuh",
               "tv_host.h"],
     "pq": ["tv_pq.cu", "tv_coop.cuh", "tv_dp.cuh", "tv_launch.cuh", "tv_host.h"],

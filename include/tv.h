@@ -391,19 +391,21 @@ tv_status tv_set_batched_graph(int on);
 /*
  * Tuning knobs set by the autotuner (the paper has no counterpart): warps per block
  * of the batched phase kernels (1, 2, 4 or 8), and the largest chain batch solved
- * with one warp per chain instead of one thread per chain. 0 restores the defaults:
- * 4096 chains, and 2048 for tv_chain_solve batches of uniform rows of at least 64
- * nodes, a multiple of 4, with 16-byte aligned arrays (the one-thread-per-half kernel
- * stages those 16 bytes at a time and is the faster one from about 2048 chains on).
+ * with warps per chain instead of one thread per chain. 0 restores the defaults. For chains
+ * of 64 to 4096 nodes in the default solve mode (tv_set_coop_split) those follow the chain
+ * length, the staging and the weights (the thread kernels are the faster ones beyond 2048 to
+ * 8192 chains of uniform rows of a multiple of 4 nodes with 16-byte aligned arrays, later or
+ * never for others); otherwise 4096 chains, and 2048 for tv_chain_solve batches of such rows.
  * A value set here applies to every batch.
  */
 tv_status tv_set_batched_warps(int warps_per_block);
 tv_status tv_set_coop_max_chains(int64_t max_chains);
-/* How a chain of 64 nodes or more is solved when its batch runs one warp per chain:
- * 0 by the whole warp from one end; 1 (the default) rooted at its middle node, the two
- * halves' forward passes run at once by the warp's two 16-lane halves (Algorithm 2
- * allows any root); 2 rooted at its middle node by two warps. All give the same
- * solution up to FP32 rounding. */
+/* How a chain of 64 nodes or more is solved when its batch runs warps per chain: 1 (the
+ * default) by threshold splitting for TV-l2 chains of up to 4096 nodes (1, 2 or 4 warps), and
+ * for others rooted at its middle node, the two halves' forward passes run at once by the
+ * warp's two 16-lane halves (Algorithm 2 allows any root); 0 by the whole warp from one end;
+ * 2 rooted at its middle node by two warps. All give the same solution up to FP32
+ * rounding. */
 tv_status tv_set_coop_split(int mode);
 /* How batches that run one thread per chain (tv_chain_solve with chains of 64 nodes or
  * more, and the thread path of tv2d_denoise_batched) solve a chain: 1 (the default)
