@@ -1174,7 +1174,7 @@ __global__ void __launch_bounds__(NTHR)
 //    and writes p = lambda tanh(o) on the vertical edges (rows 0 .. H - 2, 0 on the last
 //    row) for the dual head; in training (lam null) it writes o itself.
 // Training runs the forward layers in the grouped layout and the backward-data ones with
-// the taps reversed as the weights are staged (TwTrain); TW_IMAGE with lam null reads the
+// the taps reversed as the weights are staged (TR); TW_IMAGE with lam null reads the
 // one-channel gradient of o that way. Each accumulator adds its taps and K steps in the
 // order of the mma.sync kernel and gets the same bits (measured over whole gradients, three
 // batch shapes).
@@ -1254,14 +1254,14 @@ __device__ __forceinline__ TwChunk tw_chunk(long long c, int cpc, int L, int til
     return r;
 }
 
-// What training adds to the convolution (all null / false at inference). Only the sign of
-// a pre-activation is needed again on the way back, so a layer leaves one word per pixel
-// (bit c: channel c > 0, exact) instead of its 32 FP32 pre-activations.
-struct TwTrain {
-    unsigned *mask_out;       // forward: the ReLU masks of this layer's 32 outputs
-    const unsigned *mask_in;  // backward data: the masks its 32 outputs are multiplied by
-    bool flip;                // backward data: Wt is the forward layer's [CIN][3][3][COUT]
-};
+// What training adds to the convolution (TR). Only the sign of a pre-activation is needed
+// again on the way back, so a layer leaves one word per pixel (bit c: channel c > 0, exact)
+// instead of its 32 FP32 pre-activations. Instantiations of their own: with the masks' 64
+// instructions per pixel behind runtime tests, inference at 1024 x 1024 took 127 us, not 108.
+//   TW_FORWARD: mask receives the ReLU masks of this layer's 32 outputs;
+//   TW_BACKWARD: the 32 outputs are multiplied by the masks in mask; Wt is the forward
+//   layer's [CIN][3][3][COUT].
+constexpr int TW_PLAIN = 0, TW_FORWARD = 1, TW_BACKWARD = 2;
 
 // Walks the input rows of a block's chunks in load order (n + 2 rows per chunk).
 struct TwRows {
@@ -1297,13 +1297,14 @@ __device__ __forceinline__ int tw_block(unsigned o)
     return R - 1 - (int)(o % R);
 }
 
-template <int CIN, int COUT, int IO>
+template <int CIN, int COUT, int IO, int TR>
 __global__ void __launch_bounds__(TW_THREADS, 4)
     conv3x3_tw(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap_tail,
                int B, int H, int W, int L, const __nv_bfloat16 *Wt, const float *bias, int relu,
                float *pre_out, __nv_bfloat16 *act_out, const float *img, const float *lam, float *p_out,
-               TwTrain tr)
+               [[maybe_unused]] unsigned *mask)
 {
+    static_assert(TR == TW_PLAIN || COUT == 32, "a mask word holds 32 channels");
     static_assert(IO != TW_IMAGE || CIN == 16, "the image input has 16 (2 non-zero) channels");
     static_assert(IO != TW_HEAD || COUT == 16, "the head reads a 16-channel output");
     constexpr int TW_NR = tw_nr(IO), TW_R = tw_r(COUT);
@@ -1363,7 +1364,7 @@ __global__ void __launch_bounds__(TW_THREADS, 4)
     for (int t = tid; t < 9 * KG * COUT; t += TW_THREADS) {
         const int co = t % COUT, dy = (t / COUT) % 3, g = (t / (3 * COUT)) % KG, dx = t / (3 * COUT * KG);
         uint4 *dst = reinterpret_cast<uint4 *>(bbuf + (size_t)t * 16);
-        if (tr.flip) {  // the taps in reverse, the channel roles swapped
+        if constexpr (TR == TW_BACKWARD) {  // the taps in reverse, the channel roles swapped
             unsigned u[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -1614,8 +1615,8 @@ __global__ void __launch_bounds__(TW_THREADS, 4)
                 const int k = tw_block<TW_R>(o);
                 const long long row = (long long)ch.b * H + ch.y0 + j;
                 const int x = ch.x0 + lg * 32 + lane;
-                unsigned keep = 0xffffffffu;  // read ahead of the wait
-                if (tr.mask_in && x < W) keep = tr.mask_in[row * W + x];
+                [[maybe_unused]] unsigned keep = 0u;  // read ahead of the wait
+                if (TR == TW_BACKWARD && x < W) keep = mask[row * W + x];
                 int got = 1;
                 if (lane == 0) got = tw_wait(c_full(k), (o / TW_R) & 1u, bad) ? 1 : 0;
                 got = __shfl_sync(0xffffffffu, got, 0);
@@ -1637,16 +1638,24 @@ __global__ void __launch_bounds__(TW_THREADS, 4)
                     p_out[row * W + x] = !lam ? o0 : ch.y0 + j < H - 1 ? lam[ch.b] * tanhf(o0) : 0.f;
                 } else if (x < W) {
                     const long long pbase = (row * W + x) * COUT;
-                    unsigned signs = 0u;
+#pragma unroll
+                    for (int c = 0; c < COUT; ++c) v[c] += bias_s[c];
+                    if constexpr (TR == TW_FORWARD) {
+                        unsigned signs = 0u;  // 0 - v is negative exactly where v > 0
+#pragma unroll
+                        for (int c = COUT - 1; c >= 0; --c)
+                            signs = __funnelshift_l(__float_as_uint(0.f - v[c]), signs, 1);
+                        mask[row * W + x] = signs;
+                    }
+                    if constexpr (TR == TW_BACKWARD) {
+#pragma unroll
+                        for (int c = 0; c < COUT; ++c) v[c] = keep >> c & 1u ? v[c] : 0.f;
+                    }
 #pragma unroll
                     for (int c = 0; c < COUT; c += 8) {
                         float q[8];
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            q[e] = v[c + e] + bias_s[c + e];
-                            signs |= q[e] > 0.f ? 1u << (c + e) : 0u;
-                            if (!(keep >> (c + e) & 1u)) q[e] = 0.f;
-                        }
+                        for (int e = 0; e < 8; ++e) q[e] = v[c + e];
                         if (pre_out) {
                             *reinterpret_cast<float4 *>(pre_out + pbase + c) = make_float4(q[0], q[1], q[2], q[3]);
                             *reinterpret_cast<float4 *>(pre_out + pbase + c + 4) = make_float4(q[4], q[5], q[6], q[7]);
@@ -1668,7 +1677,6 @@ __global__ void __launch_bounds__(TW_THREADS, 4)
                             *reinterpret_cast<uint4 *>(act_out + o8) = make_uint4(u[0], u[1], u[2], u[3]);
                         }
                     }
-                    if (tr.mask_out) tr.mask_out[row * W + x] = signs;
                 }
             }
         }
@@ -1927,11 +1935,11 @@ CUresult grouped_map(TmapEncodeFn enc, CUtensorMap *map, const __nv_bfloat16 *X,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
-template <int CIN, int COUT, int IO>
+template <int CIN, int COUT, int IO, int TR = TW_PLAIN>
 tv_status launch_conv_tw(const __nv_bfloat16 *X, int B, int H, int W, const __nv_bfloat16 *Wt,
                          const float *bias, int relu, float *pre_out, __nv_bfloat16 *act_out,
                          cudaStream_t s, const float *img = nullptr, const float *lam = nullptr,
-                         float *p_out = nullptr, TwTrain tr = {nullptr, nullptr, false})
+                         float *p_out = nullptr, unsigned *mask = nullptr)
 {
     TmapEncodeFn enc = tmap_encoder();
     if (!enc) {
@@ -1964,7 +1972,7 @@ tv_status launch_conv_tw(const __nv_bfloat16 *X, int B, int H, int W, const __nv
         set_error("tv_net_conv3x3: cuTensorMapEncodeTiled rejected the activation layout");
         return TV_ERR_INVALID;
     }
-    auto kern = conv3x3_tw<CIN, COUT, IO>;
+    auto kern = conv3x3_tw<CIN, COUT, IO, TR>;
     constexpr size_t smem = conv_tw_smem<CIN, COUT, IO>();
     static bool attr = false;
     if (!attr) {
@@ -2009,7 +2017,7 @@ tv_status launch_conv_tw(const __nv_bfloat16 *X, int B, int H, int W, const __nv
     PdlScope pdl(true);
     tv_status st = check_cuda(launch_k(kern, dim3((unsigned)blocks), dim3(TW_THREADS), smem, s, tmap,
                                        tmap_tail, B, H, W, (int)L, Wt, bias, relu, pre_out, act_out,
-                                       img, lam, p_out, tr),
+                                       img, lam, p_out, mask),
                               "conv launch");
     if (st == TV_OK) note_launch();
     return st;
@@ -2485,9 +2493,11 @@ tv_status tv_net_train_layer(const void *d_x, const float *d_f, const float *d_l
     auto X = static_cast<const __nv_bfloat16 *>(d_x);
     auto Wt = static_cast<const __nv_bfloat16 *>(d_w);
     auto A = static_cast<__nv_bfloat16 *>(d_act_out);
-    const TwTrain tr{d_mask_out, nullptr, false};
-    if (X) return launch_conv_tw<32, 32, TW_GROUPED>(X, B, H, W, Wt, d_bias, 1, nullptr, A, s, nullptr, nullptr, nullptr, tr);
-    return launch_conv_tw<16, 32, TW_IMAGE>(nullptr, B, H, W, Wt, d_bias, 1, nullptr, A, s, d_f, d_lam, nullptr, tr);
+    if (X)
+        return launch_conv_tw<32, 32, TW_GROUPED, TW_FORWARD>(X, B, H, W, Wt, d_bias, 1, nullptr, A, s, nullptr,
+                                                              nullptr, nullptr, d_mask_out);
+    return launch_conv_tw<16, 32, TW_IMAGE, TW_FORWARD>(nullptr, B, H, W, Wt, d_bias, 1, nullptr, A, s, d_f,
+                                                        d_lam, nullptr, d_mask_out);
 }
 
 tv_status tv_net_train_head(const void *d_x, int B, int H, int W, const void *d_w, const float *d_bias,
@@ -2543,18 +2553,21 @@ tv_status tv_net_train_backward(const void *d_x, const float *d_f, const float *
     float *P = static_cast<float *>(d_ws);
     if (!d_x)  // the first layer: no gradient of its input
         return launch_wgrad_plane<true>(d_dy, d_f, d_lam, B, H, W, d_dw, d_db, P, s);
-    const TwTrain tr{nullptr, d_mask, true};
+    unsigned *mask = const_cast<uint32_t *>(d_mask);  // read only in TW_BACKWARD
     auto Wt = static_cast<const __nv_bfloat16 *>(d_w);
     auto dX = static_cast<__nv_bfloat16 *>(d_dx);
     tv_status st;
     if (d_grad_o) {  // the last layer: one channel of dY
         st = launch_wgrad_plane<false>(d_x, d_grad_o, nullptr, B, H, W, d_dw, d_db, P, s);
         if (st != TV_OK) return st;
-        return launch_conv_tw<16, 32, TW_IMAGE>(nullptr, B, H, W, Wt, nullptr, 0, nullptr, dX, s, d_grad_o, nullptr, nullptr, tr);
+        return launch_conv_tw<16, 32, TW_IMAGE, TW_BACKWARD>(nullptr, B, H, W, Wt, nullptr, 0, nullptr, dX, s,
+                                                             d_grad_o, nullptr, nullptr, mask);
     }
     st = launch_wgrad_tc(static_cast<const __nv_bfloat16 *>(d_x), static_cast<const __nv_bfloat16 *>(d_dy), B, H, W, d_dw, d_db, P, s);
     if (st != TV_OK) return st;
-    return launch_conv_tw<32, 32, TW_GROUPED>(static_cast<const __nv_bfloat16 *>(d_dy), B, H, W, Wt, nullptr, 0, nullptr, dX, s, nullptr, nullptr, nullptr, tr);
+    return launch_conv_tw<32, 32, TW_GROUPED, TW_BACKWARD>(static_cast<const __nv_bfloat16 *>(d_dy), B, H, W, Wt,
+                                                           nullptr, 0, nullptr, dX, s, nullptr, nullptr, nullptr,
+                                                           mask);
 }
 
 tv_status tv_net_adam(float *d_w, float *d_m, float *d_v, float *d_g, int64_t n, float lr,
