@@ -42,11 +42,12 @@ inline bool split_takes(long long max_len, long long chains, long long max_chain
 //    nodes 248 / 266 for 65536, 1023 nodes 61 / 167 for 4096;
 //  - columns (the thread kernel runs one thread per chain): at 1024 nodes 57 / 889 for 4096 and
 //    650 / 1119 for 65536, at 100 nodes 56 / 93 for 16384 and 195 / 114 for 65536.
-// Chains of under 64 nodes leave most of a warp idle. Up to 2048 chains the alternative is
+// Chains of under 64 nodes leave most of a warp idle: at 16 nodes 16.6 / 14.7 (the
+// warp-per-chain kernel) for 4096 chains, 13.7 / 13.8 for 2048. Up to 2048 chains the alternative is
 // another warp-per-chain kernel, which is never faster.
 inline long long split_max_chains(long long len, bool cols, bool vec, bool has_w)
 {
-    if (len < 64) return kCoopMaxChainsDefault;
+    if (len < 64) return len < 32 && !cols ? 2048 : kCoopMaxChainsDefault;
     if (cols) return len < 256 ? 16384 : INT64_MAX;
     if (vec) return std::max(2048LL, std::min(28 * len, has_w ? 6144LL : 8192LL));
     if (has_w) return len < 192 ? 150 * len : INT64_MAX;
