@@ -37,7 +37,6 @@ using namespace tvh;
 namespace {
 
 constexpr int kGradWarps = 4;
-constexpr int kGradSmemNodes = 4096;  // g and segment means of one chain: 8 bytes per node
 constexpr int kGradUnroll = 4;        // steps whose loads are in flight together
 
 struct GradArgs {
@@ -46,13 +45,13 @@ struct GradArgs {
     long long nchains;
     int maxlen;
     float *gy, *gw;
-    int smem_nodes;
     bool full;  // also write gw (0) at a chain's last node
 };
 
+// GW: with grad_w.
+template <bool GW>
 __global__ void __launch_bounds__(kGradWarps * WARP) chain_vjp_kernel(GradArgs a, WsHeader *hdr)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & (WARP - 1);
     const int warp = threadIdx.x / WARP;
     const long long k = (long long)blockIdx.x * kGradWarps + warp;
@@ -74,10 +73,7 @@ __global__ void __launch_bounds__(kGradWarps * WARP) chain_vjp_kernel(GradArgs a
     if (n == 0) return;
     const float *x = a.x + start, *g = a.g + start;
     float *gy = a.gy + start;
-    // per-node segment means: shared memory when the chain fits, else grad_y itself
-    float *mean = (n <= a.smem_nodes)
-                      ? reinterpret_cast<float *>(smem_raw) + (size_t)warp * a.smem_nodes
-                      : gy;
+    float *mean = gy;  // segment means wait in grad_y itself
     const int nblk = (n + WARP - 1) / WARP;
 
     // ---- forward: segmented (sum, count); the mean lands on each segment's last node
@@ -132,9 +128,8 @@ __global__ void __launch_bounds__(kGradWarps * WARP) chain_vjp_kernel(GradArgs a
     }
     __syncwarp();
     // ---- backward: every node takes the mean stored at its segment's last node
-    // (a batch's tail means are read before any of its outputs is written: for a chain
-    // longer than the shared-memory records the means live in grad_y itself, each at its
-    // segment's last node, inside the step that owns that node)
+    // (a batch's tail means are read before any of its outputs is written: the means live in
+    // grad_y itself, each at its segment's last node, inside the step that owns that node)
     float carry_m = 0.f;
     for (int b0 = nblk - 1; b0 >= 0; b0 -= U) {
         float xv[U], xn[U], mv[U];
@@ -167,13 +162,13 @@ __global__ void __launch_bounds__(kGradWarps * WARP) chain_vjp_kernel(GradArgs a
             if (in) {
                 gy[i] = m;
                 // jump edge i -> i+1: sign * (mean left - mean right); fused edges: 0
-                if (a.gw && a.full && i + 1 == n) a.gw[start + i] = 0.f;
-                if (a.gw && i + 1 < n)
+                if (GW && i + 1 < n)
                     a.gw[start + i] = tail ? ((xnext > xi ? 1.f : -1.f) * (m - mright)) : 0.f;
             }
             carry_m = __shfl_sync(FULL, m, 0);
         }
     }
+    if (GW && a.full && lane == 0) a.gw[start + n - 1] = 0.f;
 }
 
 // Exchange between the warps of one chain.
@@ -516,7 +511,7 @@ tv_status solve_backward(const float *d_x, const float *d_grad_x, const int64_t 
         auto al = [](const void *q) { return ((uintptr_t)q & 15) == 0; };
         const bool vec = !d_offsets && max_len % 4 == 0 && al(d_x) && al(d_grad_x) &&
                          al(d_grad_y) && al(d_grad_w);
-        GradArgs a{d_x, d_grad_x, d_offsets, num_chains, (int)max_len, d_grad_y, d_grad_w, 0,
+        GradArgs a{d_x, d_grad_x, d_offsets, num_chains, (int)max_len, d_grad_y, d_grad_w,
                    full};
         const bool prof = prof_on();
         if (prof) prof_mark(PK_GRAD, s, true);
@@ -524,18 +519,12 @@ tv_status solve_backward(const float *d_x, const float *d_grad_x, const int64_t 
         if (prof) prof_mark(PK_GRAD, s, false);
         return st;
     }
-    const int smem_nodes = max_len <= kGradSmemNodes ? (int)max_len : 0;
-    const size_t smem = (size_t)kGradWarps * smem_nodes * sizeof(float);
-    st = check_cuda(cudaFuncSetAttribute(chain_vjp_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                    "cudaFuncSetAttribute");
-    if (st != TV_OK) return st;
-    GradArgs a{d_x, d_grad_x, d_offsets, num_chains, (int)max_len, d_grad_y, d_grad_w, smem_nodes,
-               full};
+    GradArgs a{d_x, d_grad_x, d_offsets, num_chains, (int)max_len, d_grad_y, d_grad_w, full};
     const long long blocks = (num_chains + kGradWarps - 1) / kGradWarps;
     const bool prof = prof_on();
     if (prof) prof_mark(PK_GRAD, s, true);
-    chain_vjp_kernel<<<(unsigned)blocks, kGradWarps * WARP, smem, s>>>(a, hdr);
+    auto kern = d_grad_w ? chain_vjp_kernel<true> : chain_vjp_kernel<false>;
+    kern<<<(unsigned)blocks, kGradWarps * WARP, 0, s>>>(a, hdr);
     st = check_cuda(cudaGetLastError(), "backward kernel launch");
     if (st == TV_OK) note_launch();
     if (prof) prof_mark(PK_GRAD, s, false);
