@@ -444,13 +444,12 @@ tv_status launch_runs(const GradArgs &a, int nmax, bool vec, WsHeader *hdr, int 
     const int cpb = W == 1 ? 2 : 1;  // chains per block
     const int l = run_pick<W>(nmax), cs = 32 * W * ((l / 4) % 2 == 1 ? l : l + 4);
     const size_t smem = 2 * sizeof(float) * (size_t)cs * cpb;
+    // no opt-in (a limit that belongs to the kernel, which calls on other threads would move)
+    static_assert(2 * sizeof(float) * 36 * 32 * W * (W == 1 ? 2 : 1) + sizeof(RunX<W>) <= 48 * 1024,
+                  "shared memory of the largest block");
     auto kern = vec ? run_means_kernel<W, true> : run_means_kernel<W, false>;
-    tv_status st = check_cuda(
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-        "cudaFuncSetAttribute");
-    if (st != TV_OK) return st;
     kern<<<(unsigned)((a.nchains + cpb - 1) / cpb), cpb * W * WARP, smem, s>>>(a, hdr, cs, n_lo);
-    st = check_cuda(cudaGetLastError(), "backward kernel launch");
+    tv_status st = check_cuda(cudaGetLastError(), "backward kernel launch");
     if (st == TV_OK) note_launch();
     return st;
 }

@@ -107,16 +107,18 @@ tv_status launch_coop(const P &p, long long nchains, int max_len, float2 *rec, f
     const long long blocks = (nchains + cpb - 1) / cpb;
     // records in shared memory when a block's share fits in ~200 KB, else in the workspace
     const size_t xchg = mode != 0 ? cpb * sizeof(tvk::PairXchg) : 0;
+    constexpr size_t kMost = 200 * 1024;
     const bool fits = max_len <= kCoopSmemNodes &&
-                      xchg + cpb * tvk::coop_smem_per_warp<P>(max_len) <= (size_t)200 * 1024;
+                      xchg + cpb * tvk::coop_smem_per_warp<P>(max_len) <= kMost;
     const int smem_nodes = fits ? max_len : 0;
     const size_t smem = xchg + cpb * tvk::coop_smem_per_warp<P>(smem_nodes);
     auto kern = mode == 1 ? tvk::coop_chain_kernel<P, true> : tvk::coop_chain_kernel<P, false>;
     if constexpr (!tvk::has_unary_g<P>::value) {
         if (pair) kern = tvk::coop_pair_kernel<P>;
     }
+    // the most of any launch: the limit is the kernel's, and calls on other threads share it
     tv_status st = check_cuda(
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMost),
         "cudaFuncSetAttribute");
     if (st != TV_OK) return st;
     const bool prof = prof_on();

@@ -46,7 +46,8 @@ constexpr int kNcMaxWarps = 4;
 
 // warps per block: as many as fit three message buffers each in ~220 KB of shared memory
 // (at least the two warps of one chain: 2 * 24 * 4096 bytes fit)
-int nc_warps(int T) { return std::max(2, std::min(kNcMaxWarps, (220 * 1024) / (24 * T))); }
+constexpr int kNcMaxBuffers = 220 * 1024;
+int nc_warps(int T) { return std::max(2, std::min(kNcMaxWarps, kNcMaxBuffers / (24 * T))); }
 
 struct NcArgs {
     const int64_t *uoff;  // node -> first breakpoint (N + 1 entries), or NULL: grid unaries
@@ -700,8 +701,10 @@ tv_status tv_chain_solve_nonconvex(const int64_t *d_uoff, const float *d_ulam,
     const int wpb = 2 * pairs;
     const size_t smem = ((pairs * sizeof(NcPairXchg) + 15) & ~(size_t)15) +
                         (size_t)wpb * 3 * max_breakpoints * sizeof(float2);
+    // the most of any launch: the limit is the kernel's, and calls on other threads share it
+    constexpr int most = kNcMaxBuffers + (kNcMaxWarps / 2 * (int)sizeof(NcPairXchg) + 15) / 16 * 16;
     st = check_cuda(cudaFuncSetAttribute(nc_chain_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, most),
                     "cudaFuncSetAttribute");
     if (st != TV_OK) return st;
     const long long blocks = (num_chains + pairs - 1) / pairs;

@@ -16,8 +16,11 @@ tv_status launch_w(SRC src, int lmax, int nch, WsHeader *hdr, cudaStream_t s)
     const size_t smem = 2 * (size_t)nch * cs * sizeof(float);
     auto kern = split_kernel<W, UNI, SRC>;
     tv_status st = TV_OK;
-    if (smem > 47 * 1024)  // beyond what needs no opt-in (with the exchange): a call less, 1 us
-        st = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+    // Beyond what needs no opt-in (with the exchange; a call less, 1 us). The limit is the kernel's,
+    // not the launch's: always the most, so that no other thread's call lowers it meanwhile.
+    if (smem > 47 * 1024)
+        st = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)split_smem_most<W>()),
                         "cudaFuncSetAttribute");
     if (st != TV_OK) return st;
     long long blocks = (src.nchains + nch - 1) / nch;
