@@ -178,6 +178,13 @@ struct RunX {
     unsigned char cut[W];
 };
 
+// Mean of a run inside a lane. A sum that is not finite is the mean: mean_of's residual would
+// turn an infinite one into NaN.
+__device__ __forceinline__ float run_mean(float s, float k)
+{
+    return fabsf(s) < INFINITY ? mean_of(s, k) : s;
+}
+
 template <int L, int W, bool VEC>
 __device__ __forceinline__ void run_means(const GradArgs &a, long long start, int n, float *sx,
                                           float *sg, RunX<W> *xc)
@@ -326,7 +333,7 @@ __device__ __forceinline__ void run_means(const GradArgs &a, long long start, in
         for (int j = L - 1; j >= 0; --j) {
             s = cut[j] ? y[j] : s + y[j];
             k = cut[j] ? 1.f : k + 1.f;
-            m[j] = mean_of(s, k);
+            m[j] = run_mean(s, k);
         }
     }
     const unsigned LC = C & (0u - C);
