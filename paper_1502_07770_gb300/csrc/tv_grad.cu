@@ -174,15 +174,16 @@ __global__ void __launch_bounds__(kGradWarps * WARP) chain_vjp_kernel(GradArgs a
 // Exchange between the warps of one chain.
 template <int W>
 struct RunX {
-    float R[W], K[W], St[W], Kt[W], z[W];
+    Sum2 R[W], St[W];
+    float K[W], Kt[W], z[W];
     unsigned char cut[W];
 };
 
-// Mean of a run inside a lane. A sum that is not finite is the mean: mean_of's residual would
-// turn an infinite one into NaN.
-__device__ __forceinline__ float run_mean(float s, float k)
+// Mean of a run. A sum that is not finite is the mean: the residual would turn an infinite one
+// into NaN.
+__device__ __forceinline__ float run_mean(Sum2 s, float k)
 {
-    return fabsf(s) < INFINITY ? mean_of(s, k) : s;
+    return fabsf(s.hi) < INFINITY ? mean_of(s, k) : s.hi;
 }
 
 template <int L, int W, bool VEC>
@@ -253,33 +254,46 @@ __device__ __forceinline__ void run_means(const GradArgs &a, long long start, in
         }
     }
     sync();  // the slots are written below
-    // (selected, not multiplied by 0: an infinite or NaN gradient stays in its own run)
-    float Sh = 0.f, St = 0.f;  // to the lane's first cut; after its last one
+    // One walk from the right, restarting at cuts (selected, not multiplied by 0: an infinite or
+    // NaN gradient stays in its own run), gives the sum to the lane's first cut, the one after
+    // its last cut, and the means of the runs that lie in the lane, at their first nodes. Sums
+    // are carried in two floats: node after node in one float a mean was off by a third more
+    // than from the step-wise kernel's tree of sums.
+    const Sum2 zero{0.f, 0.f};
+    Sum2 Sh = zero, St = zero;
+    float m[L];
+    {
+        float k = 0.f;
 #pragma unroll
-    for (int j = L - 1; j >= 0; --j) {
-        if ((C & ((2u << (L - 1 - j)) - 1u)) == 0) St += y[j];
-        Sh = cut[j] ? y[j] : Sh + y[j];
+        for (int j = L - 1; j >= 0; --j) {
+            Sh = pick(cut[j], zero, Sh) + Sum2{y[j], 0.f};
+            k = cut[j] ? 1.f : k + 1.f;
+            m[j] = run_mean(Sh, k);
+            if ((C & ((2u << (L - 1 - j)) - 1u)) == 0) St = Sh;
+        }
     }
     const unsigned bc = __ballot_sync(FULL, C != 0);
     const float kh = C ? (float)(__clz(C) - (31 - L)) : (float)L;
     const float kt = (float)(__ffs(C) - 1);
     // R, K: sum and count from the lane's first node to the end of its run
-    float R = Sh;
+    Sum2 R = Sh;
     const unsigned ahead = bc >> lane;
     const int pe = ahead ? lane + __ffs(ahead) - 1 : WARP;
 #pragma unroll
     for (int o = 1; o < WARP; o <<= 1) {
-        const float r2 = __shfl_down_sync(FULL, R, o);
-        if (lane + o < WARP && lane + o <= pe) R += r2;
+        const Sum2 r2 = shfl_down(R, o);
+        if (lane + o < WARP && lane + o <= pe) R = R + r2;
     }
     const float kp = __shfl_sync(FULL, kh, pe & (WARP - 1));
     float K = pe < WARP ? (float)((pe - lane) * L) + kp : (float)((WARP - lane) * L);
     const int lq = bc ? 31 - __clz(bc) : 0;  // the warp's last lane with a cut
-    float tS = St, tK = kt, Rin = 0.f, Kin = 0.f, zprev = 0.f;
+    Sum2 tS = St, Rin = zero;
+    float tK = kt, Kin = 0.f, zprev = 0.f;
     if constexpr (W > 1) {
-        const float Rq = __shfl_down_sync(FULL, R, 1), Kq = __shfl_down_sync(FULL, K, 1);
+        const Sum2 Rq = shfl_down(R, 1);
+        const float Kq = __shfl_down_sync(FULL, K, 1);
         if (lane < WARP - 1) {
-            tS += Rq;
+            tS = tS + Rq;
             tK += Kq;
         }
         if (lane == lq) {
@@ -292,50 +306,41 @@ __device__ __forceinline__ void run_means(const GradArgs &a, long long start, in
             xc->cut[wi] = bc != 0;
         }
         __syncthreads();
-        float rr = 0.f, kk = 0.f;  // from warp q's first node to the end of its run
-        bool enters = true;        // the run that enters warp wi is not found yet
+        Sum2 rr = zero;      // from warp q's first node to the end of its run
+        float kk = 0.f;
+        bool enters = true;  // the run that enters warp wi is not found yet
 #pragma unroll
         for (int q = W - 1; q >= 0; --q) {
             const bool e = xc->cut[q] != 0;
             if (q < wi && enters && e) {
-                zprev = __fdiv_rn(xc->St[q] + rr, xc->Kt[q] + kk);
+                zprev = run_mean(xc->St[q] + rr, xc->Kt[q] + kk);
                 enters = false;
             }
-            rr = xc->R[q] + (e ? 0.f : rr);
+            rr = xc->R[q] + pick(e, zero, rr);
             kk = xc->K[q] + (e ? 0.f : kk);
             if (q == wi + 1) {
                 Rin = rr;
                 Kin = kk;
             }
         }
-        if (enters) zprev = __fdiv_rn(rr, kk);
+        if (enters) zprev = run_mean(rr, kk);
         if (pe == WARP) {
-            R += Rin;
+            R = R + Rin;
             K += Kin;
         }
     }
-    float Rn = __shfl_down_sync(FULL, R, 1), Kn = __shfl_down_sync(FULL, K, 1);
+    Sum2 Rn = shfl_down(R, 1);
+    float Kn = __shfl_down_sync(FULL, K, 1);
     if (lane == WARP - 1) {
         Rn = Rin;
         Kn = Kin;
     }
     const bool out = W > 1 && lane == lq;  // its last run leaves the warp
-    const float zt = __fdiv_rn((out ? tS : St) + (out ? Rin : Rn), (out ? tK : kt) + (out ? Kin : Kn));
-    const float zh = __fdiv_rn(R, K);
+    const float zt = run_mean(pick(out, tS, St) + pick(out, Rin, Rn), (out ? tK : kt) + (out ? Kin : Kn));
+    const float zh = run_mean(R, K);
     const unsigned before = bc & ((1u << lane) - 1u);
     float zr = __shfl_sync(FULL, C || W > 1 ? zt : zh, before ? 31 - __clz(before) : 0);
     if (W > 1 ? !before : lane == 0) zr = W > 1 ? zprev : zh;
-    // means of the runs that begin in the lane, at their first nodes, then spread
-    float m[L];
-    {
-        float s = 0.f, k = 0.f;
-#pragma unroll
-        for (int j = L - 1; j >= 0; --j) {
-            s = cut[j] ? y[j] : s + y[j];
-            k = cut[j] ? 1.f : k + 1.f;
-            m[j] = run_mean(s, k);
-        }
-    }
     const unsigned LC = C & (0u - C);
 #pragma unroll
     for (int j = 0; j < L; ++j) {

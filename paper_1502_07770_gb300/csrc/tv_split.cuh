@@ -163,6 +163,30 @@ __device__ __forceinline__ float mean_of(float s, float k)
     return fmaf(fmaf(-q, k, s), rc, q);
 }
 
+// A sum carried in two floats: hi the running FP32 sum, lo what its roundings left out.
+struct Sum2 {
+    float hi, lo;
+};
+__device__ __forceinline__ Sum2 operator+(Sum2 a, Sum2 b)
+{
+    const float t = a.hi + b.hi, u = t - a.hi;
+    return Sum2{t, ((a.hi - (t - u)) + (b.hi - u)) + (a.lo + b.lo)};
+}
+__device__ __forceinline__ Sum2 pick(bool c, Sum2 a, Sum2 b)
+{
+    return Sum2{c ? a.hi : b.hi, c ? a.lo : b.lo};
+}
+__device__ __forceinline__ Sum2 shfl_down(Sum2 a, int o)
+{
+    return Sum2{__shfl_down_sync(FULL, a.hi, o), __shfl_down_sync(FULL, a.lo, o)};
+}
+// s / k to within a little over half an ulp: the residual takes up the low part
+__device__ __forceinline__ float mean_of(Sum2 s, float k)
+{
+    const float rc = rcp_approx(k), q = s.hi * rc;
+    return fmaf(fmaf(-q, k, s.hi) + s.lo, rc, q);
+}
+
 template <int W>
 __device__ __forceinline__ void split_sync(int bar)
 {
