@@ -173,10 +173,9 @@ __global__ void __launch_bounds__(kGradWarps * WARP) chain_vjp_kernel(GradArgs a
 
 // Exchange between the warps of one chain.
 template <int W>
-struct RunX {
-    Sum2 R[W], St[W];
-    float K[W], Kt[W], z[W];
-    unsigned char cut[W];
+struct MeansX {
+    RunX<W, Sum2> run;
+    float z[W];
 };
 
 // Mean of a run. A sum that is not finite is the mean: the residual would turn an infinite one
@@ -188,7 +187,7 @@ __device__ __forceinline__ float run_mean(Sum2 s, float k)
 
 template <int L, int W, bool VEC>
 __device__ __forceinline__ void run_means(const GradArgs &a, long long start, int n, float *sx,
-                                          float *sg, RunX<W> *xc)
+                                          float *sg, MeansX<W> *xc)
 {
     constexpr int LP = split_lp<L>();
     constexpr int T = W * WARP;
@@ -273,79 +272,13 @@ __device__ __forceinline__ void run_means(const GradArgs &a, long long start, in
         }
     }
     const unsigned bc = __ballot_sync(FULL, C != 0);
-    const float kh = C ? (float)(__clz(C) - (31 - L)) : (float)L;
-    const float kt = (float)(__ffs(C) - 1);
-    // R, K: sum and count from the lane's first node to the end of its run
-    Sum2 R = Sh;
-    const unsigned ahead = bc >> lane;
-    const int pe = ahead ? lane + __ffs(ahead) - 1 : WARP;
-#pragma unroll
-    for (int o = 1; o < WARP; o <<= 1) {
-        const Sum2 r2 = shfl_down(R, o);
-        if (lane + o < WARP && lane + o <= pe) R = R + r2;
-    }
-    const float kp = __shfl_sync(FULL, kh, pe & (WARP - 1));
-    float K = pe < WARP ? (float)((pe - lane) * L) + kp : (float)((WARP - lane) * L);
-    const int lq = bc ? 31 - __clz(bc) : 0;  // the warp's last lane with a cut
-    Sum2 tS = St, Rin = zero;
-    float tK = kt, Kin = 0.f, zprev = 0.f;
-    if constexpr (W > 1) {
-        const Sum2 Rq = shfl_down(R, 1);
-        const float Kq = __shfl_down_sync(FULL, K, 1);
-        if (lane < WARP - 1) {
-            tS = tS + Rq;
-            tK += Kq;
-        }
-        if (lane == lq) {
-            xc->St[wi] = tS;
-            xc->Kt[wi] = tK;
-        }
-        if (lane == 0) {
-            xc->R[wi] = R;
-            xc->K[wi] = K;
-            xc->cut[wi] = bc != 0;
-        }
-        __syncthreads();
-        Sum2 rr = zero;      // from warp q's first node to the end of its run
-        float kk = 0.f;
-        bool enters = true;  // the run that enters warp wi is not found yet
-#pragma unroll
-        for (int q = W - 1; q >= 0; --q) {
-            const bool e = xc->cut[q] != 0;
-            if (q < wi && enters && e) {
-                zprev = run_mean(xc->St[q] + rr, xc->Kt[q] + kk);
-                enters = false;
-            }
-            rr = xc->R[q] + pick(e, zero, rr);
-            kk = xc->K[q] + (e ? 0.f : kk);
-            if (q == wi + 1) {
-                Rin = rr;
-                Kin = kk;
-            }
-        }
-        if (enters) zprev = run_mean(rr, kk);
-        if (pe == WARP) {
-            R = R + Rin;
-            K += Kin;
-        }
-    }
-    Sum2 Rn = shfl_down(R, 1);
-    float Kn = __shfl_down_sync(FULL, K, 1);
-    if (lane == WARP - 1) {
-        Rn = Rin;
-        Kn = Kin;
-    }
-    const bool out = W > 1 && lane == lq;  // its last run leaves the warp
-    const float zt = run_mean(pick(out, tS, St) + pick(out, Rin, Rn), (out ? tK : kt) + (out ? Kin : Kn));
-    const float zh = run_mean(R, K);
-    const unsigned before = bc & ((1u << lane) - 1u);
-    float zr = __shfl_sync(FULL, C || W > 1 ? zt : zh, before ? 31 - __clz(before) : 0);
-    if (W > 1 ? !before : lane == 0) zr = W > 1 ? zprev : zh;
+    const RunEnds<Sum2> run = join_runs<L, W>(Sh, St, C, bc, lane, wi, &xc->run, run_mean, sync);
+    float zr = run.zr;
     const unsigned LC = C & (0u - C);
 #pragma unroll
     for (int j = 0; j < L; ++j) {
         if (j > 0 && cut[j > 0 ? j - 1 : 0]) zr = m[j];
-        if (j > 0 && (LC & (1u << (L - j)))) zr = zt;
+        if (j > 0 && (LC & (1u << (L - j)))) zr = run.zt;
         m[j] = zr;
     }
 #pragma unroll
@@ -417,7 +350,7 @@ __global__ void __launch_bounds__(W <= 2 ? 64 : W * WARP)
     run_means_kernel(GradArgs a, WsHeader *hdr, int cs, int n_lo)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ RunX<W> xc;
+    __shared__ MeansX<W> xc;
     const int warp = threadIdx.x / WARP;
     const long long k = W == 1 ? (long long)blockIdx.x * (blockDim.x / WARP) + warp : blockIdx.x;
     if (k >= a.nchains) return;
@@ -457,7 +390,7 @@ tv_status launch_runs(const GradArgs &a, int nmax, bool vec, WsHeader *hdr, int 
     const int l = run_pick<W>(nmax), cs = 32 * W * ((l / 4) % 2 == 1 ? l : l + 4);
     const size_t smem = 2 * sizeof(float) * (size_t)cs * cpb;
     // no opt-in (a limit that belongs to the kernel, which calls on other threads would move)
-    static_assert(2 * sizeof(float) * 36 * 32 * W * (W == 1 ? 2 : 1) + sizeof(RunX<W>) <= 48 * 1024,
+    static_assert(2 * sizeof(float) * 36 * 32 * W * (W == 1 ? 2 : 1) + sizeof(MeansX<W>) <= 48 * 1024,
                   "shared memory of the largest block");
     auto kern = vec ? run_means_kernel<W, true> : run_means_kernel<W, false>;
     kern<<<(unsigned)((a.nchains + cpb - 1) / cpb), cpb * W * WARP, smem, s>>>(a, hdr, cs, n_lo);

@@ -132,19 +132,6 @@ static __device__ __noinline__ void split_fallback(const SplitView &v, long long
                      (float *)nullptr, spill, hdr);
 }
 
-// Exchange between the warps of one chain (W > 1).
-template <int W>
-struct SplitX {
-    float a[W], lo[W], hi[W];     // composed map of each warp
-    float R[W], St[W], Kt[W];     // head sum, tail sum and count of each warp
-    float K[W];                   // head count
-    float u[W], u2[W];            // flow of a (new) cut after the warp's last node
-    float re[W];                  // r of that node
-    unsigned amax[W];
-    unsigned char cut[W], side[W], more[W], heavy[W];  // heavy: 1; the stop flag: 2
-    int bad;                      // the chain goes to the fallback, or was stopped
-};
-
 __device__ __forceinline__ float rcp_approx(float v)
 {
     float r;
@@ -180,12 +167,35 @@ __device__ __forceinline__ Sum2 shfl_down(Sum2 a, int o)
 {
     return Sum2{__shfl_down_sync(FULL, a.hi, o), __shfl_down_sync(FULL, a.lo, o)};
 }
+__device__ __forceinline__ float pick(bool c, float a, float b) { return c ? a : b; }
+__device__ __forceinline__ float shfl_down(float a, int o) { return __shfl_down_sync(FULL, a, o); }
 // s / k to within a little over half an ulp: the residual takes up the low part
 __device__ __forceinline__ float mean_of(Sum2 s, float k)
 {
     const float rc = rcp_approx(k), q = s.hi * rc;
     return fmaf(fmaf(-q, k, s.hi) + s.lo, rc, q);
 }
+
+// Sums of the runs that leave a warp, for the other warps of its chain (W > 1).
+template <int W, class T>
+struct RunX {
+    T R[W], St[W];        // head sum and tail sum of each warp
+    float K[W], Kt[W];    // and their counts
+    unsigned char cut[W];
+};
+
+// Exchange between the warps of one chain (W > 1).
+template <int W>
+struct SplitX {
+    float a[W], lo[W], hi[W];     // composed map of each warp
+    RunX<W, float> run;           // of a round
+    RunX<W, Sum2> sum;            // of the solution
+    float u[W], u2[W];            // flow of a (new) cut after the warp's last node
+    float re[W];                  // r of that node
+    unsigned amax[W];
+    unsigned char side[W], more[W], heavy[W];  // heavy: 1; the stop flag: 2
+    int bad;                      // the chain goes to the fallback, or was stopped
+};
 
 template <int W>
 __device__ __forceinline__ void split_sync(int bar)
@@ -200,6 +210,106 @@ __device__ __forceinline__ void split_sync(int bar)
         else if (bar == 2) asm volatile("bar.sync 3, %0;" ::"n"(W * WARP) : "memory");
         else asm volatile("bar.sync 4, %0;" ::"n"(W * WARP) : "memory");
     }
+}
+
+// The runs of one chain of lanes of L nodes, joined across its lanes and warps. C: the lane's
+// cuts (node j is bit L-1-j, cut after it), bc the lanes of the warp with one; Sh the sum to the
+// lane's first cut (or of all its nodes), St after its last one. mean(s, k): value of a run.
+template <class T>
+struct RunEnds {
+    T Rn;          // sum and count from the next lane's first node to the end of its run
+    float Kn;
+    float zr, zt;  // value of the run at the lane's first node; of the one after its last cut
+};
+template <int L, int W, class T, class MEAN, class SYNC>
+__device__ __forceinline__ RunEnds<T> join_runs(T Sh, T St, unsigned C, unsigned bc, int lane, int wi,
+                                                RunX<W, T> *xc, MEAN mean, SYNC sync)
+{
+    const float kh = C ? (float)(__clz(C) - (31 - L)) : (float)L;  // nodes of the head
+    const float kt = (float)(__ffs(C) - 1);                       // nodes after the last cut
+    RunEnds<T> e;
+    // R, K: sum and count from the lane's first node to the end of its run
+    T R = Sh;
+    float K = kh;
+    int pe = lane;
+    if (bc != FULL) {
+        const unsigned ahead = bc >> lane;
+        pe = ahead ? lane + __ffs(ahead) - 1 : WARP;  // lane where that run ends
+#pragma unroll
+        for (int o = 1; o < WARP; o <<= 1) {
+            const T r2 = shfl_down(R, o);
+            if (lane + o < WARP && lane + o <= pe) R = R + r2;
+        }
+        const float kp = __shfl_sync(FULL, kh, pe & (WARP - 1));
+        K = pe < WARP ? (float)((pe - lane) * L) + kp : (float)((WARP - lane) * L);
+    }
+    const unsigned before = bc & ((1u << lane) - 1u);
+    const int src = before ? 31 - __clz(before) : 0;
+    if constexpr (W == 1) {
+        e.Rn = shfl_down(R, 1);
+        e.Kn = __shfl_down_sync(FULL, K, 1);
+        e.zt = mean(St + e.Rn, kt + e.Kn);  // (unused in the last lane)
+        const float zh = mean(R, K);        // of the lane's first node, if a run begins there
+        e.zr = __shfl_sync(FULL, C ? e.zt : zh, src);
+        if (lane == 0) e.zr = zh;
+        if (lane == WARP - 1) {
+            e.Rn = T{};
+            e.Kn = 0.f;
+        }
+    } else {
+        // Every warp forms the sum of a run that crosses warps in the same order (tail of
+        // the warp it begins in, plus the head sums folded from the right), so that all its
+        // nodes get the same bits.
+        const int lq = bc ? 31 - __clz(bc) : 0;
+        const T Rq = shfl_down(R, 1);
+        const float Kq = __shfl_down_sync(FULL, K, 1);
+        const T tS = pick(lane < WARP - 1, St + Rq, St);
+        const float tK = lane < WARP - 1 ? kt + Kq : kt;
+        if (lane == lq) {
+            xc->St[wi] = tS;
+            xc->Kt[wi] = tK;
+        }
+        if (lane == 0) {
+            xc->R[wi] = R;
+            xc->K[wi] = K;
+            xc->cut[wi] = bc != 0;
+        }
+        sync();
+        T Rin{}, rr{};               // the same for the next warp's first node; from warp q's
+        float Kin = 0.f, kk = 0.f;   // first node to the end of its run
+        float zprev = 0.f;           // value of the run that enters this warp
+        bool enters = true;          // which is not found yet
+#pragma unroll
+        for (int q = W - 1; q >= 0; --q) {
+            const bool c = xc->cut[q] != 0;
+            if (q < wi && enters && c) {
+                zprev = mean(xc->St[q] + rr, xc->Kt[q] + kk);
+                enters = false;
+            }
+            rr = xc->R[q] + pick(c, T{}, rr);
+            kk = xc->K[q] + (c ? 0.f : kk);
+            if (q == wi + 1) {
+                Rin = rr;
+                Kin = kk;
+            }
+        }
+        if (enters) zprev = mean(rr, kk);  // the chain's first run
+        if (pe == WARP) {
+            R = R + Rin;
+            K += Kin;
+        }
+        e.Rn = shfl_down(R, 1);
+        e.Kn = __shfl_down_sync(FULL, K, 1);
+        if (lane == WARP - 1) {
+            e.Rn = Rin;
+            e.Kn = Kin;
+        }
+        const bool out = lane == lq;  // its last run leaves the warp
+        e.zt = mean(pick(out, tS, St) + pick(out, Rin, e.Rn), (out ? tK : kt) + (out ? Kin : e.Kn));
+        e.zr = __shfl_sync(FULL, e.zt, src);
+        if (!before) e.zr = zprev;
+    }
+    return e;
 }
 
 // Lane slots of L nodes in shared memory, padded so that the lanes' 16-byte accesses do not
@@ -345,7 +455,7 @@ __device__ __forceinline__ int split_solve(const float *sc, float *sx, SplitX<W>
         if (lane > 0) re = rq;
         else if (W > 1 && wi > 0) re = xc->re[wi - 1];
     }
-    bool more = true;
+    auto sync = [&] { split_sync<W>(bar); };
     for (;;) {
         // ---- sums of the runs across lanes ----
         float Sh = 0.f, St = 0.f, b = 1.f;  // to the lane's first cut; after its last one
@@ -356,116 +466,12 @@ __device__ __forceinline__ int split_solve(const float *sc, float *sx, SplitX<W>
             b *= rj;
             St = fmaf(b, y[j], St);
         }
-        const float kh = C ? (float)(__clz(C) - (31 - L)) : (float)L;  // nodes of the head
-        const float kt = (float)(__ffs(C) - 1);                       // nodes after the last cut
-        // R, K: sum and count from the lane's first node to the end of its run
-        float R = Sh, K = kh;
-        int pe = lane;
-        if (bc != FULL) {
-            const unsigned ahead = bc >> lane;
-            pe = ahead ? lane + __ffs(ahead) - 1 : WARP;  // lane where that run ends
-#pragma unroll
-            for (int o = 1; o < WARP; o <<= 1) {
-                const float r2 = __shfl_down_sync(FULL, R, o);
-                if (lane + o < WARP && lane + o <= pe) R += r2;
-            }
-            const float kp = __shfl_sync(FULL, kh, pe & (WARP - 1));
-            K = pe < WARP ? (float)((pe - lane) * L) + kp : (float)((WARP - lane) * L);
-        }
-        float Rn, Kn;       // the same for the next lane's first node
-        float zprev = 0.f;  // value of the run that enters this warp
-        float zt;           // value of the run after the lane's last cut
-        if constexpr (W == 1) {
-            Rn = __shfl_down_sync(FULL, R, 1);
-            Kn = __shfl_down_sync(FULL, K, 1);
-            zt = mean_of(St + Rn, kt + Kn);  // (unused in the last lane)
-        } else {
-            // Every warp forms the sum of a run that crosses warps in the same order (tail of
-            // the warp it begins in, plus the head sums folded from the right), so that all its
-            // nodes get the same bits.
-            const int lq = bc ? 31 - __clz(bc) : 0;
-            const float Rq = __shfl_down_sync(FULL, R, 1), Kq = __shfl_down_sync(FULL, K, 1);
-            const float tS = lane < WARP - 1 ? St + Rq : St, tK = lane < WARP - 1 ? kt + Kq : kt;
-            if (lane == lq) {
-                xc->St[wi] = tS;
-                xc->Kt[wi] = tK;
-            }
-            if (lane == 0) {
-                xc->R[wi] = R;
-                xc->K[wi] = K;
-                xc->cut[wi] = bc != 0;
-            }
-            split_sync<W>(bar);
-            float Rin = 0.f, Kin = 0.f;  // the same for the next warp's first node
-            float rr = 0.f, kk = 0.f;    // from warp q's first node to the end of its run
-            bool enters = true;          // the run that enters warp wi is not found yet
-#pragma unroll
-            for (int q = W - 1; q >= 0; --q) {
-                const bool e = xc->cut[q] != 0;
-                if (q < wi && enters && e) {
-                    zprev = mean_of(xc->St[q] + rr, xc->Kt[q] + kk);
-                    enters = false;
-                }
-                rr = xc->R[q] + (e ? 0.f : rr);
-                kk = xc->K[q] + (e ? 0.f : kk);
-                if (q == wi + 1) {
-                    Rin = rr;
-                    Kin = kk;
-                }
-            }
-            if (enters) zprev = mean_of(rr, kk);  // the chain's first run
-            if (pe == WARP) {
-                R += Rin;
-                K += Kin;
-            }
-            Rn = __shfl_down_sync(FULL, R, 1);
-            Kn = __shfl_down_sync(FULL, K, 1);
-            if (lane == WARP - 1) {
-                Rn = Rin;
-                Kn = Kin;
-            }
-            const bool out = lane == lq;  // its last run leaves the warp
-            zt = mean_of((out ? tS : St) + (out ? Rin : Rn), (out ? tK : kt) + (out ? Kin : Kn));
-        }
-        // zr: value of the run at the lane's first node
-        const unsigned before = bc & ((1u << lane) - 1u);
-        float zr;
-        if constexpr (W == 1) {
-            const float zh = mean_of(R, K);  // of the lane's first node, if a run begins there
-            zr = __shfl_sync(FULL, C ? zt : zh, before ? 31 - __clz(before) : 0);
-            if (lane == 0) zr = zh;
-        } else {
-            zr = __shfl_sync(FULL, zt, before ? 31 - __clz(before) : 0);
-            if (!before) zr = zprev;
-        }
+        const RunEnds<float> run = join_runs<L, W>(
+            Sh, St, C, bc, lane, wi, &xc->run, [](float s, float k) { return mean_of(s, k); }, sync);
+        float zr = run.zr;
 
         // ---- mean of every run that begins in the lane, at its first node ----
-        float s = Rn, k = Kn;
-        if (W == 1 && lane == WARP - 1) s = k = 0.f;
-        if (!more) {  // no cut in the last round: the runs are the solution
-#pragma unroll
-            for (int j = L - 1; j >= 0; --j) {
-                const float rj = keep(j);
-                s = fmaf(s, rj, y[j]);
-                k = fmaf(k, rj, 1.f);
-                z[j] = mean_of(s, k);
-            }
-            const unsigned LC = C & (0u - C);
-            float4 *xp = reinterpret_cast<float4 *>(sx + (wi * WARP + lane) * LP);
-#pragma unroll
-            for (int q = 0; q < L / 4; ++q) {
-                float v[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int j = 4 * q + e;
-                    if (j > 0 && (C & (1u << (L - j)))) zr = z[j];
-                    if (j > 0 && (LC & (1u << (L - j)))) zr = zt;  // the bits other lanes have
-                    v[e] = zr;
-                }
-                xp[q] = make_float4(v[0], v[1], v[2], v[3]);
-            }
-            return SPLIT_DONE;
-        }
+        float s = run.Rn, k = run.Kn;
 #pragma unroll
         for (int j = L - 1; j >= 0; --j) {
             const float rj = keep(j);
@@ -611,7 +617,7 @@ __device__ __forceinline__ int split_solve(const float *sc, float *sx, SplitX<W>
         // ---- new cuts: fold their flows into the values ----
         const unsigned upf = fresh & low;
         const unsigned bf = __ballot_sync(FULL, fresh != 0);
-        more = bf != 0;
+        bool more = bf != 0;
         bc |= bf;
         // the flow of a cut after the lane's last node (UNI: 2 with its half, 1 without)
         float ue;
@@ -659,33 +665,67 @@ __device__ __forceinline__ int split_solve(const float *sc, float *sx, SplitX<W>
         }
         if (STOP && halt) return SPLIT_STOPPED;
         if (hv) return SPLIT_FALLBACK;
-        if constexpr (UNI) {
-            if (!more) {  // the values as they came, with the flows of all cuts
-                const unsigned ends = last >= L ? 0u : ML >> max(0, min(31, last));
-                const unsigned F = C & ~ends;  // cuts that carry a flow
-                float u = (F & 1u) ? ((UP & 1u) ? lamw : -lamw) : 0.f;
-                float ul = __shfl_up_sync(FULL, u, 1);
-                if (lane == 0) ul = 0.f;
-                if constexpr (W > 1) {
-                    if (lane == WARP - 1) xc->u2[wi] = u;
-                    split_sync<W>(bar);
-                    if (lane == 0 && wi > 0) ul = xc->u2[wi - 1];
-                }
+        if (!more) break;  // the runs are the solution
+    }
+
+    // ---- values of the runs: sums in two floats (in one, x was further off than the dynamic
+    // program's: 4.7e-8 against 3.2e-8 for 512 x 256, now 2.3e-8) ----
+    {
+        if constexpr (UNI) {  // of the values as they came, with the flows of all cuts
+            const unsigned ends = last >= L ? 0u : ML >> max(0, min(31, last));
+            const unsigned F = C & ~ends;  // cuts that carry a flow
+            float u = (F & 1u) ? ((UP & 1u) ? lamw : -lamw) : 0.f;
+            float ul = __shfl_up_sync(FULL, u, 1);
+            if (lane == 0) ul = 0.f;
+            if constexpr (W > 1) {
+                if (lane == WARP - 1) xc->u2[wi] = u;
+                sync();
+                if (lane == 0 && wi > 0) ul = xc->u2[wi - 1];
+            }
 #pragma unroll
-                for (int q = 0; q < L / 4; ++q) {
-                    const float4 t = yp[q];
-                    const float v[4] = {t.x, t.y, t.z, t.w};
+            for (int q = 0; q < L / 4; ++q) {
+                const float4 t = yp[q];
+                const float v[4] = {t.x, t.y, t.z, t.w};
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const unsigned bit = 1u << (L - 1 - (4 * q + e));
-                        u = (F & bit) ? ((UP & bit) ? lamw : -lamw) : 0.f;
-                        y[4 * q + e] = v[e] + (u - ul);  // equal flows cancel exactly
-                        ul = u;
-                    }
+                for (int e = 0; e < 4; ++e) {
+                    const unsigned bit = 1u << (L - 1 - (4 * q + e));
+                    u = (F & bit) ? ((UP & bit) ? lamw : -lamw) : 0.f;
+                    y[4 * q + e] = v[e] + (u - ul);  // equal flows cancel exactly
+                    ul = u;
                 }
             }
         }
+        Sum2 Sh{0.f, 0.f}, St{0.f, 0.f};
+        float k = 0.f, b = 1.f;
+#pragma unroll
+        for (int j = L - 1; j >= 0; --j) {
+            const float rj = keep(j);
+            const Sum2 before{Sh.hi * rj, Sh.lo * rj};
+            Sh = before + Sum2{y[j], 0.f};
+            k = fmaf(k, rj, 1.f);
+            z[j] = mean_of(Sh, k);  // of a run that ends in the lane
+            b *= rj;
+            St = pick(b != 0.f, Sh, St);
+        }
+        const RunEnds<Sum2> run = join_runs<L, W>(
+            Sh, St, C, bc, lane, wi, &xc->sum, [](Sum2 s, float n) { return mean_of(s, n); }, sync);
+        float zr = run.zr;
+        const unsigned LC = C & (0u - C);
+        float4 *xp = reinterpret_cast<float4 *>(sx + (wi * WARP + lane) * LP);
+#pragma unroll
+        for (int q = 0; q < L / 4; ++q) {
+            float v[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int j = 4 * q + e;
+                if (j > 0 && (C & (1u << (L - j)))) zr = z[j];
+                if (j > 0 && (LC & (1u << (L - j)))) zr = run.zt;  // the bits other lanes have
+                v[e] = zr;
+            }
+            xp[q] = make_float4(v[0], v[1], v[2], v[3]);
+        }
     }
+    return SPLIT_DONE;
 }
 
 struct UnitStride {  // of rows: known at compile time

@@ -18,7 +18,8 @@ tv_status launch_w(SRC src, int lmax, int nch, WsHeader *hdr, cudaStream_t s)
     tv_status st = TV_OK;
     // Beyond what needs no opt-in (with the exchange; a call less, 1 us). The limit is the kernel's,
     // not the launch's: always the most, so that no other thread's call lowers it meanwhile.
-    if (smem > 47 * 1024)
+    static_assert(sizeof(SplitX<W>) * (split_threads<W>() / (WARP * W)) <= 1536, "static shared memory");
+    if (smem > 46 * 1024)
         st = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)split_smem_most<W>()),
                         "cudaFuncSetAttribute");
