@@ -25,8 +25,9 @@
 //
 // Solutions are sums of the values of a run over its length: all nodes of a run are bitwise
 // equal, and the rounding is that of one mean. The folded flows cost eps * |u| per run, so a
-// chain that is to be cut at a flow above 16 max |y|, or whose values are not finite, goes to the warp's dynamic program
-// (coop_solve_chain, records and reserve in the workspace) instead.
+// chain that is to be cut at a flow above 16 max |y|, or whose values are not finite or near the
+// ends of FP32's range, goes to the warp's dynamic program (coop_solve_chain, records and reserve
+// in the workspace) instead.
 #pragma once
 #include "tv2d_common.cuh"
 #include "tv2d_gap.cuh"
@@ -37,6 +38,9 @@ namespace tvk {
 constexpr int kSplitMaxLen = 4096;     // nodes of the longest chain (4 warps x 32 lanes x 32)
 constexpr float kSplitHeavy = 16.f;
 constexpr float kSplitTiny = 1e-37f;  // weights up to here decouple
+// Largest |value| of a chain that is split. Above, the sums of 4096 values, each with two flows of
+// up to 16 times as much folded in, could overflow; below, weights that decouple would count.
+constexpr float kSplitMost = 1e32f, kSplitLeast = 1e-28f;
 
 // What a chain's nodes are made of. PLAIN: c = y. INIT, ROW, COL: the set-up of the phases
 // of eq. pd (x^0 rows, primal rows, dual columns).
@@ -415,8 +419,9 @@ __device__ __forceinline__ int split_solve(const float *sc, float *sx, SplitX<W>
 #pragma unroll
         for (int q = 0; q < W; ++q) ab = max(ab, xc->amax[q]);
     }
-    if (ab >= 0x7f800000u) return SPLIT_FALLBACK;  // not finite: as the dynamic program has it
     const float amax = __uint_as_float(ab);
+    // not finite, or beyond what the sums hold: as the dynamic program has it
+    if (!(amax <= kSplitMost && (amax >= kSplitLeast || amax == 0.f))) return SPLIT_FALLBACK;
     unsigned H = 0;   // edges whose flow would swamp the values
     unsigned UP = 0;  // UNI: cuts with flow +w
     if constexpr (UNI) {
