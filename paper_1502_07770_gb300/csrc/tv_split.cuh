@@ -25,8 +25,8 @@
 //
 // Solutions are sums of the values of a run over its length: all nodes of a run are bitwise
 // equal, and the rounding is that of one mean. The folded flows cost eps * |u| per run, so a
-// chain that is to be cut at a flow above 16 max |y|, or whose values are not finite or near the
-// ends of FP32's range, goes to the warp's dynamic program (coop_solve_chain, records and reserve
+// chain that is to be cut at a flow above 16 max |y|, that has a NaN weight, or whose values are
+// not finite or near the ends of FP32's range, goes to the warp's dynamic program (coop_solve_chain, records and reserve
 // in the workspace) instead.
 #pragma once
 #include "tv2d_common.cuh"
@@ -404,6 +404,10 @@ __device__ __forceinline__ int split_solve(const float *sc, float *sx, SplitX<W>
             w[4 * q + 2] = e.z;
             w[4 * q + 3] = e.w;
         }
+        float sum = 0.f;  // NaN if a weight is (weights are >= 0)
+#pragma unroll
+        for (int j = 0; j < L; ++j) sum += w[j];
+        if (sum != sum) ab = 0x7fffffffu;
 #pragma unroll
         for (int j = 0; j < L; ++j) {
             const bool cut = !(w[j] > kSplitTiny);

@@ -33,3 +33,29 @@ def test_scales(scale, edges):
                                      lam=float(lam)).cpu().numpy().T
         for got in (x, xc):
             assert np.abs(got / scale - ref / scale).max() <= TOL, n
+
+
+@pytest.mark.parametrize("n", [48, 300, 1024, 1500, 2600])
+def test_nan_weights_go_to_the_dynamic_program(n):
+    """A NaN weight is no cut: its chain gives what the warp's dynamic program (solve mode 0)
+    makes of it, bit for bit; the entry at a chain's last node is not read. The other chains are
+    untouched."""
+    y = synth.chain_batch(9, n, seed0=n)
+    w = np.full(y.shape, 0.2, np.float32)
+    clean = _lib.chain_prox(_gpu(y), _gpu(w)).cpu().numpy()
+    w[3, n // 3] = w[7, 0] = np.nan
+    w[5, -1] = np.nan
+    lib = _lib.load()
+    try:
+        _lib._check(lib.tv_set_coop_split(0))
+        want = _lib.chain_prox(_gpu(y), _gpu(w)).cpu().numpy()
+        wantc = _lib.chain_prox_columns(_gpu(y.T), _gpu(w.T)).cpu().numpy().T
+    finally:
+        _lib._check(lib.tv_set_coop_split(1))
+    x = _lib.chain_prox(_gpu(y), _gpu(w)).cpu().numpy()
+    xc = _lib.chain_prox_columns(_gpu(y.T), _gpu(w.T)).cpu().numpy().T
+    for k in (3, 7):
+        assert np.array_equal(x[k], want[k], equal_nan=True)
+        assert np.array_equal(xc[k], wantc[k], equal_nan=True)
+    rest = [k for k in range(9) if k not in (3, 7)]
+    assert np.array_equal(x[rest], clean[rest]) and np.array_equal(xc[rest], clean[rest])
