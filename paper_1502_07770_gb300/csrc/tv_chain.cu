@@ -809,7 +809,7 @@ tv_status tv_chain_solve(const float *d_y, const float *d_w, float lambda,
     if (st != TV_OK) return st;
     const bool vec_w = vec_ok(d_offsets, max_len, d_y, d_w, d_x);
     if (split_takes(max_len, num_chains,
-                    split_max_chains(max_len, false, vec_w, d_w != nullptr))) {
+                    split_max_chains(max_len, false, vec_w, d_w != nullptr, d_offsets != nullptr))) {
         SplitSrc src{};
         src.v.mode = SPLIT_PLAIN;
         src.v.p0 = d_y;

@@ -45,8 +45,26 @@ inline bool split_takes(long long max_len, long long chains, long long max_chain
 // Chains of under 64 nodes leave most of a warp idle: at 16 nodes 16.6 / 14.7 (the
 // warp-per-chain kernel) for 4096 chains, 13.7 / 13.8 for 2048. Up to 2048 chains the alternative is
 // another warp-per-chain kernel, which is never faster.
-inline long long split_max_chains(long long len, bool cols, bool vec, bool has_w)
+//
+// CSR batches (`csr`; `len` is their longest chain): a short chain still takes its warps, and one
+// of more than 256 nodes is solved at the longest chain's nodes a lane, while the thread kernels
+// take the time of the longest chain or that of all nodes. The line is the lowest crossover over
+// lengths spread evenly up to `len`, all near it, or far below it but for one (us, splitting /
+// thread kernel): 260 nodes 38 / 42 for 5000 chains and 73 / 54 for 10000, 400 nodes 60 / 57 for
+// 5000, 600 nodes 61 / 80 and 127 / 108, 1000 nodes 130 / 126 for 7000 and 196 / 182 for 10000,
+// 1600 nodes 240 / 286 for 10000 and 384 / 292 for 14000, 2400 nodes 335 / 416 and 485 / 443, 4096
+// nodes (1200 on average) 360 / 480 and 523 / 487. With a weight per edge, where the thread
+// kernels are slower: 150 nodes 73 / 87 for 20000 and 163 / 119 for 50000, 400 nodes 231 / 220
+// for 20000, 600 nodes 341 / 330 for 28000, 1000 nodes 311 / 536 for 20000, 1600 nodes 484 / 617
+// and 732 / 646 for 28000, 4096 nodes (1200 on average) 702 / 995 and 1051 / 953 for 28000.
+// (Limits from rows of the longest length sent 65536 chains of up to 900 nodes, 400 on average,
+// here: 1258 us for 494, and a million of 20 nodes but for one of 700: 2455 for 319.)
+inline long long split_max_chains(long long len, bool cols, bool vec, bool has_w, bool csr = false)
 {
+    if (csr && len >= 64) {
+        if (has_w) return len <= 256 ? 120 * len : std::min(47 * len, 22000LL);
+        return std::max(4096LL, len <= 256 ? 23 * len : len <= 1024 ? 9 * len : std::min(2 * len + 7000, 13500LL));
+    }
     if (len < 64) return len < 32 && !cols ? 2048 : kCoopMaxChainsDefault;
     if (cols) return len < 256 ? 16384 : INT64_MAX;
     if (vec) return std::max(2048LL, std::min(28 * len, has_w ? 6144LL : 8192LL));
