@@ -13,7 +13,7 @@
 // copies x_{i+1} into x_i whenever the clip is inactive, so fused neighbours are
 // bitwise equal.
 //
-// Chains of at most kSplitMaxLen nodes (run_means_kernel): the chain lies in the registers of
+// Chains of at most kSplitMaxLen nodes (run_means_kernel; not large batches of short ones): the chain lies in the registers of
 // one warp (2 or 4 for more than 1024 nodes), L consecutive nodes a lane, loaded and stored
 // through padded slots in shared memory so that global accesses are whole lines. Run sums are
 // walks that restart behind a run's last node, joined across lanes by one segmented scan
@@ -21,7 +21,7 @@
 // and one or two writes bound the kernel. 4096 x 1024 with both gradients: 31 -> 14.7 us (4.6
 // TB/s) against the step-wise kernel; 16384 x 1024 50.6 us (5.3 TB/s).
 //
-// Longer chains (chain_vjp_kernel): one warp per chain, 32 nodes per step: a forward segmented
+// Others (chain_vjp_kernel): one warp per chain, 32 nodes per step: a forward segmented
 // scan of (sum, count) with a carry across steps yields each segment's mean at its last node;
 // a reverse segmented scan spreads it over the segment. The loads of kGradUnroll steps are
 // issued together before their scans run one after another: with one step's loads in flight
@@ -414,9 +414,21 @@ tv_status launch_run_classes(const GradArgs &a, bool vec, WsHeader *hdr, cudaStr
     return st;
 }
 
-}  // namespace
-
-namespace {
+// Largest batch for the register kernel. A chain takes a warp (and its shared memory) however
+// short it is, and a CSR batch a launch over all chains for every class of lengths, so the
+// step-wise kernel is the faster one for large batches of short chains. Measured (us, step-wise /
+// register kernel; chain_prox_backward called from Python, about 20 us of which are the call):
+//  - rows: 20 nodes 21 / 24 for 20000 chains and 314 / 807 for a million, 60 nodes 22 / 24 for
+//    20000 and 48 / 82 for 100000, 150 nodes 27 / 25 and 91 / 93, 400 nodes 49 / 35 and 194 / 146;
+//  - CSR, lengths spread evenly up to 300 nodes 32 / 32 for 20000 chains and 106 / 119 for 100000,
+//    800 nodes 24 / 24 for 3000 and 60 / 69 for 20000, 1600 nodes 35 / 31 and 127 / 131 (142 / 180
+//    with grad_w), 4000 nodes 112 / 56 and 630 / 246; short chains but for one of 4096 nodes
+//    67 / 58 for 20000 and 98 / 218 for 100000.
+long long runs_max_chains(long long max_len, bool csr)
+{
+    if (!csr) return max_len < 128 ? 4096 : INT64_MAX;
+    return max_len <= 1024 ? 2048 : max_len <= 2048 ? 4096 : 24000;
+}
 
 tv_status solve_backward(const float *d_x, const float *d_grad_x, const int64_t *d_offsets,
                          int64_t num_chains, int64_t max_len, float *d_grad_y, float *d_grad_w,
@@ -446,7 +458,8 @@ tv_status solve_backward(const float *d_x, const float *d_grad_x, const int64_t 
     cudaStream_t s = (cudaStream_t)stream;
     WsHeader *hdr = static_cast<WsHeader *>(d_workspace);
     tv_status st = TV_OK;
-    const bool runs = max_len >= 1 && max_len <= kSplitMaxLen;
+    const bool runs = max_len >= 1 && max_len <= kSplitMaxLen &&
+                      num_chains <= runs_max_chains(max_len, d_offsets != nullptr);
     if (d_offsets || !runs) {
         st = check_cuda(cudaMemsetAsync(hdr, 0, sizeof(WsHeader), s), "memset header");
         if (st != TV_OK) return st;
