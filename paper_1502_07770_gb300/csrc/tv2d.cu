@@ -642,9 +642,17 @@ SplitSrc split_src(SplitMode mode, const float *img, const float *w, float lam, 
     return src;
 }
 
+// Rows: the phases' thread kernel is slower than tv_chain_solve's, so the splitting kernel is the
+// faster one for larger batches (ms, four iterations, thread / splitting kernel: 16384 x 1024
+// 8.9 / 5.4, 65536 x 1024 26.5 / 20.9, 32768 x 512 9.8 / 8.2, 30000 x 200 6.6 / 6.7; with edge
+// weights 65536 x 512 25.6 / 22.4, 30000 x 200 9.6 / 9.2).
 bool split_rows(long long H, long long W, const float *wh)
 {
-    return split_takes(W, H, split_max_chains(W, false, false, wh != nullptr));
+    long long most = INT64_MAX;
+    if (W < 64) most = W < 32 ? 2048 : kCoopMaxChainsDefault;
+    else if (wh) most = W < 192 ? 150 * W : INT64_MAX;
+    else if (W < 640) most = W < 400 ? std::max(2048LL, 23 * W) : 32768;
+    return split_takes(W, H, most);
 }
 bool split_cols(long long H, long long W, const float *wv)
 {

@@ -30,21 +30,26 @@ inline bool split_takes(long long max_len, long long chains, long long max_chain
 //    about the same for any short chain, the thread kernel in proportion to its length, so the
 //    line goes with the length: 64 nodes 17 / 18 for 2048 chains and 21 / 16 for 4096, 128 nodes
 //    22 / 22 for 4096 and 28 / 23 for 6144, 192 nodes 25 / 29 and 32 / 30 for 6000, 256 nodes
-//    32 / 37 for 6000 and 40 / 37 for 8192. Long ones: at 512 nodes 54 / 64 for 8192 and 95 / 91
-//    for 16384, at 1024 nodes 91 / 122 and 180 / 177, at 4096 nodes 441 / 475 and 853 / 675. With
-//    a weight per edge as above up to 256 nodes, then at 1024 nodes 86 / 126 for 6000 and
-//    129 / 129 for 8192.
+//    35 / 39 for 6000, 300 nodes 40 / 44 for 6000 and 50 / 44 for 8192, 400 nodes 46 / 54 and
+//    58 / 54. Long ones: at 512 nodes 57 / 66 for 8192 and 95 / 91 for 16384, at 1024 nodes
+//    101 / 127 and 180 / 177, at 4096 nodes 470 / 484 and 853 / 675. With a weight per edge as
+//    above up to 256 nodes, then at 1024 nodes 92 / 129 for 6000 and 129 / 129 for 8192.
 //  - other rows, one weight: 130 nodes 24 / 23 for 3072 chains, 201 nodes 27 / 31 for 4096 and
-//    36 / 35 for 6144, 257 nodes 41 / 41 for 6144, 385 nodes 48 / 59 and 62 / 60 for 8192, 514
-//    nodes 239 / 266 for 32768 and 469 / 449 for 65536, 770 nodes 636 / 708 for 65536;
+//    36 / 35 for 6144, 257 nodes 45 / 44 for 6000, 385 nodes 52 / 61 for 6000 and 66 / 62 for
+//    8192, 514 nodes 155 / 190 for 20000 and 469 / 449 for 65536, 770 nodes 563 / 582 for 50000.
+//    Just above what one warp or two hold the kernel pays for half-empty warps: 1027 nodes
+//    126 / 145 for 6000, 168 / 152 for 8192 and 984 / 752 for 50000, 2050 nodes 245 / 278 and
+//    328 / 292; 3001 nodes 870 / 1170 for 20000.
 //  - other rows with a weight per edge (the thread kernel stages those worst): 65 nodes 31 / 39
 //    for 8192 and 51 / 41 for 16384, 130 nodes 66 / 78 for 16384 and 120 / 91 for 32768, 201
-//    nodes 248 / 266 for 65536, 1023 nodes 61 / 167 for 4096;
+//    nodes 86 / 122 for 20000 and 198 / 175 for 50000, 257 nodes 104 / 156 and 246 / 213, 385
+//    nodes 313 / 313 for 50000 and 916 / 881 for 150000, 1023 nodes 65 / 167 for 4096;
 //  - columns (the thread kernel runs one thread per chain): at 1024 nodes 57 / 889 for 4096 and
-//    650 / 1119 for 65536, at 100 nodes 56 / 93 for 16384 and 195 / 114 for 65536.
+//    650 / 1119 for 65536, at 300 nodes 180 / 258 for 40000 and 638 / 554 for 150000, at 100
+//    nodes 56 / 93 for 16384 and 195 / 114 for 65536.
 // Chains of under 64 nodes leave most of a warp idle: at 16 nodes 16.6 / 14.7 (the
-// warp-per-chain kernel) for 4096 chains, 13.7 / 13.8 for 2048. Up to 2048 chains the alternative is
-// another warp-per-chain kernel, which is never faster.
+// warp-per-chain kernel; columns 20.4 / 16.3) for 4096 chains, 13.7 / 13.8 for 2048. Up to 2048
+// chains the alternative is another warp-per-chain kernel, which is never faster.
 //
 // CSR batches (`csr`; `len` is their longest chain): a short chain still takes its warps, and one
 // of more than 256 nodes is solved at the longest chain's nodes a lane, while the thread kernels
@@ -65,11 +70,12 @@ inline long long split_max_chains(long long len, bool cols, bool vec, bool has_w
         if (has_w) return len <= 256 ? 120 * len : std::min(47 * len, 22000LL);
         return std::max(4096LL, len <= 256 ? 23 * len : len <= 1024 ? 9 * len : std::min(2 * len + 7000, 13500LL));
     }
-    if (len < 64) return len < 32 && !cols ? 2048 : kCoopMaxChainsDefault;
-    if (cols) return len < 256 ? 16384 : INT64_MAX;
-    if (vec) return std::max(2048LL, std::min(28 * len, has_w ? 6144LL : 8192LL));
-    if (has_w) return len < 192 ? 150 * len : INT64_MAX;
-    if (len < 400) return std::max(2048LL, 23 * len);
+    if (len < 64) return len < 32 ? 2048 : kCoopMaxChainsDefault;
+    if (cols) return len < 256 ? 16384 : len < 512 ? 250 * len : INT64_MAX;
+    if (vec) return std::max(2048LL, std::min(28 * len, has_w ? 6144LL : len < 512 ? 6800LL : 8192LL));
+    if (has_w) return len < 384 ? 150 * len : INT64_MAX;
+    if (len < 400) return std::max(2048LL, std::min(23 * len, 7000LL));
+    if ((len > 1024 && len <= 1536) || (len > 2048 && len <= 2560)) return 7000;
     return len < 640 ? 32768 : INT64_MAX;
 }
 
