@@ -851,6 +851,33 @@ void plan_split(const tv_image_desc *d, int n, Plan &plan)
     }
 }
 
+// The splitting kernel's first phases read the caller's duals in place. One that overlaps the
+// output x of an image, which the initial rows write, is copied into the image's own y instead.
+tv_status copy_overlapped_duals(const tv_image_desc *d, int n, Plan &plan, cudaStream_t s)
+{
+    typedef std::pair<uintptr_t, uintptr_t> Range;
+    auto range = [&](const float *p, int m) {
+        return Range((uintptr_t)p, (uintptr_t)(p + (size_t)d[m].H * d[m].W));
+    };
+    if (std::none_of(d, d + n, [](const tv_image_desc &q) { return q.y0 != nullptr; })) return TV_OK;
+    std::vector<Range> xs;
+    for (int m = 0; m < n; ++m) xs.push_back(range(d[m].x, m));
+    std::sort(xs.begin(), xs.end());
+    for (size_t q = 1; q < xs.size(); ++q) xs[q].second = std::max(xs[q].second, xs[q - 1].second);
+    for (int m = 0; m < n; ++m) {
+        if (!d[m].y0) continue;
+        const Range y = range(d[m].y0, m);
+        // outputs that begin before the dual ends, and how far they reach
+        const auto after = std::lower_bound(xs.begin(), xs.end(), Range(y.second, 0));
+        if (after == xs.begin() || (after - 1)->second <= y.first) continue;
+        const tv_status st = check_cuda(cudaMemcpyAsync(plan.imgs[m].y, d[m].y0, y.second - y.first,
+                                                        cudaMemcpyDeviceToDevice, s), "copy y0");
+        if (st != TV_OK) return st;
+        plan.imgs[m].y0 = plan.imgs[m].y;
+    }
+    return TV_OK;
+}
+
 int g_batched_wpb = 4;  // warps per block of the phase kernels (tunable)
 
 template <int PHASE>
@@ -1118,6 +1145,7 @@ tv_status tv2d_denoise_batched(const tv_image_desc *imgs, int n_imgs, int max_it
     build_plan(imgs, n_imgs, plan);
     cudaStream_t s = (cudaStream_t)stream;
     tv_status st;
+    if (plan.split && (st = copy_overlapped_duals(imgs, n_imgs, plan, s)) != TV_OK) return st;
     if ((st = upload(ws.imgs, plan.imgs, s)) != TV_OK) return st;
     if (!plan.split) {
         if ((st = upload(ws.cols, plan.cols, s)) != TV_OK) return st;
