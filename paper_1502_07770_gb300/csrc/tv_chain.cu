@@ -43,6 +43,25 @@ int sm_count_current()
     return sms > 0 ? sms : 148;
 }
 
+// (cuCtxGetId through the runtime's driver entry point, so that the library needs no link to
+// the driver library)
+bool current_context_id(unsigned long long *id)
+{
+    typedef int (*CtxGetId)(void *, unsigned long long *);
+    static CtxGetId fn = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) !=
+                cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            (void)cudaGetLastError();
+            return (CtxGetId) nullptr;
+        }
+        return (CtxGetId)f;
+    }();
+    return fn != nullptr && fn(nullptr, id) == 0;
+}
+
 // ---------------------------------------------------------- launch accounting --
 static std::atomic<long long> g_launches{0};
 static std::mutex g_prof_mu;
@@ -990,26 +1009,6 @@ struct NoAllocSlot {
     unsigned long long ctx;  // id of the context the address was looked up in
 };
 NoAllocSlot g_noalloc[kNoAllocMaxDevices];
-
-// Unique id of the current context (cuCtxGetId through the runtime's driver entry
-// point, so that the library needs no link to the driver library); false if there is
-// no current context or the driver has no such call.
-bool current_context_id(unsigned long long *id)
-{
-    typedef int (*CtxGetId)(void *, unsigned long long *);
-    static CtxGetId fn = [] {
-        void *f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) !=
-                cudaSuccess ||
-            q != cudaDriverEntryPointSuccess) {
-            (void)cudaGetLastError();
-            return (CtxGetId) nullptr;
-        }
-        return (CtxGetId)f;
-    }();
-    return fn != nullptr && fn(nullptr, id) == 0;
-}
 
 tv_status noalloc_scratch(void **out)
 {

@@ -42,4 +42,8 @@ struct Shape {
 Shape batch_shape(long long warps, int sm_count);
 int sm_count_current();
 
+// Unique id of the current context; false if there is no current context or the driver cannot
+// tell.
+bool current_context_id(unsigned long long *id);
+
 }  // namespace tvh

@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 
 #include "tv_launch.cuh"
+#include "tv_once.h"
 
 using namespace tvk;
 using namespace tvh;
@@ -542,6 +543,23 @@ __global__ void __launch_bounds__(RED_E * RED_G)
     }
 }
 
+// A kernel's opt-in to `smem` bytes of shared memory per block, at the largest carve-out so that
+// several blocks fit an SM.
+template <class K>
+tv_status smem_opt_in(K kern, size_t smem, OncePerContext &once)
+{
+    return once.run(current_context_id, [&] {
+        tv_status st = check_cuda(
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+            "cudaFuncSetAttribute");
+        if (st == TV_OK)
+            st = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                                 (int)cudaSharedmemCarveoutMaxShared),
+                            "cudaFuncSetAttribute");
+        return st;
+    });
+}
+
 // Blocks of the weight-gradient kernel for a B x H x W batch.
 long long wgrad_blocks(int B, int H, int W)
 {
@@ -556,16 +574,11 @@ tv_status launch_conv(const __nv_bfloat16 *X, int B, int H, int W, const __nv_bf
 {
     auto kern = conv3x3_persist<CIN, COUT, MODE>;
     constexpr size_t smem = conv_persist_smem<CIN, COUT>();
-    static int per_sm = 0;  // resident blocks per SM (occupancy, computed once per kernel)
+    static OncePerContext once;
+    tv_status st0 = smem_opt_in(kern, smem, once);
+    if (st0 != TV_OK) return st0;
+    static std::atomic<int> per_sm{0};  // resident blocks per SM (occupancy, computed once per kernel)
     if (per_sm == 0) {
-        tv_status st0 = check_cuda(
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-            "cudaFuncSetAttribute");
-        if (st0 != TV_OK) return st0;
-        st0 = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                              (int)cudaSharedmemCarveoutMaxShared),
-                         "cudaFuncSetAttribute");
-        if (st0 != TV_OK) return st0;
         int b = 0;
         st0 = check_cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, NTHR, smem),
                          "occupancy");
@@ -599,18 +612,9 @@ tv_status launch_wgrad(const void *X, const void *dY, int B, int H, int W, float
 {
     using G = Wgrad<CIN, COUT>;
     auto kern = conv3x3_wgrad<CIN, COUT>;
-    static bool attr = false;
-    if (!attr) {
-        tv_status st0 = check_cuda(
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem),
-            "cudaFuncSetAttribute");
-        if (st0 != TV_OK) return st0;
-        st0 = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                              (int)cudaSharedmemCarveoutMaxShared),
-                         "cudaFuncSetAttribute");
-        if (st0 != TV_OK) return st0;
-        attr = true;
-    }
+    static OncePerContext once;
+    const tv_status st0 = smem_opt_in(kern, G::smem, once);
+    if (st0 != TV_OK) return st0;
     const long long blocks = wgrad_blocks(B, H, W);
     kern<<<(unsigned)blocks, NTHR, G::smem, s>>>(static_cast<const __nv_bfloat16 *>(X),
                                                  static_cast<const __nv_bfloat16 *>(dY), B, H, W, P);
@@ -1974,25 +1978,16 @@ tv_status launch_conv_tw(const __nv_bfloat16 *X, int B, int H, int W, const __nv
     }
     auto kern = conv3x3_tw<CIN, COUT, IO, TR>;
     constexpr size_t smem = conv_tw_smem<CIN, COUT, IO>();
-    static bool attr = false;
-    if (!attr) {
-        tv_status st0 = check_cuda(
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-            "cudaFuncSetAttribute");
-        if (st0 != TV_OK) return st0;
-        st0 = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                              (int)cudaSharedmemCarveoutMaxShared),
-                         "cudaFuncSetAttribute");
-        if (st0 != TV_OK) return st0;
-        attr = true;
-    }
+    static OncePerContext once;
+    tv_status st0 = smem_opt_in(kern, smem, once);
+    if (st0 != TV_OK) return st0;
     // resident blocks per SM from registers, shared memory and TMEM columns (the occupancy
     // query reports one block for a kernel that allocates TMEM, whatever it allocates)
-    static int per_sm = 0;
+    static std::atomic<int> per_sm{0};
     if (per_sm == 0) {
         cudaFuncAttributes fa;
         int dev = 0, smem_sm = 0, regs_sm = 0;
-        tv_status st0 = check_cuda(cudaFuncGetAttributes(&fa, kern), "cudaFuncGetAttributes");
+        st0 = check_cuda(cudaFuncGetAttributes(&fa, kern), "cudaFuncGetAttributes");
         if (st0 == TV_OK) st0 = check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
         if (st0 == TV_OK)
             st0 = check_cuda(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev),
@@ -2038,18 +2033,9 @@ tv_status launch_wgrad_tc(const __nv_bfloat16 *X, const __nv_bfloat16 *dY, int B
         set_error("weight gradient: cuTensorMapEncodeTiled rejected the activation layout");
         return TV_ERR_INVALID;
     }
-    static bool attr = false;
-    if (!attr) {
-        tv_status st0 = check_cuda(
-            cudaFuncSetAttribute(wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WT_SMEM),
-            "cudaFuncSetAttribute");
-        if (st0 != TV_OK) return st0;
-        st0 = check_cuda(cudaFuncSetAttribute(wgrad_tc, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                              (int)cudaSharedmemCarveoutMaxShared),
-                         "cudaFuncSetAttribute");
-        if (st0 != TV_OK) return st0;
-        attr = true;
-    }
+    static OncePerContext once;
+    const tv_status st0 = smem_opt_in(wgrad_tc, WT_SMEM, once);
+    if (st0 != TV_OK) return st0;
     // two blocks per SM (shared memory and TMEM), no more than steps or rows of P
     const long long steps = (long long)B * ((W + TC_M - 1) / TC_M) * ((H + 1) / 2);
     const long long blocks = std::min(std::min(2LL * sm_count_current(), steps), wgrad_blocks(B, H, W));
@@ -2069,22 +2055,13 @@ tv_status launch_conv_tc(const __nv_bfloat16 *X, int B, int H, int W, const __nv
 {
     auto kern = conv3x3_tc<CIN, COUT>;
     constexpr size_t smem = conv_tc_smem<CIN, COUT>();
-    static int per_sm = 0;
-    if (per_sm == 0) {
-        tv_status st0 = check_cuda(
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-            "cudaFuncSetAttribute");
-        if (st0 != TV_OK) return st0;
-        // the whole unified memory as shared memory, so that several blocks fit per SM
-        st0 = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                              (int)cudaSharedmemCarveoutMaxShared),
-                         "cudaFuncSetAttribute");
-        if (st0 != TV_OK) return st0;
-        // blocks per SM from the shared memory (the occupancy query does not see that
-        // a block holds only 64 of the 512 TMEM columns); at most 4, 256 columns
-        const int b = (int)((227 * 1024) / (smem + 1024));
-        per_sm = b < 1 ? 1 : (b > 4 ? 4 : b);
-    }
+    static OncePerContext once;
+    const tv_status st0 = smem_opt_in(kern, smem, once);
+    if (st0 != TV_OK) return st0;
+    // blocks per SM from the shared memory (the occupancy query does not see that
+    // a block holds only 64 of the 512 TMEM columns); at most 4, 256 columns
+    constexpr int fit = (int)((227 * 1024) / (smem + 1024));
+    constexpr int per_sm = fit < 1 ? 1 : (fit > 4 ? 4 : fit);
     const long long ntiles = (long long)B * H * ((W + TC_M - 1) / TC_M);
     long long blocks = (long long)per_sm * sm_count_current();
     if (blocks > ntiles) blocks = ntiles;
