@@ -1,10 +1,13 @@
 """Autotuner for the launch choices of the TV library.
 
 Two choices are measured on the running GPU and applied through the C ABI:
-  * the largest batch of chains solved with one warp per chain (latency-bound
-    batches) rather than one thread per chain (throughput-bound batches): the
-    crossover is timed on uniform batches of 256- and 1024-node chains;
-  * the warps per block of the persistent kernels of the batched 2D solver.
+  * the largest batch of chains solved with warps per chain (latency-bound batches)
+    rather than one thread per chain (throughput-bound batches). The library's own
+    limits go with the chain length, the layout and the weights; one number for every
+    batch, the crossover timed on uniform batches of 256- and 1024-node chains, takes
+    their place only where it is the faster choice over batches of all kinds;
+  * the warps per block of the batched 2D solver's persistent kernels, which run images
+    with a side above 4096 pixels (others are on the splitting kernel).
 Results are cached as JSON keyed by the GPU name and library version, in
 ``$TV_AUTOTUNE_CACHE`` or ``~/.cache/tv_gb300/autotune.json``.
 """
@@ -22,6 +25,8 @@ BATCHES = (512, 1024, 2048, 4096, 8192)
 LENGTHS = (256, 1024)
 FORCE_COOP = 1 << 40
 FORCE_THREAD = 1
+# a GPU keeps the library's limits unless one crossover beats them by more than this
+MARGIN = 0.02
 
 
 def cache_path() -> str:
@@ -65,6 +70,40 @@ def choose_crossover(timings):
     return best
 
 
+def keep_limits(own, crossover):
+    """Whether the library's own limits stay: times of the same batches with them and with one
+    crossover, compared by their geometric means."""
+    ratio = np.exp(np.mean(np.log(np.asarray(own, float) / np.asarray(crossover, float))))
+    return bool(ratio <= 1.0 / (1.0 - MARGIN))
+
+
+def _mixed_batches(dev):
+    """Batches of every kind around the library's limits, as calls."""
+    import torch
+    rng = np.random.default_rng(7)
+
+    def rows(chains, n, edges):
+        y = torch.from_numpy(np.tile(synth.chain_batch(50, n, seed0=n), (-(-chains // 50), 1))[:chains]).to(dev)
+        w = torch.full_like(y, 0.15) if edges else None
+        x = torch.empty_like(y)
+        return lambda: _lib.chain_prox(y, w=w, lam=0.15, out=x)
+
+    def columns(n, chains):
+        y = torch.from_numpy(np.tile(synth.chain_batch(50, n, seed0=n), (chains // 50, 1)).T.copy()).to(dev)
+        x = torch.empty_like(y)
+        return lambda: _lib.chain_prox_columns(y, lam=0.15, out=x)
+
+    def ragged(chains, longest):
+        off = np.r_[0, np.cumsum(rng.integers(1, longest + 1, chains))]
+        y = torch.from_numpy(np.resize(synth.chain_batch(50, 4096, seed0=3), off[-1])).to(dev)
+        w, o = torch.full_like(y, 0.15), torch.from_numpy(off).to(dev)
+        x = torch.empty_like(y)
+        return lambda: _lib.chain_prox(y, w=w, offsets=o, max_len=longest, out=x)
+
+    return [rows(512, 256, False), rows(4096, 1024, False), rows(16384, 512, False), rows(4096, 1023, True),
+            rows(8192, 385, True), columns(512, 8000), ragged(6000, 2500), ragged(20000, 200)]
+
+
 def measure(device=0):
     import torch
     dev = torch.device("cuda", device)
@@ -81,8 +120,13 @@ def measure(device=0):
             timings[(B, n)] = tuple(res)
     _lib.set_coop_max_chains(0)
     crossover = choose_crossover(timings)
-    # warps per block of the batched solver, on a small uneven batch
-    sizes, lams = synth.uneven_image_sizes(6, seed=5, w_range=(128, 768), h_range=(96, 576))
+    batches = _mixed_batches(dev)
+    own = [_time_ms(fn) for fn in batches]
+    _lib.set_coop_max_chains(max(crossover, 1))
+    single = [_time_ms(fn) for fn in batches]
+    _lib.set_coop_max_chains(0)
+    # warps per block of the batched solver, on a small uneven batch of wide images
+    sizes, lams = synth.uneven_image_sizes(6, seed=5, w_range=(4100, 4600), h_range=(32, 128))
     imgs = [torch.from_numpy(synth.shapes_image(h, w, seed=200 + i, n_shapes=40)[1]).to(dev)
             for i, (h, w) in enumerate(sizes)]
     wpb_ms = {}
@@ -92,12 +136,14 @@ def measure(device=0):
                                                                  tol=1e-4), reps=3, warm=1)
     best_wpb = min(wpb_ms, key=wpb_ms.get)
     return {"coop_max_chains": int(max(crossover, 1)), "batched_warps": int(best_wpb),
+            "keep_limits": keep_limits(own, single),
+            "mixed_ms": {"own_limits": own, "coop_max_chains": single},
             "chain_timings_ms": {f"{b}x{n}": list(v) for (b, n), v in timings.items()},
             "batched_warps_ms": {str(k): v for k, v in wpb_ms.items()}}
 
 
 def apply(params):
-    _lib.set_coop_max_chains(int(params["coop_max_chains"]))
+    _lib.set_coop_max_chains(0 if params.get("keep_limits") else int(params["coop_max_chains"]))
     _lib.set_batched_warps(int(params["batched_warps"]))
 
 

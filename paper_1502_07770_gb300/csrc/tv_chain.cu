@@ -659,7 +659,7 @@ extern "C" {
 
 const char *tv_last_error(void) { return tvh::g_err; }
 
-int tv_version(void) { return 100; }
+int tv_version(void) { return 101; }  // 0.1.1
 
 int64_t tv_launch_count(void) { return (int64_t)tvh::g_launches.load(); }
 
