@@ -849,13 +849,11 @@ tv_status tv2d_denoise(const float *d_img, int64_t H, int64_t W, const float *d_
               : launch_init<false>(d_img, d_wh, lambda, H, W, d_x, ws, s);
     if (st != TV_OK) return st;
 
-    // Each iteration: column (dual) phase, row (primal) phase, gap. Iterations are
-    // launched in small batches (4, then 2 at a time); the device stop flag turns the
-    // rest of a batch into immediate returns, and the host checks it once per batch.
-    // Iterations go out in batches, each followed by the conditional result copy and one
-    // read of the device state (the only host synchronisation): a first batch of 6 (the
-    // usual iteration count of 1e-4 solves is 3 to 7; iterations launched after
-    // convergence return at once), then batches of 3.
+    // Each iteration: column (dual) phase, row (primal) phase, gap. Iterations go out in
+    // batches, each followed by the conditional result copy and one read of the device state
+    // (the only host synchronisation): a first batch of 6 (the usual iteration count of 1e-4
+    // solves is 3 to 7; the device stop flag turns iterations launched after convergence into
+    // immediate returns), then batches of 3.
     const long long N = H * W;
     const int copy_blocks = (int)std::min<long long>((N / 4 + 255) / 256 + 1, 4LL * sm_count_current());
     auto launch_copy = [&]() -> tv_status {

@@ -131,9 +131,10 @@ tv_status launch_coop(const P &p, long long nchains, int max_len, float2 *rec, f
     return st;
 }
 
-// Batches of fewer chains than this run one warp per chain (the update of one
-// chain is then latency-bound, and a warp shortens its critical path); larger
-// batches run one thread per chain.
+// Chains that the splitting kernel does not take (tv_split_launch.h: TV-l2 chains of 2 to 4096
+// nodes in the default solve mode, up to a batch size of its own): batches of up to this many run
+// one warp per chain by the dynamic program (the update of one chain is then latency-bound, and a
+// warp shortens its critical path); larger ones run one thread per chain or chain half.
 constexpr long long kCoopMaxChainsDefault = 4096;
 // The same for tv_chain_solve batches that the fixed-shape thread kernel stages 16 bytes
 // at a time (uniform rows of >= 64 nodes, a multiple of 4, 16-byte aligned arrays):
