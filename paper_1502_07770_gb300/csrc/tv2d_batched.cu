@@ -6,7 +6,7 @@
 // phase of an iteration goes over the chains of all images still running, longest
 // first. With every side up to 4096 pixels that is one launch of the threshold-splitting
 // kernel per number of warps a chain takes (tv_split.cuh; a block takes neighbouring rows
-// or columns of one image): 64 uneven images with weights per edge 16.0 ms, against 23.4 on
+// or columns of one image): 64 uneven images with weights per edge 16.2 ms, against 23.4 on
 // the lockstep halves. Otherwise it is ONE launch, for small batches persistent with warps
 // taking chains (one warp per chain, tv_coop.cuh) from an atomic work counter, for larger
 // ones a thread per chain half (tv_halves.cuh). A gap launch tiles all images; the

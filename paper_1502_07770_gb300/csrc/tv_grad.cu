@@ -13,13 +13,14 @@
 // copies x_{i+1} into x_i whenever the clip is inactive, so fused neighbours are
 // bitwise equal.
 //
-// Chains of at most kSplitMaxLen nodes (run_means_kernel; not large batches of short ones): the chain lies in the registers of
-// one warp (2 or 4 for more than 1024 nodes), L consecutive nodes a lane, loaded and stored
-// through padded slots in shared memory so that global accesses are whole lines. Run sums are
-// walks that restart behind a run's last node, joined across lanes by one segmented scan
-// (as the sums of tv_split.cuh), so that a node costs about 25 instructions and the two reads
-// and one or two writes bound the kernel. 4096 x 1024 with both gradients: 31 -> 14.7 us (4.6
-// TB/s) against the step-wise kernel; 16384 x 1024 50.6 us (5.3 TB/s).
+// Chains of at most kSplitMaxLen nodes (run_means_kernel; not large batches of short ones): the
+// chain lies in the shared memory of one warp (2 or 4 for more than 1024 nodes), L consecutive
+// nodes a lane in padded slots, through which global accesses are whole lines. Run sums are walks
+// that restart behind a run's last node, joined across lanes by one segmented scan (join_runs of
+// tv_split.cuh), and are carried in two floats. The two reads and one or two writes bound the
+// kernel from about 16384 chains on, before that the walks' latency. 4096 x 1024 with both
+// gradients: 31 -> 14.4 us against the step-wise kernel (back to back; 16.2 with the walks
+// unrolled over the chain in registers); 16384 x 1024 55 us (4.9 TB/s).
 //
 // Others (chain_vjp_kernel): one warp per chain, 32 nodes per step: a forward segmented
 // scan of (sum, count) with a carry across steps yields each segment's mean at its last node;
@@ -233,77 +234,81 @@ __device__ __forceinline__ void run_means(const GradArgs &a, long long start, in
         }
     }
     sync();
-    // node j of the lane is bit L-1-j: C the runs' last nodes, UP where the solution rises
-    float y[L];
-    bool cut[L];
-    unsigned C = 0, UP = 0;
-    const int last = n - 1 - ll * L;
-    {
-        float xv = sx[ll * LP];
-#pragma unroll
-        for (int j = 0; j < L; ++j) {
-            float xn = 0.f;
-            if (j + 1 < L) xn = sx[ll * LP + j + 1];
-            else if (ll + 1 < T) xn = sx[(ll + 1) * LP];
-            cut[j] = j >= last || xv != xn;
-            C = C << 1 | (cut[j] ? 1u : 0u);
-            UP = UP << 1 | (xn > xv ? 1u : 0u);
-            y[j] = sg[ll * LP + j];
-            xv = xn;
-        }
-    }
-    sync();  // the slots are written below
     // One walk from the right, restarting at cuts (selected, not multiplied by 0: an infinite or
     // NaN gradient stays in its own run), gives the sum to the lane's first cut, the one after
     // its last cut, and the means of the runs that lie in the lane, at their first nodes. Sums
     // are carried in two floats: node after node in one float a mean was off by a third more
-    // than from the step-wise kernel's tree of sums.
+    // than from the step-wise kernel's tree of sums. (Loops of four nodes, the values in shared
+    // memory: unrolled, the code that runs once per chain took longer to fetch than to run.)
+    // node j of the lane is bit L-1-j: C the runs' last nodes, UP where the solution rises
+    float4 *xs = reinterpret_cast<float4 *>(sx + ll * LP), *gs = reinterpret_cast<float4 *>(sg + ll * LP);
+    const int last = n - 1 - ll * L;
     const Sum2 zero{0.f, 0.f};
     Sum2 Sh = zero, St = zero;
-    float m[L];
-    {
-        float k = 0.f;
+    float k = 0.f;
+    bool open = true;  // no cut at or after the node
+    unsigned C = 0, UP = 0;
+    float xn = ll + 1 < T ? sx[(ll + 1) * LP] : 0.f;
+#pragma unroll 1
+    for (int q = L / 4 - 1; q >= 0; --q) {
+        const float4 xq = xs[q], gq = gs[q];
+        const float xv[4] = {xq.x, xq.y, xq.z, xq.w}, g4[4] = {gq.x, gq.y, gq.z, gq.w};
+        float m[4];
+        unsigned c4 = 0, u4 = 0;
 #pragma unroll
-        for (int j = L - 1; j >= 0; --j) {
-            Sh = pick(cut[j], zero, Sh) + Sum2{y[j], 0.f};
-            k = cut[j] ? 1.f : k + 1.f;
-            m[j] = run_mean(Sh, k);
-            if ((C & ((2u << (L - 1 - j)) - 1u)) == 0) St = Sh;
+        for (int e = 3; e >= 0; --e) {
+            const bool cut = 4 * q + e >= last || xv[e] != xn;
+            c4 |= cut ? 8u >> e : 0u;
+            u4 |= xn > xv[e] ? 8u >> e : 0u;
+            xn = xv[e];
+            Sh = pick(cut, zero, Sh) + g4[e];
+            k = cut ? 1.f : k + 1.f;
+            m[e] = run_mean(Sh, k);
+            open = open && !cut;
+            if (open) St = Sh;
         }
+        C |= c4 << (L - 4 - 4 * q);
+        UP |= u4 << (L - 4 - 4 * q);
+        gs[q] = make_float4(m[0], m[1], m[2], m[3]);
     }
     const unsigned bc = __ballot_sync(FULL, C != 0);
     const RunEnds<Sum2> run = join_runs<L, W>(Sh, St, C, bc, lane, wi, &xc->run, run_mean, sync);
     float zr = run.zr;
-    const unsigned LC = C & (0u - C);
-#pragma unroll
-    for (int j = 0; j < L; ++j) {
-        if (j > 0 && cut[j > 0 ? j - 1 : 0]) zr = m[j];
-        if (j > 0 && (LC & (1u << (L - j)))) zr = run.zt;
-        m[j] = zr;
-    }
-#pragma unroll
-    for (int q = 0; q < L / 4; ++q)
-        *reinterpret_cast<float4 *>(sg + ll * LP + 4 * q) =
-            make_float4(m[4 * q], m[4 * q + 1], m[4 * q + 2], m[4 * q + 3]);
+    float zn = 0.f;  // mean of the node after the lane's last
     if (a.gw) {
-        float zn = __shfl_down_sync(FULL, m[0], 1);  // mean of the node after the lane's last
+        zn = __shfl_down_sync(FULL, zr, 1);
         if constexpr (W > 1) {
-            if (lane == 0) xc->z[wi] = m[0];
-            __syncthreads();
+            if (lane == 0) xc->z[wi] = zr;
+        }
+        sync();  // every lane has read its neighbour's x, and the warps' first means are there
+        if constexpr (W > 1) {
             if (lane == WARP - 1) zn = wi + 1 < W ? xc->z[wi + 1 < W ? wi + 1 : 0] : 0.f;
         }
-        // a jump edge: sign * (mean left - mean right); fused edges: 0
+    }
+    const unsigned LC = C & (0u - C);
+#pragma unroll 1
+    for (int q = 0; q < L / 4; ++q) {
+        const int s4 = L - 4 - 4 * q;
+        const unsigned c4 = C >> s4, l4 = LC >> s4, u4 = UP >> s4;
+        const float4 t = gs[q];
+        float v[5] = {t.x, t.y, t.z, t.w, zn};
 #pragma unroll
-        for (int q = 0; q < L / 4; ++q) {
-            float v[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int j = 4 * q + e;
-                const float d = m[j] - (j + 1 < L ? m[j + 1 < L ? j + 1 : 0] : zn);
-                v[e] = !cut[j] || j >= last ? 0.f : ((UP & (1u << (L - 1 - j))) ? d : -d);
-            }
-            *reinterpret_cast<float4 *>(sx + ll * LP + 4 * q) = make_float4(v[0], v[1], v[2], v[3]);
+        for (int e = 0; e < 4; ++e) {
+            if (c4 & (16u >> e)) zr = v[e];    // a run begins
+            if (l4 & (16u >> e)) zr = run.zt;  // the bits other lanes have
+            v[e] = zr;
         }
+        gs[q] = make_float4(v[0], v[1], v[2], v[3]);
+        if (!a.gw) continue;
+        if (q + 1 < L / 4) v[4] = (l4 & 1u) ? run.zt : (c4 & 1u) ? gs[q + 1].x : zr;
+        float d[4];  // a jump edge: sign * (mean left - mean right); fused edges: 0
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const unsigned bit = 8u >> e;
+            const float h = v[e] - v[e + 1];
+            d[e] = !(c4 & bit) || 4 * q + e >= last ? 0.f : (u4 & bit) ? h : -h;
+        }
+        xs[q] = make_float4(d[0], d[1], d[2], d[3]);
     }
     sync();
     float *gy = a.gy + start, *gw = a.gw ? a.gw + start : nullptr;

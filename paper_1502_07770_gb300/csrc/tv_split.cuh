@@ -20,7 +20,7 @@
 // warp scan (across W warps: a shared-memory exchange) gives each lane its incoming m, a
 // second walk gives the sides as two bit masks, and the undecided bits are filled from the
 // right by one carry-propagating addition. The mean of every run comes from a walk from the
-// right and a segmented scan over the lanes. Cut flows are folded into the values at the cut
+// right and a segmented scan over the lanes (join_runs). Cut flows are folded into the values at the cut
 // (y_i += u, y_{i+1} -= u, w_i = 0), after which a cut needs no special case.
 //
 // Solutions are sums of the values of a run over its length: all nodes of a run are bitwise
@@ -162,6 +162,11 @@ __device__ __forceinline__ Sum2 operator+(Sum2 a, Sum2 b)
 {
     const float t = a.hi + b.hi, u = t - a.hi;
     return Sum2{t, ((a.hi - (t - u)) + (b.hi - u)) + (a.lo + b.lo)};
+}
+__device__ __forceinline__ Sum2 operator+(Sum2 a, float b)
+{
+    const float t = a.hi + b, u = t - a.hi;
+    return Sum2{t, ((a.hi - (t - u)) + (b - u)) + a.lo};
 }
 __device__ __forceinline__ Sum2 pick(bool c, Sum2 a, Sum2 b)
 {
@@ -678,61 +683,73 @@ __device__ __forceinline__ int split_solve(const float *sc, float *sx, SplitX<W>
     }
 
     // ---- values of the runs: sums in two floats (in one, x was further off than the dynamic
-    // program's: 4.7e-8 against 3.2e-8 for 512 x 256, now 2.3e-8) ----
-    {
-        if constexpr (UNI) {  // of the values as they came, with the flows of all cuts
-            const unsigned ends = last >= L ? 0u : ML >> max(0, min(31, last));
-            const unsigned F = C & ~ends;  // cuts that carry a flow
-            float u = (F & 1u) ? ((UP & 1u) ? lamw : -lamw) : 0.f;
-            float ul = __shfl_up_sync(FULL, u, 1);
-            if (lane == 0) ul = 0.f;
-            if constexpr (W > 1) {
-                if (lane == WARP - 1) xc->u2[wi] = u;
-                sync();
-                if (lane == 0 && wi > 0) ul = xc->u2[wi - 1];
-            }
-#pragma unroll
-            for (int q = 0; q < L / 4; ++q) {
-                const float4 t = yp[q];
-                const float v[4] = {t.x, t.y, t.z, t.w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const unsigned bit = 1u << (L - 1 - (4 * q + e));
-                    u = (F & bit) ? ((UP & bit) ? lamw : -lamw) : 0.f;
-                    y[4 * q + e] = v[e] + (u - ul);  // equal flows cancel exactly
-                    ul = u;
-                }
-            }
+    // program's: 4.7e-8 against 3.2e-8 for 512 x 256, now 2.3e-8). Loops of four nodes, the values
+    // in shared memory: unrolled like the rounds this was 16 KB of code that runs once (1024 x 1024
+    // with cold caches 30 us, now 26; 4096 x 1023 with weights per edge 65 us, now 62) ----
+    float4 *slots = reinterpret_cast<float4 *>(sx + (wi * WARP + lane) * LP);
+    unsigned F = 0;  // UNI: cuts that carry a flow; the values as they came, with the flows of all cuts
+    float ul = 0.f;  // flow of the cut before the lane's first node
+    if constexpr (UNI) {
+        const unsigned ends = last >= L ? 0u : ML >> max(0, min(31, last));
+        F = C & ~ends;
+        const float u = (F & 1u) ? ((UP & 1u) ? lamw : -lamw) : 0.f;
+        ul = __shfl_up_sync(FULL, u, 1);
+        if (lane == 0) ul = 0.f;
+        if constexpr (W > 1) {
+            if (lane == WARP - 1) xc->u2[wi] = u;
+            sync();
+            if (lane == 0 && wi > 0) ul = xc->u2[wi - 1];
         }
-        Sum2 Sh{0.f, 0.f}, St{0.f, 0.f};
-        float k = 0.f, b = 1.f;
+    } else {
 #pragma unroll
-        for (int j = L - 1; j >= 0; --j) {
-            const float rj = keep(j);
-            const Sum2 before{Sh.hi * rj, Sh.lo * rj};
-            Sh = before + Sum2{y[j], 0.f};
-            k = fmaf(k, rj, 1.f);
-            z[j] = mean_of(Sh, k);  // of a run that ends in the lane
-            b *= rj;
-            St = pick(b != 0.f, Sh, St);
-        }
-        const RunEnds<Sum2> run = join_runs<L, W>(
-            Sh, St, C, bc, lane, wi, &xc->sum, [](Sum2 s, float n) { return mean_of(s, n); }, sync);
-        float zr = run.zr;
-        const unsigned LC = C & (0u - C);
-        float4 *xp = reinterpret_cast<float4 *>(sx + (wi * WARP + lane) * LP);
+        for (int q = 0; q < L / 4; ++q)
+            slots[q] = make_float4(y[4 * q], y[4 * q + 1], y[4 * q + 2], y[4 * q + 3]);
+    }
+    Sum2 Sh{0.f, 0.f}, St{0.f, 0.f};
+    float k = 0.f;
+    bool open = true;  // no cut at or after the node
+#pragma unroll 1
+    for (int q = L / 4 - 1; q >= 0; --q) {
+        const int s4 = L - 4 - 4 * q;  // node 4 q + e is bit 3 - e
+        const unsigned c4 = C >> s4, f4 = F >> s4, p4 = UP >> s4;
+        const float4 t = UNI ? yp[q] : slots[q];
+        const float v[4] = {t.x, t.y, t.z, t.w};
+        float m[4], u = 0.f;
+        auto flow = [&](unsigned bit) { return (f4 & bit) ? ((p4 & bit) ? lamw : -lamw) : 0.f; };
+        if constexpr (UNI) u = flow(1u);
 #pragma unroll
-        for (int q = 0; q < L / 4; ++q) {
-            float v[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int j = 4 * q + e;
-                if (j > 0 && (C & (1u << (L - j)))) zr = z[j];
-                if (j > 0 && (LC & (1u << (L - j)))) zr = run.zt;  // the bits other lanes have
-                v[e] = zr;
+        for (int e = 3; e >= 0; --e) {
+            float c = v[e];
+            if constexpr (UNI) {
+                const float before = e == 0 && q == 0 ? ul : flow(16u >> e);
+                c += u - before;  // equal flows cancel exactly
+                u = before;
             }
-            xp[q] = make_float4(v[0], v[1], v[2], v[3]);
+            const bool cut = c4 & (8u >> e);
+            Sh = pick(cut, Sum2{0.f, 0.f}, Sh) + c;
+            k = cut ? 1.f : k + 1.f;
+            m[e] = mean_of(Sh, k);  // of a run that ends in the lane
+            open = open && !cut;
+            if (open) St = Sh;
         }
+        slots[q] = make_float4(m[0], m[1], m[2], m[3]);
+    }
+    const RunEnds<Sum2> run = join_runs<L, W>(
+        Sh, St, C, bc, lane, wi, &xc->sum, [](Sum2 a, float n) { return mean_of(a, n); }, sync);
+    float zr = run.zr;
+    const unsigned LC = C & (0u - C);
+#pragma unroll 1
+    for (int q = 0; q < L / 4; ++q) {
+        const unsigned c4 = C >> (L - 4 - 4 * q), l4 = LC >> (L - 4 - 4 * q);
+        const float4 t = slots[q];
+        float v[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if (c4 & (16u >> e)) zr = v[e];    // a run begins
+            if (l4 & (16u >> e)) zr = run.zt;  // the bits other lanes have
+            v[e] = zr;
+        }
+        slots[q] = make_float4(v[0], v[1], v[2], v[3]);
     }
     return SPLIT_DONE;
 }
