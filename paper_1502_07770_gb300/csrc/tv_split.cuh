@@ -20,14 +20,14 @@
 // warp scan (across W warps: a shared-memory exchange) gives each lane its incoming m, a
 // second walk gives the sides as two bit masks, and the undecided bits are filled from the
 // right by one carry-propagating addition. The mean of every run comes from a walk from the
-// right and a segmented scan over the lanes (join_runs). Cut flows are folded into the values at the cut
-// (y_i += u, y_{i+1} -= u, w_i = 0), after which a cut needs no special case.
+// right and a segmented scan over the lanes (join_runs). Cut flows are folded into the values at
+// the cut (y_i += u, y_{i+1} -= u, w_i = 0), after which a cut needs no special case.
 //
 // Solutions are sums of the values of a run over its length: all nodes of a run are bitwise
 // equal, and the rounding is that of one mean. The folded flows cost eps * |u| per run, so a
 // chain that is to be cut at a flow above 16 max |y|, that has a NaN weight, or whose values are
-// not finite or near the ends of FP32's range, goes to the warp's dynamic program (coop_solve_chain, records and reserve
-// in the workspace) instead.
+// not finite or near the ends of FP32's range, goes to the warp's dynamic program
+// (coop_solve_chain, records and reserve in the workspace) instead.
 #pragma once
 #include "tv2d_common.cuh"
 #include "tv2d_gap.cuh"
