@@ -395,9 +395,10 @@ tv_status tv_set_batched_graph(int on);
  * of 64 to 4096 nodes in the default solve mode (tv_set_coop_split) those follow the chain
  * length, the staging and the weights (the thread kernels are the faster ones beyond 2048 to
  * 8192 chains of uniform rows of a multiple of 4 nodes with 16-byte aligned arrays, beyond
- * 4096 to 30000 of CSR batches, later or never for others); otherwise 4096 chains, and 2048 for tv_chain_solve batches of such rows.
- * A value set here applies to every batch. (The autotuner sets one only where that is faster
- * than the defaults; the warps per block concern images with a side above 4096.)
+ * 4096 to 30000 of CSR batches, later or never for others); otherwise 4096 chains, and 2048
+ * for tv_chain_solve batches of such rows. A value set here applies to every batch. (The
+ * autotuner sets one only where that is faster than the defaults; the warps per block concern
+ * images with a side above 4096.)
  */
 tv_status tv_set_batched_warps(int warps_per_block);
 tv_status tv_set_coop_max_chains(int64_t max_chains);

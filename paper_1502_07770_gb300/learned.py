@@ -337,9 +337,9 @@ def denoise_warm(net, f, lam: float, lam_t=None, tol=1e-4, max_iters=400, first_
     thus costs at most two short runs of ``first_check`` iterations. ``lam_t``: the same
     lambda as a (1,) CUDA tensor (made here if None).
 
-    Whether it pays is the caller's choice: on a GB300 24 images of 512 x 512 take 0.287 ms
-    warm against 0.321 from y^0 = 0, one of 1024 x 1024 0.357 against 0.337 (the network's
-    0.107 ms are more than the two iterations that it saves).
+    Whether it pays is the caller's choice: on a GB300 an image of 512 x 512 takes 0.287 ms
+    warm against 0.321 from y^0 = 0 (means of 24), one of 1024 x 1024 0.357 against 0.337
+    (the network's 0.107 ms are more than the two iterations that it saves).
 
     Returns (x, outer iterations of every run, gap, converged, used_fallback)."""
     if lam_t is None:

@@ -46,10 +46,11 @@ def test_runs_are_bitwise_equal(n, edges):
 
 
 @pytest.mark.parametrize("edges", [False, True])
-@pytest.mark.parametrize("shape", [(12, 4500), (4500, 12), (4097, 33), (33, 4097)])
-def test_images_with_one_side_beyond_the_longest_chain(shape, edges):
-    """One direction on the splitting kernel, the other on the warp- or thread-per-chain phases,
-    the step counter advanced by the gap pass and the row phase."""
+@pytest.mark.parametrize("shape", [(300, 4500), (4500, 300), (70, 4097), (4097, 70), (16, 3000), (12, 4500)])
+def test_images_with_one_direction_on_the_splitting_kernel(shape, edges):
+    """Rows or columns beyond 4096 nodes, or too many short columns, on the warp- or
+    thread-per-chain phases and the other direction on the splitting kernel, the step counter
+    advanced by the gap pass and the row phase; both on the old phases (12 x 4500)."""
     f = synth.shapes_image(*shape, seed=sum(shape), n_shapes=60)[1]
     wh, wv = synth.edge_aware_weights(f, 0.2) if edges else (None, None)
     for iters, tol in ((60, 1e-4), (7, 0.0)):
