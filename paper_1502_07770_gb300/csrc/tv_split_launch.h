@@ -47,9 +47,13 @@ inline bool split_takes(long long max_len, long long chains, long long max_chain
 //  - columns (the thread kernel runs one thread per chain): at 1024 nodes 57 / 889 for 4096 and
 //    650 / 1119 for 65536, at 300 nodes 180 / 258 for 40000 and 638 / 554 for 150000, at 100
 //    nodes 56 / 93 for 16384 and 195 / 114 for 65536.
-// Chains of under 64 nodes leave most of a warp idle: at 16 nodes 16.6 / 14.7 (the
-// warp-per-chain kernel; columns 20.4 / 16.3) for 4096 chains, 13.7 / 13.8 for 2048. Up to 2048
-// chains the alternative is another warp-per-chain kernel, which is never faster.
+// Chains of under 64 nodes leave most of a warp idle. There, and up to 4096 chains otherwise, the
+// alternative is a warp per chain by the dynamic program, whose time goes with the length (us,
+// splitting / dynamic program, device time of a call): rows of 8 nodes 8.2 / 6.2 for 20 to 1000
+// chains and 14.4 / 8.4 for 4000, 16 nodes 8.3 / 8.2 and 14.4 / 12.3, 24 nodes 8.3 / 9.0 and
+// 14.7 / 16.4, 63 nodes 9.0 / 16.4 and 16.4 / 33.0; columns of 16 nodes 8.2 / 6.4 and 16.3 / 11.2, 24
+// nodes 8.3 / 8.2 and 16.4 / 14.4, 32 nodes 8.5 / 8.4 and 16.4 / 17.6, 63 nodes 8.3 / 12.4 and
+// 17.1 / 30.7.
 //
 // CSR batches (`csr`; `len` is their longest chain): a short chain still takes its warps, and one
 // of more than 256 nodes is solved at the longest chain's nodes a lane, while the thread kernels
@@ -70,7 +74,7 @@ inline long long split_max_chains(long long len, bool cols, bool vec, bool has_w
         if (has_w) return len <= 256 ? 120 * len : std::min(47 * len, 22000LL);
         return std::max(4096LL, len <= 256 ? 23 * len : len <= 1024 ? 9 * len : std::min(2 * len + 7000, 13500LL));
     }
-    if (len < 64) return len < 32 ? 2048 : kCoopMaxChainsDefault;
+    if (len < 64) return len < (cols ? 32 : 20) ? 0 : kCoopMaxChainsDefault;
     if (cols) return len < 256 ? 16384 : len < 512 ? 250 * len : INT64_MAX;
     if (vec) return std::max(2048LL, std::min(28 * len, has_w ? 6144LL : len < 512 ? 6800LL : 8192LL));
     if (has_w) return len < 384 ? 150 * len : INT64_MAX;

@@ -34,3 +34,28 @@ def test_route(cols, n, chains, edges, split):
         _lib.set_coop_max_chains(0)
     assert not torch.equal(forced["split"], forced["thread"])
     assert torch.equal(default, forced["split" if split else "thread"])
+
+
+@pytest.mark.parametrize("edges", [False, True])
+@pytest.mark.parametrize("cols,n,split", [(False, 8, False), (False, 19, False), (False, 20, True), (False, 40, True),
+                                          (True, 8, False), (True, 31, False), (True, 32, True), (True, 48, True)])
+def test_short_chains(cols, n, split, edges):
+    """Short chains stay on the warp's dynamic program (below 64 nodes solve mode 0 is the
+    default's), which is the faster one for them."""
+    chains = 3000
+    g = torch.Generator(device=DEV).manual_seed(n)
+    shape = (n, chains) if cols else (chains, n)
+    y = torch.rand(shape, generator=g, device=DEV)
+    w = 0.1 * torch.rand(shape, generator=g, device=DEV) if edges else None
+    solve = _lib.chain_prox_columns if cols else _lib.chain_prox
+    default = solve(y, w, lam=0.07)
+    try:
+        _lib.set_coop_max_chains(1 << 40)
+        splitting = solve(y, w, lam=0.07)
+        _lib.set_coop_split(0)
+        program = solve(y, w, lam=0.07)
+    finally:
+        _lib.set_coop_max_chains(0)
+        _lib.set_coop_split(1)
+    assert not torch.equal(splitting, program)
+    assert torch.equal(default, splitting if split else program)
